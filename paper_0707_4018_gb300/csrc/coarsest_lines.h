@@ -1,0 +1,54 @@
+// Direct solve of a small periodic coarse stencil by cyclic reduction over lattice lines
+// (coarsest_lines.cu), with the dense LU of the same matrix behind it.
+#pragma once
+
+#include <vector>
+
+#include "common.cuh"
+
+namespace mg {
+
+// one level of the reduction: a ring of r lines of b dofs; line p couples to p +- 1 (mod r)
+struct LineLevel {
+  int r = 0, K = 0, E = 0;  // lines, kept (even positions), eliminated (odd positions)
+  Cx<double> *D = nullptr, *R = nullptr, *L = nullptr;        // [r] blocks: self, next, previous (r <= 2: R holds both)
+  Cx<double> *Dinv = nullptr, *WL = nullptr, *WR = nullptr;   // [E]: D^-1, D^-1 L, D^-1 R (r = 1: Dinv of the last line)
+  long long rhs = 0, y = 0, x = 0;                            // offsets of the level's vectors in the workspace
+  long long w_jobs = 0, u_jobs = 0;                           // first product of the level in the job list
+  int n_w = 0, n_u = 0;
+};
+
+// C = I1 + I2 + sgn (A1 B1 + A2 B2) on b x b row-major blocks (null terms left out)
+struct LineJob {
+  Cx<double> *C;
+  const Cx<double> *I1, *I2, *A1, *B1, *A2, *B2;
+  double sgn;
+};
+
+struct LineSolver {
+  int N = 0, L0 = 0, L1 = 0, n = 0;
+  int axis = 1, Q = 0, b = 0;  // line coordinate (1: lines along x0, one per x1), sites per line, dofs per line
+  bool lines = false;          // the factors in use: cyclic reduction, or the dense LU
+  bool planned = false;
+  std::vector<LineLevel> lv;
+  std::vector<LineJob> jobs;
+  DevBuf<Cx<double>> mem, tmp, pinv, chk;
+  DevBuf<LineJob> jobs_dev;
+  DevBuf<Cx<double>> LU;
+  DevBuf<int> ipiv, info;      // info[0]: singular pivot seen
+  DevBuf<double> berr;         // backward error of the check
+};
+
+// entries of the vector workspace that line_solve needs per right-hand side (shared between the
+// solvers of one lattice; at least n, for the dense path)
+long long line_work_size(Geo2 g, int N);
+// Factors the 5-point stencil Y[j][dir][col][row] + shift (nine = false) or the 9-point stencil
+// Y[j][o][row][col] (nine = true). work: workspace of one right-hand side. Synchronises s.
+// Returns true when the kind of factors changed (a graph captured with the old ones is stale);
+// fails with MG_ERR_NAN ("... zero pivot at column k") on a singular matrix.
+bool line_factor(LineSolver &f, const Cx<double> *Y, Geo2 g, int N, bool nine, double shift, Cx<double> *work,
+                 cudaStream_t s, const char *what);
+// x_v = A^{-1} b_v for nvec vectors of stride n (b and x may be equal); work: nvec workspaces
+void line_solve(const LineSolver &f, const Cx<double> *b, Cx<double> *x, int nvec, Cx<double> *work, cudaStream_t s);
+
+}  // namespace mg

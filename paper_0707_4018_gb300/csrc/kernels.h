@@ -218,6 +218,8 @@ void launch_gaussian(Cx<double> *out, long long n, unsigned long long seed, int 
 // ---- coarsest level: dense LU with partial pivoting, column-major ----
 // dense matrix of the stencil plus shift * identity
 void launch_dense_from_stencil(const Cx<double> *Y, Cx<double> *A, Geo2 g, int N, cudaStream_t s, double shift = 0.0);
+// the same for a 9-point stencil Y[j][o][row][col] (mgcg.cu)
+void launch_dense_from_stencil9(const Cx<double> *Y, Cx<double> *A, Geo2 g, int N, cudaStream_t s);
 // factor in place; ipiv[k] = pivot row of step k; info_dev[0] = 1 + first zero pivot (0 if none)
 void lu_factor(Cx<double> *A, int n, int *ipiv, int *info_dev, cudaStream_t s);
 // x = A^{-1} b with the factors; work: n entries, must alias neither b nor x (b may equal work)

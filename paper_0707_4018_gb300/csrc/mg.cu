@@ -21,6 +21,7 @@
 #include <thread>
 #include <vector>
 
+#include "coarsest_lines.h"
 #include "kernels.h"
 #include "mg4d.h"
 #include "nullnet.h"
@@ -117,8 +118,8 @@ struct mg_ctx {
   // coarsest
   bool use_lu = false;
   int nc = 0;
-  mg::DevBuf<mg::Cx<double>> LU, lu_work;
-  mg::DevBuf<int> ipiv, info;
+  mg::LineSolver lu;                           // exact coarsest solve at the context mass
+  mg::DevBuf<mg::Cx<double>> lu_work;          // nbatch workspaces
   mg::DevBuf<mg::Cx<double>> cZ, cW, cr, cb, cx;
   mg::DevBuf<double> cg_partials, cg_rel;
   mg::DevBuf<mg::Cx<double>> cg_Minv, cg_Yt, cg_work, cg_y;
@@ -147,8 +148,7 @@ struct mg_ctx {
   mg::DevBuf<double> shift_dev;
   std::vector<double> slot_shift;     // shift each slot was prepared for (NaN: not prepared)
   mg::DevBuf<mg::Cx<double>> bMinv, bYt;               // per slot (iterative coarsest)
-  std::vector<mg::DevBuf<mg::Cx<double>>> bLU;         // per slot (dense coarsest)
-  std::vector<mg::DevBuf<int>> bipiv;
+  std::vector<mg::LineSolver> blu;                     // per slot (exact coarsest)
   bool cg_batch = false;  // batched shared-memory coarsest kernel usable
   mg::DevBuf<mg::Cx<double>> cgb_u, cgb_x;
   mg::DevBuf<double> cgb_partials;
@@ -429,9 +429,7 @@ static void coarsest_solve64(mg_ctx &c, const Cx<double> *b, Cx<double> *x, int 
   const int l = c.p.levels - 1;
   const Level &L = c.lv[l];
   if (c.use_lu) {
-    const Cx<double> *LU = slot == 0 ? c.LU.p : c.bLU[slot - 1].p;
-    const int *piv = slot == 0 ? c.ipiv.p : c.bipiv[slot - 1].p;
-    lu_solve_ws(LU, piv, c.nc, b, x, c.lu_work.p, c.s);
+    line_solve(slot == 0 ? c.lu : c.blu[slot - 1], b, x, 1, c.lu_work.p, c.s);
     c.apps[l]++;
     return;
   }
@@ -466,6 +464,11 @@ static void coarsest_vectors64(mg_ctx &c, const Cx<double> *b, Cx<double> *x, in
   const Level &L = c.lv[l];
   const long long n = L.n;
   const bool batch = c.cur_shift != nullptr;
+  if (c.use_lu && !batch) {
+    line_solve(c.lu, b, x, nvec, c.lu_work.p, c.s);
+    c.apps[l] += nvec;
+    return;
+  }
   if (c.cg_cluster && nvec > 1 && !batch) {
     // every vector at the context mass: one cluster per vector, all in one launch
     launch_coarsest_gcr_cluster(c.cl_Yr.p, c.cg_Minv.p, L.geo, nvec, b, x, c.cl_rpub.p, c.cl_ypub.p,
@@ -631,6 +634,14 @@ static void precondition(mg_ctx &c, const Cx<double> *r, Cx<double> *z) {
 // batched solves: nb systems (D + shift_v) psi_v = chi_v sharing one hierarchy
 // ---------------------------------------------------------------------------
 
+// the captured V-cycles hold the launches of one kind of coarsest solve: dropped when it changes
+static void reset_graphs(mg_ctx &c) {
+  for (GraphCache &g : c.pre) g.reset();
+  for (auto &v : c.preb)
+    for (GraphCache &g : v) g.reset();
+  for (GraphCache &g : c.setup_vc) g.reset();
+}
+
 // coarsest slots 1..nb for the shifts (prepared again only when a shift changed)
 static void prepare_slots(mg_ctx &c, int nb, const double *shift) {
   Level &L = c.lv.back();
@@ -638,17 +649,9 @@ static void prepare_slots(mg_ctx &c, int nb, const double *shift) {
   for (int v = 0; v < nb; ++v) {
     if (c.slot_shift[v] == shift[v]) continue;
     if (c.use_lu) {
-      if (c.bLU[v].p == nullptr) {
-        c.bLU[v].alloc((size_t)c.nc * c.nc);
-        c.bipiv[v].alloc(c.nc);
-        pool_ready();
-      }
-      launch_dense_from_stencil(L.Y64.p, c.bLU[v].p, L.geo, L.nint, c.s, shift[v]);
-      lu_factor(c.bLU[v].p, c.nc, c.bipiv[v].p, c.info.p, c.s);
-      int info = 0;
-      MG_CUDA(cudaMemcpyAsync(&info, c.info.p, sizeof(int), cudaMemcpyDeviceToHost, c.s));
-      MG_CUDA(cudaStreamSynchronize(c.s));
-      if (info != 0) fail(MG_ERR_NAN, "coarsest LU (batched mass): zero pivot at column " + std::to_string(info - 1));
+      if (line_factor(c.blu[v], L.Y64.p, L.geo, L.nint, false, shift[v], c.lu_work.p, c.s,
+                      "coarsest LU (batched mass)"))
+        reset_graphs(c);
     } else {
       prepare_coarsest_gcr(L.Y64.p, L.geo, L.nint, c.bMinv.p + v * m2, c.cg_batch ? nullptr : c.bYt.p + v * 5 * m2,
                            c.cg_work.p, c.cg_info.p, c.s, shift[v]);
@@ -1115,12 +1118,7 @@ static void prepare_coarsest(mg_ctx &c) {
     if (info != 0) fail(MG_ERR_NAN, "coarsest level: a self block is singular");
     return;
   }
-  launch_dense_from_stencil(L.Y64.p, c.LU.p, L.geo, L.nint, c.s);
-  lu_factor(c.LU.p, c.nc, c.ipiv.p, c.info.p, c.s);
-  int info = 0;
-  MG_CUDA(cudaMemcpyAsync(&info, c.info.p, sizeof(int), cudaMemcpyDeviceToHost, c.s));
-  MG_CUDA(cudaStreamSynchronize(c.s));
-  if (info != 0) fail(MG_ERR_NAN, "coarsest LU: zero pivot at column " + std::to_string(info - 1));
+  if (line_factor(c.lu, L.Y64.p, L.geo, L.nint, false, 0.0, c.lu_work.p, c.s, "coarsest LU")) reset_graphs(c);
 }
 
 // block Gram-Schmidt of the level's vectors and the Galerkin operator of l+1
@@ -1267,8 +1265,7 @@ static void alloc_batch(mg_ctx &c) {
   const size_t nr = (size_t)c.p.max_rhs;
   const size_t m2 = (size_t)Cst.geo.nsites * Cst.nint * Cst.nint;
   if (c.use_lu) {
-    c.bLU.resize(nr);
-    c.bipiv.resize(nr);
+    c.blu.resize(nr);
   } else {
     c.bMinv.alloc(nr * m2);
     if (!c.cg_batch) c.bYt.alloc(nr * 5 * m2);
@@ -1387,10 +1384,7 @@ static std::unique_ptr<mg_ctx> create(const mg_geom *g, double m, const mg_param
   c->nc = (int)Cst.n;
   c->use_lu = Cst.n <= p->coarsest_lu_max;
   if (c->use_lu) {
-    c->LU.alloc((size_t)Cst.n * Cst.n);
-    c->lu_work.alloc(Cst.n);
-    c->ipiv.alloc(Cst.n);
-    c->info.alloc(1);
+    c->lu_work.alloc((size_t)c->nbatch * line_work_size(Cst.geo, Cst.nint));
   } else {
     c->cZ.alloc((size_t)p->coarsest_restart * Cst.n);
     c->cW.alloc((size_t)p->coarsest_restart * Cst.n);

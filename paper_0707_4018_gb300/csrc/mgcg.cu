@@ -18,6 +18,7 @@
 #include <memory>
 #include <vector>
 
+#include "coarsest_lines.h"
 #include "kernels.h"
 
 namespace mg {
@@ -141,6 +142,12 @@ unsigned int blocks_for(long long n) {
 
 }  // namespace
 
+void launch_dense_from_stencil9(const Cx<double> *Y, Cx<double> *A, Geo2 g, int N, cudaStream_t s) {
+  const long long n = g.nsites * N;
+  dense_from_stencil9_kernel<<<grid_for(n * n, 256), 256, 0, s>>>(Y, A, g.L0, g.L1, N);
+  MG_LAUNCHED();
+}
+
 // ---------------------------------------------------------------------------
 // the engine
 // ---------------------------------------------------------------------------
@@ -166,8 +173,8 @@ struct CgEngine {
   cudaEvent_t ev = nullptr;
   DevBuf<Cx<double>> U, tmp;  // links; fine scratch of the D^dagger D apply
   std::vector<CgLevel> lv;
-  DevBuf<Cx<double>> LU, lu_work;
-  DevBuf<int> ipiv, info;
+  LineSolver coarsest;
+  DevBuf<Cx<double>> lu_work;
   DevBuf<double> partials, mgs_min, dots;
   DevBuf<unsigned int> tickets;
   ReduceWs ws{};
@@ -236,7 +243,7 @@ static void frozen_smooth(CgEngine &e, int l, const Cx<double> *b, Cx<double> *x
 static void cg_vcycle(CgEngine &e, int l, const Cx<double> *b, Cx<double> *x) {
   CgLevel &L = e.lv[l];
   if (l + 1 == (int)e.lv.size()) {
-    lu_solve_ws(e.LU.p, e.ipiv.p, (int)L.n, b, x, e.lu_work.p, e.s);
+    line_solve(e.coarsest, b, x, 1, e.lu_work.p, e.s);
     return;
   }
   CgLevel &C = e.lv[l + 1];
@@ -312,15 +319,7 @@ static void cg_prepare(CgEngine &e) {
     }
   }
   CgLevel &C = e.lv.back();
-  const int n = (int)C.n;
-  dense_from_stencil9_kernel<<<grid_for((long long)n * n, 256), 256, 0, e.s>>>(C.Y.p, e.LU.p, C.geo.L0, C.geo.L1,
-                                                                              C.nint);
-  MG_LAUNCHED();
-  lu_factor(e.LU.p, n, e.ipiv.p, e.info.p, e.s);
-  int info = 0;
-  MG_CUDA(cudaMemcpyAsync(&info, e.info.p, sizeof(int), cudaMemcpyDeviceToHost, e.s));
-  MG_CUDA(cudaStreamSynchronize(e.s));
-  if (info != 0) fail(MG_ERR_NAN, "MG-CG: coarsest LU hit a zero pivot");
+  line_factor(e.coarsest, C.Y.p, C.geo, C.nint, true, 0.0, e.lu_work.p, e.s, "MG-CG: coarsest LU");
 }
 
 
@@ -369,10 +368,7 @@ static std::unique_ptr<CgEngine> cg_create(const mg_geom *g, const void *U, doub
   }
   const long long nc = e->lv.back().n;
   if (nc > 4096) fail(MG_ERR_UNSUPPORTED, "MG-CG: the coarsest level is solved by dense LU (at most 4096 dofs)");
-  e->LU.alloc((size_t)(nc * nc));
-  e->lu_work.alloc((size_t)nc);
-  e->ipiv.alloc((size_t)nc);
-  e->info.alloc(1);
+  e->lu_work.alloc((size_t)line_work_size(e->lv.back().geo, e->lv.back().nint));
   const long long nf = e->lv[0].n;
   e->U.alloc((size_t)e->lv[0].geo.nsites * 2);
   e->tmp.alloc((size_t)nf);
