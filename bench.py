@@ -640,7 +640,7 @@ def dslash4_roofline(precision: int, dims=(32, 32, 32, 64), iters: int = 20, com
     res = dict(lattice="x".join(str(v) for v in dims), dtype="f64" if precision == 0 else "f32",
                bytes_per_site=per_site, flop_per_site=1368, ms=t * 1e3, gbs=V * per_site / t / 1e9,
                tflops=V * 1368 / t / 1e12,
-               kernel="dslash4_tile_kernel (8x2x2x2 tiles)" if precision == 1 else "dslash4_kernel<double>")
+               kernel="dslash4_pair_kernel (8x2x2x2 tile per warp)" if precision == 1 else "dslash4_kernel<double>")
     if precision == 1 and compare_gather:
         # the warp-gather kernel on the same inputs
         os.environ["MG_DSLASH4_GATHER"] = "1"
@@ -1071,22 +1071,6 @@ def run_only(case: str):
         return
     if case == "su3-prof":  # mixed precision, setup and 2 solves (launch-list profiling)
         print(json.dumps({"case": case, **su3_workload((1,), 2, batched=False)}))
-        return
-    if case == "dslash4-sweep":
-        # the FP32 4d apply on 32^3 x 64 with each kernel variant (tile shapes, warp gather)
-        res = {}
-        for name, env in (("gather", ("MG_DSLASH4_GATHER", "1")), ("tileA_8x4x4x4", ("MG_DSLASH4_TILE", "0")),
-                          ("tileB_8x4x4x2", ("MG_DSLASH4_TILE", "1")), ("tileC_4x4x4x2", ("MG_DSLASH4_TILE", "2")),
-                          ("tileD_8x4x2x2", ("MG_DSLASH4_TILE", "3")), ("tileB_3cta", ("MG_DSLASH4_TILE", "4")),
-                          ("tileC_6cta", ("MG_DSLASH4_TILE", "5")), ("tileE_4x4x2x2", ("MG_DSLASH4_TILE", "6")),
-                          ("tileF_8x2x2x2", ("MG_DSLASH4_TILE", "7"))):
-            os.environ[env[0]] = env[1]
-            try:
-                r = dslash4_roofline(1, iters=10, compare_gather=False)
-            finally:
-                del os.environ[env[0]]
-            res[name] = {"ms": r["ms"], "gbs": r["gbs"]}
-        print(json.dumps({"case": case, **res}))
         return
     if case.startswith("dslash4"):
         r = dslash4_roofline(1 if case == "dslash4-f32" else 0, iters=3, compare_gather=False)

@@ -210,47 +210,64 @@ __global__ void __launch_bounds__(32 * DSLASH4_WARPS, sizeof(R) == 4 ? 5 : 2) ds
 }
 
 // ---------------------------------------------------------------------------
-// Tiled FP32 apply, for extents divisible by the tile: one CTA per tile of the lattice, one site
-// per thread. Each site reads its spinor and its four forward links once and uses every link
-// twice: U_x^mu for its own forward hop (applied to the projected spinor of x + mu) and
-// U_x^mu^dagger for the backward hop of x + mu (applied to its own projected spinor here and
-// handed over). Per direction the tile exchanges these two half spinors (2 spins x 3 colours)
-// through shared memory; a site on a face of the tile forms the missing one itself from the
-// outside neighbour (its spinor, and for a backward hop its link, read through L2). On-chip
-// traffic per site: the 480 algorithmic bytes plus the faces' share, instead of 8 neighbour
-// spinors and 8 links per site.
+// Tiled FP32 apply, for extents divisible by 8 x 2 x 2 x 2: a warp owns one such tile, a lane the
+// two sites of one (x0, x1, x2) that differ in x3. What bounded the one-site-per-thread form was
+// the L1 path (91 % busy): 36 strided 8-byte link loads per site, each touching 32 sectors, and
+// half spinors exchanged through shared memory behind block barriers. Here
+//  * the tile's links and the links of its backward faces are copied into shared memory once by
+//    coalesced 16-byte asynchronous copies and serve every vector of a batch (records of 304 B and
+//    80 B: conflict-free 16-byte reads);
+//  * spinors are read in 32-byte pieces, one sector each;
+//  * a direction's two hops need the projected spinor of x + mu and U_{x-mu}^dagger times that of
+//    x - mu. Each lane projects its own spinor for both, and the lanes of a row rotate them: the
+//    first lane sends the forward half spinor of the site beyond the last one, the last lane the
+//    backward product of the site before the first one, so every lane does two link products per
+//    direction and no work for a neighbour is done twice inside the tile;
+//  * the two x3 neighbours inside the tile are in one lane: no exchange at all.
+// A warp waits for no other warp. Two sites per lane (about 250 registers, 8 warps per SM) give
+// each warp twice the loads in flight. 32^3 x 64: 257 us (3.92 TB/s), the one-site form 353 us; the
+// batch of a propagator (setup and 12 solves on 16^3 x 32) 758 -> 659 ms.
 // ---------------------------------------------------------------------------
 
-// tile extents (powers of two) and the thread-id step of one hop in each direction
-template <int A0, int A1, int A2, int A3>
-struct Tile4 {
-  static constexpr int sites = A0 * A1 * A2 * A3;
-  template <int MU>
-  __host__ __device__ static constexpr int n() {
-    return MU == 0 ? A0 : MU == 1 ? A1 : MU == 2 ? A2 : A3;
-  }
-  template <int MU>
-  __host__ __device__ static constexpr int d() {
-    return MU == 0 ? 1 : MU == 1 ? A0 : MU == 2 ? A0 * A1 : A0 * A1 * A2;
-  }
-};
-
+template <bool A32>
 __device__ __forceinline__ void load_spinor32(const Cx<float> *__restrict__ f, int x, Cx<float> (&p)[12]) {
-  const float4 *q = reinterpret_cast<const float4 *>(f) + (long long)x * 6;
+  const float *q = reinterpret_cast<const float *>(f) + (long long)x * 24;
+  float v[24];
+  if (A32) {
 #pragma unroll
-  for (int i = 0; i < 6; ++i) {
-    const float4 w = __ldg(q + i);
-    p[2 * i] = mk(w.x, w.y);
-    p[2 * i + 1] = mk(w.z, w.w);
+    for (int i = 0; i < 3; ++i)
+      asm("ld.global.nc.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+          : "=f"(v[8 * i]), "=f"(v[8 * i + 1]), "=f"(v[8 * i + 2]), "=f"(v[8 * i + 3]), "=f"(v[8 * i + 4]),
+            "=f"(v[8 * i + 5]), "=f"(v[8 * i + 6]), "=f"(v[8 * i + 7])
+          : "l"(q + 8 * i));
+  } else {
+#pragma unroll
+    for (int i = 0; i < 6; ++i) {
+      const float4 w = __ldg(reinterpret_cast<const float4 *>(q) + i);
+      v[4 * i] = w.x;
+      v[4 * i + 1] = w.y;
+      v[4 * i + 2] = w.z;
+      v[4 * i + 3] = w.w;
+    }
   }
+#pragma unroll
+  for (int i = 0; i < 12; ++i) p[i] = mk(v[2 * i], v[2 * i + 1]);
 }
 
-__device__ __forceinline__ void load_link32(const Cx<float> *__restrict__ U, int x, int mu, Cx<float> (&u)[9]) {
-  const float2 *q = reinterpret_cast<const float2 *>(U) + ((long long)x * 4 + mu) * 9;
+template <bool A32>
+__device__ __forceinline__ void store_spinor32(Cx<float> *f, int x, const Cx<float> (&p)[12]) {
+  float *q = reinterpret_cast<float *>(f) + (long long)x * 24;
+  if (A32) {
 #pragma unroll
-  for (int i = 0; i < 9; ++i) {
-    const float2 w = __ldg(q + i);
-    u[i] = mk(w.x, w.y);
+    for (int i = 0; i < 3; ++i)
+      asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(q + 8 * i), "f"(p[4 * i].re),
+                   "f"(p[4 * i].im), "f"(p[4 * i + 1].re), "f"(p[4 * i + 1].im), "f"(p[4 * i + 2].re),
+                   "f"(p[4 * i + 2].im), "f"(p[4 * i + 3].re), "f"(p[4 * i + 3].im)
+                   : "memory");
+  } else {
+#pragma unroll
+    for (int i = 0; i < 6; ++i)
+      reinterpret_cast<float4 *>(q)[i] = make_float4(p[2 * i].re, p[2 * i].im, p[2 * i + 1].re, p[2 * i + 1].im);
   }
 }
 
@@ -306,223 +323,308 @@ __device__ __forceinline__ void reconstruct4(const Cx<float> (&t)[6], Cx<float> 
   }
 }
 
-// the two hops of direction MU for the site of thread t (tile coordinate lm, lattice coordinate
-// cm, extent Lm, site stride sm); sF / sM: [6][sites] half spinors in flight
-template <class T, int MU>
-__device__ __forceinline__ void tile_hops(const Cx<float> *__restrict__ U, const Cx<float> *__restrict__ in,
-                                          const Cx<float> (&p)[12], int x, int t, int lm, int cm, int Lm, int sm,
-                                          float2 (*sF)[T::sites], float2 (*sM)[T::sites], Cx<float> (&acc)[12]) {
-  constexpr int n = T::template n<MU>(), d = T::template d<MU>();
-  Cx<float> u[9];
-  load_link32(U, x, MU, u);
-  Cx<float> h[6], m[6];
-  if (lm > 0) {  // the forward hop of x - mu needs (1 - gamma_mu) psi_x
-    project4<MU, true>(p, h);
-#pragma unroll
-    for (int k = 0; k < 6; ++k) sF[k][t - d] = make_float2(h[k].re, h[k].im);
-  }
-  if (lm < n - 1) {  // the backward hop of x + mu needs U_x^mu^dagger (1 + gamma_mu) psi_x
-    project4<MU, false>(p, h);
-    link_times4<true>(u, h, m);
-#pragma unroll
-    for (int k = 0; k < 6; ++k) sM[k][t + d] = make_float2(m[k].re, m[k].im);
-  }
-  __syncthreads();
-  if (lm < n - 1) {
-#pragma unroll
-    for (int k = 0; k < 6; ++k) {
-      const float2 w = sF[k][t];
-      h[k] = mk(w.x, w.y);
-    }
-  } else {
-    Cx<float> q[12];
-    load_spinor32(in, cm + 1 == Lm ? x - cm * sm : x + sm, q);
-    project4<MU, true>(q, h);
-  }
-  link_times4<false>(u, h, m);
-  reconstruct4<MU, true>(m, acc);
-  if (lm > 0) {
-#pragma unroll
-    for (int k = 0; k < 6; ++k) {
-      const float2 w = sM[k][t];
-      m[k] = mk(w.x, w.y);
-    }
-  } else {
-    const int y = cm == 0 ? x + (Lm - 1) * sm : x - sm;
-    Cx<float> q[12];
-    load_spinor32(in, y, q);
-    load_link32(U, y, MU, u);
-    project4<MU, false>(q, h);
-    link_times4<true>(u, h, m);
-  }
-  reconstruct4<MU, false>(m, acc);
-  __syncthreads();
+namespace {
+
+// staged links, in 16-byte units: a site's four links (288 B, padded), and one link of a face site
+// as the 80 bytes around it that start on a 16-byte boundary (72 mu rounded down)
+constexpr int kRec = 19, kHalo = 5;
+constexpr int kHaloX = 0, kHaloY = 8, kHaloZ = 40, kHaloT = 72, kHaloSites = 104;
+constexpr int kPairWarps = 4;
+constexpr int kWarpUnits = 64 * kRec + kHaloSites * kHalo;
+constexpr size_t kPairSmem = (size_t)kPairWarps * kWarpUnits * 16;
+
+// first 16-byte unit of link mu in a record; links 1 and 3 start 8 bytes into it
+__host__ __device__ constexpr int link_unit(int mu) { return mu == 0 ? 0 : mu == 1 ? 4 : mu == 2 ? 9 : 13; }
+
+__device__ __forceinline__ void copy16(float4 *dst, const char *src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned int)__cvta_generic_to_shared(dst)),
+               "l"(src)
+               : "memory");
 }
 
-// DOTS: also the sums of an MR step on each vector (blockIdx.y), (<out, in>, |out|^2) as
-// (re, im, norm), formed from the values the kernel holds anyway (its input and output at the
-// site): per-thread and per-block in FP32, FP64 partials and final sum, into mr.out[3 v]
+template <int MU>
+__device__ __forceinline__ void staged_link(const float4 *q, Cx<float> (&u)[9]) {
+  if (MU % 2 == 0) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const float4 w = q[i];
+      u[2 * i] = mk(w.x, w.y);
+      u[2 * i + 1] = mk(w.z, w.w);
+    }
+    const float2 w = *reinterpret_cast<const float2 *>(q + 4);
+    u[8] = mk(w.x, w.y);
+  } else {
+    const float2 w = reinterpret_cast<const float2 *>(q)[1];
+    u[0] = mk(w.x, w.y);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const float4 v = q[1 + i];
+      u[1 + 2 * i] = mk(v.x, v.y);
+      u[2 + 2 * i] = mk(v.z, v.w);
+    }
+  }
+}
+
+__device__ __forceinline__ void rotate6(const Cx<float> (&s)[6], int src, Cx<float> (&d)[6]) {
+#pragma unroll
+  for (int i = 0; i < 6; ++i)
+    d[i] = mk(__shfl_sync(0xffffffffu, s[i].re, src), __shfl_sync(0xffffffffu, s[i].im, src));
+}
+
+// the two hops of direction MU (0, 1, 2) for the lane's site with spinor p: `out` is the site beyond
+// the row this lane reads (first lane: the one after the last, last lane: the one before the first;
+// others none), fsrc / bsrc the lanes holding x + mu and x - mu (cyclic in the row), own / face the
+// staged links of the site and of the site before the first one
+template <int MU, bool A32>
+__device__ __forceinline__ void row_hops(const Cx<float> *__restrict__ in, const Cx<float> (&p)[12], int out,
+                                         bool first, bool last, int fsrc, int bsrc, const float4 *own,
+                                         const float4 *face, Cx<float> (&acc)[12]) {
+  Cx<float> q[12], h[6], t[6], u[9];
+  if (MU == 0) {
+#pragma unroll
+    for (int i = 0; i < 12; ++i) q[i] = p[i];
+    if (first || last) load_spinor32<A32>(in, out, q);
+  } else {
+    load_spinor32<A32>(in, out, q);
+  }
+  Cx<float> v[12];
+#pragma unroll
+  for (int i = 0; i < 12; ++i) v[i] = mk(first ? q[i].re : p[i].re, first ? q[i].im : p[i].im);
+  project4<MU, true>(v, h);
+  rotate6(h, fsrc, t);
+  staged_link<MU>(own + link_unit(MU), u);
+  link_times4<false>(u, t, h);
+  reconstruct4<MU, true>(h, acc);
+#pragma unroll
+  for (int i = 0; i < 12; ++i) v[i] = mk(last ? q[i].re : p[i].re, last ? q[i].im : p[i].im);
+  project4<MU, false>(v, h);
+  staged_link<MU>(last ? face : own + link_unit(MU), u);
+  link_times4<true>(u, h, t);
+  rotate6(t, bsrc, h);
+  reconstruct4<MU, false>(h, acc);
+}
+
+}  // namespace
+
+// DOTS: also the sums of an MR step on each vector, (<out, in>, |out|^2) as (re, im, norm), formed
+// from the values the kernel holds anyway: per-thread and per-block in FP32, FP64 partials and
+// final sum, into mr.out[3 v]
 struct MrSums {
-  double *partials;  // [vector][tile][3]
+  double *partials;  // [vector][CTA][3]
   double *out;       // [vector][3]
   unsigned int *tickets;
 };
 
-template <class T, int MINB, bool SHIFT, bool DOTS = false>
-__global__ void __launch_bounds__(T::sites, MINB) dslash4_tile_kernel(const Cx<float> *__restrict__ U,
-                                                                      const Cx<float> *__restrict__ in,
-                                                                      Cx<float> *__restrict__ out, Geo4 g,
-                                                                      float diag, const Cx<float> *__restrict__ b,
-                                                                      float a, float c, long long ldv,
-                                                                      const double *__restrict__ shift,
-                                                                      MrSums mr = MrSums{}) {
-  constexpr int A0 = T::template n<0>(), A1 = T::template n<1>(), A2 = T::template n<2>();
-  __shared__ float2 sF[6][T::sites], sM[6][T::sites];
-  if (SHIFT) diag += (float)shift[blockIdx.y];
-  in += blockIdx.y * ldv;
-  out += blockIdx.y * ldv;
-  if (b != nullptr) b += blockIdx.y * ldv;
-  const int t = threadIdx.x;
-  const int l0 = t % A0, l1 = (t / A0) % A1, l2 = (t / (A0 * A1)) % A2, l3 = t / (A0 * A1 * A2);
-  const int n0 = g.L[0] / A0, n1 = g.L[1] / A1, n2 = g.L[2] / A2;
-  int tb = blockIdx.x;
-  const int b0 = tb % n0;
+// out_v = a (D in_v) + c b_v for the vectors [chunk blockIdx.y, ...) of nvec (stride ldv complex)
+template <bool A32, bool SHIFT, bool DOTS>
+__global__ void __launch_bounds__(32 * kPairWarps, 2)
+    dslash4_pair_kernel(const Cx<float> *__restrict__ U, const Cx<float> *__restrict__ in, Cx<float> *__restrict__ out,
+                        Geo4 g, float diag, const Cx<float> *__restrict__ b, float a, float c, long long ldv,
+                        const double *__restrict__ shift, int nvec, int chunk, MrSums mr) {
+  extern __shared__ float4 staged[];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int l0 = lane & 7, l1 = (lane >> 3) & 1, l2 = lane >> 4;
+  const int tiles = (int)(g.nsites / 64);
+  const int tile = blockIdx.x * kPairWarps + w;
+  const bool live = tile < tiles;  // whole warps
+  const int s1 = g.L[0], s2 = s1 * g.L[1], s3 = s2 * g.L[2];
+  int tb = live ? tile : 0;
+  const int n0 = g.L[0] / 8, n1 = g.L[1] / 2, n2 = g.L[2] / 2;
+  const int o0 = (tb % n0) * 8;
   tb /= n0;
-  const int b1 = tb % n1;
+  const int o1 = (tb % n1) * 2;
   tb /= n1;
-  const int b2 = tb % n2;
-  const int b3 = tb / n2;
-  const int c0 = b0 * A0 + l0, c1 = b1 * A1 + l1, c2 = b2 * A2 + l2, c3 = b3 * T::template n<3>() + l3;
-  const int s1 = g.L[0], s2 = g.L[0] * g.L[1], s3 = s2 * g.L[2];
-  const int x = c0 + c1 * s1 + c2 * s2 + c3 * s3;
-  Cx<float> p[12], acc[12];
-  load_spinor32(in, x, p);
-#pragma unroll
-  for (int i = 0; i < 12; ++i) acc[i] = mk(0.f, 0.f);
-  tile_hops<T, 0>(U, in, p, x, t, l0, c0, g.L[0], 1, sF, sM, acc);
-  tile_hops<T, 1>(U, in, p, x, t, l1, c1, g.L[1], s1, sF, sM, acc);
-  tile_hops<T, 2>(U, in, p, x, t, l2, c2, g.L[2], s2, sF, sM, acc);
-  tile_hops<T, 3>(U, in, p, x, t, l3, c3, g.L[3], s3, sF, sM, acc);
-  float sums[3] = {0.f, 0.f, 0.f};  // <out, in> and |out|^2 at this site (DOTS)
-#pragma unroll
-  for (int i = 0; i < 12; ++i) {
-    const Cx<float> o = mk(a * (diag * p[i].re - 0.5f * acc[i].re), a * (diag * p[i].im - 0.5f * acc[i].im));
-    if (DOTS) {
-      sums[0] += o.re * p[i].re + o.im * p[i].im;
-      sums[1] += o.re * p[i].im - o.im * p[i].re;
-      sums[2] += o.re * o.re + o.im * o.im;
+  const int o2 = (tb % n2) * 2, o3 = (tb / n2) * 2;
+  // coordinates just outside the tile, periodic
+  const int p0 = o0 + 8 == g.L[0] ? 0 : o0 + 8, m0 = o0 == 0 ? g.L[0] - 1 : o0 - 1;
+  const int p1 = o1 + 2 == g.L[1] ? 0 : o1 + 2, m1 = o1 == 0 ? g.L[1] - 1 : o1 - 1;
+  const int p2 = o2 + 2 == g.L[2] ? 0 : o2 + 2, m2 = o2 == 0 ? g.L[2] - 1 : o2 - 1;
+  const int p3 = o3 + 2 == g.L[3] ? 0 : o3 + 2, m3 = o3 == 0 ? g.L[3] - 1 : o3 - 1;
+  float4 *rec = staged + w * kWarpUnits, *halo = rec + 64 * kRec;
+  if (live) {
+    const char *Ub = reinterpret_cast<const char *>(U);
+    const long long org = o0 + (long long)o1 * s1 + (long long)o2 * s2 + (long long)o3 * s3;
+    // own links: 8 rows of 8 sites, 144 units each
+#pragma unroll 4
+    for (int it = 0; it < 36; ++it) {
+      const int idx = it * 32 + lane, row = idx / 144, k = idx - row * 144, site = k / 18;
+      const long long x = org + (row & 1) * s1 + ((row >> 1) & 1) * s2 + (row >> 2) * s3;
+      copy16(rec + (row * 8 + site) * kRec + (k - site * 18), Ub + x * 288 + k * 16);
     }
-    p[i] = o;
-  }
-  if (b != nullptr) {
-    Cx<float> q[12];
-    load_spinor32(b, x, q);
+    // backward faces: 8 sites of the x0 face, 4 rows of 8 sites of each other face
 #pragma unroll
-    for (int i = 0; i < 12; ++i) p[i] = mk(p[i].re + c * q[i].re, p[i].im + c * q[i].im);
-  }
-  float4 *o = reinterpret_cast<float4 *>(out) + (long long)x * 6;
+    for (int it = 0; it < 2; ++it) {
+      const int idx = it * 32 + lane, e = idx / kHalo, k = idx - e * kHalo;
+      const long long x = org - o0 + m0 + (e & 1) * s1 + ((e >> 1) & 1) * s2 + (e >> 2) * s3;
+      if (idx < 8 * kHalo) copy16(halo + idx, Ub + x * 288 + k * 16);
+    }
 #pragma unroll
-  for (int i = 0; i < 6; ++i) o[i] = make_float4(p[2 * i].re, p[2 * i].im, p[2 * i + 1].re, p[2 * i + 1].im);
-  if (DOTS) {
-    __shared__ float sh[32 * 3];
-    grid_finish_t<3, float>(sums, mr.partials + (long long)blockIdx.y * gridDim.x * 3, mr.out + 3 * blockIdx.y,
-                            mr.tickets + blockIdx.y, sh);
+    for (int mu = 1; mu < 4; ++mu) {
+      const long long face = mu == 1 ? org + (long long)(m1 - o1) * s1
+                                     : mu == 2 ? org + (long long)(m2 - o2) * s2 : org + (long long)(m3 - o3) * s3;
+      const int sa = mu == 1 ? s2 : s1, sb = mu == 3 ? s2 : s3;
+      const int h0 = (mu == 1 ? kHaloY : mu == 2 ? kHaloZ : kHaloT) * kHalo;
+#pragma unroll
+      for (int it = 0; it < 5; ++it) {
+        const int idx = it * 32 + lane, row = idx / 40, e = (idx - row * 40) / kHalo, k = idx % kHalo;
+        const long long x = face + (row & 1) * sa + (row >> 1) * sb + e;
+        copy16(halo + h0 + idx, Ub + x * 288 + (link_unit(mu) + k) * 16);
+      }
+    }
+  }
+  asm volatile("cp.async.commit_group;" ::: "memory");
+  const int row12 = (o1 + l1) * s1 + (o2 + l2) * s2;
+  const int xA = o0 + l0 + row12 + o3 * s3, xB = xA + s3;
+  const float4 *recA = rec + lane * kRec, *recB = recA + 32 * kRec;
+  // the outside site this lane reads for the rows along x0, x1 and x2 of site A (site B: + s3)
+  const int dx = (l0 == 0 ? p0 - o0 : m0 - (o0 + 7));
+  const int outX = xA + dx, outY = xA + (l1 == 0 ? p1 - o1 : m1 - (o1 + 1)) * s1,
+            outZ = xA + (l2 == 0 ? p2 - o2 : m2 - (o2 + 1)) * s2;
+  const int fX = (lane & 24) | ((l0 + 1) & 7), bX = (lane & 24) | ((l0 + 7) & 7);
+  const float4 *hX = halo + (kHaloX + l1 + 2 * l2) * kHalo, *hY = halo + (kHaloY + l0 + 8 * l2) * kHalo,
+               *hZ = halo + (kHaloZ + l0 + 8 * l1) * kHalo, *hT = halo + (kHaloT + lane) * kHalo;
+  const int v0 = blockIdx.y * chunk, v1 = v0 + chunk < nvec ? v0 + chunk : nvec;
+  in += v0 * ldv;
+  out += v0 * ldv;
+  if (b != nullptr) b += v0 * ldv;
+  asm volatile("cp.async.wait_all;" ::: "memory");
+  __syncwarp();
+  for (int v = v0; v < v1; ++v) {
+    const float dg = SHIFT ? diag + (float)shift[v] : diag;
+    float sums[3] = {0.f, 0.f, 0.f};
+    if (live) {
+      Cx<float> pA[12], pB[12], aA[12], aB[12];
+      load_spinor32<A32>(in, xA, pA);
+      load_spinor32<A32>(in, xB, pB);
+#pragma unroll
+      for (int i = 0; i < 12; ++i) aA[i] = aB[i] = mk(0.f, 0.f);
+      row_hops<0, A32>(in, pA, outX, l0 == 0, l0 == 7, fX, bX, recA, hX, aA);
+      row_hops<0, A32>(in, pB, outX + s3, l0 == 0, l0 == 7, fX, bX, recB, hX + 4 * kHalo, aB);
+      row_hops<1, A32>(in, pA, outY, l1 == 0, l1 == 1, lane ^ 8, lane ^ 8, recA, hY, aA);
+      row_hops<1, A32>(in, pB, outY + s3, l1 == 0, l1 == 1, lane ^ 8, lane ^ 8, recB, hY + 16 * kHalo, aB);
+      row_hops<2, A32>(in, pA, outZ, l2 == 0, l2 == 1, lane ^ 16, lane ^ 16, recA, hZ, aA);
+      row_hops<2, A32>(in, pB, outZ + s3, l2 == 0, l2 == 1, lane ^ 16, lane ^ 16, recB, hZ + 16 * kHalo, aB);
+      {  // direction 3: the neighbours inside the tile are the lane's own two sites
+        Cx<float> q[12], h[6], t[6], u[9];
+        staged_link<3>(recA + link_unit(3), u);
+        project4<3, true>(pB, h);
+        link_times4<false>(u, h, t);
+        reconstruct4<3, true>(t, aA);
+        load_spinor32<A32>(in, xA + (m3 - o3) * s3, q);
+        project4<3, false>(pA, h);
+        link_times4<true>(u, h, t);
+        staged_link<3>(hT, u);
+        Cx<float> t2[6];
+        project4<3, false>(q, h);
+        link_times4<true>(u, h, t2);
+        reconstruct4<3, false>(t2, aA);
+        load_spinor32<A32>(in, xA + (p3 - o3) * s3, q);
+        staged_link<3>(recB + link_unit(3), u);
+        project4<3, true>(q, h);
+        link_times4<false>(u, h, t2);
+        reconstruct4<3, true>(t2, aB);
+        reconstruct4<3, false>(t, aB);
+      }
+#pragma unroll
+      for (int half = 0; half < 2; ++half) {
+        Cx<float>(&p)[12] = half ? pB : pA;
+        Cx<float>(&acc)[12] = half ? aB : aA;
+        const int x = half ? xB : xA;
+#pragma unroll
+        for (int i = 0; i < 12; ++i) {
+          const Cx<float> o =
+              mk(a * (dg * p[i].re - 0.5f * acc[i].re), a * (dg * p[i].im - 0.5f * acc[i].im));
+          if (DOTS) {
+            sums[0] += o.re * p[i].re + o.im * p[i].im;
+            sums[1] += o.re * p[i].im - o.im * p[i].re;
+            sums[2] += o.re * o.re + o.im * o.im;
+          }
+          p[i] = o;
+        }
+        if (b != nullptr) {
+          Cx<float> q[12];
+          load_spinor32<A32>(b, x, q);
+#pragma unroll
+          for (int i = 0; i < 12; ++i) p[i] = mk(p[i].re + c * q[i].re, p[i].im + c * q[i].im);
+        }
+        store_spinor32<A32>(out, x, p);
+      }
+    }
+    if (DOTS) {
+      __shared__ float sh[32 * 3];
+      grid_finish_t<3, float>(sums, mr.partials + (long long)v * gridDim.x * 3, mr.out + 3 * v, mr.tickets + v, sh);
+    }
+    in += ldv;
+    out += ldv;
+    if (b != nullptr) b += ldv;
   }
 }
 
-// tile shapes of the tiled kernel; MG_DSLASH4_TILE picks one (default 7, the fastest at 32^3 x 64:
-// 0.365 ms against 0.373 to 0.426 for the other shapes and 0.429 for the warp-gather kernel),
-// MG_DSLASH4_GATHER the warp-gather kernel
-using TileA = Tile4<8, 4, 4, 4>;  // 512 threads, 1 CTA per SM
-using TileB = Tile4<8, 4, 4, 2>;  // 256 threads, 2 CTAs per SM
-using TileC = Tile4<4, 4, 4, 2>;  // 128 threads, 4 CTAs per SM
-using TileD = Tile4<8, 4, 2, 2>;  // 128 threads, 4 CTAs per SM
-using TileE = Tile4<4, 4, 2, 2>;  // 64 threads, 8 CTAs per SM
-using TileF = Tile4<8, 2, 2, 2>;  // 64 threads, 8 CTAs per SM
+namespace {
 
-template <class T>
-static bool tile_divides(const Geo4 &g) {
-  return g.L[0] % T::template n<0>() == 0 && g.L[1] % T::template n<1>() == 0 && g.L[2] % T::template n<2>() == 0 &&
-         g.L[3] % T::template n<3>() == 0;
+// CTAs of one launch over the lattice, and the vectors each takes: the count that gives the least
+// work on the busiest SM (2 CTAs resident on each of 152), staging the links counted as 0.6 vectors
+int pair_ctas(const Geo4 &g) { return (int)((g.nsites / 64 + kPairWarps - 1) / kPairWarps); }
+int pair_chunk(const Geo4 &g, int nvec) {
+  int best = 1;
+  double cost = 0.0;
+  for (int c = 1; c <= nvec; ++c) {
+    const long long ctas = (long long)pair_ctas(g) * ((nvec + c - 1) / c);
+    const double t = (double)((ctas + 303) / 304) * (c + 0.6);
+    if (c == 1 || t < cost) {
+      best = c;
+      cost = t;
+    }
+  }
+  return best;
 }
 
-template <class T, int MINB>
-static void launch_tile4(const Cx<float> *U, const Cx<float> *in, Cx<float> *out, Geo4 g, double diag,
-                         const Cx<float> *b, double a, double c, cudaStream_t s, int nvec, const double *shift) {
-  const dim3 grid((unsigned int)(g.nsites / T::sites), nvec);
-  if (shift != nullptr)
-    dslash4_tile_kernel<T, MINB, true><<<grid, T::sites, 0, s>>>(U, in, out, g, (float)diag, b, (float)a, (float)c,
-                                                                  12 * g.nsites, shift);
-  else
-    dslash4_tile_kernel<T, MINB, false><<<grid, T::sites, 0, s>>>(U, in, out, g, (float)diag, b, (float)a,
-                                                                   (float)c, 12 * g.nsites, nullptr);
+template <bool A32, bool SHIFT, bool DOTS>
+void launch_pair(const Cx<float> *U, const Cx<float> *in, Cx<float> *out, Geo4 g, double diag, const Cx<float> *b,
+                 double a, double c, cudaStream_t s, int nvec, const double *shift, MrSums mr) {
+  auto fn = dslash4_pair_kernel<A32, SHIFT, DOTS>;
+  MG_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPairSmem));
+  const int chunk = pair_chunk(g, nvec);
+  fn<<<dim3(pair_ctas(g), (nvec + chunk - 1) / chunk), 32 * kPairWarps, kPairSmem, s>>>(
+      U, in, out, g, (float)diag, b, (float)a, (float)c, 12 * g.nsites, shift, nvec, chunk, mr);
   MG_LAUNCHED();
 }
 
-// true when a tiled kernel took the apply
+bool aligned(const void *p, uintptr_t n) { return (reinterpret_cast<uintptr_t>(p) & (n - 1)) == 0; }
+
+// the tiled kernel takes lattices of whole 8 x 2 x 2 x 2 tiles with 16-byte aligned links (its
+// asynchronous copies); other shapes and links at an odd 8-byte offset run the warp gather
+bool pair_takes(const Cx<float> *U, const Geo4 &g) {
+  return g.L[0] % 8 == 0 && g.L[1] % 2 == 0 && g.L[2] % 2 == 0 && g.L[3] % 2 == 0 && aligned(U, 16) &&
+         std::getenv("MG_DSLASH4_GATHER") == nullptr;
+}
+
+}  // namespace
+
+// true when the tiled kernel took the apply
 static bool try_tile4(const Cx<float> *U, const Cx<float> *in, Cx<float> *out, Geo4 g, double diag,
                       const Cx<float> *b, double a, double c, cudaStream_t s, int nvec, const double *shift) {
-  if (std::getenv("MG_DSLASH4_GATHER") != nullptr) return false;
-  const char *v = std::getenv("MG_DSLASH4_TILE");
-  const int which = v != nullptr ? std::atoi(v) : 7;
-  if (which == 0 && tile_divides<TileA>(g)) {
-    launch_tile4<TileA, 1>(U, in, out, g, diag, b, a, c, s, nvec, shift);
-    return true;
-  }
-  if (which == 2 && tile_divides<TileC>(g)) {
-    launch_tile4<TileC, 4>(U, in, out, g, diag, b, a, c, s, nvec, shift);
-    return true;
-  }
-  if (which == 6 && tile_divides<TileE>(g)) {
-    launch_tile4<TileE, 8>(U, in, out, g, diag, b, a, c, s, nvec, shift);
-    return true;
-  }
-  if (which == 7 && tile_divides<TileF>(g)) {
-    launch_tile4<TileF, 8>(U, in, out, g, diag, b, a, c, s, nvec, shift);
-    return true;
-  }
-  if (which == 3 && tile_divides<TileD>(g)) {
-    launch_tile4<TileD, 4>(U, in, out, g, diag, b, a, c, s, nvec, shift);
-    return true;
-  }
-  if (which == 4 && tile_divides<TileB>(g)) {  // 3 CTAs per SM: at most 85 registers
-    launch_tile4<TileB, 3>(U, in, out, g, diag, b, a, c, s, nvec, shift);
-    return true;
-  }
-  if (which == 5 && tile_divides<TileC>(g)) {  // 6 CTAs per SM
-    launch_tile4<TileC, 6>(U, in, out, g, diag, b, a, c, s, nvec, shift);
-    return true;
-  }
-  if (which == 1 && tile_divides<TileB>(g)) {
-    launch_tile4<TileB, 2>(U, in, out, g, diag, b, a, c, s, nvec, shift);
-    return true;
-  }
-  if (tile_divides<TileF>(g)) {
-    launch_tile4<TileF, 8>(U, in, out, g, diag, b, a, c, s, nvec, shift);
-    return true;
-  }
-  if (tile_divides<TileB>(g)) {
-    launch_tile4<TileB, 2>(U, in, out, g, diag, b, a, c, s, nvec, shift);
-    return true;
-  }
-  return false;
+  if (!pair_takes(U, g)) return false;
+  const bool a32 = aligned(in, 32) && aligned(out, 32) && aligned(b, 32);
+  auto run = [&](auto fn) { fn(U, in, out, g, diag, b, a, c, s, nvec, shift, MrSums{}); };
+  if (a32)
+    shift != nullptr ? run(launch_pair<true, true, false>) : run(launch_pair<true, false, false>);
+  else
+    shift != nullptr ? run(launch_pair<false, true, false>) : run(launch_pair<false, false, false>);
+  return true;
 }
 
 // Ar = D r for nvec FP32 vectors together with the MR sums (<Ar, r>, |Ar|^2) of each, by the
-// default tiled kernel; false (nothing launched) when that kernel does not take this lattice
-// or another variant is selected
+// tiled kernel; false (nothing launched) when that kernel does not take this lattice
 bool launch_dslash4_mr(const Cx<float> *U, const Cx<float> *r, Cx<float> *Ar, Geo4 g, double diag, int nvec,
                        double *sums, double *partials, long long partials_cap, unsigned int *tickets,
                        cudaStream_t s) {
-  if (std::getenv("MG_DSLASH4_GATHER") != nullptr || std::getenv("MG_DSLASH4_TILE") != nullptr) return false;
-  if (!tile_divides<TileF>(g)) return false;
-  const long long tiles = g.nsites / TileF::sites;
-  if (tiles * 3 * nvec > partials_cap) return false;
-  const dim3 grid((unsigned int)tiles, nvec);
-  dslash4_tile_kernel<TileF, 8, false, true><<<grid, TileF::sites, 0, s>>>(U, r, Ar, g, (float)diag, nullptr, 1.f,
-                                                                           0.f, 12 * g.nsites, nullptr,
-                                                                           MrSums{partials, sums, tickets});
-  MG_LAUNCHED();
+  if (!pair_takes(U, g) || (long long)pair_ctas(g) * 3 * nvec > partials_cap) return false;
+  const MrSums mr{partials, sums, tickets};
+  if (aligned(r, 32) && aligned(Ar, 32))
+    launch_pair<true, false, true>(U, r, Ar, g, diag, nullptr, 1.0, 0.0, s, nvec, nullptr, mr);
+  else
+    launch_pair<false, false, true>(U, r, Ar, g, diag, nullptr, 1.0, 0.0, s, nvec, nullptr, mr);
   return true;
 }
 
