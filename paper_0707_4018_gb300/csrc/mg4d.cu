@@ -66,6 +66,7 @@ struct Engine4 {
   // batched MR reductions (setup relaxation of the Nv vectors, V-cycle MR): per-vector
   // partials, tickets and (<Ar, r>, |Ar|^2) sums
   DevBuf<double> bpart, bsc;
+  DevBuf<float2> balpha;  // step lengths of an MR iteration
   DevBuf<unsigned int> btickets;
   DevBuf<Cx<float>> sx32, sr32, sAr32;  // setup relaxation batch (MG_FP32)
   DevBuf<Cx<double>> sr64, sAr64;       // setup relaxation batch (MG_FP64; x is the vector set itself)
@@ -562,20 +563,28 @@ void fgcr_batch(Engine4 &e, int nb, ApplyF &&apply, PrecF &&prec, const Cx<VT> *
 
 constexpr int kMrBlocks = 152 * 4;  // grid cap of the batched MR reductions
 
-// x (+)= nu MR iterations on D e = r for nvec vectors (stride nf; r updated to the
-// recurrence residual); the reductions are summed in the vectors' precision
+// x (+)= nu MR iterations on D e = b for nvec vectors (stride nf; x_zero: from x = 0; r and Ar are
+// work vectors, r may be b); the reductions are summed in the vectors' precision
 template <typename R>
-void mr_fine(Engine4 &e, Cx<R> *x, Cx<R> *r, Cx<R> *Ar, int nu, int nvec = 1) {
+void mr_fine(Engine4 &e, Cx<R> *x, const Cx<R> *b, Cx<R> *r, Cx<R> *Ar, int nu, bool x_zero, int nvec = 1) {
+  if constexpr (sizeof(R) == 4) {
+    // the tiled FP32 apply forms the step lengths in its epilogue; the first step reads b and makes
+    // x where it starts at zero, the last one leaves r alone
+    bool took = nu > 0;
+    for (int it = 0; took && it < nu; ++it) {
+      took = launch_dslash4_mr(U_of<R>(e), it == 0 ? b : r, Ar, e.fg, diag4(e), nvec, e.p.omega, e.balpha.p, e.bpart.p,
+                               e.bpart.n, e.btickets.p, e.s);
+      if (!took) break;  // on the first one: the lattice has no whole tiles
+      launch_mr_step_batch(e.balpha.p, x, x_zero && it == 0, it == 0 ? b : r, Ar, it + 1 < nu ? r : nullptr, e.nf, nvec,
+                           e.s);
+      e.apps[0] += nvec;
+    }
+    if (took) return;
+  }
+  if (x_zero) launch_zero<R>(x, e.nf * nvec, e.s);
+  if (b != r) launch_copy<R>(b, r, e.nf * nvec, e.s);
   for (int it = 0; it < nu; ++it) {
     e.apps[0] += nvec;
-    if constexpr (sizeof(R) == 4) {
-      // the tiled FP32 apply forms the MR sums in its epilogue (no second pass over r and A r)
-      if (launch_dslash4_mr(U_of<R>(e), r, Ar, e.fg, diag4(e), nvec, e.bsc.p, e.bpart.p, e.bpart.n, e.btickets.p,
-                            e.s)) {
-        launch_mr_update_batch<R>(e.bsc.p, e.p.omega, x, r, Ar, e.nf, nvec, e.s);
-        continue;
-      }
-    }
     launch_dslash4<R>(U_of<R>(e), r, Ar, e.fg, diag4(e), nullptr, 1.0, 0.0, e.s, nvec);
     launch_dot_norm_batch<R>(Ar, r, e.nf, nvec, e.bsc.p, e.bpart.p, e.btickets.p, kMrBlocks, e.s);
     launch_mr_update_batch<R>(e.bsc.p, e.p.omega, x, r, Ar, e.nf, nvec, e.s);
@@ -627,9 +636,7 @@ void vcycle(Engine4 &e, const Cx<double> *b64, Cx<double> *x64) {
   Cx<R> *r = VWork<R>::r(e), *Ar = VWork<R>::Ar(e), *x = VWork<R>::x(e), *b = VWork<R>::b(e);
   from64<R>(e, b64, b, e.nf);
   // 1. pre-smoothing from x = 0
-  launch_zero<R>(x, e.nf, e.s);
-  launch_copy<R>(b, r, e.nf, e.s);
-  mr_fine<R>(e, x, r, Ar, e.p.nu_pre);
+  mr_fine<R>(e, x, b, r, Ar, e.p.nu_pre, true);
   // 2. residual and restriction
   fine_apply<R>(e, x, r, b, -1.0, 1.0);
   Cx<R> *rc = sizeof(R) == 8 ? reinterpret_cast<Cx<R> *>(e.cb.p) : reinterpret_cast<Cx<R> *>(e.cb32.p);
@@ -648,7 +655,7 @@ void vcycle(Engine4 &e, const Cx<double> *b64, Cx<double> *x64) {
   launch_prolong4<R>(V_of<R>(e), ec, x, e.bg, e.s);
   // 5. post-smoothing on the new residual
   fine_apply<R>(e, x, r, b, -1.0, 1.0);
-  mr_fine<R>(e, x, r, Ar, e.p.nu_post);
+  mr_fine<R>(e, x, r, r, Ar, e.p.nu_post, false);
   to64<R>(e, x, x64, e.nf);
 }
 
@@ -717,11 +724,11 @@ void setup(Engine4 &e) {
   if (e.f32) {
     launch_convert<float, double>(e.nullv.p, e.sx32.p, nall, e.s);
     launch_dslash4<float>(e.U32.p, e.sx32.p, e.sr32.p, e.fg, diag4(e), nullptr, -1.0, 0.0, e.s, Nv);
-    mr_fine<float>(e, e.sx32.p, e.sr32.p, e.sAr32.p, e.p.nu_setup, Nv);
+    mr_fine<float>(e, e.sx32.p, e.sr32.p, e.sr32.p, e.sAr32.p, e.p.nu_setup, false, Nv);
     launch_convert<double, float>(e.sx32.p, e.nullv.p, nall, e.s);
   } else {
     launch_dslash4<double>(e.U64.p, e.nullv.p, e.sr64.p, e.fg, diag4(e), nullptr, -1.0, 0.0, e.s, Nv);
-    mr_fine<double>(e, e.nullv.p, e.sr64.p, e.sAr64.p, e.p.nu_setup, Nv);
+    mr_fine<double>(e, e.nullv.p, e.sr64.p, e.sr64.p, e.sAr64.p, e.p.nu_setup, false, Nv);
   }
   build(e);
   for (int pass = 2; pass <= e.p.n_pass; ++pass) {
@@ -851,6 +858,7 @@ Engine4 *engine4_create(const mg_geom *g, const void *U, double m, const mg_para
   e->bpart.alloc((size_t)nbat * std::max<long long>(kMrBlocks, e->fg.nsites / 64) * 3 + 16);
   e->bsc.alloc((size_t)nbat * 3);
   e->btickets.alloc((size_t)nbat);
+  if (e->f32) e->balpha.alloc((size_t)nbat);
   if (e->f32) {
     e->sx32.alloc((size_t)e->bg.Nv * e->nf);
     e->sr32.alloc((size_t)e->bg.Nv * e->nf);
@@ -943,9 +951,7 @@ void engine4_vcycle(Engine4 &e, const void *b, void *x) {
 
 void engine4_smooth(Engine4 &e, const void *b, void *x, int nu) {
   Cx<double> *xx = static_cast<Cx<double> *>(x);
-  launch_zero<double>(xx, e.nf, e.s);
-  launch_copy<double>(static_cast<const Cx<double> *>(b), e.vr64.p, e.nf, e.s);
-  mr_fine<double>(e, xx, e.vr64.p, e.vAr64.p, nu);
+  mr_fine<double>(e, xx, static_cast<const Cx<double> *>(b), e.vr64.p, e.vAr64.p, nu, true);
   MG_CUDA(cudaStreamSynchronize(e.s));
 }
 
@@ -1252,9 +1258,7 @@ void vcycle_batch(Engine4 &e, int nb, const Cx<double> *b64, Cx<double> *x64) {
   Cx<R> *r = BWork<R>::r(e), *Ar = BWork<R>::Ar(e), *x = BWork<R>::x(e), *b = BWork<R>::b(e);
   const long long nall = (long long)nb * e.nf;
   from64<R>(e, b64, b, nall);
-  launch_zero<R>(x, nall, e.s);
-  launch_copy<R>(b, r, nall, e.s);
-  mr_fine<R>(e, x, r, Ar, e.p.nu_pre, nb);
+  mr_fine<R>(e, x, b, r, Ar, e.p.nu_pre, true, nb);
   launch_dslash4<R>(U_of<R>(e), x, r, e.fg, diag4(e), b, -1.0, 1.0, e.s, nb);
   e.apps[0] += nb;
   // restriction in R, coarse solve in FP64
@@ -1267,7 +1271,7 @@ void vcycle_batch(Engine4 &e, int nb, const Cx<double> *b64, Cx<double> *x64) {
   launch_prolong4<R>(V_of<R>(e), ec, x, e.bg, e.s, nb);
   launch_dslash4<R>(U_of<R>(e), x, r, e.fg, diag4(e), b, -1.0, 1.0, e.s, nb);
   e.apps[0] += nb;
-  mr_fine<R>(e, x, r, Ar, e.p.nu_post, nb);
+  mr_fine<R>(e, x, r, r, Ar, e.p.nu_post, false, nb);
   to64<R>(e, x, x64, nall);
 }
 

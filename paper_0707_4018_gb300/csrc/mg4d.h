@@ -98,6 +98,10 @@ void launch_precondition4(const Cx<double> *Y, const Cx<double> *Minv, Cx<double
 template <typename R>
 void launch_dot_norm_batch(const Cx<R> *a, const Cx<R> *b, long long n, int nvec, double *out, double *partials,
                            unsigned int *tickets, int max_blocks, cudaStream_t s);
+// x_v (+)= alpha_v r_v (x_init: x_v = alpha_v r_v) and, unless r_out is null, r_out_v = r_v - alpha_v Ar_v for
+// nvec FP32 vectors of n (even) entries; r_out may be r
+void launch_mr_step_batch(const float2 *alpha, Cx<float> *x, bool x_init, const Cx<float> *r, const Cx<float> *Ar,
+                          Cx<float> *r_out, long long n, int nvec, cudaStream_t s);
 template <typename R>
 void launch_mr_update_batch(const double *sc, double omega, Cx<R> *x, Cx<R> *r, const Cx<R> *Ar, long long n,
                             int nvec, cudaStream_t s);

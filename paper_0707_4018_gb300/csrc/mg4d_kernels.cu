@@ -578,6 +578,34 @@ __global__ void __launch_bounds__(kReduceThreads) dot_norm_batch_kernel(const Cx
                       ticket + blockIdx.y, sh);
 }
 
+// One MR step on FP32 vectors (n2 pairs of complex each): x (+)= alpha r and, unless r_out is null,
+// r_out = r - alpha Ar. HBM-bound (five passes). The step length comes
+// ready from the apply: formed here, its two FP64 divisions per thread cost as much as the loads.
+__global__ void __launch_bounds__(256) mr_step_batch_kernel(const float2 *__restrict__ alpha, float4 *__restrict__ x,
+                                                            bool x_init, const float4 *r,
+                                                            const float4 *__restrict__ Ar, float4 *r_out,
+                                                            long long n2) {
+  const float2 a = alpha[blockIdx.y];
+  const long long off = blockIdx.y * n2;
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n2; i += (long long)gridDim.x * blockDim.x) {
+    float4 q = r[off + i];
+    float4 t = x_init ? make_float4(0.f, 0.f, 0.f, 0.f) : x[off + i];
+    t.x += a.x * q.x - a.y * q.y;
+    t.y += a.x * q.y + a.y * q.x;
+    t.z += a.x * q.z - a.y * q.w;
+    t.w += a.x * q.w + a.y * q.z;
+    x[off + i] = t;
+    if (r_out != nullptr) {
+      const float4 v = Ar[off + i];
+      q.x -= a.x * v.x - a.y * v.y;
+      q.y -= a.x * v.y + a.y * v.x;
+      q.z -= a.x * v.z - a.y * v.w;
+      q.w -= a.x * v.w + a.y * v.z;
+      r_out[off + i] = q;
+    }
+  }
+}
+
 template <typename R>
 __global__ void mr_update_batch_kernel(const double *__restrict__ sc, double omega, Cx<R> *__restrict__ x,
                                        Cx<R> *__restrict__ r, const Cx<R> *__restrict__ Ar, long long n) {
@@ -985,6 +1013,16 @@ void launch_mr_update_batch(const double *sc, double omega, Cx<R> *x, Cx<R> *r, 
   long long b = (n + 255) / 256;
   if (b > 152LL * 8) b = 152LL * 8;
   mr_update_batch_kernel<R><<<dim3((unsigned int)b, nvec), 256, 0, s>>>(sc, omega, x, r, Ar, n);
+  MG_LAUNCHED();
+}
+
+void launch_mr_step_batch(const float2 *alpha, Cx<float> *x, bool x_init, const Cx<float> *r, const Cx<float> *Ar,
+                          Cx<float> *r_out, long long n, int nvec, cudaStream_t s) {
+  const unsigned int b = grid_for(n / 2, 512);  // two pairs per thread
+  mr_step_batch_kernel<<<dim3(b, nvec), 256, 0, s>>>(alpha, reinterpret_cast<float4 *>(x), x_init,
+                                                     reinterpret_cast<const float4 *>(r),
+                                                     reinterpret_cast<const float4 *>(Ar),
+                                                     reinterpret_cast<float4 *>(r_out), n / 2);
   MG_LAUNCHED();
 }
 

@@ -224,9 +224,14 @@ __global__ void __launch_bounds__(32 * DSLASH4_WARPS, sizeof(R) == 4 ? 5 : 2) ds
 //    backward product of the site before the first one, so every lane does two link products per
 //    direction and no work for a neighbour is done twice inside the tile;
 //  * the two x3 neighbours inside the tile are in one lane: no exchange at all.
-// A warp waits for no other warp. Two sites per lane (about 250 registers, 8 warps per SM) give
-// each warp twice the loads in flight. 32^3 x 64: 257 us (3.92 TB/s), the one-site form 353 us; the
-// batch of a propagator (setup and 12 solves on 16^3 x 32) 758 -> 659 ms.
+// A warp waits for no other warp. Two sites per lane (about 255 registers, 8 warps per SM) give each
+// warp twice the loads in flight, and a direction's outside spinors are requested while the one
+// before it is worked on: with so few warps the loads' latency is what bounds it (L1 path 40 % busy,
+// issue slots 40 %). 32^3 x 64: 250 us (4.0 TB/s), the one-site form 353 us. 24 vectors on 16^3 x 32
+// with the MR step (mr_step_batch_kernel): 525 us, before 850 us; without the early requests and with
+// the sums met in a block reduction per vector 691 us; with the step applied while r is read (6
+// vector passes, not 7) 677 us, the doubled face loads costing what the pass saves; 12 warps of 168
+// registers sharing the staged links 718 us.
 // ---------------------------------------------------------------------------
 
 template <bool A32>
@@ -236,7 +241,7 @@ __device__ __forceinline__ void load_spinor32(const Cx<float> *__restrict__ f, i
   if (A32) {
 #pragma unroll
     for (int i = 0; i < 3; ++i)
-      asm("ld.global.nc.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+      asm volatile("ld.global.nc.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
           : "=f"(v[8 * i]), "=f"(v[8 * i + 1]), "=f"(v[8 * i + 2]), "=f"(v[8 * i + 3]), "=f"(v[8 * i + 4]),
             "=f"(v[8 * i + 5]), "=f"(v[8 * i + 6]), "=f"(v[8 * i + 7])
           : "l"(q + 8 * i));
@@ -329,9 +334,10 @@ namespace {
 // as the 80 bytes around it that start on a 16-byte boundary (72 mu rounded down)
 constexpr int kRec = 19, kHalo = 5;
 constexpr int kHaloX = 0, kHaloY = 8, kHaloZ = 40, kHaloT = 72, kHaloSites = 104;
-constexpr int kPairWarps = 4;
-constexpr int kWarpUnits = 64 * kRec + kHaloSites * kHalo;
-constexpr size_t kPairSmem = (size_t)kPairWarps * kWarpUnits * 16;
+constexpr int kTiles = 4;      // tiles of a CTA
+constexpr int kMaxChunk = 32;  // vectors of a CTA
+constexpr int kTileUnits = 64 * kRec + kHaloSites * kHalo;
+constexpr size_t kPairSmem = (size_t)kTiles * kTileUnits * 16;
 
 // first 16-byte unit of link mu in a record; links 1 and 3 start 8 bytes into it
 __host__ __device__ constexpr int link_unit(int mu) { return mu == 0 ? 0 : mu == 1 ? 4 : mu == 2 ? 9 : 13; }
@@ -371,33 +377,34 @@ __device__ __forceinline__ void rotate6(const Cx<float> (&s)[6], int src, Cx<flo
     d[i] = mk(__shfl_sync(0xffffffffu, s[i].re, src), __shfl_sync(0xffffffffu, s[i].im, src));
 }
 
-// the two hops of direction MU (0, 1, 2) for the lane's site with spinor p: `out` is the site beyond
-// the row this lane reads (first lane: the one after the last, last lane: the one before the first;
-// others none), fsrc / bsrc the lanes holding x + mu and x - mu (cyclic in the row), own / face the
-// staged links of the site and of the site before the first one
-template <int MU, bool A32>
-__device__ __forceinline__ void row_hops(const Cx<float> *__restrict__ in, const Cx<float> (&p)[12], int out,
-                                         bool first, bool last, int fsrc, int bsrc, const float4 *own,
-                                         const float4 *face, Cx<float> (&acc)[12]) {
-  Cx<float> q[12], h[6], t[6], u[9];
-  if (MU == 0) {
+// the two hops of direction MU (0, 1, 2) for the lane's site with spinor p: q is the spinor of the site
+// beyond the row that the lane read (first lane: the one after the last, last lane: the one before
+// the first; others none), fsrc / bsrc the lanes holding x + mu and x - mu (cyclic in the row), own /
+// face the staged links of the site and of the site before the first one
+template <int MU>
+__device__ __forceinline__ void row_hops(const Cx<float> (&p)[12], const Cx<float> (&q)[12], bool first, bool last,
+                                         int fsrc, int bsrc, const float4 *own, const float4 *face,
+                                         Cx<float> (&acc)[12]) {
+  Cx<float> e[6], h[6], t[6], u[9];
+  // e = (1 - gamma) q on the first lane, (1 + gamma) q on the last: only the sign of A q_dn differs
+  const float sg = first ? -1.f : 1.f;
 #pragma unroll
-    for (int i = 0; i < 12; ++i) q[i] = p[i];
-    if (first || last) load_spinor32<A32>(in, out, q);
-  } else {
-    load_spinor32<A32>(in, out, q);
+  for (int c = 0; c < 3; ++c) {
+    Cx<float> a0, a1;
+    a_times<float, MU>(q[6 + c], q[9 + c], a0, a1);
+    e[c] = mk(fmaf(sg, a0.re, q[c].re), fmaf(sg, a0.im, q[c].im));
+    e[3 + c] = mk(fmaf(sg, a1.re, q[3 + c].re), fmaf(sg, a1.im, q[3 + c].im));
   }
-  Cx<float> v[12];
+  project4<MU, true>(p, h);
 #pragma unroll
-  for (int i = 0; i < 12; ++i) v[i] = mk(first ? q[i].re : p[i].re, first ? q[i].im : p[i].im);
-  project4<MU, true>(v, h);
+  for (int i = 0; i < 6; ++i) h[i] = mk(first ? e[i].re : h[i].re, first ? e[i].im : h[i].im);
   rotate6(h, fsrc, t);
   staged_link<MU>(own + link_unit(MU), u);
   link_times4<false>(u, t, h);
   reconstruct4<MU, true>(h, acc);
+  project4<MU, false>(p, h);
 #pragma unroll
-  for (int i = 0; i < 12; ++i) v[i] = mk(last ? q[i].re : p[i].re, last ? q[i].im : p[i].im);
-  project4<MU, false>(v, h);
+  for (int i = 0; i < 6; ++i) h[i] = mk(last ? e[i].re : h[i].re, last ? e[i].im : h[i].im);
   staged_link<MU>(last ? face : own + link_unit(MU), u);
   link_times4<true>(u, h, t);
   rotate6(t, bsrc, h);
@@ -406,26 +413,27 @@ __device__ __forceinline__ void row_hops(const Cx<float> *__restrict__ in, const
 
 }  // namespace
 
-// DOTS: also the sums of an MR step on each vector, (<out, in>, |out|^2) as (re, im, norm), formed
-// from the values the kernel holds anyway: per-thread and per-block in FP32, FP64 partials and
-// final sum, into mr.out[3 v]
-struct MrSums {
-  double *partials;  // [vector][CTA][3]
-  double *out;       // [vector][3]
-  unsigned int *tickets;
+// SUMS: also the step length of an MR iteration on each vector, omega <out, in> / |out|^2, from the
+// values the kernel holds anyway: per-thread and per-block sums in FP32, FP64 partials, final sum and
+// quotient, into mr.alpha[v]
+struct MrStep {
+  double *partials;       // [vector][CTA][3]
+  unsigned int *tickets;  // [vector], zero
+  double omega;
+  float2 *alpha;          // [vector], written by the last CTA of the vector
 };
 
 // out_v = a (D in_v) + c b_v for the vectors [chunk blockIdx.y, ...) of nvec (stride ldv complex)
-template <bool A32, bool SHIFT, bool DOTS>
-__global__ void __launch_bounds__(32 * kPairWarps, 2)
+template <bool A32, bool SHIFT, bool SUMS>
+__global__ void __launch_bounds__(32 * kTiles, 2)
     dslash4_pair_kernel(const Cx<float> *__restrict__ U, const Cx<float> *__restrict__ in, Cx<float> *__restrict__ out,
                         Geo4 g, float diag, const Cx<float> *__restrict__ b, float a, float c, long long ldv,
-                        const double *__restrict__ shift, int nvec, int chunk, MrSums mr) {
+                        const double *__restrict__ shift, int nvec, int chunk, MrStep mr) {
   extern __shared__ float4 staged[];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int l0 = lane & 7, l1 = (lane >> 3) & 1, l2 = lane >> 4;
   const int tiles = (int)(g.nsites / 64);
-  const int tile = blockIdx.x * kPairWarps + w;
+  const int tile = blockIdx.x * kTiles + w;
   const bool live = tile < tiles;  // whole warps
   const int s1 = g.L[0], s2 = s1 * g.L[1], s3 = s2 * g.L[2];
   int tb = live ? tile : 0;
@@ -440,7 +448,7 @@ __global__ void __launch_bounds__(32 * kPairWarps, 2)
   const int p1 = o1 + 2 == g.L[1] ? 0 : o1 + 2, m1 = o1 == 0 ? g.L[1] - 1 : o1 - 1;
   const int p2 = o2 + 2 == g.L[2] ? 0 : o2 + 2, m2 = o2 == 0 ? g.L[2] - 1 : o2 - 1;
   const int p3 = o3 + 2 == g.L[3] ? 0 : o3 + 2, m3 = o3 == 0 ? g.L[3] - 1 : o3 - 1;
-  float4 *rec = staged + w * kWarpUnits, *halo = rec + 64 * kRec;
+  float4 *rec = staged + w * kTileUnits, *halo = rec + 64 * kRec;
   if (live) {
     const char *Ub = reinterpret_cast<const char *>(U);
     const long long org = o0 + (long long)o1 * s1 + (long long)o2 * s2 + (long long)o3 * s3;
@@ -487,8 +495,7 @@ __global__ void __launch_bounds__(32 * kPairWarps, 2)
   in += v0 * ldv;
   out += v0 * ldv;
   if (b != nullptr) b += v0 * ldv;
-  asm volatile("cp.async.wait_all;" ::: "memory");
-  __syncwarp();
+  __shared__ float sh[SUMS ? kMaxChunk : 1][kTiles][3];
   for (int v = v0; v < v1; ++v) {
     const float dg = SHIFT ? diag + (float)shift[v] : diag;
     float sums[3] = {0.f, 0.f, 0.f};
@@ -496,31 +503,46 @@ __global__ void __launch_bounds__(32 * kPairWarps, 2)
       Cx<float> pA[12], pB[12], aA[12], aB[12];
       load_spinor32<A32>(in, xA, pA);
       load_spinor32<A32>(in, xB, pB);
+      Cx<float> qA[12], qB[12], nA[12], nB[12];
+#pragma unroll
+      for (int i = 0; i < 12; ++i) qA[i] = qB[i] = mk(0.f, 0.f);
+      if (l0 == 0 || l0 == 7) {
+        load_spinor32<A32>(in, outX, qA);
+        load_spinor32<A32>(in, outX + s3, qB);
+      }
 #pragma unroll
       for (int i = 0; i < 12; ++i) aA[i] = aB[i] = mk(0.f, 0.f);
-      row_hops<0, A32>(in, pA, outX, l0 == 0, l0 == 7, fX, bX, recA, hX, aA);
-      row_hops<0, A32>(in, pB, outX + s3, l0 == 0, l0 == 7, fX, bX, recB, hX + 4 * kHalo, aB);
-      row_hops<1, A32>(in, pA, outY, l1 == 0, l1 == 1, lane ^ 8, lane ^ 8, recA, hY, aA);
-      row_hops<1, A32>(in, pB, outY + s3, l1 == 0, l1 == 1, lane ^ 8, lane ^ 8, recB, hY + 16 * kHalo, aB);
-      row_hops<2, A32>(in, pA, outZ, l2 == 0, l2 == 1, lane ^ 16, lane ^ 16, recA, hZ, aA);
-      row_hops<2, A32>(in, pB, outZ + s3, l2 == 0, l2 == 1, lane ^ 16, lane ^ 16, recB, hZ + 16 * kHalo, aB);
+      // each direction's outside spinors are requested while the one before it is worked on
+      load_spinor32<A32>(in, outY, nA);
+      load_spinor32<A32>(in, outY + s3, nB);
+      if (v == v0) {  // the links are on their way while the first spinors are
+        asm volatile("cp.async.wait_all;" ::: "memory");
+        __syncwarp();
+      }
+      row_hops<0>(pA, qA, l0 == 0, l0 == 7, fX, bX, recA, hX, aA);
+      row_hops<0>(pB, qB, l0 == 0, l0 == 7, fX, bX, recB, hX + 4 * kHalo, aB);
+      load_spinor32<A32>(in, outZ, qA);
+      row_hops<1>(pA, nA, l1 == 0, l1 == 1, lane ^ 8, lane ^ 8, recA, hY, aA);
+      load_spinor32<A32>(in, outZ + s3, qB);
+      row_hops<1>(pB, nB, l1 == 0, l1 == 1, lane ^ 8, lane ^ 8, recB, hY + 16 * kHalo, aB);
+      load_spinor32<A32>(in, xA + (m3 - o3) * s3, nA);
+      row_hops<2>(pA, qA, l2 == 0, l2 == 1, lane ^ 16, lane ^ 16, recA, hZ, aA);
+      load_spinor32<A32>(in, xA + (p3 - o3) * s3, nB);
+      row_hops<2>(pB, qB, l2 == 0, l2 == 1, lane ^ 16, lane ^ 16, recB, hZ + 16 * kHalo, aB);
       {  // direction 3: the neighbours inside the tile are the lane's own two sites
-        Cx<float> q[12], h[6], t[6], u[9];
+        Cx<float> h[6], t[6], t2[6], u[9];
         staged_link<3>(recA + link_unit(3), u);
         project4<3, true>(pB, h);
         link_times4<false>(u, h, t);
         reconstruct4<3, true>(t, aA);
-        load_spinor32<A32>(in, xA + (m3 - o3) * s3, q);
         project4<3, false>(pA, h);
         link_times4<true>(u, h, t);
         staged_link<3>(hT, u);
-        Cx<float> t2[6];
-        project4<3, false>(q, h);
+        project4<3, false>(nA, h);
         link_times4<true>(u, h, t2);
         reconstruct4<3, false>(t2, aA);
-        load_spinor32<A32>(in, xA + (p3 - o3) * s3, q);
         staged_link<3>(recB + link_unit(3), u);
-        project4<3, true>(q, h);
+        project4<3, true>(nB, h);
         link_times4<false>(u, h, t2);
         reconstruct4<3, true>(t2, aB);
         reconstruct4<3, false>(t, aB);
@@ -534,7 +556,7 @@ __global__ void __launch_bounds__(32 * kPairWarps, 2)
         for (int i = 0; i < 12; ++i) {
           const Cx<float> o =
               mk(a * (dg * p[i].re - 0.5f * acc[i].re), a * (dg * p[i].im - 0.5f * acc[i].im));
-          if (DOTS) {
+          if (SUMS) {
             sums[0] += o.re * p[i].re + o.im * p[i].im;
             sums[1] += o.re * p[i].im - o.im * p[i].re;
             sums[2] += o.re * o.re + o.im * o.im;
@@ -550,13 +572,56 @@ __global__ void __launch_bounds__(32 * kPairWarps, 2)
         store_spinor32<A32>(out, x, p);
       }
     }
-    if (DOTS) {
-      __shared__ float sh[32 * 3];
-      grid_finish_t<3, float>(sums, mr.partials + (long long)v * gridDim.x * 3, mr.out + 3 * v, mr.tickets + v, sh);
+    if (SUMS) {
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) sums[k] += __shfl_xor_sync(0xffffffffu, sums[k], o);
+        if (lane == 0) sh[v - v0][w][k] = sums[k];
+      }
     }
     in += ldv;
     out += ldv;
     if (b != nullptr) b += ldv;
+  }
+  if (SUMS) {
+    // the CTA's sums of every vector, then, in the last CTA of a vector, its FP64 sum over all CTAs
+    __shared__ bool last[kMaxChunk];
+    __syncthreads();
+    const int j = threadIdx.x;
+    if (j < v1 - v0) {
+      const int v = v0 + j;
+      double *part = mr.partials + (long long)v * gridDim.x * 3;
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
+        float t = 0.f;
+#pragma unroll
+        for (int q = 0; q < kTiles; ++q) t += sh[j][q][k];
+        part[blockIdx.x * 3 + k] = (double)t;
+      }
+      __threadfence();
+      last[j] = atomicAdd(mr.tickets + v, 1u) == gridDim.x - 1;
+    }
+    __syncthreads();
+    __shared__ double shd[32 * 3];
+    for (int i = 0; i < v1 - v0; ++i) {
+      if (!last[i]) continue;
+      const int v = v0 + i;
+      const volatile double *part = mr.partials + (long long)v * gridDim.x * 3;
+      __threadfence();
+      double s[3] = {0.0, 0.0, 0.0};
+      for (unsigned int q = threadIdx.x; q < gridDim.x; q += blockDim.x) {
+#pragma unroll
+        for (int k = 0; k < 3; ++k) s[k] += part[q * 3 + k];
+      }
+      block_sum<3>(s, shd);
+      if (threadIdx.x == 0) {
+        // a vanishing A r leaves r and x as they are
+        mr.alpha[v] = s[2] > 0.0 ? make_float2((float)(mr.omega * s[0] / s[2]), (float)(mr.omega * s[1] / s[2]))
+                                 : make_float2(0.f, 0.f);
+        mr.tickets[v] = 0u;
+      }
+    }
   }
 }
 
@@ -564,11 +629,11 @@ namespace {
 
 // CTAs of one launch over the lattice, and the vectors each takes: the count that gives the least
 // work on the busiest SM (2 CTAs resident on each of 152), staging the links counted as 0.6 vectors
-int pair_ctas(const Geo4 &g) { return (int)((g.nsites / 64 + kPairWarps - 1) / kPairWarps); }
+int pair_ctas(const Geo4 &g) { return (int)((g.nsites / 64 + kTiles - 1) / kTiles); }
 int pair_chunk(const Geo4 &g, int nvec) {
   int best = 1;
   double cost = 0.0;
-  for (int c = 1; c <= nvec; ++c) {
+  for (int c = 1; c <= nvec && c <= kMaxChunk; ++c) {
     const long long ctas = (long long)pair_ctas(g) * ((nvec + c - 1) / c);
     const double t = (double)((ctas + 303) / 304) * (c + 0.6);
     if (c == 1 || t < cost) {
@@ -579,13 +644,13 @@ int pair_chunk(const Geo4 &g, int nvec) {
   return best;
 }
 
-template <bool A32, bool SHIFT, bool DOTS>
+template <bool A32, bool SHIFT, bool SUMS>
 void launch_pair(const Cx<float> *U, const Cx<float> *in, Cx<float> *out, Geo4 g, double diag, const Cx<float> *b,
-                 double a, double c, cudaStream_t s, int nvec, const double *shift, MrSums mr) {
-  auto fn = dslash4_pair_kernel<A32, SHIFT, DOTS>;
+                 double a, double c, cudaStream_t s, int nvec, const double *shift, MrStep mr) {
+  auto fn = dslash4_pair_kernel<A32, SHIFT, SUMS>;
   MG_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPairSmem));
   const int chunk = pair_chunk(g, nvec);
-  fn<<<dim3(pair_ctas(g), (nvec + chunk - 1) / chunk), 32 * kPairWarps, kPairSmem, s>>>(
+  fn<<<dim3(pair_ctas(g), (nvec + chunk - 1) / chunk), 32 * kTiles, kPairSmem, s>>>(
       U, in, out, g, (float)diag, b, (float)a, (float)c, 12 * g.nsites, shift, nvec, chunk, mr);
   MG_LAUNCHED();
 }
@@ -606,7 +671,7 @@ static bool try_tile4(const Cx<float> *U, const Cx<float> *in, Cx<float> *out, G
                       const Cx<float> *b, double a, double c, cudaStream_t s, int nvec, const double *shift) {
   if (!pair_takes(U, g)) return false;
   const bool a32 = aligned(in, 32) && aligned(out, 32) && aligned(b, 32);
-  auto run = [&](auto fn) { fn(U, in, out, g, diag, b, a, c, s, nvec, shift, MrSums{}); };
+  auto run = [&](auto fn) { fn(U, in, out, g, diag, b, a, c, s, nvec, shift, MrStep{}); };
   if (a32)
     shift != nullptr ? run(launch_pair<true, true, false>) : run(launch_pair<true, false, false>);
   else
@@ -614,13 +679,11 @@ static bool try_tile4(const Cx<float> *U, const Cx<float> *in, Cx<float> *out, G
   return true;
 }
 
-// Ar = D r for nvec FP32 vectors together with the MR sums (<Ar, r>, |Ar|^2) of each, by the
-// tiled kernel; false (nothing launched) when that kernel does not take this lattice
 bool launch_dslash4_mr(const Cx<float> *U, const Cx<float> *r, Cx<float> *Ar, Geo4 g, double diag, int nvec,
-                       double *sums, double *partials, long long partials_cap, unsigned int *tickets,
+                       double omega, float2 *alpha, double *partials, long long partials_cap, unsigned int *tickets,
                        cudaStream_t s) {
   if (!pair_takes(U, g) || (long long)pair_ctas(g) * 3 * nvec > partials_cap) return false;
-  const MrSums mr{partials, sums, tickets};
+  const MrStep mr{partials, tickets, omega, alpha};
   if (aligned(r, 32) && aligned(Ar, 32))
     launch_pair<true, false, true>(U, r, Ar, g, diag, nullptr, 1.0, 0.0, s, nvec, nullptr, mr);
   else
