@@ -8,6 +8,7 @@
 // Bytes per coarse site: 5 N^2 complex of Y plus 2 N of x, y (N = 8: 5.4 KB in
 // FP64, 2.7 KB in FP32).
 #include "kernels.h"
+#include "stencil8.cuh"
 
 namespace mg {
 
@@ -101,12 +102,58 @@ __global__ void __launch_bounds__(256) coarse_apply8_kernel(const Cx<R> *__restr
   out[t] = o;
 }
 
+// the same in FP32: a warp per site and VB vectors (stencil8.cuh)
+template <int VB>
+__global__ void __launch_bounds__(256) coarse_apply8_f32_kernel(const Cx<float> *__restrict__ Y,
+                                                                const Cx<float> *__restrict__ in,
+                                                                Cx<float> *__restrict__ out, int L0, int L1,
+                                                                const Cx<float> *__restrict__ b, float a, float c,
+                                                                long long ldv, const double *__restrict__ shift,
+                                                                int nvec) {
+  const Lane8 l;
+  const int j = blockIdx.x * 8 + (threadIdx.x >> 5);
+  if (j >= L0 * L1) return;  // whole warps
+  const Site8 st(j, L0, L1);
+  float4 y[5];
+  load_blocks8(Y, j, l, y);
+#pragma unroll
+  for (int u = 0; u < VB; ++u) {
+    const int v = blockIdx.y * VB + u;
+    if (VB > 1 && v >= nvec) break;
+    const Cx<float> *iv = in + v * ldv;
+    float2 w[5];
+#pragma unroll
+    for (int d = 0; d < 5; ++d) w[d] = load_col8(iv, st.nb[d], l.q);
+    float k = stencil8(y, w, l);
+    const long long e = (v * ldv + (long long)j * 8 + l.row) * 2 + l.im;
+    if (l.writes) {
+      if (shift != nullptr) k = fmaf((float)shift[v], reinterpret_cast<const float *>(in)[e], k);
+      k *= a;
+      if (b != nullptr) k += c * reinterpret_cast<const float *>(b)[e];
+      reinterpret_cast<float *>(out)[e] = k;
+    }
+  }
+}
+
 template <typename R>
 void launch_coarse_apply(const Cx<R> *Y, const Cx<R> *in, Cx<R> *out, Geo2 g, int N, const Cx<R> *b, double a,
                          double c, cudaStream_t s, int nvec, const double *shift) {
   const int threads = 256;
   const dim3 grid(grid_for(g.nsites * N, threads), nvec);
   const long long ldv = g.nsites * N;
+  if constexpr (sizeof(R) == 4) {
+    if (N == 8) {
+      const unsigned int nb = grid_for(g.nsites * 32, threads);
+      if (nvec > 1 && (long long)nb * ((nvec + 3) / 4) >= 304)
+        coarse_apply8_f32_kernel<4><<<dim3(nb, (nvec + 3) / 4), threads, 0, s>>>(Y, in, out, g.L0, g.L1, b, (float)a,
+                                                                                (float)c, ldv, shift, nvec);
+      else
+        coarse_apply8_f32_kernel<1><<<dim3(nb, nvec), threads, 0, s>>>(Y, in, out, g.L0, g.L1, b, (float)a, (float)c,
+                                                                       ldv, shift, nvec);
+      MG_LAUNCHED();
+      return;
+    }
+  }
   if (N == 8)
     coarse_apply8_kernel<R><<<dim3(grid_for(g.nsites * 32, threads), nvec), threads, 0, s>>>(Y, in, out, g.L0, g.L1, b,
                                                                                             (R)a, (R)c, ldv, shift);

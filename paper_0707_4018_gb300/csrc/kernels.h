@@ -81,7 +81,6 @@ void launch_dslash_half(const void *U, const void *in, void *out, Geo2 g, double
 // fine level of FP32 V-cycles with half storage (MG_FP16 contexts; wilson_half.cu): the fused MR
 // iteration and its last step on half r / A r fields (12 V bytes per field of a batch), the
 // residual apply on FP32 vectors with half links
-int mr_half_grid(Geo2 g);
 void launch_mr_iteration_half(const void *U16, Geo2 g, double diag, const double *shift, bool step,
                               const Cx<float> *b, void *r_old, void *Ar_old, const float *part_in, double omega,
                               Cx<float> *x, bool x_init, void *r_new, void *Ar_new, float *part_out,

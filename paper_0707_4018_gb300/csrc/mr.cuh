@@ -32,6 +32,14 @@ __device__ __forceinline__ void block_reduce(T (&v)[NOUT], T *sh) {
   }
 }
 
+// Blocks of one MR launch per vector; a block strides over the rest of a larger lattice. Every block of
+// the next launch sums all of a vector's partials, so one block per 256 units would make that sum
+// quadratic in the lattice: at 1024 x 768 it was 60 to 75 % of an iteration (level 0: 45 us with it,
+// 11 without; level 1: 121 and 47). Up to 1216 partials (5 loads per thread) it is small beside the
+// rest: a solve there took 122 ms without the cap, 100 with it, 108 / 112 / 111 with 608 / 304 / 2432.
+constexpr int kMrGrid = 1216;
+inline int mr_blocks(long long full) { return (int)(full < kMrGrid ? full : kMrGrid); }
+
 // this block's (<A r, r> re, im, |A r|^2) into part_out[3 blockIdx.x ..]
 template <typename R>
 __device__ __forceinline__ void mr_publish(R (&v)[3], R *part_out, R *sh) {

@@ -229,7 +229,7 @@ __device__ __forceinline__ Pair<float> load_pair(const Cx<float> *f, long long x
 // STEP = false: r_new = b (rounded to half) and Ar_new = A b, partials of (<A b, b>, |A b|^2).
 // STEP = true: alpha from part_in, x (+)= alpha r_old at the site, r_new = r_old - alpha Ar_old
 // (formed at the five sites the stencil needs), Ar_new = A r_new, partials to part_out.
-template <bool STEP>
+template <bool STEP, bool LOOP>
 __global__ void __launch_bounds__(256) mr_wilson_half_kernel(const __half2 *__restrict__ U,
                                                              const Cx<float> *__restrict__ b, void *r_old,
                                                              void *Ar_old, const float *part_in, int nb_in,
@@ -240,60 +240,66 @@ __global__ void __launch_bounds__(256) mr_wilson_half_kernel(const __half2 *__re
   const int v = blockIdx.y;
   if (shift != nullptr) diag += (float)shift[v];
   const long long V = (long long)L0 * L1;
-  const long long s = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  const bool live = s < V;
   const Cx<float> z = mk(0.f, 0.f);
-  Pair<float> w[5], a[5];  // self, +0, +1, -0, -1
-#pragma unroll
-  for (int k = 0; k < 5; ++k) w[k].a = w[k].b = a[k].a = a[k].b = z;
-  Pair<float> xs;
-  xs.a = xs.b = z;
-  Cx<float> ux0 = z, ux1 = z, ub0 = z, ub1 = z;
-  if (live) {
-    const Nbr n = neighbours(s, L0, L1);
-    const long long nb[5] = {s, n.p0, n.p1, n.m0, n.m1};
-    if (STEP) {
-      const HalfField ro = half_field(r_old, V, v), ao = half_field(Ar_old, V, v);
-#pragma unroll
-      for (int k = 0; k < 5; ++k) {
-        w[k] = load_site(ro.h, ro.n, nb[k]);
-        a[k] = load_site(ao.h, ao.n, nb[k]);
-      }
-      if (!x_init) xs = load_pair(x + 2 * V * v, s);
-    } else {
-      const Cx<float> *bv = b + 2 * V * v;
-#pragma unroll
-      for (int k = 0; k < 5; ++k) w[k] = load_pair(bv, nb[k]);
-    }
-    ux0 = h2c(U[2 * s], 1.f);
-    ux1 = h2c(U[2 * s + 1], 1.f);
-    ub0 = h2c(U[2 * n.m0], 1.f);
-    ub1 = h2c(U[2 * n.m1 + 1], 1.f);
-  }
   Cx<float> alpha = z;
-  if (STEP) alpha = mr_alpha<float>(part_in + 3LL * nb_in * v, nb_in, omega, sh);  // all threads of the block
   float acc[3] = {0.f, 0.f, 0.f};
-  if (live) {
-    if (STEP) {
-      cmac(xs.a, alpha, w[0].a);
-      cmac(xs.b, alpha, w[0].b);
-      reinterpret_cast<Pair<float> *>(x + 2 * V * v)[s] = xs;
-      const Cx<float> ma = mk(-alpha.re, -alpha.im);
+  const long long sb = blockIdx.x * 256LL;
+  long long s0 = sb;
+  do {
+    const long long s = s0 + threadIdx.x;
+    const bool live = s < V;
+    Pair<float> w[5], a[5];  // self, +0, +1, -0, -1
 #pragma unroll
-      for (int k = 0; k < 5; ++k) {
-        w[k].a = mr_step(w[k].a, a[k].a, ma);
-        w[k].b = mr_step(w[k].b, a[k].b, ma);
+    for (int k = 0; k < 5; ++k) w[k].a = w[k].b = a[k].a = a[k].b = z;
+    Pair<float> xs;
+    xs.a = xs.b = z;
+    Cx<float> ux0 = z, ux1 = z, ub0 = z, ub1 = z;
+    if (live) {
+      const Nbr n = neighbours(s, L0, L1);
+      const long long nb[5] = {s, n.p0, n.p1, n.m0, n.m1};
+      if (STEP) {
+        const HalfField ro = half_field(r_old, V, v), ao = half_field(Ar_old, V, v);
+#pragma unroll
+        for (int k = 0; k < 5; ++k) {
+          w[k] = load_site(ro.h, ro.n, nb[k]);
+          a[k] = load_site(ao.h, ao.n, nb[k]);
+        }
+        if (!x_init) xs = load_pair(x + 2 * V * v, s);
+      } else {
+        const Cx<float> *bv = b + 2 * V * v;
+#pragma unroll
+        for (int k = 0; k < 5; ++k) w[k] = load_pair(bv, nb[k]);
       }
+      ux0 = h2c(U[2 * s], 1.f);
+      ux1 = h2c(U[2 * s + 1], 1.f);
+      ub0 = h2c(U[2 * n.m0], 1.f);
+      ub1 = h2c(U[2 * n.m1 + 1], 1.f);
     }
-    const HalfField rn = half_field(r_new, V, v), an = half_field(Ar_new, V, v);
-    store_site(rn.h, rn.n, s, w[0].a, w[0].b);
-    const Pair<float> o = wilson_at(w[0], w[1], w[2], w[3], w[4], ux0, ux1, ub0, ub1, diag);
-    store_site(an.h, an.n, s, o.a, o.b);
-    const Cx<float> s0 = w[0].a, s1 = w[0].b, a0 = o.a, a1 = o.b;
-    acc[0] = a0.re * s0.re + a0.im * s0.im + a1.re * s1.re + a1.im * s1.im;
-    acc[1] = a0.re * s0.im - a0.im * s0.re + a1.re * s1.im - a1.im * s1.re;
-    acc[2] = a0.re * a0.re + a0.im * a0.im + a1.re * a1.re + a1.im * a1.im;
-  }
+    if (STEP && (!LOOP || s0 == sb))
+      alpha = mr_alpha<float>(part_in + 3LL * nb_in * v, nb_in, omega, sh);  // all threads of the block
+    if (live) {
+      if (STEP) {
+        cmac(xs.a, alpha, w[0].a);
+        cmac(xs.b, alpha, w[0].b);
+        reinterpret_cast<Pair<float> *>(x + 2 * V * v)[s] = xs;
+        const Cx<float> ma = mk(-alpha.re, -alpha.im);
+#pragma unroll
+        for (int k = 0; k < 5; ++k) {
+          w[k].a = mr_step(w[k].a, a[k].a, ma);
+          w[k].b = mr_step(w[k].b, a[k].b, ma);
+        }
+      }
+      const HalfField rn = half_field(r_new, V, v), an = half_field(Ar_new, V, v);
+      store_site(rn.h, rn.n, s, w[0].a, w[0].b);
+      const Pair<float> o = wilson_at(w[0], w[1], w[2], w[3], w[4], ux0, ux1, ub0, ub1, diag);
+      store_site(an.h, an.n, s, o.a, o.b);
+      const Cx<float> p0 = w[0].a, p1 = w[0].b, a0 = o.a, a1 = o.b;
+      acc[0] += a0.re * p0.re + a0.im * p0.im + a1.re * p1.re + a1.im * p1.im;
+      acc[1] += a0.re * p0.im - a0.im * p0.re + a1.re * p1.im - a1.im * p1.re;
+      acc[2] += a0.re * a0.re + a0.im * a0.im + a1.re * a1.re + a1.im * a1.im;
+    }
+    s0 += gridDim.x * 256LL;
+  } while (LOOP && s0 < V);
   mr_publish<float>(acc, part_out + 3LL * gridDim.x * v, sh);
 }
 
@@ -406,7 +412,7 @@ void launch_half_convert(int what, int precision, const void *in, void *out, lon
   MG_LAUNCHED();
 }
 
-int mr_half_grid(Geo2 g) { return (int)grid_for(g.nsites, 256); }
+static int mr_half_grid(Geo2 g) { return mr_blocks((g.nsites + 255) / 256); }
 
 void launch_mr_iteration_half(const void *U16, Geo2 g, double diag, const double *shift, bool step,
                               const Cx<float> *b, void *r_old, void *Ar_old, const float *part_in, double omega,
@@ -417,21 +423,22 @@ void launch_mr_iteration_half(const void *U16, Geo2 g, double diag, const double
   if (3LL * nb * nvec > part_capacity) fail(MG_ERR_STATE, "MR reduction workspace too small");
   const dim3 grid(nb, nvec);
   const __half2 *U = static_cast<const __half2 *>(U16);
-  if (step)
-    mr_wilson_half_kernel<true><<<grid, 256, 0, s>>>(U, nullptr, r_old, Ar_old, part_in, nb, omega, x, x_init ? 1 : 0,
-                                                     r_new, Ar_new, g.L0, g.L1, (float)diag, part_out, shift);
+  auto run = [&](auto kernel) {
+    kernel<<<grid, 256, 0, s>>>(U, b, r_old, Ar_old, part_in, nb, omega, x, step && x_init ? 1 : 0, r_new, Ar_new,
+                                g.L0, g.L1, (float)diag, part_out, shift);
+  };
+  if (nb * 256LL < g.nsites)  // the blocks stride
+    step ? run(mr_wilson_half_kernel<true, true>) : run(mr_wilson_half_kernel<false, true>);
   else
-    mr_wilson_half_kernel<false><<<grid, 256, 0, s>>>(U, b, nullptr, nullptr, nullptr, nb, omega, nullptr, 0, r_new,
-                                                      Ar_new, g.L0, g.L1, (float)diag, part_out, shift);
+    step ? run(mr_wilson_half_kernel<true, false>) : run(mr_wilson_half_kernel<false, false>);
   MG_LAUNCHED();
 }
 
 void launch_mr_last_half(void *r_old, void *Ar_old, const float *part_in, double omega, Cx<float> *x, bool x_init,
                          Cx<float> *r_out, Geo2 g, cudaStream_t s, int nvec) {
-  long long blocks = (g.nsites + 255) / 256;
-  if (blocks > 152LL * 16) blocks = 152LL * 16;
-  mr_last_half_kernel<<<dim3((unsigned int)(blocks < 1 ? 1 : blocks), nvec), 256, 0, s>>>(
-      r_old, Ar_old, part_in, mr_half_grid(g), omega, x, x_init ? 1 : 0, r_out, g.nsites);
+  const int blocks = mr_half_grid(g);
+  mr_last_half_kernel<<<dim3((unsigned int)blocks, nvec), 256, 0, s>>>(
+      r_old, Ar_old, part_in, blocks, omega, x, x_init ? 1 : 0, r_out, g.nsites);
   MG_LAUNCHED();
 }
 
