@@ -23,6 +23,7 @@
 #include <mutex>
 
 #include "kernels.h"
+#include "stencil8.cuh"
 
 namespace mg {
 
@@ -352,6 +353,181 @@ __global__ void __launch_bounds__(256) coarsest_gcr_kernel(CgArgs<VT> a) {
 }
 
 // ---------------------------------------------------------------------------
+// The same solve for FP32 vectors and N = 8 (mixed-precision cycles, loose tolerance, coarsest levels
+// above the cluster kernel's 8192 dofs). A CTA owns a contiguous chunk of sites: the stencil by a warp
+// per site with 16-byte loads, the next site's blocks requested while one is summed (stencil8.cuh),
+// the vector work by a thread per dof. Gram-Schmidt is classical in one pass, with a second one only
+// where |w'|^2 < |w|^2 / 2 (every CTA decides from the same sums), so an iteration is one grid sum
+// and one barrier; sums inside a warp are FP32, across warps and CTAs FP64, as in the cluster kernel.
+// The thread-per-row form on a quarter of the SMs, two passes always, took 563 us per solve at 98304
+// dofs (1024 x 768 fine lattice), this one 200 us (a whole fine solve 81.5 -> 64.5 ms; on half or a
+// quarter of the SMs 65.9 and 68.6 ms).
+// ---------------------------------------------------------------------------
+constexpr int kGcr8Warps = 16;
+
+__device__ __forceinline__ void warp_put32(float t, int s, double *swarp) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+  if ((threadIdx.x & 31) == 0) swarp[(threadIdx.x >> 5) * kSlots + s] = (double)t;
+}
+
+// f(j, value) for every site j of the chunk: the lane's component of (A M v)_j (v through L2: other
+// CTAs wrote the neighbours' values)
+template <typename F>
+__device__ __forceinline__ void chunk_stencil8(const CgArgs<float> &a, const Cx<float> *v, int j0, int j1,
+                                               const Lane8 &l, F &&f) {
+  int j = j0 + (int)(threadIdx.x >> 5);
+  float4 y[5], yn[5];
+  if (j < j1) load_blocks8(a.Y, j, l, y);
+  for (; j < j1; j += kGcr8Warps) {
+    const Site8 st(j, a.L0, a.L1);
+    float2 w[5];
+#pragma unroll
+    for (int d = 0; d < 5; ++d) w[d] = __ldcg(reinterpret_cast<const float2 *>(v) + (long long)st.nb[d] * 8 + l.q);
+    if (j + kGcr8Warps < j1) load_blocks8(a.Y, j + kGcr8Warps, l, yn);
+    f(j, stencil8(y, w, l));
+#pragma unroll
+    for (int d = 0; d < 5; ++d) y[d] = yn[d];
+  }
+}
+
+__global__ void __launch_bounds__(32 * kGcr8Warps, 1) coarsest_gcr8_kernel(CgArgs<float> a) {
+  extern __shared__ double sdyn[];
+  double *swarp = sdyn;                        // kGcr8Warps x kSlots
+  double *sres = sdyn + kGcr8Warps * kSlots;   // kSlots
+  double *stage = sres + kSlots;               // G x kSlots
+  const Lane8 l;
+  const int sites = a.L0 * a.L1, per = (sites + (int)gridDim.x - 1) / (int)gridDim.x;
+  const int j0 = min(sites, (int)blockIdx.x * per), j1 = min(sites, j0 + per);
+  const long long n = a.n, d0 = (long long)j0 * 8 + threadIdx.x, d1 = (long long)j1 * 8;
+  constexpr int kStep = 32 * kGcr8Warps;
+  bool ok = true;
+
+  double t0 = 0.0;
+  for (long long i = d0; i < d1; i += kStep) {
+    const Cx<double> bi = a.b[i];
+    a.y[i] = mk(0.f, 0.f);
+    a.r[i] = cvt<float, double>(bi);
+    t0 += norm2(bi);
+  }
+  warp_put(t0, 0, swarp);
+  grid_sum(a, 1, swarp, stage, sres, ok);
+  if (!ok) return;
+  const double bn2 = sres[0];
+  const double tol2 = a.tol * a.tol * bn2;
+  int it = 0;
+  bool converged = !(bn2 > 0.0);
+  double rn2 = bn2;
+  while (!converged && it < a.max_iter) {
+    for (int k = 0; k < a.restart && it < a.max_iter; ++k) {
+      Cx<float> *Zk = a.Z + (long long)k * n, *Wk = a.W + (long long)k * n;
+      // w = (A M) r, z = r
+      chunk_stencil8(a, a.r, j0, j1, l, [&](int j, float v) {
+        if (l.writes) reinterpret_cast<float *>(Wk)[((long long)j * 8 + l.row) * 2 + l.im] = v;
+      });
+      for (long long i = d0; i < d1; i += kStep) Zk[i] = a.r[i];
+      bool breakdown = false;
+      double inv = 0.0, ar = 0.0, ai = 0.0;
+      for (int pass = 0;; ++pass) {
+        __syncthreads();
+        for (int q = 0; q < k; ++q) {
+          const Cx<float> *Wq = a.W + (long long)q * n;
+          float re = 0.f, im = 0.f;
+          for (long long i = d0; i < d1; i += kStep) {
+            const Cx<float> wj = Wq[i], w = Wk[i];
+            re = fmaf(wj.re, w.re, fmaf(wj.im, w.im, re));
+            im = fmaf(wj.re, w.im, fmaf(-wj.im, w.re, im));
+          }
+          warp_put32(re, 3 + 2 * q, swarp);
+          warp_put32(im, 4 + 2 * q, swarp);
+        }
+        float nn = 0.f, wr = 0.f, wi = 0.f;
+        for (long long i = d0; i < d1; i += kStep) {
+          const Cx<float> w = Wk[i], ri = a.r[i];
+          nn = fmaf(w.re, w.re, fmaf(w.im, w.im, nn));
+          wr = fmaf(w.re, ri.re, fmaf(w.im, ri.im, wr));
+          wi = fmaf(w.re, ri.im, fmaf(-w.im, ri.re, wi));
+        }
+        warp_put32(nn, 0, swarp);
+        warp_put32(wr, 1, swarp);
+        warp_put32(wi, 2, swarp);
+        grid_sum(a, 3 + 2 * k, swarp, stage, sres, ok);
+        if (!ok) return;
+        double nw2 = sres[0];
+        for (int q = 0; q < k; ++q) nw2 -= sres[3 + 2 * q] * sres[3 + 2 * q] + sres[4 + 2 * q] * sres[4 + 2 * q];
+        const bool again = pass == 0 && k > 0 && !(nw2 > 0.5 * sres[0]);
+        breakdown = !(nw2 > 1e-28 * sres[0]);
+        inv = breakdown ? 0.0 : 1.0 / sqrt(nw2);
+        ar = sres[1] * inv;  // <w_hat, r>
+        ai = sres[2] * inv;
+        if (!again) break;
+        for (long long i = d0; i < d1; i += kStep) {  // project, then take fresh coefficients
+          Cx<float> w = Wk[i], z = Zk[i];
+          for (int q = 0; q < k; ++q) {
+            const Cx<float> bj = mk((float)-sres[3 + 2 * q], (float)-sres[4 + 2 * q]);
+            cmac(w, bj, a.W[(long long)q * n + i]);
+            cmac(z, bj, a.Z[(long long)q * n + i]);
+          }
+          Wk[i] = w;
+          Zk[i] = z;
+        }
+      }
+      const Cx<float> alpha = mk((float)ar, (float)ai);
+      const float vinv = (float)inv;
+      for (long long i = d0; i < d1; i += kStep) {
+        Cx<float> w = Wk[i], z = Zk[i];
+        for (int q = 0; q < k; ++q) {
+          const Cx<float> bj = mk((float)-sres[3 + 2 * q], (float)-sres[4 + 2 * q]);
+          cmac(w, bj, a.W[(long long)q * n + i]);
+          cmac(z, bj, a.Z[(long long)q * n + i]);
+        }
+        w = vinv * w;
+        z = vinv * z;
+        Wk[i] = w;
+        Zk[i] = z;
+        cmac(a.y[i], alpha, z);
+        Cx<float> ri = a.r[i];
+        cmac(ri, mk(-alpha.re, -alpha.im), w);
+        a.r[i] = ri;
+      }
+      rn2 = fmax(rn2 - (ar * ar + ai * ai), 0.0);
+      ++it;
+      grid_sync(a, ok);
+      if (!ok) return;
+      if (rn2 <= tol2 || breakdown) break;
+    }
+    // true residual r = b - (A M) y; the CTA's own r is read by no other CTA until the sum below
+    chunk_stencil8(a, a.y, j0, j1, l, [&](int j, float v) {
+      const long long e = ((long long)j * 8 + l.row) * 2 + l.im;
+      if (l.writes) reinterpret_cast<float *>(a.r)[e] = (float)(reinterpret_cast<const double *>(a.b)[e] - (double)v);
+    });
+    __syncthreads();
+    float tr = 0.f;
+    for (long long i = d0; i < d1; i += kStep) tr += norm2(a.r[i]);
+    warp_put32(tr, 0, swarp);
+    grid_sum(a, 1, swarp, stage, sres, ok);
+    if (!ok) return;
+    rn2 = sres[0];
+    converged = rn2 <= tol2;
+    if (!(rn2 == rn2)) break;  // NaN: stop; reported through out_rel
+  }
+  // x = M y (site-local)
+  for (long long i = d0; i < d1; i += kStep) {
+    const long long j = i >> 3;
+    const Cx<double> *Mj = a.Minv + j * 64 + (i & 7);
+    Cx<double> acc = mk(0.0, 0.0);
+#pragma unroll
+    for (int c = 0; c < 8; ++c) cmac(acc, Mj[c * 8], cvt<double, float>(a.y[j * 8 + c]));
+    a.x[i] = acc;
+  }
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    atomicAdd(a.out, it);
+    if (!converged) atomicAdd(a.out + 2, 1);
+    a.out_rel[0] = bn2 > 0.0 ? sqrt(rn2 / bn2) : 0.0;
+  }
+}
+
+// ---------------------------------------------------------------------------
 // block-Jacobi preparation: Minv_j = X_j^{-1} (Gauss-Jordan with partial
 // pivoting, one thread per coarse site) and the stencil A M
 // ---------------------------------------------------------------------------
@@ -506,8 +682,15 @@ static void coarsest_gcr_go(const Cx<VT> *Yt, const Cx<double> *Minv, Geo2 g, in
   int threads = (int)((per + 31) / 32) * 32;
   if (threads < 64) threads = 64;
   if (threads > 256) threads = 256;
-  const size_t smem = (size_t)(9 + grid) * kSlots * sizeof(double);
-  const void *fn = (N == 8) ? (const void *)coarsest_gcr_kernel<8, VT> : (const void *)coarsest_gcr_kernel<0, VT>;
+  size_t smem = (size_t)(9 + grid) * kSlots * sizeof(double);
+  const void *fn = (const void *)coarsest_gcr_kernel<0, VT>;
+  if constexpr (sizeof(VT) == 8) {
+    if (N == 8) fn = (const void *)coarsest_gcr_kernel<8, VT>;
+  } else if (N == 8) {
+    fn = (const void *)coarsest_gcr8_kernel;
+    threads = 32 * kGcr8Warps;
+    smem = (size_t)(kGcr8Warps + 1 + grid) * kSlots * sizeof(double);
+  }
   MG_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   int per_sm = 0;
   MG_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessorWithFlags(&per_sm, fn, threads, smem, 0));

@@ -445,11 +445,9 @@ static void coarsest_solve64(mg_ctx &c, const Cx<double> *b, Cx<double> *x, int 
                              c.p.coarsest_tol, c.p.coarsest_restart, c.p.coarsest_max_iter, c.cg_out.p, c.cg_rel.p,
                              c.cg_grid, c.s);
   else if (c.cg_large32 && slot == 0)
-    // a quarter of the SMs: the FP32 solve is latency-bound (grid barriers over fewer CTAs are
-    // cheaper), and the other SMs stay free for the non-cooperative work of concurrent streams
     launch_coarsest_gcr32(c.cg_Yt32.p, Minv, L.geo, L.nint, b, x, c.cy32.p, c.cr32.p, c.cZ32.p, c.cW32.p,
                           c.cg_partials.p, c.cg_bar.p, c.p.coarsest_tol, c.p.coarsest_restart, c.p.coarsest_max_iter,
-                          c.cg_out.p, c.cg_rel.p, std::max(1, c.cg_grid / 4), c.s);
+                          c.cg_out.p, c.cg_rel.p, c.cg_grid, c.s);
   else
     launch_coarsest_gcr(Yt, Minv, L.geo, L.nint, b, x, c.cg_y.p, c.cr.p, c.cZ.p, c.cW.p,
                         c.cg_partials.p, c.cg_bar.p, c.p.coarsest_tol, c.p.coarsest_restart, c.p.coarsest_max_iter,

@@ -56,3 +56,22 @@ def test_fp32_batches_match_single_solves(nrhs):
         # both residuals at 1e-12, |D^-1| below 10 at these masses
         assert np.linalg.norm(to_host(psi)[v] - to_host(one)) < 1e-10 * np.linalg.norm(to_host(one))
     ctx.close()
+
+
+@pytest.mark.parametrize("tol", [0.2, 1e-3, 1e-5])
+@pytest.mark.parametrize("ext", [(41, 35), (64, 48)])
+def test_fp32_large_coarsest_solve_meets_its_tolerance(ext, tol):
+    # more dofs than the cluster and the shared-memory kernels take (9728), chunks of sites of uneven length
+    import torch
+    import paper_0707_4018_gb300 as mg
+    dims = (4 * ext[0], 4 * ext[1])
+    p = mg.mg_default_params(levels=2, blocks=[(4, 4)], Nv=[8], n_pass=1, precision=mg.MG_FP32, coarsest_tol=tol)
+    ctx = mg.Context.setup(to_dev(inputs.hot_links(*dims, seed=28)), 0.2, dims, p)
+    b = to_dev(inputs.gaussian_spinor(ext[0] * ext[1], 8, 29, 0))
+    x, y = torch.empty_like(b), torch.empty_like(b)
+    iters, _ = ctx.coarsest_solve(b, x)
+    ctx.level_apply(1, x, y)
+    # the kernel's true residual is taken in FP32: 40 products and sums per dof, rounding below 1e-5 of |A| |x|
+    assert iters > 0
+    assert float(torch.linalg.norm(b - y) / torch.linalg.norm(b)) <= tol + 1e-5
+    ctx.close()
