@@ -79,6 +79,38 @@ __global__ void mr_update_kernel(const double *__restrict__ sc, double omega, Cx
   }
 }
 
+// This thread's part of <a, b> (SAME: |a|^2, real): the FP64 rate bounds these reductions (two multiply-adds
+// per clock and SM), so exactly four of them per complex product, two for a norm; as sums of products
+// they were six DP instructions for every row. Four elements are in flight per thread.
+template <typename VT>
+__device__ __forceinline__ void dot_part(const Cx<VT> *__restrict__ a, const Cx<VT> *__restrict__ b, bool same,
+                                         long long n, VT &t0, VT &t1) {
+  const long long step = (long long)gridDim.x * blockDim.x;
+  long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  if (same) {
+#pragma unroll 4
+    for (; i < n; i += step) {
+      const Cx<VT> x = a[i];
+      t0 = fma(x.re, x.re, t0);
+      t0 = fma(x.im, x.im, t0);
+    }
+  } else {
+#pragma unroll 4
+    for (; i < n; i += step) {
+      const Cx<VT> x = a[i], y = b[i];
+      t0 = fma(x.re, y.re, t0);
+      t1 = fma(x.re, y.im, t1);
+      t0 = fma(x.im, y.im, t0);
+      t1 = fma(-x.im, y.re, t1);
+    }
+  }
+}
+
+// Blocks per reduction: at least eight elements per thread, so that the block and grid trees (FP64
+// too) stay small beside the products; one element per thread and 512 blocks per row took 50 us at
+// n = 131072 (256^2), more than its products by a factor of eight.
+static int dot_blocks(long long n, int per) { return reduce_blocks((n + 7) / 8, per); }
+
 // rows j < k: <W_j, w>; row k: <w, w>; row k + 1: <w, r>; row k + 2: <r, r>  (blockIdx.y = row)
 // (VT = float: FP32 vectors; each thread sums its few products in FP32, the block and grid
 // trees sum in FP64)
@@ -97,11 +129,7 @@ __global__ void __launch_bounds__(kReduceThreads) gcr_dots_kernel(const Cx<VT> *
   const Cx<VT> *a = row < k ? W + (long long)row * n : (row == k + 2 ? r : w);
   const Cx<VT> *b = row > k ? r : w;
   VT t0 = (VT)0, t1 = (VT)0;
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-    const Cx<VT> x = a[i], y = b[i];
-    t0 += x.re * y.re + x.im * y.im;
-    t1 += x.re * y.im - x.im * y.re;
-  }
+  dot_part<VT>(a, b, row == k || row == k + 2, n, t0, t1);
   double v[2] = {(double)t0, (double)t1};
   grid_finish<2>(v, partials + (long long)row * pstride, out + 2 * row, ticket + row, sh);
 }
@@ -140,7 +168,7 @@ static void gcr_dots_any(const Cx<VT> *W, const Cx<VT> *w, const Cx<VT> *r, int 
   int per = (int)(ws.capacity / (2 * rows));
   if (per > ws.max_blocks) per = ws.max_blocks;
   if (per < 1) per = 1;
-  dim3 grid(reduce_blocks(n, per), rows);
+  dim3 grid(dot_blocks(n, per), rows);
   gcr_dots_kernel<VT><<<grid, kReduceThreads, 0, s>>>(W, w, r, k, nullptr, n, ws.partials, out, ws.ticket,
                                                       2 * (int)grid.x);
   MG_LAUNCHED();
@@ -155,7 +183,7 @@ void launch_gcr_dots_kdev(const Cx<VT> *W, const Cx<VT> *w, const Cx<VT> *r, con
   int per = (int)(ws.capacity / (2 * rows));
   if (per > ws.max_blocks) per = ws.max_blocks;
   if (per < 1) per = 1;
-  dim3 grid(reduce_blocks(n, per), rows);
+  dim3 grid(dot_blocks(n, per), rows);
   gcr_dots_kernel<VT><<<grid, kReduceThreads, 0, s>>>(W, w, r, 0, kdev, n, ws.partials, out, ws.ticket,
                                                       2 * (int)grid.x);
   MG_LAUNCHED();
@@ -228,11 +256,7 @@ __global__ void __launch_bounds__(kReduceThreads) gcr_dots_batch_kernel(const Cx
   const Cx<VT> *a = row < k ? W + ((long long)row * nb + v) * n : (row == k + 2 ? rv : w);
   const Cx<VT> *b = row > k ? rv : w;
   VT t0 = (VT)0, t1 = (VT)0;
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-    const Cx<VT> x = a[i], y = b[i];
-    t0 += x.re * y.re + x.im * y.im;
-    t1 += x.re * y.im - x.im * y.re;
-  }
+  dot_part<VT>(a, b, row == k || row == k + 2, n, t0, t1);
   double acc[2] = {(double)t0, (double)t1};
   const long long slot = (long long)v * rows + row;
   grid_finish<2>(acc, partials + slot * 2 * gridDim.x, out + 2 * slot, ticket + slot, sh);
@@ -350,7 +374,7 @@ void launch_gcr_dots_batch(const Cx<VT> *W, const Cx<VT> *r, int k, int nb, long
   int per = (int)(ws.capacity / (2LL * rows * nb));
   if (per > ws.max_blocks) per = ws.max_blocks;
   if (per < 1) fail(MG_ERR_STATE, "gcr_dots_batch: reduction workspace too small");
-  gcr_dots_batch_kernel<VT><<<dim3(reduce_blocks(n, per), rows, nb), kReduceThreads, 0, s>>>(W, r, k, nb, n,
+  gcr_dots_batch_kernel<VT><<<dim3(dot_blocks(n, per), rows, nb), kReduceThreads, 0, s>>>(W, r, k, nb, n,
                                                                                              ws.partials, out,
                                                                                              ws.ticket);
   MG_LAUNCHED();
@@ -451,7 +475,7 @@ template void launch_convert<double, float>(const Cx<float> *, Cx<double> *, lon
 namespace mg {
 
 // rows j < k: <W_j, w>; row k: |w|^2; row k + 1: <w, r>; row k + 2: |r|^2, with k = ctl[1];
-// the grid has restart + 3 rows, the rows above k + 2 only finish their (empty) reduction
+// the grid has restart + 3 rows, those above k + 2 return at once (all blocks alike: their tickets stay)
 __global__ void __launch_bounds__(kReduceThreads) gcr_dots_devk_kernel(const Cx<double> *__restrict__ W,
                                                                        const Cx<double> *__restrict__ w,
                                                                        const Cx<double> *__restrict__ r,
@@ -460,17 +484,11 @@ __global__ void __launch_bounds__(kReduceThreads) gcr_dots_devk_kernel(const Cx<
                                                                        unsigned int *ticket, int pstride) {
   __shared__ double sh[32 * 2];
   const int row = blockIdx.y, k = ctl[1];
+  if (row > k + 2) return;
+  const Cx<double> *a = row < k ? W + (long long)row * n : (row == k + 2 ? r : w);
+  const Cx<double> *b = row > k ? r : w;
   double v[2] = {0.0, 0.0};
-  if (row <= k + 2) {
-    const Cx<double> *a = row < k ? W + (long long)row * n : (row == k + 2 ? r : w);
-    const Cx<double> *b = row > k ? r : w;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
-         i += (long long)gridDim.x * blockDim.x) {
-      const Cx<double> x = a[i], y = b[i];
-      v[0] += x.re * y.re + x.im * y.im;
-      v[1] += x.re * y.im - x.im * y.re;
-    }
-  }
+  dot_part<double>(a, b, row == k || row == k + 2, n, v[0], v[1]);
   grid_finish<2>(v, partials + (long long)row * pstride, out + 2 * row, ticket + row, sh);
 }
 
@@ -548,7 +566,7 @@ void launch_gcr_dots_devk(const Cx<double> *W, const Cx<double> *w, const Cx<dou
   int per = (int)(ws.capacity / (2 * rows));
   if (per > ws.max_blocks) per = ws.max_blocks;
   if (per < 1) per = 1;
-  dim3 grid(reduce_blocks(n, per), rows);
+  dim3 grid(dot_blocks(n, per), rows);
   gcr_dots_devk_kernel<<<grid, kReduceThreads, 0, s>>>(W, w, r, ctl, n, ws.partials, out, ws.ticket, 2 * (int)grid.x);
   MG_LAUNCHED();
 }
@@ -604,11 +622,7 @@ __global__ void __launch_bounds__(kReduceThreads) gcr_dots_batch_devk_kernel(
   const Cx<VT> *a = row < k ? W + ((long long)row * nb + v) * n : (row == k + 2 ? rv : wv);
   const Cx<VT> *b = row > k ? rv : wv;
   VT t0 = (VT)0, t1 = (VT)0;
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-    const Cx<VT> x = a[i], y = b[i];
-    t0 += x.re * y.re + x.im * y.im;
-    t1 += x.re * y.im - x.im * y.re;
-  }
+  dot_part<VT>(a, b, row == k || row == k + 2, n, t0, t1);
   double acc[2] = {(double)t0, (double)t1};
   const long long slot = (long long)v * rows + row;
   grid_finish<2>(acc, partials + slot * 2 * gridDim.x, out + 2 * slot, ticket + slot, sh);
@@ -706,7 +720,7 @@ void launch_gcr_dots_batch_devk(const Cx<VT> *W, const Cx<VT> *w, const Cx<VT> *
   if (per > ws.max_blocks) per = ws.max_blocks;
   if (per < 1) per = 1;
   if ((long long)rows * nb > ws.tickets) fail(MG_ERR_UNSUPPORTED, "gcr_dots_batch: too many reduction slots");
-  gcr_dots_batch_devk_kernel<VT><<<dim3(reduce_blocks(n, per), rows, nb), kReduceThreads, 0, s>>>(
+  gcr_dots_batch_devk_kernel<VT><<<dim3(dot_blocks(n, per), rows, nb), kReduceThreads, 0, s>>>(
       W, w, r, ctl, nb, restart, n, ws.partials, out, ws.ticket);
   MG_LAUNCHED();
 }
