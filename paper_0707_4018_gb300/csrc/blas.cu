@@ -134,29 +134,38 @@ __global__ void __launch_bounds__(kReduceThreads) gcr_dots_kernel(const Cx<VT> *
   grid_finish<2>(v, partials + (long long)row * pstride, out + 2 * row, ticket + row, sh);
 }
 
-// w <- (w - sum_j beta_j W_j) * inv, z likewise; W_k = w, Z_k = z; x += alpha z; r -= alpha w
-__global__ void gcr_project_update_kernel(const Cx<double> *__restrict__ W, Cx<double> *__restrict__ Wk,
-                                          const Cx<double> *__restrict__ Z, Cx<double> *__restrict__ Zk, int k,
+// W_k <- (W_k - sum_j beta_j W_j) inv; with update_r also r -= alpha W_k (the solution is formed at the end of
+// the cycle, krylov.h)
+__global__ void gcr_project_update_kernel(const Cx<double> *__restrict__ W, Cx<double> *__restrict__ Wk, int k,
                                           const double *__restrict__ beta, double inv, double are, double aim,
-                                          Cx<double> *__restrict__ x, Cx<double> *__restrict__ r, long long n,
-                                          int update_xr) {
+                                          Cx<double> *__restrict__ r, long long n, int update_r) {
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-    Cx<double> w = Wk[i], z = Zk[i];
-    for (int j = 0; j < k; ++j) {
-      const Cx<double> bj = mk(-beta[2 * j], -beta[2 * j + 1]);
-      cmac(w, bj, W[(long long)j * n + i]);
-      cmac(z, bj, Z[(long long)j * n + i]);
-    }
+    Cx<double> w = Wk[i];
+#pragma unroll 4
+    for (int j = 0; j < k; ++j) cmac(w, mk(-beta[2 * j], -beta[2 * j + 1]), W[(long long)j * n + i]);
     w = inv * w;
-    z = inv * z;
     Wk[i] = w;
-    Zk[i] = z;
-    if (update_xr) {
-      cmac(x[i], mk(are, aim), z);
+    if (update_r) {
       Cx<double> ri = r[i];
       cmac(ri, mk(-are, -aim), w);
       r[i] = ri;
     }
+  }
+}
+
+// x_v += sum_j<k y_j Z_j,v for vector v = blockIdx.y (y: 2 k doubles per vector; Z[j][v][n], nb vectors)
+template <typename VT>
+__global__ void gcr_solution_kernel(const Cx<VT> *__restrict__ Z, int k, int nb, const double *__restrict__ y,
+                                    Cx<VT> *__restrict__ x, long long n) {
+  const int v = blockIdx.y;
+  y += 2LL * k * v;
+  x += (long long)v * n;
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
+    Cx<VT> t = x[i];
+#pragma unroll 4
+    for (int j = 0; j < k; ++j)
+      cmac(t, mk((VT)y[2 * j], (VT)y[2 * j + 1]), Z[((long long)j * nb + v) * n + i]);
+    x[i] = t;
   }
 }
 
@@ -201,16 +210,27 @@ void launch_gcr_dots(const Cx<float> *W, const Cx<float> *w, const Cx<float> *r,
   gcr_dots_any<float>(W, w, r, k, n, out, ws, s);
 }
 
-void launch_gcr_project_update(const Cx<double> *W, Cx<double> *Wk, const Cx<double> *Z, Cx<double> *Zk, int k,
-                               const double *beta_dev, double inv, double are, double aim, Cx<double> *x,
-                               Cx<double> *r, long long n, bool update_xr, cudaStream_t s) {
+void launch_gcr_project_update(const Cx<double> *W, Cx<double> *Wk, int k, const double *beta_dev, double inv,
+                               double are, double aim, Cx<double> *r, long long n, bool update_r, cudaStream_t s) {
   long long b = (n + 255) / 256;
   if (b > 152LL * 16) b = 152LL * 16;
-  gcr_project_update_kernel<<<(unsigned int)(b < 1 ? 1 : b), 256, 0, s>>>(W, Wk, Z, Zk, k, beta_dev, inv, are, aim, x,
-                                                                          r, n, update_xr ? 1 : 0);
+  gcr_project_update_kernel<<<(unsigned int)(b < 1 ? 1 : b), 256, 0, s>>>(W, Wk, k, beta_dev, inv, are, aim, r, n,
+                                                                          update_r ? 1 : 0);
   MG_LAUNCHED();
 }
 
+template <typename VT>
+void launch_gcr_solution(const Cx<VT> *Z, int k, int nb, const double *y_dev, Cx<VT> *x, long long n,
+                         cudaStream_t s) {
+  long long b = (n + 255) / 256;
+  if (b > 152LL * 16) b = 152LL * 16;
+  gcr_solution_kernel<VT><<<dim3((unsigned int)(b < 1 ? 1 : b), nb), 256, 0, s>>>(Z, k, nb, y_dev, x, n);
+  MG_LAUNCHED();
+}
+template void launch_gcr_solution<double>(const Cx<double> *, int, int, const double *, Cx<double> *, long long,
+                                          cudaStream_t);
+template void launch_gcr_solution<float>(const Cx<float> *, int, int, const double *, Cx<float> *, long long,
+                                         cudaStream_t);
 
 // ---------------------------------------------------------------------------
 // batched outer GCR (FP64): nb systems in lockstep, vector v of a batch at v * n;
@@ -262,35 +282,27 @@ __global__ void __launch_bounds__(kReduceThreads) gcr_dots_batch_kernel(const Cx
   grid_finish<2>(acc, partials + slot * 2 * gridDim.x, out + 2 * slot, ticket + slot, sh);
 }
 
-// per vector v (blockIdx.y), coef[4 v .. 4 v + 3] = (inv, alpha re, alpha im, mode):
-// mode 0 leaves the vector alone; mode 2 projects w_k, z_k against the basis with beta_j =
-// dots[v * 2 (k + 3) + 2 j]; mode 1 projects, scales both by inv and updates x += alpha z_k,
-// r -= alpha w_k
+// per vector v (blockIdx.y), coef[4 v .. 4 v + 3] = (inv, alpha re, alpha im, mode): mode 0 leaves the
+// vector alone; mode 2 projects w_k against the basis with beta_j = dots[v * 2 (k + 3) + 2 j]; mode 1
+// projects, scales by inv and updates r -= alpha w_k
 template <typename VT>
-__global__ void gcr_update_batch_kernel(Cx<VT> *__restrict__ W, Cx<VT> *__restrict__ Z, int k, int nb,
-                                        const double *__restrict__ dots, const double *__restrict__ coef,
-                                        Cx<VT> *__restrict__ x, Cx<VT> *__restrict__ r, long long n) {
+__global__ void gcr_update_batch_kernel(Cx<VT> *__restrict__ W, int k, int nb, const double *__restrict__ dots,
+                                        const double *__restrict__ coef, Cx<VT> *__restrict__ r, long long n) {
   const int v = blockIdx.y;
   const int mode = (int)coef[4 * v + 3];
   if (mode == 0) return;
   const double *beta = dots + (long long)v * 2 * (k + 3);
   const VT inv = (VT)(mode == 1 ? coef[4 * v] : 1.0);
   const Cx<VT> alpha = mk((VT)coef[4 * v + 1], (VT)coef[4 * v + 2]);
-  Cx<VT> *Wk = W + ((long long)k * nb + v) * n, *Zk = Z + ((long long)k * nb + v) * n;
+  Cx<VT> *Wk = W + ((long long)k * nb + v) * n;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-    Cx<VT> w = Wk[i], z = Zk[i];
-    for (int j = 0; j < k; ++j) {
-      const Cx<VT> bj = mk((VT)-beta[2 * j], (VT)-beta[2 * j + 1]);
-      const long long o = ((long long)j * nb + v) * n + i;
-      cmac(w, bj, W[o]);
-      cmac(z, bj, Z[o]);
-    }
+    Cx<VT> w = Wk[i];
+#pragma unroll 4
+    for (int j = 0; j < k; ++j)
+      cmac(w, mk((VT)-beta[2 * j], (VT)-beta[2 * j + 1]), W[((long long)j * nb + v) * n + i]);
     w = inv * w;
-    z = inv * z;
     Wk[i] = w;
-    Zk[i] = z;
     if (mode == 1) {
-      cmac(x[(long long)v * n + i], alpha, z);
       Cx<VT> ri = r[(long long)v * n + i];
       cmac(ri, mk(-alpha.re, -alpha.im), w);
       r[(long long)v * n + i] = ri;
@@ -305,41 +317,32 @@ __global__ void gcr_update_batch_kernel(Cx<VT> *__restrict__ W, Cx<VT> *__restri
 constexpr int kLanes = 4;
 
 template <typename VT>
-__global__ void gcr_update_batch_split_kernel(Cx<VT> *__restrict__ W, Cx<VT> *__restrict__ Z, int k, int nb,
-                                              const double *__restrict__ dots, const double *__restrict__ coef,
-                                              Cx<VT> *__restrict__ x, Cx<VT> *__restrict__ r, long long n) {
+__global__ void gcr_update_batch_split_kernel(Cx<VT> *__restrict__ W, int k, int nb, const double *__restrict__ dots,
+                                              const double *__restrict__ coef, Cx<VT> *__restrict__ r, long long n) {
   const int v = blockIdx.y;
   const int mode = (int)coef[4 * v + 3];
   if (mode == 0) return;
   const double *beta = dots + (long long)v * 2 * (k + 3);
   const VT inv = (VT)(mode == 1 ? coef[4 * v] : 1.0);
   const Cx<VT> alpha = mk((VT)coef[4 * v + 1], (VT)coef[4 * v + 2]);
-  Cx<VT> *Wk = W + ((long long)k * nb + v) * n, *Zk = Z + ((long long)k * nb + v) * n;
+  Cx<VT> *Wk = W + ((long long)k * nb + v) * n;
   const int sub = threadIdx.x % kLanes, lane = threadIdx.x & 31;
   const long long stride = (long long)gridDim.x * (blockDim.x / kLanes);
   long long i = (blockIdx.x * (long long)blockDim.x + threadIdx.x) / kLanes;
   for (long long i0 = i - lane / kLanes; i0 < n; i0 += stride, i += stride) {
     const bool valid = i < n;
-    Cx<VT> pw = mk((VT)0, (VT)0), pz = mk((VT)0, (VT)0);
-    for (int j = sub; valid && j < k; j += kLanes) {
-      const Cx<VT> bj = mk((VT)-beta[2 * j], (VT)-beta[2 * j + 1]);
-      const long long o = ((long long)j * nb + v) * n + i;
-      cmac(pw, bj, W[o]);
-      cmac(pz, bj, Z[o]);
-    }
+    Cx<VT> pw = mk((VT)0, (VT)0);
+    for (int j = sub; valid && j < k; j += kLanes)
+      cmac(pw, mk((VT)-beta[2 * j], (VT)-beta[2 * j + 1]), W[((long long)j * nb + v) * n + i]);
 #pragma unroll
     for (int o = kLanes / 2; o > 0; o >>= 1) {
       pw.re += __shfl_xor_sync(0xffffffffu, pw.re, o);
       pw.im += __shfl_xor_sync(0xffffffffu, pw.im, o);
-      pz.re += __shfl_xor_sync(0xffffffffu, pz.re, o);
-      pz.im += __shfl_xor_sync(0xffffffffu, pz.im, o);
     }
     if (valid && sub == 0) {
-      const Cx<VT> w = inv * (Wk[i] + pw), z = inv * (Zk[i] + pz);
+      const Cx<VT> w = inv * (Wk[i] + pw);
       Wk[i] = w;
-      Zk[i] = z;
       if (mode == 1) {
-        cmac(x[(long long)v * n + i], alpha, z);
         Cx<VT> ri = r[(long long)v * n + i];
         cmac(ri, mk(-alpha.re, -alpha.im), w);
         r[(long long)v * n + i] = ri;
@@ -381,15 +384,14 @@ void launch_gcr_dots_batch(const Cx<VT> *W, const Cx<VT> *r, int k, int nb, long
 }
 
 template <typename VT>
-void launch_gcr_update_batch(Cx<VT> *W, Cx<VT> *Z, int k, int nb, const double *dots, const double *coef, Cx<VT> *x,
-                             Cx<VT> *r, long long n, cudaStream_t s) {
+void launch_gcr_update_batch(Cx<VT> *W, int k, int nb, const double *dots, const double *coef, Cx<VT> *r, long long n,
+                             cudaStream_t s) {
   if (n < (1LL << 18)) {  // short (coarse) vectors: kLanes lanes per element
-    gcr_update_batch_split_kernel<VT><<<dim3(stream_grid(n * kLanes), nb), 256, 0, s>>>(W, Z, k, nb, dots, coef, x,
-                                                                                        r, n);
+    gcr_update_batch_split_kernel<VT><<<dim3(stream_grid(n * kLanes), nb), 256, 0, s>>>(W, k, nb, dots, coef, r, n);
     MG_LAUNCHED();
     return;
   }
-  gcr_update_batch_kernel<VT><<<dim3(stream_grid(n), nb), 256, 0, s>>>(W, Z, k, nb, dots, coef, x, r, n);
+  gcr_update_batch_kernel<VT><<<dim3(stream_grid(n), nb), 256, 0, s>>>(W, k, nb, dots, coef, r, n);
   MG_LAUNCHED();
 }
 
@@ -398,8 +400,8 @@ void launch_gcr_update_batch(Cx<VT> *W, Cx<VT> *Z, int k, int nb, const double *
   template void launch_norm2_batch<VT>(const Cx<VT> *, long long, int, double *, const ReduceWs &, cudaStream_t); \
   template void launch_gcr_dots_batch<VT>(const Cx<VT> *, const Cx<VT> *, int, int, long long, double *,          \
                                           const ReduceWs &, cudaStream_t);                                         \
-  template void launch_gcr_update_batch<VT>(Cx<VT> *, Cx<VT> *, int, int, const double *, const double *,          \
-                                            Cx<VT> *, Cx<VT> *, long long, cudaStream_t);
+  template void launch_gcr_update_batch<VT>(Cx<VT> *, int, int, const double *, const double *, Cx<VT> *,           \
+                                            long long, cudaStream_t);
 MG_INST_BATCH(double)
 MG_INST_BATCH(float)
 #undef MG_INST_BATCH

@@ -163,11 +163,13 @@ void launch_gcr_dots(const Cx<float> *W, const Cx<float> *w, const Cx<float> *r,
 template <typename VT>
 void launch_gcr_dots_kdev(const Cx<VT> *W, const Cx<VT> *w, const Cx<VT> *r, const int *kdev, int kmax, long long n,
                           double *out, const ReduceWs &ws, cudaStream_t s);
-// w = (w - sum beta_j W_j) inv and z likewise (written to Wk / Zk); then, if update_xr,
-// x += alpha z and r -= alpha w. beta_dev: 2k doubles on the device.
-void launch_gcr_project_update(const Cx<double> *W, Cx<double> *Wk, const Cx<double> *Z, Cx<double> *Zk, int k,
-                               const double *beta_dev, double inv, double are, double aim, Cx<double> *x,
-                               Cx<double> *r, long long n, bool update_xr, cudaStream_t s);
+// W_k = (W_k - sum beta_j W_j) inv; then, if update_r, r -= alpha W_k. beta_dev: 2k doubles on the device.
+void launch_gcr_project_update(const Cx<double> *W, Cx<double> *Wk, int k, const double *beta_dev, double inv,
+                               double are, double aim, Cx<double> *r, long long n, bool update_r, cudaStream_t s);
+// end of a cycle of k steps (krylov.h): x_v += sum_j y_j Z_j,v for nb vectors (Z[j][v][n]); y_dev: 2 k
+// doubles per vector on the device, zeros for the steps a vector did not take
+template <typename VT>
+void launch_gcr_solution(const Cx<VT> *Z, int k, int nb, const double *y_dev, Cx<VT> *x, long long n, cudaStream_t s);
 
 // batched outer GCR over nb systems (vector v at v * n; bases W[j][v][n], Z[j][v][n]):
 // y_v = mask bit v ? x_v : 0
@@ -180,11 +182,11 @@ void launch_norm2_batch(const Cx<VT> *a, long long n, int nb, double *out, const
 template <typename VT>
 void launch_gcr_dots_batch(const Cx<VT> *W, const Cx<VT> *r, int k, int nb, long long n, double *out,
                            const ReduceWs &ws, cudaStream_t s);
-// per vector, coef[4 v .. 4 v + 3] = (inv, alpha, mode): mode 0 skip, 2 project W_k / Z_k
-// with the betas in dots, 1 project, scale by inv, x += alpha Z_k, r -= alpha W_k
+// per vector, coef[4 v .. 4 v + 3] = (inv, alpha, mode): mode 0 skip, 2 project W_k with the betas in dots,
+// 1 project, scale by inv, r -= alpha W_k
 template <typename VT>
-void launch_gcr_update_batch(Cx<VT> *W, Cx<VT> *Z, int k, int nb, const double *dots, const double *coef,
-                             Cx<VT> *x, Cx<VT> *r, long long n, cudaStream_t s);
+void launch_gcr_update_batch(Cx<VT> *W, int k, int nb, const double *dots, const double *coef, Cx<VT> *r, long long n,
+                             cudaStream_t s);
 
 // ---- transfer between levels ----
 // coarse[b][k] = sum_i conj(V[b][k][i]) fine[site(b,s)][a]

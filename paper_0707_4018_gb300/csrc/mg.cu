@@ -23,6 +23,7 @@
 
 #include "coarsest_lines.h"
 #include "kernels.h"
+#include "krylov.h"
 #include "mg4d.h"
 #include "nullnet.h"
 
@@ -373,8 +374,10 @@ static GcrOut outer_fgcr(mg_ctx &c, const Cx<double> *b, Cx<double> *x, double t
     return out;
   }
   double rn2 = bn2, rel = 1.0;
+  KrylovCycle kc(restart);
   while (out.iters < max_iter) {
     int k = 0;
+    kc.reset();
     for (; k < restart && out.iters < max_iter; ++k) {
       Cx<double> *z = Z + (long long)k * n, *w = W + (long long)k * n;
       precondition(c, r, z);
@@ -385,9 +388,11 @@ static GcrOut outer_fgcr(mg_ctx &c, const Cx<double> *b, Cx<double> *x, double t
       double nw0 = h[2 * k], nw2 = nw0;
       for (int j = 0; j < k; ++j) nw2 -= h[2 * j] * h[2 * j] + h[2 * j + 1] * h[2 * j + 1];
       double wr = h[2 * k + 2], wi = h[2 * k + 3];
+      kc.open(k);
       if (k > 0 && !(nw2 > 0.5 * nw0)) {
         // cancellation: project once, then take fresh coefficients for a second projection
-        launch_gcr_project_update(W, w, Z, z, k, dots, 1.0, 0.0, 0.0, x, r, n, false, c.s);
+        kc.project(k, h);
+        launch_gcr_project_update(W, w, k, dots, 1.0, 0.0, 0.0, r, n, false, c.s);
         launch_gcr_dots(W, w, r, k, n, dots, c.ws, c.s);
         fetch(2 * (k + 3));
         nw0 = h[2 * k];
@@ -399,7 +404,9 @@ static GcrOut outer_fgcr(mg_ctx &c, const Cx<double> *b, Cx<double> *x, double t
       if (!(nw2 > 1e-28 * nw0)) break;  // breakdown: restart from the true residual
       const double inv = 1.0 / std::sqrt(nw2);
       const double are = wr * inv, aim = wi * inv;
-      launch_gcr_project_update(W, w, Z, z, k, dots, inv, are, aim, x, r, n, true, c.s);
+      kc.project(k, h);
+      kc.close(k, inv, are, aim);
+      launch_gcr_project_update(W, w, k, dots, inv, are, aim, r, n, true, c.s);
       rn2 = std::max(rr - (are * are + aim * aim), 0.0);
       ++out.iters;
       rel = std::sqrt(rn2 / bn2);
@@ -407,6 +414,11 @@ static GcrOut outer_fgcr(mg_ctx &c, const Cx<double> *b, Cx<double> *x, double t
         ++k;
         break;
       }
+    }
+    if (kc.columns() > 0) {  // x += Z y
+      kc.solution(h);
+      MG_CUDA(cudaMemcpyAsync(dots, h, 2 * kc.columns() * sizeof(double), cudaMemcpyHostToDevice, c.s));
+      launch_gcr_solution<double>(Z, kc.columns(), 1, dots, x, n, c.s);
     }
     apply_op<double>(c, 0, x, r, b, -1.0, 1.0);  // true residual r = b - D x
     launch_norm2<double>(r, n, dots, c.ws, c.s);
@@ -717,9 +729,11 @@ static void outer_fgcr_batch(mg_ctx &c, int nb, const Cx<double> *b, Cx<double> 
   const unsigned int all = nb == 32 ? 0xffffffffu : (1u << nb) - 1u;
   int iters = 0;
   std::vector<double> nw0(nb), nw2(nb), wr(nb), wi(nb), rr(nb);
+  std::vector<KrylovCycle> kc(nb, KrylovCycle(restart));
   while (done != all && iters < c.p.max_iter) {
     unsigned int act = all & ~done;
     int k = 0;
+    for (KrylovCycle &q : kc) q.reset();
     for (; k < restart && iters < c.p.max_iter && act != 0u; ++k) {
       Cx<double> *Zk = Z + (long long)k * nb * n, *Wk = W + (long long)k * nb * n;
       precondition_batch(c, nb, r, act, Zk);
@@ -736,7 +750,11 @@ static void outer_fgcr_batch(mg_ctx &c, int nb, const Cx<double> *b, Cx<double> 
         for (int j = 0; j < k; ++j) nw2[v] -= hv[2 * j] * hv[2 * j] + hv[2 * j + 1] * hv[2 * j + 1];
         wr[v] = hv[2 * k + 2];
         wi[v] = hv[2 * k + 3];
-        if (((act >> v) & 1u) && k > 0 && !(nw2[v] > 0.5 * nw0[v])) cancel |= 1u << v;
+        kc[v].open(k);
+        if (((act >> v) & 1u) && k > 0 && !(nw2[v] > 0.5 * nw0[v])) {
+          cancel |= 1u << v;
+          kc[v].project(k, hv);
+        }
       }
       if (cancel != 0u) {
         // cancellation: project those vectors once, then take fresh coefficients for them
@@ -746,7 +764,7 @@ static void outer_fgcr_batch(mg_ctx &c, int nb, const Cx<double> *b, Cx<double> 
           hcoef[4 * v + 3] = ((cancel >> v) & 1u) ? 2.0 : 0.0;
         }
         MG_CUDA(cudaMemcpyAsync(c.bcoef.p, hcoef, 4 * nb * sizeof(double), cudaMemcpyHostToDevice, c.s));
-        launch_gcr_update_batch(W, Z, k, nb, c.bdots.p, c.bcoef.p, x, r, n, c.s);
+        launch_gcr_update_batch(W, k, nb, c.bdots.p, c.bcoef.p, r, n, c.s);
         launch_gcr_dots_batch(W, r, k, nb, n, c.bdots.p, c.ws, c.s);
         fetch(c.bdots.p, nb * stride);
         for (int v = 0; v < nb; ++v) {
@@ -772,6 +790,8 @@ static void outer_fgcr_batch(mg_ctx &c, int nb, const Cx<double> *b, Cx<double> 
         hcoef[4 * v + 1] = are;
         hcoef[4 * v + 2] = aim;
         hcoef[4 * v + 3] = 1.0;
+        kc[v].project(k, h + v * stride);
+        kc[v].close(k, inv, are, aim);
         rn2[v] = std::max(rr[v] - (are * are + aim * aim), 0.0);
         ++out[v].iters;
         if (std::sqrt(rn2[v] / bn2[v]) <= tol) act &= ~(1u << v);
@@ -779,8 +799,14 @@ static void outer_fgcr_batch(mg_ctx &c, int nb, const Cx<double> *b, Cx<double> 
       // mode 1 projects with the betas now in bdots: fresh ones for the vectors that were
       // projected once already, the original ones (the same reduction again) for the others
       MG_CUDA(cudaMemcpyAsync(c.bcoef.p, hcoef, 4 * nb * sizeof(double), cudaMemcpyHostToDevice, c.s));
-      launch_gcr_update_batch(W, Z, k, nb, c.bdots.p, c.bcoef.p, x, r, n, c.s);
+      launch_gcr_update_batch(W, k, nb, c.bdots.p, c.bcoef.p, r, n, c.s);
       ++iters;
+    }
+    if (k > 0) {  // x_v += Z_v y_v, zeros beyond the steps a vector took
+      std::fill(h, h + 2 * k * nb, 0.0);
+      for (int v = 0; v < nb; ++v) kc[v].solution(h + 2 * k * v);
+      MG_CUDA(cudaMemcpyAsync(c.bdots.p, h, 2 * k * nb * sizeof(double), cudaMemcpyHostToDevice, c.s));
+      launch_gcr_solution<double>(Z, k, nb, c.bdots.p, x, n, c.s);
     }
     // true residuals r = b - D x of every unfinished vector (defect correction)
     apply_op<double>(c, 0, x, r, b, -1.0, 1.0, nb);

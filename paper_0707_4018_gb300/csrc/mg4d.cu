@@ -21,6 +21,7 @@
 
 #include <cstdlib>
 
+#include "krylov.h"
 #include "mg4d.h"
 
 namespace mg {
@@ -174,8 +175,10 @@ Gcr fgcr(Engine4 &e, ApplyF &&apply, PrecF &&prec, const Cx<double> *b, Cx<doubl
     return out;
   }
   double rel = 1.0;
+  KrylovCycle kc(restart);
   while (out.iters < max_iter) {
     int k = 0;
+    kc.reset();
     for (; k < restart && out.iters < max_iter; ++k) {
       Cx<double> *z = Z + (long long)k * n, *w = W + (long long)k * n;
       prec(r, z);
@@ -186,8 +189,10 @@ Gcr fgcr(Engine4 &e, ApplyF &&apply, PrecF &&prec, const Cx<double> *b, Cx<doubl
       double nw0 = h[2 * k], nw2 = nw0;
       for (int j = 0; j < k; ++j) nw2 -= h[2 * j] * h[2 * j] + h[2 * j + 1] * h[2 * j + 1];
       double wr = h[2 * k + 2], wi = h[2 * k + 3];
+      kc.open(k);
       if (k > 0 && !(nw2 > 0.5 * nw0)) {
-        launch_gcr_project_update(W, w, Z, z, k, dots, 1.0, 0.0, 0.0, x, r, n, false, e.s);
+        kc.project(k, h);
+        launch_gcr_project_update(W, w, k, dots, 1.0, 0.0, 0.0, r, n, false, e.s);
         launch_gcr_dots(W, w, r, k, n, dots, e.ws, e.s);
         fetch(2 * (k + 3));
         nw0 = h[2 * k];
@@ -199,13 +204,20 @@ Gcr fgcr(Engine4 &e, ApplyF &&apply, PrecF &&prec, const Cx<double> *b, Cx<doubl
       if (!(nw2 > 1e-28 * nw0)) break;
       const double inv = 1.0 / std::sqrt(nw2);
       const double are = wr * inv, aim = wi * inv;
-      launch_gcr_project_update(W, w, Z, z, k, dots, inv, are, aim, x, r, n, true, e.s);
+      kc.project(k, h);
+      kc.close(k, inv, are, aim);
+      launch_gcr_project_update(W, w, k, dots, inv, are, aim, r, n, true, e.s);
       ++out.iters;
       rel = std::sqrt(std::max(rr - (are * are + aim * aim), 0.0) / bn2);
       if (rel <= tol) {
         ++k;
         break;
       }
+    }
+    if (kc.columns() > 0) {  // x += Z y
+      kc.solution(h);
+      MG_CUDA(cudaMemcpyAsync(dots, h, 2 * kc.columns() * sizeof(double), cudaMemcpyHostToDevice, e.s));
+      launch_gcr_solution<double>(Z, kc.columns(), 1, dots, x, n, e.s);
     }
     apply(x, r, b);  // r = b - A x
     launch_norm2<double>(r, n, dots, e.ws, e.s);
@@ -487,9 +499,11 @@ void fgcr_batch(Engine4 &e, int nb, ApplyF &&apply, PrecF &&prec, const Cx<VT> *
       out[v].converged = true;
     }
   int iters = 0;
+  std::vector<KrylovCycle> kc(nb, KrylovCycle(restart));
   while (done != all && iters < max_iter) {
     unsigned int act = all & ~done;
     int k = 0;
+    for (KrylovCycle &q : kc) q.reset();
     for (; k < restart && iters < max_iter && act != 0u; ++k) {
       Cx<VT> *Zk = Z + (long long)k * nb * n, *Wk = W + (long long)k * nb * n;
       launch_copy_masked(r, rin, n, nb, act, e.s);
@@ -506,7 +520,11 @@ void fgcr_batch(Engine4 &e, int nb, ApplyF &&apply, PrecF &&prec, const Cx<VT> *
         for (int j = 0; j < k; ++j) nw2[v] -= hv[2 * j] * hv[2 * j] + hv[2 * j + 1] * hv[2 * j + 1];
         wr[v] = hv[2 * k + 2];
         wi[v] = hv[2 * k + 3];
-        if (((act >> v) & 1u) && k > 0 && !(nw2[v] > reproject * nw0[v])) cancel |= 1u << v;
+        kc[v].open(k);
+        if (((act >> v) & 1u) && k > 0 && !(nw2[v] > reproject * nw0[v])) {
+          cancel |= 1u << v;
+          kc[v].project(k, hv);
+        }
       }
       if (cancel != 0u) {  // project those vectors once, then take fresh coefficients for them
         for (int v = 0; v < nb; ++v) {
@@ -515,7 +533,7 @@ void fgcr_batch(Engine4 &e, int nb, ApplyF &&apply, PrecF &&prec, const Cx<VT> *
           hcoef[4 * v + 3] = ((cancel >> v) & 1u) ? 2.0 : 0.0;
         }
         MG_CUDA(cudaMemcpyAsync(coef, hcoef, 4 * nb * sizeof(double), cudaMemcpyHostToDevice, e.s));
-        launch_gcr_update_batch(W, Z, k, nb, dots, coef, x, r, n, e.s);
+        launch_gcr_update_batch(W, k, nb, dots, coef, r, n, e.s);
         launch_gcr_dots_batch(W, r, k, nb, n, dots, ws, e.s);
         fetch(nb * stride);
         for (int v = 0; v < nb; ++v) {
@@ -538,13 +556,21 @@ void fgcr_batch(Engine4 &e, int nb, ApplyF &&apply, PrecF &&prec, const Cx<VT> *
         hcoef[4 * v + 1] = are;
         hcoef[4 * v + 2] = aim;
         hcoef[4 * v + 3] = 1.0;
+        kc[v].project(k, h + v * stride);
+        kc[v].close(k, inv, are, aim);
         rn2[v] = std::max(rr[v] - (are * are + aim * aim), 0.0);
         ++out[v].iters;
         if (std::sqrt(rn2[v] / bn2[v]) <= tol) act &= ~(1u << v);
       }
       MG_CUDA(cudaMemcpyAsync(coef, hcoef, 4 * nb * sizeof(double), cudaMemcpyHostToDevice, e.s));
-      launch_gcr_update_batch(W, Z, k, nb, dots, coef, x, r, n, e.s);
+      launch_gcr_update_batch(W, k, nb, dots, coef, r, n, e.s);
       ++iters;
+    }
+    if (k > 0) {  // x_v += Z_v y_v, zeros beyond the steps a vector took
+      std::fill(h, h + 2 * k * nb, 0.0);
+      for (int v = 0; v < nb; ++v) kc[v].solution(h + 2 * k * v);
+      MG_CUDA(cudaMemcpyAsync(dots, h, 2 * k * nb * sizeof(double), cudaMemcpyHostToDevice, e.s));
+      launch_gcr_solution<VT>(Z, k, nb, dots, x, n, e.s);
     }
     apply(x, r, b);  // true residuals r = b - A x
     launch_norm2_batch(r, n, nb, dots, ws, e.s);
