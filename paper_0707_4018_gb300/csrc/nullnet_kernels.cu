@@ -11,7 +11,6 @@
 //
 // Layouts: activations h[f][x][2 C] as bfloat16 pairs (re, im); pre-activations and
 // gradients float2 [f][x][2 C]; links float2 [f][x][2]; weights float2 [5][2 co][2 ci].
-// One warp owns one site; lane l holds channel-spin entry l (2 C <= 32).
 #include <cuda_bf16.h>
 
 #include "nullnet.h"
@@ -20,9 +19,12 @@ namespace mg {
 
 namespace {
 
+// the roundings are spelled out: a transported input that moves by one bit can move the bfloat16
+// activation behind it by 2^-9, so every kernel that transports must round alike
 __device__ __forceinline__ float2 cmulf(float2 a, float2 b) {
-  return make_float2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
+  return make_float2(fmaf(a.x, b.x, -__fmul_rn(a.y, b.y)), fmaf(a.x, b.y, __fmul_rn(a.y, b.x)));
 }
+__device__ __forceinline__ float norm2f(float2 a) { return fmaf(a.x, a.x, __fmul_rn(a.y, a.y)); }
 // acc += a * b
 __device__ __forceinline__ void cmacf(float2 &acc, float2 a, float2 b) {
   acc.x = fmaf(a.x, b.x, acc.x);
@@ -38,9 +40,6 @@ __device__ __forceinline__ void cmacf_conj(float2 &acc, float2 a, float2 b) {
   acc.y = fmaf(-a.y, b.x, acc.y);
 }
 __device__ __forceinline__ float2 conjf2(float2 a) { return make_float2(a.x, -a.y); }
-__device__ __forceinline__ float2 shfl2(float2 v, int src) {
-  return make_float2(__shfl_sync(0xffffffffu, v.x, src), __shfl_sync(0xffffffffu, v.y, src));
-}
 __device__ __forceinline__ float2 bf2f(__nv_bfloat162 v) {
   return make_float2(__bfloat162float(v.x), __bfloat162float(v.y));
 }
@@ -95,108 +94,144 @@ __device__ __forceinline__ void adj_hop(int dir, int z0, int z1, int L0, int L1,
   }
 }
 
-constexpr int kWarps = 8;
+// ---------------------------------------------------------------------------
+// The transported convolution as a tiled product: for a tile of S sites and one direction the
+// transported inputs v_x[k] = phase_x in_{nb(x)}[k] are staged in shared memory (site fastest), the
+// weights of all directions once per CTA, and a thread accumulates the two spin rows of one channel
+// at four sites: one 16-byte weight load and two 16-byte input loads for 8 complex multiply-adds.
+// FP32 issue bounds it; with a warp per site and a lane per output row the weights' rows met in one
+// bank and every input took two shuffles (16 fields of 128^2, one layer: 2.1 ms forward, 2.5 ms
+// backward; a whole gradient, with the loss and weight kernels below, 22.1 ms before and 6.3 now). Every output sums its terms in the order direction, input, as fused multiply-adds, so
+// the values that are rounded to bfloat16 do not depend on the tiling.
+// ---------------------------------------------------------------------------
+enum class Conv {
+  kHidden,  // bf16 in; gated bf16 out, pre-activation out if asked for
+  kLast,    // bf16 in; float2 out
+  kAdjoint  // float2 in (dL/da^* of the layer), conj(W)^T, adjoint hops; dL/da^* of the layer before (through its gate)
+};
 
-// One layer forward. h_in: [f][x][ci2] bf16 pairs; out: pre-activation a (float2, may be null),
-// gated bf16 h_out (hidden layers) or float2 y (last layer, LAST).
-template <bool LAST>
-__global__ void __launch_bounds__(256) ptconv_fwd_kernel(const __nv_bfloat162 *__restrict__ h_in,
-                                                         const float2 *__restrict__ U, const int *__restrict__ fmap,
-                                                         const float2 *__restrict__ W, int ci2, int co2, int L0,
-                                                         int L1, float2 *__restrict__ a_out,
-                                                         __nv_bfloat162 *__restrict__ h_out) {
-  __shared__ float2 Ws[5 * 32 * 32];
-  for (int q = threadIdx.x; q < 5 * co2 * ci2; q += blockDim.x) {
-    const int dir = q / (co2 * ci2), r = q - dir * co2 * ci2, lo = r / ci2, li = r - lo * ci2;
-    Ws[(dir * 32 + lo) * 32 + li] = W[q];
-  }
-  __syncthreads();
-  const int f = blockIdx.y;
-  const long long V = (long long)L0 * L1;
-  const float2 *Uf = U + (size_t)(fmap ? fmap[f] : f) * 2 * V;
-  const __nv_bfloat162 *hin = h_in + (size_t)f * V * ci2;
-  const int lane = threadIdx.x & 31;
-  const long long wstride = (long long)gridDim.x * kWarps;
-  for (long long x = (long long)blockIdx.x * kWarps + (threadIdx.x >> 5); x < V; x += wstride) {
-    const int x1 = (int)(x / L0), x0 = (int)(x - (long long)x1 * L0);
-    float2 acc = make_float2(0.f, 0.f);
-#pragma unroll
-    for (int dir = 0; dir < 5; ++dir) {
-      long long nb;
-      float2 ph;
-      fwd_hop(dir, x0, x1, L0, L1, Uf, nb, ph);
-      float2 v = lane < ci2 ? bf2f(hin[nb * ci2 + lane]) : make_float2(0.f, 0.f);
-      v = cmulf(ph, v);
-      const float2 *wrow = Ws + (dir * 32 + (lane < co2 ? lane : 0)) * 32;
-      for (int li = 0; li < ci2; ++li) cmacf(acc, wrow[li], shfl2(v, li));
-    }
-    const size_t o = (size_t)f * V * co2 + (size_t)x * co2 + lane;
-    if (LAST) {
-      if (lane < co2) a_out[o] = acc;
-    } else {
-      if (a_out != nullptr && lane < co2) a_out[o] = acc;
-      float s = acc.x * acc.x + acc.y * acc.y;
-      s += __shfl_xor_sync(0xffffffffu, s, 1);
-      const float g = rsqrtf(1.f + s);
-      if (lane < co2) h_out[o] = f2bf(make_float2(acc.x * g, acc.y * g));
-    }
-  }
+constexpr int kConvThreads = 256;
+constexpr int kSites = 4;      // sites of a thread
+constexpr int kMaxTile = 128;  // sites of a tile
+
+// sites of a tile for `channels` output channels
+__host__ __device__ inline int conv_tile(int channels) {
+  const int s = kConvThreads / channels * kSites;
+  return s < kMaxTile ? s : kMaxTile;
 }
 
-// dL/dh^* of a layer's input from dL/da^* of its output, then (GATE_PREV) through the gate of
-// the previous layer: ga_prev = g gh + 2 g'(s) Re(a^dagger gh)_c a
-template <bool GATE_PREV>
-__global__ void __launch_bounds__(256) ptconv_bwd_data_kernel(const float2 *__restrict__ ga,
-                                                              const float2 *__restrict__ U,
+__device__ __forceinline__ void load_pair(const __nv_bfloat162 *p, float2 &a, float2 &b) {
+  const uint2 w = *reinterpret_cast<const uint2 *>(p);
+  a = bf2f(*reinterpret_cast<const __nv_bfloat162 *>(&w.x));
+  b = bf2f(*reinterpret_cast<const __nv_bfloat162 *>(&w.y));
+}
+__device__ __forceinline__ void load_pair(const float2 *p, float2 &a, float2 &b) {
+  const float4 w = *reinterpret_cast<const float4 *>(p);
+  a = make_float2(w.x, w.y);
+  b = make_float2(w.z, w.w);
+}
+
+// kin / kout: channel-spin entries (even) of the input and output of this product
+template <Conv M, typename TI>
+__global__ void __launch_bounds__(kConvThreads, 3) ptconv_kernel(const TI *__restrict__ in, const float2 *__restrict__ U,
                                                               const int *__restrict__ fmap,
-                                                              const float2 *__restrict__ W, int ci2, int co2, int L0,
+                                                              const float2 *__restrict__ W, int kin, int kout, int L0,
                                                               int L1, const float2 *__restrict__ a_prev,
-                                                              float2 *__restrict__ ga_prev) {
-  __shared__ float2 Ws[5 * 32 * 32];
-  for (int q = threadIdx.x; q < 5 * co2 * ci2; q += blockDim.x) {
-    const int dir = q / (co2 * ci2), r = q - dir * co2 * ci2, lo = r / ci2, li = r - lo * ci2;
-    Ws[(dir * 32 + li) * 32 + lo] = W[q];  // transposed: row li holds W[dir][.][li]
-  }
-  __syncthreads();
-  const int f = blockIdx.y;
-  const long long V = (long long)L0 * L1;
-  const float2 *Uf = U + (size_t)(fmap ? fmap[f] : f) * 2 * V;
-  const float2 *gaf = ga + (size_t)f * V * co2;
-  const int lane = threadIdx.x & 31;
-  const long long wstride = (long long)gridDim.x * kWarps;
-  for (long long z = (long long)blockIdx.x * kWarps + (threadIdx.x >> 5); z < V; z += wstride) {
-    const int z1 = (int)(z / L0), z0 = (int)(z - (long long)z1 * L0);
-    float2 acc = make_float2(0.f, 0.f);
-#pragma unroll
-    for (int dir = 0; dir < 5; ++dir) {
-      long long src;
-      float2 ph;
-      adj_hop(dir, z0, z1, L0, L1, Uf, src, ph);
-      const float2 g = lane < co2 ? gaf[src * co2 + lane] : make_float2(0.f, 0.f);
-      const float2 *wcol = Ws + (dir * 32 + (lane < ci2 ? lane : 0)) * 32;
-      float2 t = make_float2(0.f, 0.f);
-      for (int lo = 0; lo < co2; ++lo) cmacf_conj(t, wcol[lo], shfl2(g, lo));
-      cmacf(acc, ph, t);
+                                                              float2 *__restrict__ a_out,
+                                                              __nv_bfloat162 *__restrict__ h_out) {
+  extern __shared__ float4 conv_smem[];
+  const int C = kout / 2, S = conv_tile(C), V = L0 * L1, f = blockIdx.y;
+  float2 *Ws = reinterpret_cast<float2 *>(conv_smem);  // [dir][k][out]
+  float2 *Vs = Ws + 5 * kin * kout;                    // [k][S]
+  for (int q = threadIdx.x; q < 5 * kin * kout; q += kConvThreads) {
+    const int dir = q / (kin * kout), r = q - dir * kin * kout;
+    if (M == Conv::kAdjoint) {  // W[dir][k][out]: rows of the layer's weights are this product's inputs
+      Ws[q] = conjf2(W[q]);
+    } else {  // W[dir][out][k]
+      const int o = r / kin, k = r - o * kin;
+      Ws[(dir * kin + k) * kout + o] = W[q];
     }
-    const size_t o = (size_t)f * V * ci2 + (size_t)z * ci2 + lane;
-    if (GATE_PREV) {
-      const float2 a = lane < ci2 ? a_prev[o] : make_float2(0.f, 0.f);
-      float s = a.x * a.x + a.y * a.y;
-      s += __shfl_xor_sync(0xffffffffu, s, 1);
-      float re = a.x * acc.x + a.y * acc.y;
-      re += __shfl_xor_sync(0xffffffffu, re, 1);
-      const float g = rsqrtf(1.f + s);
-      const float dg2 = -g * g * g * re;  // 2 g'(s) Re(a^dagger gh), g' = -g^3 / 2
-      if (lane < ci2) ga_prev[o] = make_float2(g * acc.x + dg2 * a.x, g * acc.y + dg2 * a.y);
-    } else if (lane < ci2) {
-      ga_prev[o] = acc;
+  }
+  const float2 *Uf = U + (size_t)(fmap ? fmap[f] : f) * 2 * V;
+  in += (size_t)f * V * kin;
+  const int c = threadIdx.x % C, grp = threadIdx.x / C;
+  const bool works = grp * kSites < S;
+  for (int x0 = blockIdx.x * S; x0 < V; x0 += gridDim.x * S) {
+    float2 acc[kSites][2];
+#pragma unroll
+    for (int s = 0; s < kSites; ++s) acc[s][0] = acc[s][1] = make_float2(0.f, 0.f);
+    for (int dir = 0; dir < 5; ++dir) {
+      __syncthreads();
+      // a thread stages the two entries of a channel at a site; consecutive threads, consecutive sites
+      for (int q = threadIdx.x; q < S * (kin / 2); q += kConvThreads) {
+        const int ch = q / S, s = q - ch * S, x = x0 + s;
+        float2 a = make_float2(0.f, 0.f), b = a;
+        if (x < V) {
+          const int y1 = x / L0, y0 = x - y1 * L0;
+          long long nb;
+          float2 ph;
+          if (M == Conv::kAdjoint)
+            adj_hop(dir, y0, y1, L0, L1, Uf, nb, ph);
+          else
+            fwd_hop(dir, y0, y1, L0, L1, Uf, nb, ph);
+          load_pair(in + nb * kin + 2 * ch, a, b);
+          a = cmulf(ph, a);
+          b = cmulf(ph, b);
+        }
+        Vs[2 * ch * S + s] = a;
+        Vs[(2 * ch + 1) * S + s] = b;
+      }
+      __syncthreads();
+      if (works) {
+        const float4 *wp = reinterpret_cast<const float4 *>(Ws + dir * kin * kout) + c;
+        const float4 *vp = reinterpret_cast<const float4 *>(Vs) + grp * (kSites / 2);
+#pragma unroll 4
+        for (int k = 0; k < kin; ++k) {
+          const float4 w = wp[k * C], v01 = vp[k * (S / 2)], v23 = vp[k * (S / 2) + 1];
+          const float2 v[kSites] = {make_float2(v01.x, v01.y), make_float2(v01.z, v01.w), make_float2(v23.x, v23.y),
+                                    make_float2(v23.z, v23.w)};
+#pragma unroll
+          for (int s = 0; s < kSites; ++s) {
+            cmacf(acc[s][0], make_float2(w.x, w.y), v[s]);
+            cmacf(acc[s][1], make_float2(w.z, w.w), v[s]);
+          }
+        }
+      }
+    }
+    if (!works) continue;
+#pragma unroll
+    for (int s = 0; s < kSites; ++s) {
+      const int x = x0 + grp * kSites + s;
+      if (x >= V) break;
+      const float2 p = acc[s][0], q = acc[s][1];
+      const size_t o = ((size_t)f * V + x) * kout + 2 * c;
+      if (M == Conv::kAdjoint) {
+        const float4 a = *reinterpret_cast<const float4 *>(a_prev + o);
+        const float sq = (a.x * a.x + a.y * a.y) + (a.z * a.z + a.w * a.w);
+        const float re = (a.x * p.x + a.y * p.y) + (a.z * q.x + a.w * q.y);
+        const float g = rsqrtf(1.f + sq);
+        const float dg2 = -g * g * g * re;  // 2 g'(s) Re(a^dagger gh), g' = -g^3 / 2
+        *reinterpret_cast<float4 *>(a_out + o) =
+            make_float4(g * p.x + dg2 * a.x, g * p.y + dg2 * a.y, g * q.x + dg2 * a.z, g * q.y + dg2 * a.w);
+      } else {
+        if (M == Conv::kLast || a_out != nullptr)
+          *reinterpret_cast<float4 *>(a_out + o) = make_float4(p.x, p.y, q.x, q.y);
+        if (M == Conv::kHidden) {
+          const float s0 = norm2f(p), s1 = norm2f(q);
+          const float g = rsqrtf(1.f + (s0 + s1));
+          __nv_bfloat162 h[2] = {f2bf(make_float2(p.x * g, p.y * g)), f2bf(make_float2(q.x * g, q.y * g))};
+          *reinterpret_cast<uint2 *>(h_out + o) = *reinterpret_cast<const uint2 *>(h);
+        }
+      }
     }
   }
 }
 
 // Per-CTA partial sums of dL/dW^*[dir][lo][li] = sum_x ga_x[lo] conj(T_dir h_x[li]) over a
 // contiguous range of (field, site) pairs; partials[cta][entry] (entry = (dir co2 + lo) ci2 + li)
-constexpr int kWG = 8;  // sites staged per group
+// A thread owns input entry li (its lane) and output rows lo0 .. lo0 + 3 of every direction: per staged
+// site two 16-byte broadcast loads of g and five loads of T h for 20 complex multiply-adds.
+constexpr int kWG = 16;  // sites staged per group
 __global__ void __launch_bounds__(256) ptconv_bwd_weight_kernel(const float2 *__restrict__ ga,
                                                                 const __nv_bfloat162 *__restrict__ h_in,
                                                                 const float2 *__restrict__ U,
@@ -209,24 +244,26 @@ __global__ void __launch_bounds__(256) ptconv_bwd_weight_kernel(const float2 *__
   const long long per = (total + gridDim.x - 1) / gridDim.x;
   const long long p0 = (long long)blockIdx.x * per, p1 = p0 + per < total ? p0 + per : total;
   const int ne = 5 * co2 * ci2;
-  constexpr int kEnt = 20;  // 5 * 32 * 32 / 256
-  float2 acc[kEnt];
+  float2 acc[5][4];
 #pragma unroll
-  for (int e = 0; e < kEnt; ++e) acc[e] = make_float2(0.f, 0.f);
+  for (int d = 0; d < 5; ++d)
+#pragma unroll
+    for (int e = 0; e < 4; ++e) acc[d][e] = make_float2(0.f, 0.f);
   const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
   for (long long g0 = p0; g0 < p1; g0 += kWG) {
     __syncthreads();
-    // warp w stages site g0 + w: its gradient row and its five transported inputs
-    const long long p = g0 + wid;
-    if (wid < kWG) {
+    // warp w stages sites g0 + w, g0 + w + 8: the gradient row and the five transported inputs
+#pragma unroll
+    for (int s = wid; s < kWG; s += 8) {
+      const long long p = g0 + s;
       float2 gv = make_float2(0.f, 0.f);
       float2 tv[5];
 #pragma unroll
       for (int d = 0; d < 5; ++d) tv[d] = make_float2(0.f, 0.f);
       if (p < p1) {
         const int f = (int)(p / V);
-        const long long x = p - (long long)f * V;
-        const int x1 = (int)(x / L0), x0 = (int)(x - (long long)x1 * L0);
+        const int x = (int)(p - (long long)f * V);
+        const int x1 = x / L0, x0 = x - x1 * L0;
         const float2 *Uf = U + (size_t)(fmap ? fmap[f] : f) * 2 * V;
         if (lane < co2) gv = ga[(size_t)p * co2 + lane];
 #pragma unroll
@@ -237,25 +274,35 @@ __global__ void __launch_bounds__(256) ptconv_bwd_weight_kernel(const float2 *__
           if (lane < ci2) tv[d] = cmulf(ph, bf2f(h_in[((size_t)f * V + nb) * ci2 + lane]));
         }
       }
-      gs[wid][lane] = gv;
+      gs[s][lane] = gv;
 #pragma unroll
-      for (int d = 0; d < 5; ++d) Ts[wid][d][lane] = tv[d];
+      for (int d = 0; d < 5; ++d) Ts[s][d][lane] = tv[d];
     }
     __syncthreads();
+    if (4 * wid < co2) {
+#pragma unroll 4
+      for (int s = 0; s < kWG; ++s) {
+        const float4 g01 = *reinterpret_cast<const float4 *>(&gs[s][4 * wid]);
+        const float4 g23 = *reinterpret_cast<const float4 *>(&gs[s][4 * wid + 2]);
+        const float2 g[4] = {make_float2(g01.x, g01.y), make_float2(g01.z, g01.w), make_float2(g23.x, g23.y),
+                             make_float2(g23.z, g23.w)};
 #pragma unroll
-    for (int e = 0; e < kEnt; ++e) {
-      const int q = threadIdx.x + 256 * e;
-      if (q < ne) {
-        const int dir = q / (co2 * ci2), r = q - dir * co2 * ci2, lo = r / ci2, li = r - lo * ci2;
+        for (int d = 0; d < 5; ++d) {
+          const float2 t = Ts[s][d][lane];
 #pragma unroll
-        for (int s = 0; s < kWG; ++s) cmacf_conj(acc[e], Ts[s][dir][li], gs[s][lo]);
+          for (int e = 0; e < 4; ++e) cmacf_conj(acc[d][e], t, g[e]);
+        }
       }
     }
   }
+  if (lane < ci2) {
 #pragma unroll
-  for (int e = 0; e < kEnt; ++e) {
-    const int q = threadIdx.x + 256 * e;
-    if (q < ne) partials[(size_t)blockIdx.x * ne + q] = acc[e];
+    for (int d = 0; d < 5; ++d)
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const int lo = 4 * wid + e;
+        if (lo < co2) partials[(size_t)blockIdx.x * ne + (d * co2 + lo) * ci2 + lane] = acc[d][e];
+      }
   }
 }
 
@@ -273,146 +320,153 @@ __global__ void sum_partials_kernel(const float2 *__restrict__ partials, int npa
   gW[q] = make_float2((float)re, (float)im);
 }
 
-// Rotation-invariant block loss and dL/dy^*: one warp per (field, block), lane r = 2 i + s
-// (site i of the block, spin s). G = W^dagger W and C = W^dagger V in FP32 warp sums, then the
-// small dense algebra in FP64: G = L L^dagger (a relative ridge of 1e-7 tr G / nv keeps FP32
-// round-off from breaking it), A = G^{-1} C, L_b = nv - Re tr(C^dagger A); grad = -(V - W A) A^dagger.
+// Rotation-invariant block loss and dL/dy^*, four blocks per warp. G = W^dagger W and C = W^dagger V in
+// FP32 (a lane forms two entries of each over the block's rows, staged in shared memory), then the small
+// dense algebra in FP64: G = L L^dagger (a relative ridge of 1e-7 tr G / nv keeps FP32 round-off from
+// breaking it), A = G^{-1} C, L_b = nv - Re tr(C^dagger A); grad = -(V - W A) A^dagger. Eight lanes share
+// a block's FP64 work (row i of L, then column i of A), so a warp's FP64 instructions, which bound the
+// kernel, serve four blocks; a serial factorisation by one lane per warp and block took 2.2 ms for 16
+// fields of 128^2.
 constexpr int kMaxNv = 8;
-__global__ void __launch_bounds__(128) nullnet_loss_kernel(const float2 *__restrict__ y,
-                                                           const float2 *__restrict__ target,
-                                                           const int *__restrict__ fmap, int nv, BlockGeo bg,
-                                                           float scale, float2 *__restrict__ gy,
-                                                           double *__restrict__ lossb) {
-  __shared__ double Gs[4][kMaxNv * kMaxNv * 2];
-  __shared__ double Cs[4][kMaxNv * kMaxNv * 2];
-  __shared__ double As[4][kMaxNv * kMaxNv * 2];
+constexpr int kLossWarps = 4, kLossBlocks = 4;
+struct LossSmem {
+  float2 w[32][kMaxNv + 1], v[32][kMaxNv + 1];  // rows of the block in work
+  double2 G[kLossBlocks][kMaxNv * kMaxNv];      // G, then L below the diagonal
+  double2 C[kLossBlocks][kMaxNv * kMaxNv];
+  float2 A[kLossBlocks][kMaxNv * kMaxNv];
+};
+
+__global__ void __launch_bounds__(32 * kLossWarps) nullnet_loss_kernel(const float2 *__restrict__ y,
+                                                                       const float2 *__restrict__ target,
+                                                                       const int *__restrict__ fmap, int nv,
+                                                                       BlockGeo bg, float scale,
+                                                                       float2 *__restrict__ gy,
+                                                                       double *__restrict__ lossb) {
+  extern __shared__ float4 loss_smem[];
   const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const long long nb = bg.nblocks;
-  const long long wglob = (long long)blockIdx.x * 4 + wid;
+  LossSmem &sm = reinterpret_cast<LossSmem *>(loss_smem)[wid];
   const int f = blockIdx.y;
   const long long V = (long long)bg.L0 * bg.L1;
-  if (wglob >= nb) return;  // whole warps leave together
-  const long long b = wglob;
-  const int rows = bg.bvol * 2;
+  const long long first = ((long long)blockIdx.x * kLossWarps + wid) * kLossBlocks;
+  const int count = bg.nblocks - first < kLossBlocks ? (int)(bg.nblocks - first) : kLossBlocks;
+  if (count <= 0) return;  // whole warps leave together
+  const int rows = bg.bvol * 2, sp = lane & 1;
   const bool act = lane < rows;
-  long long site = 0;
-  int sp = 0;
-  if (act) {
-    site = fine_site_of(bg, b, lane >> 1);
-    sp = lane & 1;
-  }
   const float2 *yf = y + (size_t)f * V * 2 * nv;
   const float2 *tf = target + (size_t)(fmap ? fmap[f] : f) * nv * V * 2;
-  float2 w[kMaxNv], v[kMaxNv];
+  const float2 zero = make_float2(0.f, 0.f);
+  // entries [lane] and [lane + 32] of each block's G and C
+  for (int b = 0; b < count; ++b) {
+    const long long site = act ? fine_site_of(bg, first + b, lane >> 1) : 0;
+    __syncwarp();
 #pragma unroll
-  for (int k = 0; k < kMaxNv; ++k) {
-    w[k] = (act && k < nv) ? yf[(size_t)site * 2 * nv + 2 * k + sp] : make_float2(0.f, 0.f);
-    v[k] = (act && k < nv) ? tf[((size_t)k * V + site) * 2 + sp] : make_float2(0.f, 0.f);
-  }
-  double *G = Gs[wid], *C = Cs[wid], *A = As[wid];
-  for (int k = 0; k < nv; ++k) {
-    for (int j = 0; j < nv; ++j) {
-      float2 g = make_float2(0.f, 0.f), c = make_float2(0.f, 0.f);
-      cmacf_conj(g, w[k], w[j]);
-      cmacf_conj(c, w[k], v[j]);
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        g.x += __shfl_xor_sync(0xffffffffu, g.x, o);
-        g.y += __shfl_xor_sync(0xffffffffu, g.y, o);
-        c.x += __shfl_xor_sync(0xffffffffu, c.x, o);
-        c.y += __shfl_xor_sync(0xffffffffu, c.y, o);
-      }
-      if (lane == 0) {
-        G[(k * nv + j) * 2] = g.x;
-        G[(k * nv + j) * 2 + 1] = g.y;
-        C[(k * nv + j) * 2] = c.x;
-        C[(k * nv + j) * 2 + 1] = c.y;
-      }
+    for (int k = 0; k < kMaxNv; ++k) {
+      sm.w[lane][k] = (act && k < nv) ? yf[(size_t)site * 2 * nv + 2 * k + sp] : zero;
+      sm.v[lane][k] = (act && k < nv) ? tf[((size_t)k * V + site) * 2 + sp] : zero;
     }
+    __syncwarp();
+    const int k0 = lane >> 3, j = lane & 7;
+    float2 g0 = zero, g1 = zero, c0 = zero, c1 = zero;
+#pragma unroll 4
+    for (int r = 0; r < rows; ++r) {
+      const float2 a = sm.w[r][k0], e = sm.w[r][k0 + 4], wj = sm.w[r][j], vj = sm.v[r][j];
+      cmacf_conj(g0, a, wj);
+      cmacf_conj(g1, e, wj);
+      cmacf_conj(c0, a, vj);
+      cmacf_conj(c1, e, vj);
+    }
+    // unused vectors: an identity block, so that the factorisation runs over all eight rows
+    const bool in0 = k0 < nv && j < nv, in1 = k0 + 4 < nv && j < nv;
+    sm.G[b][lane] = in0 ? make_double2(g0.x, g0.y) : make_double2(k0 == j ? 1.0 : 0.0, 0.0);
+    sm.G[b][lane + 32] = in1 ? make_double2(g1.x, g1.y) : make_double2(k0 + 4 == j ? 1.0 : 0.0, 0.0);
+    sm.C[b][lane] = make_double2(c0.x, c0.y);
+    sm.C[b][lane + 32] = make_double2(c1.x, c1.y);
   }
   __syncwarp();
-  if (lane == 0) {
-    // Cholesky G = L L^dagger in place (lower triangle), with the ridge
+  {
+    const int q = lane >> 3, i = lane & 7;  // block of the warp; row of L and column of A
+    const bool mine = q < count;
+    const int b = mine ? q : 0;  // idle lanes shadow block 0 and write nothing
+    double2 *G = sm.G[b], *C = sm.C[b];
     double tr = 0.0;
-    for (int k = 0; k < nv; ++k) tr += G[(k * nv + k) * 2];
+    for (int k = 0; k < nv; ++k) tr += G[k * kMaxNv + k].x;
     const double ridge = 1e-7 * tr / nv + 1e-30;
-    for (int k = 0; k < nv; ++k) G[(k * nv + k) * 2] += ridge;
-    for (int j = 0; j < nv; ++j) {
-      double d = G[(j * nv + j) * 2];
-      for (int k = 0; k < j; ++k) d -= G[(j * nv + k) * 2] * G[(j * nv + k) * 2] + G[(j * nv + k) * 2 + 1] * G[(j * nv + k) * 2 + 1];
-      d = sqrt(fmax(d, 1e-300));
-      G[(j * nv + j) * 2] = d;
-      G[(j * nv + j) * 2 + 1] = 0.0;
-      for (int i = j + 1; i < nv; ++i) {
-        // L_ij = (G_ij - sum_k L_ik conj(L_jk)) / L_jj, G_ij = conj(G_ji) read from the upper part
-        double re = G[(j * nv + i) * 2], im = -G[(j * nv + i) * 2 + 1];
-        for (int k = 0; k < j; ++k) {
-          const double ar = G[(i * nv + k) * 2], ai = G[(i * nv + k) * 2 + 1];
-          const double br = G[(j * nv + k) * 2], bi = G[(j * nv + k) * 2 + 1];
-          re -= ar * br + ai * bi;
-          im -= ai * br - ar * bi;
-        }
-        G[(i * nv + j) * 2] = re / d;
-        G[(i * nv + j) * 2 + 1] = im / d;
-      }
-    }
-  }
-  __syncwarp();
-  // column j of A = G^{-1} C by lane j: L u = c_j, then L^dagger a = u
-  if (lane < nv) {
-    const int j = lane;
-    double ur[kMaxNv], ui[kMaxNv];
-    for (int i = 0; i < nv; ++i) {
-      double re = C[(i * nv + j) * 2], im = C[(i * nv + j) * 2 + 1];
-      for (int k = 0; k < i; ++k) {
-        const double lr = G[(i * nv + k) * 2], li = G[(i * nv + k) * 2 + 1];
-        re -= lr * ur[k] - li * ui[k];
-        im -= lr * ui[k] + li * ur[k];
-      }
-      const double d = G[(i * nv + i) * 2];
-      ur[i] = re / d;
-      ui[i] = im / d;
-    }
-    for (int i = nv - 1; i >= 0; --i) {
-      double re = ur[i], im = ui[i];
-      for (int k = i + 1; k < nv; ++k) {
-        // (L^dagger)_ik = conj(L_ki)
-        const double lr = G[(k * nv + i) * 2], li = -G[(k * nv + i) * 2 + 1];
-        re -= lr * A[(k * nv + j) * 2] - li * A[(k * nv + j) * 2 + 1];
-        im -= lr * A[(k * nv + j) * 2 + 1] + li * A[(k * nv + j) * 2];
-      }
-      const double d = G[(i * nv + i) * 2];
-      A[(i * nv + j) * 2] = re / d;
-      A[(i * nv + j) * 2 + 1] = im / d;
-    }
-  }
-  __syncwarp();
-  if (lane == 0) {
-    double tr = 0.0;  // Re tr(C^dagger A) = sum_ij Re(conj(C_ij) A_ij)
-    for (int q = 0; q < nv * nv; ++q) tr += C[2 * q] * A[2 * q] + C[2 * q + 1] * A[2 * q + 1];
-    lossb[(size_t)f * nb + b] = (double)nv - tr;
-  }
-  if (!act) return;
-  // R = V - W A, grad_k' = -sum_k R_k conj(A_k'k)
-  float2 r[kMaxNv];
+    double rinv[kMaxNv];
+    double2 L[kMaxNv];  // row i of L
 #pragma unroll
-  for (int k = 0; k < kMaxNv; ++k) {
-    if (k >= nv) break;
-    float2 t = v[k];
-    for (int q = 0; q < nv; ++q) {
-      const float2 a = make_float2((float)A[(q * nv + k) * 2], (float)A[(q * nv + k) * 2 + 1]);
-      cmacf(t, make_float2(-w[q].x, -w[q].y), a);
+    for (int j = 0; j < kMaxNv; ++j) {
+      // L_ij = (G_ij - sum_k L_ik conj(L_jk)) / L_jj, G_ij = conj(G_ji) read from the upper part
+      double re = G[j * kMaxNv + i].x, im = -G[j * kMaxNv + i].y;
+      if (i == j) re += ridge;
+#pragma unroll
+      for (int k = 0; k < j; ++k) {
+        const double2 ljk = G[j * kMaxNv + k];
+        re = fma(-L[k].x, ljk.x, fma(-L[k].y, ljk.y, re));
+        im = fma(-L[k].y, ljk.x, fma(L[k].x, ljk.y, im));
+      }
+      const double d = sqrt(fmax(__shfl_sync(0xffffffffu, re, 8 * q + j), 1e-300));
+      rinv[j] = 1.0 / d;
+      L[j] = make_double2(re * rinv[j], im * rinv[j]);
+      __syncwarp();
+      if (mine && i > j) G[i * kMaxNv + j] = L[j];
+      __syncwarp();
     }
-    r[k] = t;
+    // column i of A = G^{-1} C: L u = c, then L^dagger a = u
+    double2 u[kMaxNv];
+#pragma unroll
+    for (int r = 0; r < kMaxNv; ++r) {
+      double re = C[r * kMaxNv + i].x, im = C[r * kMaxNv + i].y;
+#pragma unroll
+      for (int k = 0; k < r; ++k) {
+        const double2 l = G[r * kMaxNv + k];
+        re = fma(-l.x, u[k].x, fma(l.y, u[k].y, re));
+        im = fma(-l.x, u[k].y, fma(-l.y, u[k].x, im));
+      }
+      u[r] = make_double2(re * rinv[r], im * rinv[r]);
+    }
+    double t = 0.0;  // Re tr(C^dagger A) = sum_ij Re(conj(C_ij) A_ij)
+#pragma unroll
+    for (int r = kMaxNv - 1; r >= 0; --r) {
+      double re = u[r].x, im = u[r].y;
+#pragma unroll
+      for (int k = r + 1; k < kMaxNv; ++k) {
+        const double2 l = G[k * kMaxNv + r];  // (L^dagger)_rk = conj(L_kr)
+        re = fma(-l.x, u[k].x, fma(-l.y, u[k].y, re));
+        im = fma(-l.x, u[k].y, fma(l.y, u[k].x, im));
+      }
+      u[r] = make_double2(re * rinv[r], im * rinv[r]);
+      t = fma(C[r * kMaxNv + i].x, u[r].x, fma(C[r * kMaxNv + i].y, u[r].y, t));
+      if (mine) sm.A[b][r * kMaxNv + i] = make_float2((float)u[r].x, (float)u[r].y);
+    }
+#pragma unroll
+    for (int o = 1; o < 8; o <<= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    if (mine && i == 0) lossb[(size_t)f * bg.nblocks + first + b] = (double)nv - t;
   }
+  __syncwarp();
+  if (!act) return;
   float2 *gf = gy + (size_t)f * V * 2 * nv;
-  for (int kp = 0; kp < nv; ++kp) {
-    float2 t = make_float2(0.f, 0.f);
-    for (int k = 0; k < nv; ++k) {
-      const float2 a = make_float2((float)A[(kp * nv + k) * 2], (float)A[(kp * nv + k) * 2 + 1]);
-      cmacf(t, r[k], conjf2(a));
+  for (int b = 0; b < count; ++b) {
+    const long long site = fine_site_of(bg, first + b, lane >> 1);
+    const float2 *A = sm.A[b];
+    float2 w[kMaxNv], r[kMaxNv];
+#pragma unroll
+    for (int k = 0; k < kMaxNv; ++k) {
+      w[k] = k < nv ? yf[(size_t)site * 2 * nv + 2 * k + sp] : zero;
+      r[k] = k < nv ? tf[((size_t)k * V + site) * 2 + sp] : zero;
     }
-    gf[(size_t)site * 2 * nv + 2 * kp + sp] = make_float2(-scale * t.x, -scale * t.y);
+    // R = V - W A, grad_k' = -sum_k R_k conj(A_k'k)
+#pragma unroll
+    for (int k = 0; k < kMaxNv; ++k)
+#pragma unroll
+      for (int q = 0; q < kMaxNv; ++q) cmacf(r[k], make_float2(-w[q].x, -w[q].y), A[q * kMaxNv + k]);
+#pragma unroll
+    for (int kp = 0; kp < kMaxNv; ++kp) {
+      if (kp >= nv) break;
+      float2 t = zero;
+#pragma unroll
+      for (int k = 0; k < kMaxNv; ++k) cmacf(t, r[k], conjf2(A[kp * kMaxNv + k]));
+      gf[(size_t)site * 2 * nv + 2 * kp + sp] = make_float2(-scale * t.x, -scale * t.y);
+    }
   }
 }
 
@@ -464,33 +518,36 @@ __global__ void to_float2_kernel(const Cx<double> *__restrict__ a, long long n, 
 
 int blocks_for(long long n, int t) { return (int)((n + t - 1) / t); }
 
-int site_grid(long long V) {
-  const long long want = (V + kWarps - 1) / kWarps;
-  return (int)(want < 152 * 16 ? want : 152 * 16);
+// CTAs per field: three resident on each of 152 SMs over all fields (each stages the weights once)
+template <Conv M, typename TI>
+void conv_launch(const TI *in, const float2 *U, const int *fmap, const float2 *W, int kin, int kout, int L0, int L1,
+                 int nf, const float2 *a_prev, float2 *a_out, __nv_bfloat162 *h_out, cudaStream_t s) {
+  auto fn = ptconv_kernel<M, TI>;
+  const int S = conv_tile(kout / 2);
+  const size_t smem = ((size_t)5 * kin * kout + (size_t)kin * S) * sizeof(float2);
+  MG_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  const long long tiles = ((long long)L0 * L1 + S - 1) / S;
+  long long gx = (152 * 3 + nf - 1) / nf;
+  if (gx > tiles) gx = tiles;
+  fn<<<dim3((unsigned int)gx, nf), kConvThreads, smem, s>>>(in, U, fmap, W, kin, kout, L0, L1, a_prev, a_out, h_out);
+  MG_LAUNCHED();
 }
 
 }  // namespace
 
 void launch_ptconv_fwd(const void *h_in, const float2 *U, const int *fmap, const float2 *W, int ci2, int co2,
                        int L0, int L1, int nf, bool last, float2 *a_out, void *h_out, cudaStream_t s) {
-  const dim3 grid(site_grid((long long)L0 * L1), nf);
   const auto *hi = static_cast<const __nv_bfloat162 *>(h_in);
   if (last)
-    ptconv_fwd_kernel<true><<<grid, 256, 0, s>>>(hi, U, fmap, W, ci2, co2, L0, L1, a_out, nullptr);
+    conv_launch<Conv::kLast>(hi, U, fmap, W, ci2, co2, L0, L1, nf, nullptr, a_out, nullptr, s);
   else
-    ptconv_fwd_kernel<false><<<grid, 256, 0, s>>>(hi, U, fmap, W, ci2, co2, L0, L1, a_out,
-                                                   static_cast<__nv_bfloat162 *>(h_out));
-  MG_LAUNCHED();
+    conv_launch<Conv::kHidden>(hi, U, fmap, W, ci2, co2, L0, L1, nf, nullptr, a_out,
+                               static_cast<__nv_bfloat162 *>(h_out), s);
 }
 
 void launch_ptconv_bwd_data(const float2 *ga, const float2 *U, const int *fmap, const float2 *W, int ci2, int co2,
                             int L0, int L1, int nf, const float2 *a_prev, float2 *ga_prev, cudaStream_t s) {
-  const dim3 grid(site_grid((long long)L0 * L1), nf);
-  if (a_prev != nullptr)
-    ptconv_bwd_data_kernel<true><<<grid, 256, 0, s>>>(ga, U, fmap, W, ci2, co2, L0, L1, a_prev, ga_prev);
-  else
-    ptconv_bwd_data_kernel<false><<<grid, 256, 0, s>>>(ga, U, fmap, W, ci2, co2, L0, L1, nullptr, ga_prev);
-  MG_LAUNCHED();
+  conv_launch<Conv::kAdjoint>(ga, U, fmap, W, co2, ci2, L0, L1, nf, a_prev, ga_prev, nullptr, s);
 }
 
 void launch_ptconv_bwd_weight(const float2 *ga, const void *h_in, const float2 *U, const int *fmap, int nf, int ci2,
@@ -505,8 +562,10 @@ void launch_ptconv_bwd_weight(const float2 *ga, const void *h_in, const float2 *
 
 void launch_nullnet_loss(const float2 *y, const float2 *target, const int *fmap, int nv, const BlockGeo &bg, int nf,
                          float scale, float2 *gy, double *lossb, cudaStream_t s) {
-  const dim3 grid(blocks_for(bg.nblocks, 4), nf);
-  nullnet_loss_kernel<<<grid, 128, 0, s>>>(y, target, fmap, nv, bg, scale, gy, lossb);
+  const dim3 grid(blocks_for(bg.nblocks, kLossWarps * kLossBlocks), nf);
+  const int smem = kLossWarps * (int)sizeof(LossSmem);
+  MG_CUDA(cudaFuncSetAttribute(nullnet_loss_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+  nullnet_loss_kernel<<<grid, 32 * kLossWarps, smem, s>>>(y, target, fmap, nv, bg, scale, gy, lossb);
   MG_LAUNCHED();
 }
 
