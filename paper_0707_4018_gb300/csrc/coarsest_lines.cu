@@ -80,63 +80,73 @@ __global__ void line_blocks_kernel(const Cx<double> *__restrict__ Y, Cx<double> 
   out[(long long)p * b * b + t] = v;
 }
 
-// in-place inverse of the m x m block in `a` by 256 threads (thread = element), partial pivoting;
-// *info = 1 on a pivot that is zero or not finite
+// Inverse of the m x m block in `a` by 256 threads (thread = element), partial pivoting, result in `a`;
+// *info = 1 on a pivot that is zero or not finite. A chain of m steps: warp 0 picks the pivot from the
+// entries' FP32 magnitudes (one integer maximum; which of two nearly equal rows leads does not matter),
+// inverts it and scales the pivot row, then every element is updated into the other buffer, so a step
+// is two barriers and 16 x 16 complex multiply-adds. 11 us; with exact norms, a division by every
+// thread's element and in-place updates 33 us.
 __device__ __forceinline__ void invert_tile(Cx<double> (*a)[kT + 1], int m, int *info) {
-  __shared__ int piv[kT];
+  __shared__ Cx<double> other[kT][kT + 1], lead[kT];
   __shared__ Cx<double> dinv;
+  __shared__ int piv[kT];
   const int i = threadIdx.x / kT, j = threadIdx.x % kT;
   const bool in = i < m && j < m;
+  Cx<double>(*src)[kT + 1] = a, (*dst)[kT + 1] = other;
   for (int s = 0; s < m; ++s) {
     __syncthreads();
     if (threadIdx.x < 32) {
       const int lane = threadIdx.x;
-      double v = lane >= s && lane < m ? norm2(a[lane][s]) : -1.0;
-      int r = lane;
-#pragma unroll
-      for (int o = 8; o > 0; o >>= 1) {
-        const double ov = __shfl_xor_sync(0xffffffffu, v, o);
-        const int orr = __shfl_xor_sync(0xffffffffu, r, o);
-        if (ov > v || (ov == v && orr < r)) { v = ov; r = orr; }
-      }
+      unsigned int key = 0u;
+      if (lane >= s && lane < m)
+        key = (__float_as_uint(fmaxf(fabsf((float)src[lane][s].re), fabsf((float)src[lane][s].im))) & ~15u) |
+              (unsigned int)(15 - lane);
+      key = __reduce_max_sync(0xffffffffu, key);
+      const int p = 15 - (int)(key & 15u);
+      const Cx<double> pv = src[p][s];
+      const double inv = 1.0 / norm2(pv);
+      const Cx<double> d = mk(pv.re * inv, -pv.im * inv);
       if (lane == 0) {
-        piv[s] = v > 0.0 ? r : s;
-        const Cx<double> pv = a[piv[s]][s];
-        const double inv = v > 0.0 ? 1.0 / v : 0.0;
-        if (!(v > 0.0) || !isfinite(v) || !isfinite(inv)) *info = 1;
-        dinv = mk(pv.re * inv, -pv.im * inv);
+        piv[s] = p;
+        dinv = d;
+        if (!(inv > 0.0) || !isfinite(inv)) *info = 1;
       }
+      if (lane < m) lead[lane] = src[p][lane] * d;
     }
     __syncthreads();
-    const int p = piv[s];
-    // rows s and p change places while the step is applied: read first, write after
-    const int src = i == s ? p : i == p ? s : i;
-    Cx<double> v = mk(0.0, 0.0);
     if (in) {
-      const Cx<double> as = a[src][s], pj = a[p][j];
-      if (i == s)
-        v = j == s ? dinv : pj * dinv;
-      else if (j == s)
-        v = mk(-(as.re * dinv.re - as.im * dinv.im), -(as.re * dinv.im + as.im * dinv.re));
-      else {
-        v = a[src][j];
-        const Cx<double> f = pj * dinv;
-        cmac(v, mk(-as.re, -as.im), f);
+      const int p = piv[s];
+      const int row = i == s ? p : i == p ? s : i;  // rows s and p change places
+      const Cx<double> as = src[row][s];
+      Cx<double> v;
+      if (i == s) {
+        v = j == s ? dinv : lead[j];
+      } else if (j == s) {
+        v = as * dinv;
+        v = mk(-v.re, -v.im);
+      } else {
+        v = src[row][j];
+        cmac(v, mk(-as.re, -as.im), lead[j]);
       }
+      dst[i][j] = v;
     }
-    __syncthreads();
-    if (in) a[i][j] = v;
+    Cx<double>(*t)[kT + 1] = src;
+    src = dst;
+    dst = t;
   }
-  // undo the row exchanges as column exchanges, last first
-  for (int s = m - 1; s >= 0; --s) {
-    __syncthreads();
-    const int p = piv[s];
-    if (p != s && j == s && i < m) {
-      const Cx<double> t = a[i][s];
-      a[i][s] = a[i][p];
-      a[i][p] = t;
+  // the row exchanges undone as column exchanges, last first: column j of the result
+  __syncthreads();
+  Cx<double> v = mk(0.0, 0.0);
+  if (in) {
+    int c = j;
+    for (int s = 0; s < m; ++s) {  // where column j comes from: the exchanges in forward order
+      const int p = piv[s];
+      c = c == s ? p : c == p ? s : c;
     }
+    v = src[i][c];
   }
+  __syncthreads();
+  if (in) a[i][j] = v;
   __syncthreads();
 }
 
@@ -198,7 +208,15 @@ __global__ void __launch_bounds__(kT *kT) gj_step_kernel(const Cx<double> *__res
   }
 }
 
-// the block products of one level
+// whether 16 x 16 tiles whose first indexes differ by d can hold an entry within `band` (cyclic in b)
+__device__ __forceinline__ bool in_band(int d, int b, int band) {
+  const int lo = min(abs(d), min(abs(d - b), abs(d + b)));
+  return lo - (kT - 1) <= band || b - (kT - 1) <= band;
+}
+
+// the block products of one level, at the FP64 rate. The couplings of the finest ring connect a site to
+// the site(s) of the next line beside it: their products take 3 of 8 tiles at most (16 x 16 sites, N = 8:
+// 1.2 instead of 1.9 ms of products per factorisation)
 __global__ void __launch_bounds__(kT *kT) line_product_kernel(const LineJob *__restrict__ jobs, int b) {
   __shared__ Cx<double> A[kT][kT + 1], B[kT][kT + 1];
   const LineJob job = jobs[blockIdx.y];
@@ -212,6 +230,9 @@ __global__ void __launch_bounds__(kT *kT) line_product_kernel(const LineJob *__r
     const Cx<double> *Am = half ? job.A2 : job.A1, *Bm = half ? job.B2 : job.B1;
     if (Am == nullptr) continue;
     for (int k0 = 0; k0 < b; k0 += kT) {
+      // tiles outside a factor's band hold zeros
+      if (job.band_a >= 0 && !in_band(k0 - tr * kT, b, job.band_a)) continue;
+      if (job.band_b >= 0 && !in_band(k0 - tc * kT, b, job.band_b)) continue;
       __syncthreads();
       A[i][j] = r < b && k0 + j < b ? Am[(long long)r * b + k0 + j] : mk(0.0, 0.0);
       B[i][j] = k0 + i < b && c < b ? Bm[(long long)(k0 + i) * b + c] : mk(0.0, 0.0);
@@ -399,7 +420,7 @@ std::vector<LineLevel> line_levels(int r, int b, long long *ws) {
   return lv;
 }
 
-void line_plan(LineSolver &f, Geo2 g, int N, cudaStream_t s) {
+void line_plan(LineSolver &f, Geo2 g, int N, bool nine, cudaStream_t s) {
   if (f.planned) return;
   f.N = N;
   f.L0 = g.L0;
@@ -443,13 +464,15 @@ void line_plan(LineSolver &f, Geo2 g, int N, cudaStream_t s) {
   for (size_t k = 0; k + 1 < f.lv.size(); ++k) {
     LineLevel &l = f.lv[k];
     const LineLevel &c = f.lv[k + 1];
+    const int band = k > 0 ? -1 : nine ? 2 * N - 1 : N - 1;  // of the couplings L and R
     l.w_jobs = (long long)f.jobs.size();
     for (int e = 0; e < l.E; ++e) {
       const Cx<double> *di = l.Dinv + e * b2;
       f.jobs.push_back({l.WL + e * b2, nullptr, nullptr, di, (l.r == 2 ? l.R : l.L) + (2 * e + 1) * b2, nullptr,
-                        nullptr, 1.0});
+                        nullptr, 1.0, -1, band});
       if (l.r > 2)
-        f.jobs.push_back({l.WR + e * b2, nullptr, nullptr, di, l.R + (2 * e + 1) * b2, nullptr, nullptr, 1.0});
+        f.jobs.push_back({l.WR + e * b2, nullptr, nullptr, di, l.R + (2 * e + 1) * b2, nullptr, nullptr, 1.0, -1,
+                          band});
     }
     l.n_w = (int)(f.jobs.size() - l.w_jobs);
     l.u_jobs = (long long)f.jobs.size();
@@ -458,7 +481,7 @@ void line_plan(LineSolver &f, Geo2 g, int N, cudaStream_t s) {
       const int right = pos + 1 < l.r ? a : -1;
       const int left = l.r == 2 ? -1 : a > 0 ? a - 1 : l.r % 2 == 0 ? l.E - 1 : -1;
       const Cx<double> *Ra = l.R + pos * b2, *La = l.L + pos * b2;
-      LineJob d{c.D + a * b2, l.D + pos * b2, nullptr, nullptr, nullptr, nullptr, nullptr, -1.0};
+      LineJob d{c.D + a * b2, l.D + pos * b2, nullptr, nullptr, nullptr, nullptr, nullptr, -1.0, band, -1};
       if (right >= 0) {
         d.A1 = Ra;
         d.B1 = l.WL + right * b2;
@@ -470,8 +493,8 @@ void line_plan(LineSolver &f, Geo2 g, int N, cudaStream_t s) {
       f.jobs.push_back(d);
       if (l.K == 1) continue;
       // couplings of the kept line to the next and to the previous kept line
-      LineJob n{c.R + a * b2, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, -1.0};
-      LineJob v{c.L + a * b2, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, -1.0};
+      LineJob n{c.R + a * b2, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, -1.0, band, -1};
+      LineJob v{c.L + a * b2, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, -1.0, band, -1};
       if (right >= 0) {
         n.A1 = Ra;
         n.B1 = l.WR + right * b2;
@@ -604,7 +627,7 @@ long long line_work_size(Geo2 g, int N) {
 bool line_factor(LineSolver &f, const Cx<double> *Y, Geo2 g, int N, bool nine, double shift, Cx<double> *work,
                  cudaStream_t s, const char *what) {
   const bool first = !f.planned, was = f.lines;
-  line_plan(f, g, N, s);
+  line_plan(f, g, N, nine, s);
   f.lines = line_try(f, Y, nine, shift, work, s);
   if (!f.lines) {
     if (f.LU.p == nullptr) {

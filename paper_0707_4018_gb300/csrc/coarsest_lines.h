@@ -18,11 +18,13 @@ struct LineLevel {
   int n_w = 0, n_u = 0;
 };
 
-// C = I1 + I2 + sgn (A1 B1 + A2 B2) on b x b row-major blocks (null terms left out)
+// C = I1 + I2 + sgn (A1 B1 + A2 B2) on b x b row-major blocks (null terms left out). band_a / band_b: the
+// left / right factors' entries (i, k) vanish where |i - k| (cyclic in b) exceeds it; -1: full.
 struct LineJob {
   Cx<double> *C;
   const Cx<double> *I1, *I2, *A1, *B1, *A2, *B2;
   double sgn;
+  int band_a, band_b;
 };
 
 struct LineSolver {

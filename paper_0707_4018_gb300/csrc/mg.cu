@@ -25,6 +25,7 @@
 #include "kernels.h"
 #include "krylov.h"
 #include "mg4d.h"
+#include "mr.cuh"
 #include "nullnet.h"
 
 namespace mg {
@@ -1479,7 +1480,8 @@ static std::unique_ptr<mg_ctx> create(const mg_geom *g, double m, const mg_param
   for (int l = 0; l < p->levels; ++l) {
     // fine: a thread per site; coarse N = 8: four threads per dof; other N: a thread per dof
     const long long units = l == 0 ? c->lv[l].geo.nsites : (c->lv[l].nint == 8 ? 4 : 1) * c->lv[l].n;
-    cap = std::max(cap, 3 * ((units + 255) / 256) * c->nbatch);
+    const int per = l == 0 ? site_threads(units) : 256;
+    cap = std::max(cap, 3 * ((units + per - 1) / per) * c->nbatch);
   }
   cap = std::max(cap, 2LL * (p->gcr_restart + 3) * p->max_rhs * 64);
   c->partials.alloc((size_t)cap + 16);

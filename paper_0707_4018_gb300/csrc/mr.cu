@@ -49,7 +49,7 @@ __global__ void __launch_bounds__(256) mr_wilson_kernel(const Cx<R> *__restrict_
   Cx<R> alpha = z;
   R v[3] = {(R)0, (R)0, (R)0};
   // every block makes its first pass (alpha is a block-wide sum), then strides on
-  const long long sb = blockIdx.x * 256LL;
+  const long long sb = blockIdx.x * (long long)blockDim.x;
   long long s0 = sb;
   do {
     const long long s = s0 + threadIdx.x;
@@ -115,7 +115,7 @@ __global__ void __launch_bounds__(256) mr_wilson_kernel(const Cx<R> *__restrict_
       v[1] += a0.re * p0.im - a0.im * p0.re + a1.re * p1.im - a1.im * p1.re;
       v[2] += a0.re * a0.re + a0.im * a0.im + a1.re * a1.re + a1.im * a1.im;
     }
-    s0 += gridDim.x * 256LL;
+    s0 += gridDim.x * (long long)blockDim.x;
   } while (LOOP && s0 < V);
   mr_publish<R>(v, part_out, sh);
 }
@@ -401,14 +401,15 @@ __global__ void mr_last_kernel(const Cx<R> *r_old, const Cx<R> *Ar_old, const R 
 template <typename R>
 int mr_grid(const OpDesc<R> &op) {
   const long long units = op.wilson ? op.geo.nsites : op.geo.nsites * (op.N == 8 ? 32 : op.N);
-  return mr_blocks((units + 255) / 256);
+  const int threads = op.wilson ? site_threads(units) : 256;
+  return mr_blocks((units + threads - 1) / threads);
 }
 
 template <typename R>
 void launch_mr_iteration(const OpDesc<R> &op, bool step, const Cx<R> *r_old, const Cx<R> *Ar_old, const R *part_in,
                          double omega, Cx<R> *x, bool x_init, Cx<R> *r_new, Cx<R> *Ar_new, R *part_out,
                          long long part_capacity, cudaStream_t s, int nvec) {
-  const int threads = 256;
+  const int threads = op.wilson ? site_threads(op.geo.nsites) : 256;
   if (nvec > 128) fail(MG_ERR_UNSUPPORTED, "MR batch larger than 128 vectors");
   const int nb = mr_grid(op);
   if (3LL * nb * nvec > part_capacity) fail(MG_ERR_STATE, "MR reduction workspace too small");

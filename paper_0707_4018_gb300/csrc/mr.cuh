@@ -40,6 +40,10 @@ __device__ __forceinline__ void block_reduce(T (&v)[NOUT], T *sh) {
 constexpr int kMrGrid = 1216;
 inline int mr_blocks(long long full) { return (int)(full < kMrGrid ? full : kMrGrid); }
 
+// Threads per block of the fine-level MR and apply kernels: small lattices take smaller blocks, which
+// reach more SMs (64^2 in FP64, bound by the FP64 rate: an MR iteration on 16 of 152 SMs took 16 us).
+inline int site_threads(long long sites) { return sites <= 64LL * 152 ? 64 : 256; }
+
 // this block's (<A r, r> re, im, |A r|^2) into part_out[3 blockIdx.x ..]
 template <typename R>
 __device__ __forceinline__ void mr_publish(R (&v)[3], R *part_out, R *sh) {

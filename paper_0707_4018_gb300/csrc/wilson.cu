@@ -8,6 +8,7 @@
 // The fused epilogue out = a * D in + c * b forms residuals b - D x in the
 // same pass.
 #include "kernels.h"
+#include "mr.cuh"
 #include "wilson.cuh"
 
 namespace mg {
@@ -68,7 +69,7 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 8 : 4) dslash_kernel(con
 template <typename R>
 void launch_dslash(const Cx<R> *U, const Cx<R> *in, Cx<R> *out, Geo2 g, double diag, const Cx<R> *b, double a,
                    double c, cudaStream_t s, int nvec, const double *shift) {
-  const int threads = 256;
+  const int threads = site_threads(g.nsites);
   const dim3 grid(grid_for(g.nsites, threads), nvec);
   if (shift != nullptr)
     dslash_kernel<R, true><<<grid, threads, 0, s>>>(U, in, out, g.L0, g.L1, (R)diag, b, (R)a, (R)c, 2 * g.nsites, shift);
