@@ -94,4 +94,85 @@ __device__ __forceinline__ void hop_dispatch(int hop, const Cx<R> (&p)[12], cons
   }
 }
 
+// h = psi_up - A_mu psi_dn (MINUS, the forward hop's (1 - gamma_mu)) or psi_up + A_mu psi_dn
+template <typename R, int MU, bool MINUS>
+__device__ __forceinline__ void hop_project(const Cx<R> (&p)[12], Cx<R> (&h)[2][3]) {
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    Cx<R> a0, a1;
+    a_times<R, MU>(p[6 + c], p[9 + c], a0, a1);
+    h[0][c] = MINUS ? p[c] - a0 : p[c] + a0;
+    h[1][c] = MINUS ? p[3 + c] - a1 : p[3 + c] + a1;
+  }
+}
+
+// forward hop of direction MU: t = U (1 - gamma_mu) psi_{x+mu}, upper half
+template <typename R, int MU>
+__device__ __forceinline__ void hop_fwd(const Cx<R> (&p)[12], const Cx<R> *link, Cx<R> (&t)[2][3]) {
+  Cx<R> h[2][3];
+  hop_project<R, MU, true>(p, h);
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    t[0][a] = mk((R)0, (R)0);
+    t[1][a] = mk((R)0, (R)0);
+#pragma unroll
+    for (int b = 0; b < 3; ++b) {
+      const Cx<R> u = link[a * 3 + b];  // U_ab
+      cmac(t[0][a], u, h[0][b]);
+      cmac(t[1][a], u, h[1][b]);
+    }
+  }
+}
+
+// backward hop, and both hops into the accumulators (the -1/2 is applied at the end): with the forward t and
+// the backward one t', up += t + t' and dn += A_mu^dagger (t' - t). The backward product is summed onto t
+// (s = t + t'), and t' - t = s - 2 t: 36 additions for a direction's two hops where adding each by itself
+// takes 48, in a kernel that the FP64 rate bounds.
+template <typename R, int MU>
+__device__ __forceinline__ void hop_bwd(const Cx<R> (&p)[12], const Cx<R> *link, const Cx<R> (&t)[2][3],
+                                        Cx<R> (&acc)[12]) {
+  Cx<R> h[2][3];
+  hop_project<R, MU, false>(p, h);
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    Cx<R> s0 = t[0][a], s1 = t[1][a];
+#pragma unroll
+    for (int b = 0; b < 3; ++b) {
+      const Cx<R> u = link[b * 3 + a];  // (U^dagger)_ab = conj(U_ba)
+      cmac_conj(s0, u, h[0][b]);
+      cmac_conj(s1, u, h[1][b]);
+    }
+    const R m2 = (R)-2;
+    const Cx<R> d0 = mk(fma(m2, t[0][a].re, s0.re), fma(m2, t[0][a].im, s0.im));
+    const Cx<R> d1 = mk(fma(m2, t[1][a].re, s1.re), fma(m2, t[1][a].im, s1.im));
+    Cx<R> l0, l1;
+    adag_times<R, MU>(d0, d1, l0, l1);
+    acc[a] = acc[a] + s0;
+    acc[3 + a] = acc[3 + a] + s1;
+    acc[6 + a] = acc[6 + a] + l0;
+    acc[9 + a] = acc[9 + a] + l1;
+  }
+}
+
+template <typename R>
+__device__ __forceinline__ void hop_fwd_dispatch(int mu, const Cx<R> (&p)[12], const Cx<R> *link, Cx<R> (&t)[2][3]) {
+  switch (mu) {
+    case 0: hop_fwd<R, 0>(p, link, t); break;
+    case 1: hop_fwd<R, 1>(p, link, t); break;
+    case 2: hop_fwd<R, 2>(p, link, t); break;
+    default: hop_fwd<R, 3>(p, link, t); break;
+  }
+}
+
+template <typename R>
+__device__ __forceinline__ void hop_bwd_dispatch(int mu, const Cx<R> (&p)[12], const Cx<R> *link,
+                                                 const Cx<R> (&t)[2][3], Cx<R> (&acc)[12]) {
+  switch (mu) {
+    case 0: hop_bwd<R, 0>(p, link, t, acc); break;
+    case 1: hop_bwd<R, 1>(p, link, t, acc); break;
+    case 2: hop_bwd<R, 2>(p, link, t, acc); break;
+    default: hop_bwd<R, 3>(p, link, t, acc); break;
+  }
+}
+
 }  // namespace mg
