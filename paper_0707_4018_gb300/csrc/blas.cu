@@ -39,9 +39,9 @@ __global__ void __launch_bounds__(kReduceThreads) dot_norm_kernel(const Cx<R> *_
   double v[3] = {0.0, 0.0, 0.0};
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
     const Cx<double> x = cvt<double>(a[i]), y = cvt<double>(b[i]);
-    v[0] += x.re * y.re + x.im * y.im;
-    v[1] += x.re * y.im - x.im * y.re;
-    v[2] += x.re * x.re + x.im * x.im;
+    v[0] = fma(x.re, y.re, fma(x.im, y.im, v[0]));
+    v[1] = fma(x.re, y.im, fma(-x.im, y.re, v[1]));
+    v[2] = fma(x.re, x.re, fma(x.im, x.im, v[2]));
   }
   grid_finish<3>(v, partials, out, ticket, sh);
 }
@@ -436,7 +436,7 @@ void launch_xmy(const Cx<R> *x, Cx<R> *y, long long n, cudaStream_t s) {
 }
 template <typename R>
 void launch_dot_norm(const Cx<R> *a, const Cx<R> *b, long long n, double *out, const ReduceWs &ws, cudaStream_t s) {
-  dot_norm_kernel<R><<<reduce_blocks(n, ws.max_blocks), kReduceThreads, 0, s>>>(a, b, n, ws.partials, out, ws.ticket);
+  dot_norm_kernel<R><<<dot_blocks(n, ws.max_blocks), kReduceThreads, 0, s>>>(a, b, n, ws.partials, out, ws.ticket);
   MG_LAUNCHED();
 }
 template <typename R>

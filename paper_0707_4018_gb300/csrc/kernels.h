@@ -50,6 +50,10 @@ template <typename R>
 void launch_dslash(const Cx<R> *U, const Cx<R> *in, Cx<R> *out, Geo2 g, double diag, const Cx<R> *b, double a,
                    double c, cudaStream_t s, int nvec = 1, const double *shift = nullptr);
 
+// out = gamma_5 D in (D^dagger D = gamma_5 D gamma_5 D), FP64
+void launch_dslash_g5(const Cx<double> *U, const Cx<double> *in, Cx<double> *out, Geo2 g, double diag,
+                      cudaStream_t s);
+
 // ---- fine Wilson operator (4d, SU(3), DeGrand-Rossi gammas) ----
 // out = a * D in + c * b on psi[x][4][3], U[x][4][3][3]; diagonal `diag` = 4 + m (+ shift[v])
 template <typename R>

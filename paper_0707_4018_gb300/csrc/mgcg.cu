@@ -100,15 +100,19 @@ __global__ void dense_from_stencil9_kernel(const Cx<double> *__restrict__ Y, Cx<
   A[t] = v;
 }
 
-// x += a r; r -= a w
-__global__ void step_kernel(Cx<double> *__restrict__ x, Cx<double> *__restrict__ r, const Cx<double> *__restrict__ w,
-                            double are, double aim, long long n) {
+// one MR step: x += a r (x = a r with x_init) and, unless r_out is null, r_out = r - a w (r_out may be r)
+__global__ void step_kernel(Cx<double> *__restrict__ x, const Cx<double> *r, Cx<double> *r_out,
+                            const Cx<double> *__restrict__ w, double are, double aim, int x_init, long long n) {
   const Cx<double> a = mk(are, aim), ma = mk(-are, -aim);
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-    cmac(x[i], a, r[i]);
     Cx<double> ri = r[i];
-    cmac(ri, ma, w[i]);
-    r[i] = ri;
+    Cx<double> xi = x_init ? mk(0.0, 0.0) : x[i];
+    cmac(xi, a, ri);
+    x[i] = xi;
+    if (r_out != nullptr) {
+      cmac(ri, ma, w[i]);
+      r_out[i] = ri;
+    }
   }
 }
 
@@ -122,12 +126,7 @@ __global__ void cg_update_kernel(Cx<double> *__restrict__ x, Cx<double> *__restr
   }
 }
 
-// x += t; and the CG direction p = z + beta p
-__global__ void add_kernel(Cx<double> *__restrict__ x, const Cx<double> *__restrict__ t, long long n) {
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
-    x[i] = x[i] + t[i];
-}
-
+// the CG direction p = z + beta p
 __global__ void direction_kernel(Cx<double> *__restrict__ p, const Cx<double> *__restrict__ z, double beta,
                                  long long n) {
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
@@ -203,12 +202,8 @@ static void cg_apply(CgEngine &e, int l, const Cx<double> *in, Cx<double> *out) 
   CgLevel &L = e.lv[l];
   if (l == 0) {
     const double diag = 2.0 + e.m;
-    launch_dslash<double>(e.U.p, in, e.tmp.p, L.geo, diag, nullptr, 1.0, 0.0, e.s, 1, nullptr);
-    gamma5_kernel<<<grid_for(L.geo.nsites, 256), 256, 0, e.s>>>(e.tmp.p, L.geo.nsites);
-    MG_LAUNCHED();
-    launch_dslash<double>(e.U.p, e.tmp.p, out, L.geo, diag, nullptr, 1.0, 0.0, e.s, 1, nullptr);
-    gamma5_kernel<<<grid_for(L.geo.nsites, 256), 256, 0, e.s>>>(out, L.geo.nsites);
-    MG_LAUNCHED();
+    launch_dslash_g5(e.U.p, in, e.tmp.p, L.geo, diag, e.s);
+    launch_dslash_g5(e.U.p, e.tmp.p, out, L.geo, diag, e.s);
     ++e.fine_apps;
   } else {
     stencil9_kernel<<<grid_for(L.n, 256), 256, 0, e.s>>>(L.Y.p, in, out, L.geo.L0, L.geo.L1, L.nint);
@@ -227,16 +222,20 @@ static void cg_dot(CgEngine &e, const Cx<double> *a, const Cx<double> *b, long l
   }
 }
 
-// x = R b with the frozen two-step MR polynomial; r = b - A x
-static void frozen_smooth(CgEngine &e, int l, const Cx<double> *b, Cx<double> *x, Cx<double> *r) {
+static void cg_step(CgEngine &e, Cx<double> *x, const Cx<double> *r, Cx<double> *r_out, const Cx<double> *w,
+                    double are, double aim, bool x_init, long long n) {
+  step_kernel<<<blocks_for(n), 256, 0, e.s>>>(x, r, r_out, w, are, aim, x_init ? 1 : 0, n);
+  MG_LAUNCHED();
+}
+
+// x = R b (add: x += R b) with the frozen two-step MR polynomial; r is scratch and, unless adding, ends as
+// b - A R b (b may not be r)
+static void frozen_smooth(CgEngine &e, int l, const Cx<double> *b, Cx<double> *x, Cx<double> *r, bool add) {
   CgLevel &L = e.lv[l];
-  launch_zero<double>(x, L.n, e.s);
-  launch_copy<double>(b, r, L.n, e.s);
-  for (int i = 0; i < 2; ++i) {
-    cg_apply(e, l, r, L.w.p);
-    step_kernel<<<blocks_for(L.n), 256, 0, e.s>>>(x, r, L.w.p, L.alpha[i], 0.0, L.n);
-    MG_LAUNCHED();
-  }
+  cg_apply(e, l, b, L.w.p);
+  cg_step(e, x, b, r, L.w.p, L.alpha[0], 0.0, !add, L.n);
+  cg_apply(e, l, r, L.w.p);
+  cg_step(e, x, r, add ? nullptr : r, L.w.p, L.alpha[1], 0.0, false, L.n);
 }
 
 // x = V_l b (Eq. vcycle, R = R^dagger); b must not be a buffer of level l
@@ -247,16 +246,13 @@ static void cg_vcycle(CgEngine &e, int l, const Cx<double> *b, Cx<double> *x) {
     return;
   }
   CgLevel &C = e.lv[l + 1];
-  frozen_smooth(e, l, b, x, L.r.p);
+  frozen_smooth(e, l, b, x, L.r.p, false);
   launch_restrict<double>(L.V.p, L.r.p, C.b.p, L.bg, L.Nv, e.s);
   cg_vcycle(e, l + 1, C.b.p, C.x.p);
   launch_prolong_add<double>(L.V.p, C.x.p, x, L.bg, L.Nv, e.s);
-  cg_apply(e, l, x, L.w.p);
-  launch_copy<double>(L.w.p, L.r.p, L.n, e.s);
+  cg_apply(e, l, x, L.r.p);
   launch_xmy<double>(b, L.r.p, L.n, e.s);  // r = b - A x
-  frozen_smooth(e, l, L.r.p, L.t.p, L.r2.p);
-  add_kernel<<<blocks_for(L.n), 256, 0, e.s>>>(x, L.t.p, L.n);
-  MG_LAUNCHED();
+  frozen_smooth(e, l, L.r.p, x, L.r2.p, true);
 }
 
 // the Nv vectors of level l: Philox draws relaxed by nu_setup MR iterations on A x = 0
@@ -274,9 +270,7 @@ static void cg_relax(CgEngine &e, int l) {
       double d[3];
       cg_dot(e, L.w.p, L.r.p, L.n, d);
       if (d[2] == 0.0) break;
-      step_kernel<<<blocks_for(L.n), 256, 0, e.s>>>(v, L.r.p, L.w.p, e.p.omega * d[0] / d[2], e.p.omega * d[1] / d[2],
-                                                      L.n);
-      MG_LAUNCHED();
+      cg_step(e, v, L.r.p, L.r.p, L.w.p, e.p.omega * d[0] / d[2], e.p.omega * d[1] / d[2], false, L.n);
     }
   }
 }
@@ -314,8 +308,7 @@ static void cg_prepare(CgEngine &e) {
       cg_dot(e, L.w.p, L.r.p, L.n, d);
       if (d[2] <= 0.0) fail(MG_ERR_NAN, "MG-CG: zero operator image in the smoother setup");
       L.alpha[i] = e.p.omega * d[0] / d[2];  // real for hermitian A
-      step_kernel<<<blocks_for(L.n), 256, 0, e.s>>>(L.t.p, L.r.p, L.w.p, L.alpha[i], 0.0, L.n);
-      MG_LAUNCHED();
+      cg_step(e, L.t.p, L.r.p, L.r.p, L.w.p, L.alpha[i], 0.0, true, L.n);
     }
   }
   CgLevel &C = e.lv.back();
@@ -427,9 +420,7 @@ static void cg_solve(CgEngine &e, const Cx<double> *chi, Cx<double> *psi, double
   launch_copy<double>(chi, e.cr.p, n, e.s);
   gamma5_kernel<<<grid_for(F.geo.nsites, 256), 256, 0, e.s>>>(e.cr.p, F.geo.nsites);
   MG_LAUNCHED();
-  launch_dslash<double>(e.U.p, e.cr.p, e.rhs.p, F.geo, 2.0 + e.m, nullptr, 1.0, 0.0, e.s, 1, nullptr);
-  gamma5_kernel<<<grid_for(F.geo.nsites, 256), 256, 0, e.s>>>(e.rhs.p, F.geo.nsites);
-  MG_LAUNCHED();
+  launch_dslash_g5(e.U.p, e.cr.p, e.rhs.p, F.geo, 2.0 + e.m, e.s);
   double d[3];
   cg_dot(e, e.rhs.p, e.rhs.p, n, d);
   const double bn2 = d[2];
@@ -454,13 +445,12 @@ static void cg_solve(CgEngine &e, const Cx<double> *chi, Cx<double> *psi, double
       cg_update_kernel<<<blocks_for(n), 256, 0, e.s>>>(e.cx.p, e.cr.p, e.cp.p, e.cq.p, alpha, n);
       MG_LAUNCHED();
       ++it;
-      cg_dot(e, e.cr.p, e.cr.p, n, d);
-      rn2 = d[2];
       if (precond)
         cg_vcycle(e, 0, e.cr.p, e.cz.p);
       else
         launch_copy<double>(e.cr.p, e.cz.p, n, e.s);
-      cg_dot(e, e.cr.p, e.cz.p, n, d);
+      cg_dot(e, e.cr.p, e.cz.p, n, d);  // <r, z> and |r|^2 from one reduction
+      rn2 = d[2];
       const double beta = d[0] / rz;
       rz = d[0];
       direction_kernel<<<blocks_for(n), 256, 0, e.s>>>(e.cp.p, e.cz.p, beta, n);

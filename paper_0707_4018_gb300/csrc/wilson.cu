@@ -15,7 +15,8 @@ namespace mg {
 
 // FP32: at most 32 registers, so that 8 blocks of 256 threads fit an SM (this kernel is
 // HBM-bound and needs the memory parallelism of full occupancy)
-template <typename R, bool SHIFT>
+// G5: out = gamma_5 D in (the second spin component changes sign), for the normal equations
+template <typename R, bool SHIFT, bool G5 = false>
 __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 8 : 4) dslash_kernel(const Cx<R> *__restrict__ U, const Cx<R> *__restrict__ in,
                                                      Cx<R> *__restrict__ out, int L0, int L1, R diag,
                                                      const Cx<R> *__restrict__ b, R a, R c, long long ldv,
@@ -63,7 +64,16 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 8 : 4) dslash_kernel(con
     res.a = mk(a * o0.re, a * o0.im);
     res.b = mk(a * o1.re, a * o1.im);
   }
+  if (G5) res.b = mk(-res.b.re, -res.b.im);
   reinterpret_cast<Pair<R> *>(out)[x] = res;
+}
+
+void launch_dslash_g5(const Cx<double> *U, const Cx<double> *in, Cx<double> *out, Geo2 g, double diag,
+                      cudaStream_t s) {
+  const int threads = site_threads(g.nsites);
+  dslash_kernel<double, false, true><<<grid_for(g.nsites, threads), threads, 0, s>>>(
+      U, in, out, g.L0, g.L1, diag, nullptr, 1.0, 0.0, 2 * g.nsites, nullptr);
+  MG_LAUNCHED();
 }
 
 template <typename R>
