@@ -89,97 +89,111 @@ __device__ __forceinline__ Pair<float> wilson_at(Pair<float> s, Pair<float> f0, 
   return o;
 }
 
+// ---- the apply on half fields ----
+// A site as stored; the norm multiplies the projected half spinor (two products instead of four)
+struct RawSite {
+  float2 a, b;
+  float nu;
+};
+
+__device__ __forceinline__ float2 h2f(unsigned int w) {
+  __half2 h;
+  memcpy(&h, &w, 4);
+  return __half22float2(h);
+}
+__device__ __forceinline__ RawSite raw_site(uint2 w, float nu) { return {h2f(w.x), h2f(w.y), nu}; }
+__device__ __forceinline__ RawSite raw_load(const __half2 *d, const float *nrm, unsigned int x) {
+  return raw_site(__ldg(reinterpret_cast<const uint2 *>(d) + x), __ldg(nrm + x));
+}
+__device__ __forceinline__ Cx<float> raw_link(const __half2 *U, unsigned int i) {
+  const float2 f = h2f(__ldg(reinterpret_cast<const unsigned int *>(U) + i));
+  return mk(f.x, f.y);
+}
+
+__device__ __forceinline__ Pair<float> wilson_raw(const RawSite &s, const RawSite &f0, const RawSite &f1,
+                                                  const RawSite &g0, const RawSite &g1, Cx<float> ux0, Cx<float> ux1,
+                                                  Cx<float> ub0, Cx<float> ub1, float diag) {
+  const Cx<float> t1 = ux0 * mk(f0.nu * (f0.a.x - f0.b.x), f0.nu * (f0.a.y - f0.b.y));
+  const Cx<float> t2 = cmul_conj(ub0, mk(g0.nu * (g0.a.x + g0.b.x), g0.nu * (g0.a.y + g0.b.y)));
+  const Cx<float> t3 = ux1 * mk(f1.nu * (f1.a.x - f1.b.y), f1.nu * (f1.a.y + f1.b.x));
+  const Cx<float> t4 = cmul_conj(ub1, mk(g1.nu * (g1.a.x + g1.b.y), g1.nu * (g1.a.y - g1.b.x)));
+  const Cx<float> hu = mk(t1.re + t2.re + t3.re + t4.re, t1.im + t2.im + t3.im + t4.im);
+  const Cx<float> hl = mk(-t1.re + t2.re + t3.im - t4.im, -t1.im + t2.im - t3.re + t4.re);
+  const float ds = diag * s.nu;
+  Pair<float> o;
+  o.a = mk(ds * s.a.x - 0.5f * hu.re, ds * s.a.y - 0.5f * hu.im);
+  o.b = mk(ds * s.b.x - 0.5f * hl.re, ds * s.b.y - 0.5f * hl.im);
+  return o;
+}
+
+__device__ __forceinline__ uint2 pack_site(const Pair<float> &p, float &nu) {
+  nu = fmaxf(fmaxf(fabsf(p.a.re), fabsf(p.a.im)), fmaxf(fabsf(p.b.re), fabsf(p.b.im)));
+  const float inv = nu > 1e-30f ? __frcp_rn(nu) : 0.f;
+  const __half2 a = __floats2half2_rn(p.a.re * inv, p.a.im * inv), b = __floats2half2_rn(p.b.re * inv, p.b.im * inv);
+  uint2 raw;
+  memcpy(&raw.x, &a, 4);
+  memcpy(&raw.y, &b, 4);
+  nu = inv > 0.f ? nu : 0.f;
+  return raw;
+}
+
+// One site per thread: rows of odd length (a pair of sites is then aligned in every second row only) and
+// fields that are not 16-byte aligned. Rows x1 +- 1 are x +- L0 in the linear index, modulo the volume.
 __global__ void __launch_bounds__(256, 8) dslash_half_kernel(const __half2 *__restrict__ U,
                                                              const __half2 *__restrict__ in,
                                                              const float *__restrict__ in_nrm,
                                                              __half2 *__restrict__ out, float *__restrict__ out_nrm,
-                                                             int L0, int L1, float diag) {
-  const long long x = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  const long long V = (long long)L0 * L1;
+                                                             unsigned int l0, unsigned int V, float diag) {
+  const unsigned int x = blockIdx.x * blockDim.x + threadIdx.x;
   if (x >= V) return;
-  const Nbr n = neighbours(x, L0, L1);
-  const Pair<float> self = load_site(in, in_nrm, x);
-  const Pair<float> f0 = load_site(in, in_nrm, n.p0), f1 = load_site(in, in_nrm, n.p1);
-  const Pair<float> g0 = load_site(in, in_nrm, n.m0), g1 = load_site(in, in_nrm, n.m1);
-  const Cx<float> ux0 = h2c(U[2 * x], 1.f), ux1 = h2c(U[2 * x + 1], 1.f);
-  const Cx<float> ub0 = h2c(U[2 * n.m0], 1.f), ub1 = h2c(U[2 * n.m1 + 1], 1.f);
-  const Pair<float> o = wilson_at(self, f0, f1, g0, g1, ux0, ux1, ub0, ub1, diag);
-  store_site(out, out_nrm, x, o.a, o.b);
+  const unsigned int x0 = x % l0;
+  const unsigned int up = x + l0 < V ? x + l0 : x + l0 - V, dn = x >= l0 ? x - l0 : x + V - l0;
+  const unsigned int right = x0 + 1 == l0 ? x + 1 - l0 : x + 1, left = x0 == 0 ? x + l0 - 1 : x - 1;
+  const uint2 l = __ldg(reinterpret_cast<const uint2 *>(U) + x);
+  const float2 p = h2f(l.x), q = h2f(l.y);
+  const Pair<float> o =
+      wilson_raw(raw_load(in, in_nrm, x), raw_load(in, in_nrm, right), raw_load(in, in_nrm, up),
+                 raw_load(in, in_nrm, left), raw_load(in, in_nrm, dn), mk(p.x, p.y), mk(q.x, q.y),
+                 raw_link(U, 2 * left), raw_link(U, 2 * dn + 1), diag);
+  float nu;
+  const uint2 w = pack_site(o, nu);
+  reinterpret_cast<uint2 *>(out)[x] = w;
+  out_nrm[x] = nu;
 }
 
 // two sites (x0, x0 + 1) of a row per thread, L0 even: the pair's own values, its neighbours in
 // rows x1 +- 1 and its forward links are one 16-byte load each (8-byte norm pairs), the two
 // sites are each other's x0 neighbours, and only x0 - 1 and x0 + 2 are single loads; the
 // per-thread instruction count, which bounds the one-site kernel, is about halved
-__device__ __forceinline__ void load_pair2(const __half2 *d, const float *nrm, long long x, Pair<float> &p,
-                                           Pair<float> &q) {
-  const uint4 raw = reinterpret_cast<const uint4 *>(d)[x >> 1];  // sites x, x + 1 (x even)
-  const float2 nu = reinterpret_cast<const float2 *>(nrm)[x >> 1];
-  __half2 h[4];
-  memcpy(&h[0], &raw.x, 4);
-  memcpy(&h[1], &raw.y, 4);
-  memcpy(&h[2], &raw.z, 4);
-  memcpy(&h[3], &raw.w, 4);
-  p.a = h2c(h[0], nu.x);
-  p.b = h2c(h[1], nu.x);
-  q.a = h2c(h[2], nu.y);
-  q.b = h2c(h[3], nu.y);
-}
-
-__device__ __forceinline__ void store_pair2(__half2 *d, float *nrm, long long x, const Pair<float> &p,
-                                            const Pair<float> &q) {
-  const float np = fmaxf(fmaxf(fabsf(p.a.re), fabsf(p.a.im)), fmaxf(fabsf(p.b.re), fabsf(p.b.im)));
-  const float nq = fmaxf(fmaxf(fabsf(q.a.re), fabsf(q.a.im)), fmaxf(fabsf(q.b.re), fabsf(q.b.im)));
-  const float ip = np > 1e-30f ? __frcp_rn(np) : 0.f, iq = nq > 1e-30f ? __frcp_rn(nq) : 0.f;
-  const __half2 h0 = __floats2half2_rn(p.a.re * ip, p.a.im * ip), h1 = __floats2half2_rn(p.b.re * ip, p.b.im * ip);
-  const __half2 h2 = __floats2half2_rn(q.a.re * iq, q.a.im * iq), h3 = __floats2half2_rn(q.b.re * iq, q.b.im * iq);
-  uint4 raw;
-  memcpy(&raw.x, &h0, 4);
-  memcpy(&raw.y, &h1, 4);
-  memcpy(&raw.z, &h2, 4);
-  memcpy(&raw.w, &h3, 4);
-  reinterpret_cast<uint4 *>(d)[x >> 1] = raw;
-  reinterpret_cast<float2 *>(nrm)[x >> 1] = make_float2(ip > 0.f ? np : 0.f, iq > 0.f ? nq : 0.f);
-}
-
 __global__ void __launch_bounds__(256, 6) dslash_half2_kernel(const __half2 *__restrict__ U,
                                                               const __half2 *__restrict__ in,
                                                               const float *__restrict__ in_nrm,
                                                               __half2 *__restrict__ out, float *__restrict__ out_nrm,
-                                                              int L0, int L1, float diag) {
-  const unsigned int pr = blockIdx.x * blockDim.x + threadIdx.x;  // pair index
-  const unsigned int h0 = (unsigned int)L0 >> 1;
-  if (pr >= h0 * (unsigned int)L1) return;
-  const unsigned int x1 = pr / h0, x0 = 2 * (pr - x1 * h0);
-  const unsigned int row = x1 * (unsigned int)L0;
-  const long long xa = row + x0;  // even: sites xa (a) and xa + 1 (b)
-  const long long up = (x1 + 1 == (unsigned int)L1 ? 0u : row + L0) + x0;
-  const long long dn = (x1 == 0 ? ((unsigned int)L1 - 1) * L0 : row - L0) + x0;
-  const long long am = row + (x0 == 0 ? L0 - 1 : x0 - 1);                 // a - 0
-  const long long bp = row + (x0 + 2 == (unsigned int)L0 ? 0u : x0 + 2);  // b + 0
-  Pair<float> sa, sb, ua, ub, da, db;
-  load_pair2(in, in_nrm, xa, sa, sb);
-  load_pair2(in, in_nrm, up, ua, ub);
-  load_pair2(in, in_nrm, dn, da, db);
-  const Pair<float> am_v = load_site(in, in_nrm, am), bp_v = load_site(in, in_nrm, bp);
-  // links: forward of a and b (one 16-byte load), U^1 of dn and dn + 1 (one 16-byte load), U^0 of a - 0
-  const uint4 lf = reinterpret_cast<const uint4 *>(U)[xa >> 1];
-  const uint4 ld = reinterpret_cast<const uint4 *>(U)[dn >> 1];
-  __half2 f[4], g1, g3;
-  memcpy(&f[0], &lf.x, 4);
-  memcpy(&f[1], &lf.y, 4);
-  memcpy(&f[2], &lf.z, 4);
-  memcpy(&f[3], &lf.w, 4);
-  memcpy(&g1, &ld.y, 4);
-  memcpy(&g3, &ld.w, 4);
-  const Cx<float> ua0 = h2c(f[0], 1.f), ua1 = h2c(f[1], 1.f), ub0 = h2c(f[2], 1.f), ub1 = h2c(f[3], 1.f);
-  const Cx<float> dna1 = h2c(g1, 1.f), dnb1 = h2c(g3, 1.f);
-  const Cx<float> am0 = h2c(U[2 * am], 1.f);
-  // a: +0 = b, +1 = ua, -0 = am, -1 = da; backward links U_{a-0}^0 = am0, U_{a-1}^1 = dna1
-  const Pair<float> oa = wilson_at(sa, sb, ua, am_v, da, ua0, ua1, am0, dna1, diag);
-  // b: +0 = bp, +1 = ub, -0 = a, -1 = db; backward links U_{b-0}^0 = U_a^0, U_{b-1}^1 = dnb1
-  const Pair<float> ob = wilson_at(sb, bp_v, ub, sa, db, ub0, ub1, ua0, dnb1, diag);
-  store_pair2(out, out_nrm, xa, oa, ob);
+                                                              unsigned int l0, unsigned int V, float diag) {
+  const unsigned int x = 2 * (blockIdx.x * blockDim.x + threadIdx.x);
+  if (x >= V) return;
+  const unsigned int x0 = x % l0;
+  const unsigned int up = x + l0 < V ? x + l0 : x + l0 - V, dn = x >= l0 ? x - l0 : x + V - l0;
+  const unsigned int left = x0 == 0 ? x + l0 - 1 : x - 1, right = x0 + 2 == l0 ? x + 2 - l0 : x + 2;
+  const uint4 *in4 = reinterpret_cast<const uint4 *>(in), *U4 = reinterpret_cast<const uint4 *>(U);
+  const float2 *nrm2 = reinterpret_cast<const float2 *>(in_nrm);
+  const uint4 w = __ldg(in4 + (x >> 1)), wu = __ldg(in4 + (up >> 1)), wd = __ldg(in4 + (dn >> 1));
+  const uint4 l = __ldg(U4 + (x >> 1)), ld = __ldg(U4 + (dn >> 1));
+  const float2 n = __ldg(nrm2 + (x >> 1)), nu = __ldg(nrm2 + (up >> 1)), nd = __ldg(nrm2 + (dn >> 1));
+  const RawSite a = raw_site(make_uint2(w.x, w.y), n.x), b = raw_site(make_uint2(w.z, w.w), n.y);
+  const float2 a0 = h2f(l.x), a1 = h2f(l.y), b0 = h2f(l.z), b1 = h2f(l.w), da1 = h2f(ld.y), db1 = h2f(ld.w);
+  const Pair<float> oa =
+      wilson_raw(a, b, raw_site(make_uint2(wu.x, wu.y), nu.x), raw_load(in, in_nrm, left),
+                 raw_site(make_uint2(wd.x, wd.y), nd.x), mk(a0.x, a0.y), mk(a1.x, a1.y), raw_link(U, 2 * left),
+                 mk(da1.x, da1.y), diag);
+  const Pair<float> ob =
+      wilson_raw(b, raw_load(in, in_nrm, right), raw_site(make_uint2(wu.z, wu.w), nu.y), a,
+                 raw_site(make_uint2(wd.z, wd.w), nd.y), mk(b0.x, b0.y), mk(b1.x, b1.y), mk(a0.x, a0.y),
+                 mk(db1.x, db1.y), diag);
+  float na, nb;
+  const uint2 pa = pack_site(oa, na), pb = pack_site(ob, nb);
+  reinterpret_cast<uint4 *>(out)[x >> 1] = make_uint4(pa.x, pa.y, pb.x, pb.y);
+  reinterpret_cast<float2 *>(out_nrm)[x >> 1] = make_float2(na, nb);
 }
 
 // complex (FP64 / FP32) spinor field -> half storage with per-site norms, and back
@@ -370,17 +384,17 @@ void launch_dslash_half(const void *U, const void *in, void *out, Geo2 g, double
   const long long V = g.nsites;
   const __half2 *ih = static_cast<const __half2 *>(in);
   __half2 *oh = static_cast<__half2 *>(out);
-  if ((g.L0 & 1) == 0) {
-    dslash_half2_kernel<<<grid_for(V / 2, 256), 256, 0, s>>>(static_cast<const __half2 *>(U), ih,
-                                                             reinterpret_cast<const float *>(ih + 2 * V), oh,
-                                                             reinterpret_cast<float *>(oh + 2 * V), g.L0, g.L1,
-                                                             (float)diag);
-    MG_LAUNCHED();
-    return;
-  }
-  dslash_half_kernel<<<grid_for(V, 256), 256, 0, s>>>(static_cast<const __half2 *>(U), ih,
-                                                      reinterpret_cast<const float *>(ih + 2 * V), oh,
-                                                      reinterpret_cast<float *>(oh + 2 * V), g.L0, g.L1, (float)diag);
+  const float *in_nrm = reinterpret_cast<const float *>(ih + 2 * V);
+  float *out_nrm = reinterpret_cast<float *>(oh + 2 * V);
+  const __half2 *Uh = static_cast<const __half2 *>(U);
+  const uintptr_t bits = reinterpret_cast<uintptr_t>(U) | reinterpret_cast<uintptr_t>(in) |
+                         reinterpret_cast<uintptr_t>(out);
+  if ((g.L0 & 1) == 0 && (bits & 15) == 0)
+    dslash_half2_kernel<<<grid_for(V / 2, 256), 256, 0, s>>>(Uh, ih, in_nrm, oh, out_nrm, (unsigned int)g.L0,
+                                                             (unsigned int)V, (float)diag);
+  else
+    dslash_half_kernel<<<grid_for(V, 256), 256, 0, s>>>(Uh, ih, in_nrm, oh, out_nrm, (unsigned int)g.L0,
+                                                        (unsigned int)V, (float)diag);
   MG_LAUNCHED();
 }
 
