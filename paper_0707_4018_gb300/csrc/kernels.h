@@ -219,6 +219,10 @@ void launch_prolongator_to_canonical(const Cx<double> *V, Cx<double> *out, Block
 
 // ---- random vectors: Philox4x32-10 + Box-Muller, counter (i lo, i hi, k, level) ----
 void launch_gaussian(Cx<double> *out, long long n, unsigned long long seed, int k, int level, cudaStream_t s);
+// vectors k0 .. k0 + nk - 1 of the nf seeds, out[(k - k0) * nf + f][n]; a launch takes kGaussianSeeds seeds
+constexpr int kGaussianSeeds = 64;
+void launch_gaussian(Cx<double> *out, long long n, const uint64_t *seeds, int nf, int k0, int nk, int level,
+                     cudaStream_t s);
 
 // ---- coarsest level: dense LU with partial pivoting, column-major ----
 // dense matrix of the stencil plus shift * identity

@@ -1207,7 +1207,8 @@ static void setup_level(mg_ctx &c, int l, bool full) {
   Cx<double> *V = L.nullv.p;
   const int nv = L.Nv;
   const bool f32 = c.p.precision == MG_FP32;
-  for (int k = 0; k < nv; ++k) launch_gaussian(V + (long long)k * n, n, c.p.seed, k, l, c.s);
+  const uint64_t seed = c.p.seed;
+  launch_gaussian(V, n, &seed, 1, 0, nv, l, c.s);
   if (f32)
     relax_and_adapt<float>(c, l, 1);
   else

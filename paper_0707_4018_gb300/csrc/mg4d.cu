@@ -743,7 +743,8 @@ void build(Engine4 &e) {
 
 void setup(Engine4 &e) {
   const int Nv = e.bg.Nv;
-  for (int k = 0; k < Nv; ++k) launch_gaussian(e.nullv.p + (long long)k * e.nf, e.nf, e.p.seed, k, 0, e.s);
+  const uint64_t seed = e.p.seed;
+  launch_gaussian(e.nullv.p, e.nf, &seed, 1, 0, Nv, 0, e.s);
   // relaxation of all Nv vectors as one batch: MR on D x = 0 from x = v (r = -D v); in FP32
   // on FP32 copies in mixed mode
   const long long nall = (long long)Nv * e.nf;

@@ -61,9 +61,7 @@ void nn_validate_geom(const mg_geom *g) {
 
 // noise of nf fields (seed per field) into h[0]
 void nn_noise(mg_nullnet &n, long long V, int nf, const uint64_t *seeds, cudaStream_t s) {
-  for (int f = 0; f < nf; ++f)
-    for (int c = 0; c < n.cin; ++c)
-      launch_gaussian(n.z64.p + ((size_t)c * nf + f) * V * 2, V * 2, seeds[f], c, kNullnetNoiseTag, s);
+  launch_gaussian(n.z64.p, V * 2, seeds, nf, 0, n.cin, kNullnetNoiseTag, s);
   launch_pack_noise(n.z64.p, n.cin, V, nf, n.h[0].p, s);
 }
 

@@ -156,32 +156,55 @@ __global__ void __launch_bounds__(kConvThreads, 3) ptconv_kernel(const TI *__res
   in += (size_t)f * V * kin;
   const int c = threadIdx.x % C, grp = threadIdx.x / C;
   const bool works = grp * kSites < S;
+  // raw inputs and phases of this thread's first kAhead channels of the next direction to be staged (16 fields of
+  // 128^2, 32 channels: the adjoint 470 -> 408 us)
+  constexpr int kAhead = 4;
+  float2 ra[kAhead], rb[kAhead], rp[kAhead];
+  const int work = S * (kin / 2);  // a thread stages the two entries of a channel at a site; consecutive threads,
+                                   // consecutive sites
+  auto get = [&](int q, int x0, int dir, float2 &a, float2 &b, float2 &ph) {
+    const int ch = q / S, x = x0 + q - ch * S;
+    a = b = ph = make_float2(0.f, 0.f);
+    if (q < work && x < V) {
+      const int y1 = x / L0, y0 = x - y1 * L0;
+      long long nb;
+      if (M == Conv::kAdjoint)
+        adj_hop(dir, y0, y1, L0, L1, Uf, nb, ph);
+      else
+        fwd_hop(dir, y0, y1, L0, L1, Uf, nb, ph);
+      load_pair(in + nb * kin + 2 * ch, a, b);
+    }
+  };
+  auto put = [&](int q, float2 a, float2 b, float2 ph) {
+    const int ch = q / S, s = q - ch * S;
+    Vs[2 * ch * S + s] = cmulf(ph, a);
+    Vs[(2 * ch + 1) * S + s] = cmulf(ph, b);
+  };
+  auto ahead = [&](int x0, int dir) {
+#pragma unroll
+    for (int u = 0; u < kAhead; ++u) get(threadIdx.x + u * kConvThreads, x0, dir, ra[u], rb[u], rp[u]);
+  };
+  ahead(blockIdx.x * S, 0);
   for (int x0 = blockIdx.x * S; x0 < V; x0 += gridDim.x * S) {
     float2 acc[kSites][2];
 #pragma unroll
     for (int s = 0; s < kSites; ++s) acc[s][0] = acc[s][1] = make_float2(0.f, 0.f);
     for (int dir = 0; dir < 5; ++dir) {
       __syncthreads();
-      // a thread stages the two entries of a channel at a site; consecutive threads, consecutive sites
-      for (int q = threadIdx.x; q < S * (kin / 2); q += kConvThreads) {
-        const int ch = q / S, s = q - ch * S, x = x0 + s;
-        float2 a = make_float2(0.f, 0.f), b = a;
-        if (x < V) {
-          const int y1 = x / L0, y0 = x - y1 * L0;
-          long long nb;
-          float2 ph;
-          if (M == Conv::kAdjoint)
-            adj_hop(dir, y0, y1, L0, L1, Uf, nb, ph);
-          else
-            fwd_hop(dir, y0, y1, L0, L1, Uf, nb, ph);
-          load_pair(in + nb * kin + 2 * ch, a, b);
-          a = cmulf(ph, a);
-          b = cmulf(ph, b);
-        }
-        Vs[2 * ch * S + s] = a;
-        Vs[(2 * ch + 1) * S + s] = b;
+#pragma unroll
+      for (int u = 0; u < kAhead; ++u)
+        if ((int)threadIdx.x + u * kConvThreads < work) put(threadIdx.x + u * kConvThreads, ra[u], rb[u], rp[u]);
+      for (int q = threadIdx.x + kAhead * kConvThreads; q < work; q += kConvThreads) {
+        float2 a, b, ph;
+        get(q, x0, dir, a, b, ph);
+        put(q, a, b, ph);
       }
       __syncthreads();
+      // requested while this direction's products run
+      if (dir < 4)
+        ahead(x0, dir + 1);
+      else
+        ahead(x0 + gridDim.x * S, 0);
       if (works) {
         const float4 *wp = reinterpret_cast<const float4 *>(Ws + dir * kin * kout) + c;
         const float4 *vp = reinterpret_cast<const float4 *>(Vs) + grp * (kSites / 2);
@@ -230,14 +253,15 @@ __global__ void __launch_bounds__(kConvThreads, 3) ptconv_kernel(const TI *__res
 // Per-CTA partial sums of dL/dW^*[dir][lo][li] = sum_x ga_x[lo] conj(T_dir h_x[li]) over a
 // contiguous range of (field, site) pairs; partials[cta][entry] (entry = (dir co2 + lo) ci2 + li)
 // A thread owns input entry li (its lane) and output rows lo0 .. lo0 + 3 of every direction: per staged
-// site two 16-byte broadcast loads of g and five loads of T h for 20 complex multiply-adds.
+// site two 16-byte broadcast loads of g and five loads of T h for 20 complex multiply-adds. The next group's
+// rows are requested while this one's are multiplied (16 fields of 128^2, 32 channels: 361 -> 261 us).
 constexpr int kWG = 16;  // sites staged per group
-__global__ void __launch_bounds__(256) ptconv_bwd_weight_kernel(const float2 *__restrict__ ga,
-                                                                const __nv_bfloat162 *__restrict__ h_in,
-                                                                const float2 *__restrict__ U,
-                                                                const int *__restrict__ fmap, int nf, int ci2,
-                                                                int co2, int L0, int L1,
-                                                                float2 *__restrict__ partials) {
+__global__ void __launch_bounds__(256, 2) ptconv_bwd_weight_kernel(const float2 *__restrict__ ga,
+                                                                   const __nv_bfloat162 *__restrict__ h_in,
+                                                                   const float2 *__restrict__ U,
+                                                                   const int *__restrict__ fmap, int nf, int ci2,
+                                                                   int co2, int L0, int L1,
+                                                                   float2 *__restrict__ partials) {
   __shared__ float2 gs[kWG][32];
   __shared__ float2 Ts[kWG][5][32];
   const long long V = (long long)L0 * L1, total = V * nf;
@@ -250,35 +274,47 @@ __global__ void __launch_bounds__(256) ptconv_bwd_weight_kernel(const float2 *__
 #pragma unroll
     for (int e = 0; e < 4; ++e) acc[d][e] = make_float2(0.f, 0.f);
   const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  for (long long g0 = p0; g0 < p1; g0 += kWG) {
-    __syncthreads();
-    // warp w stages sites g0 + w, g0 + w + 8: the gradient row and the five transported inputs
+  // warp w stages sites g0 + w, g0 + w + 8: the gradient row and the five transported inputs, requested a group
+  // ahead
+  float2 gv[2], ph[2][5];
+  __nv_bfloat162 hv[2][5];
+  auto request = [&](long long g0) {
 #pragma unroll
-    for (int s = wid; s < kWG; s += 8) {
-      const long long p = g0 + s;
-      float2 gv = make_float2(0.f, 0.f);
-      float2 tv[5];
+    for (int u = 0; u < 2; ++u) {
+      const long long p = g0 + wid + 8 * u;
+      gv[u] = make_float2(0.f, 0.f);
 #pragma unroll
-      for (int d = 0; d < 5; ++d) tv[d] = make_float2(0.f, 0.f);
+      for (int d = 0; d < 5; ++d) {
+        ph[u][d] = make_float2(0.f, 0.f);
+        hv[u][d] = f2bf(ph[u][d]);
+      }
       if (p < p1) {
         const int f = (int)(p / V);
         const int x = (int)(p - (long long)f * V);
         const int x1 = x / L0, x0 = x - x1 * L0;
         const float2 *Uf = U + (size_t)(fmap ? fmap[f] : f) * 2 * V;
-        if (lane < co2) gv = ga[(size_t)p * co2 + lane];
+        if (lane < co2) gv[u] = ga[(size_t)p * co2 + lane];
 #pragma unroll
         for (int d = 0; d < 5; ++d) {
           long long nb;
-          float2 ph;
-          fwd_hop(d, x0, x1, L0, L1, Uf, nb, ph);
-          if (lane < ci2) tv[d] = cmulf(ph, bf2f(h_in[((size_t)f * V + nb) * ci2 + lane]));
+          fwd_hop(d, x0, x1, L0, L1, Uf, nb, ph[u][d]);
+          if (lane < ci2) hv[u][d] = h_in[((size_t)f * V + nb) * ci2 + lane];
         }
       }
-      gs[s][lane] = gv;
+    }
+  };
+  request(p0);
+  for (long long g0 = p0; g0 < p1; g0 += kWG) {
+    __syncthreads();
 #pragma unroll
-      for (int d = 0; d < 5; ++d) Ts[s][d][lane] = tv[d];
+    for (int u = 0; u < 2; ++u) {
+      const int s = wid + 8 * u;
+      gs[s][lane] = gv[u];
+#pragma unroll
+      for (int d = 0; d < 5; ++d) Ts[s][d][lane] = cmulf(ph[u][d], bf2f(hv[u][d]));
     }
     __syncthreads();
+    request(g0 + kWG);
     if (4 * wid < co2) {
 #pragma unroll 4
       for (int s = 0; s < kWG; ++s) {
@@ -306,16 +342,28 @@ __global__ void __launch_bounds__(256) ptconv_bwd_weight_kernel(const float2 *__
   }
 }
 
-// gW[q] = sum over CTAs of partials[cta][q] (fixed order, FP64 sums)
-__global__ void sum_partials_kernel(const float2 *__restrict__ partials, int nparts, int ne,
-                                    float2 *__restrict__ gW) {
-  const int q = blockIdx.x * blockDim.x + threadIdx.x;
-  if (q >= ne) return;
+// gW[q] = sum over CTAs of partials[cta][q] (fixed order, FP64 sums): a block takes 32 entries, warp w the
+// CTAs w, w + 8, ... (a thread per entry walked all of them alone, 95 us of latency per layer)
+__global__ void __launch_bounds__(256) sum_partials_kernel(const float2 *__restrict__ partials, int nparts, int ne,
+                                                           float2 *__restrict__ gW) {
+  __shared__ double2 sh[8][32];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, q = blockIdx.x * 32 + lane;
   double re = 0.0, im = 0.0;
-  for (int c = 0; c < nparts; ++c) {
-    const float2 v = partials[(size_t)c * ne + q];
-    re += v.x;
-    im += v.y;
+  if (q < ne) {
+#pragma unroll 4
+    for (int c = w; c < nparts; c += 8) {
+      const float2 v = partials[(size_t)c * ne + q];
+      re += v.x;
+      im += v.y;
+    }
+  }
+  sh[w][lane] = make_double2(re, im);
+  __syncthreads();
+  if (w != 0 || q >= ne) return;
+#pragma unroll
+  for (int k = 1; k < 8; ++k) {
+    re += sh[k][lane].x;
+    im += sh[k][lane].y;
   }
   gW[q] = make_float2((float)re, (float)im);
 }
@@ -518,7 +566,8 @@ __global__ void to_float2_kernel(const Cx<double> *__restrict__ a, long long n, 
 
 int blocks_for(long long n, int t) { return (int)((n + t - 1) / t); }
 
-// CTAs per field: three resident on each of 152 SMs over all fields (each stages the weights once)
+// CTAs per field: at most the three resident on each of 152 SMs over all fields (each stages the weights
+// once; eight more than that ran a second wave of their own: 420 instead of 328 us a layer)
 template <Conv M, typename TI>
 void conv_launch(const TI *in, const float2 *U, const int *fmap, const float2 *W, int kin, int kout, int L0, int L1,
                  int nf, const float2 *a_prev, float2 *a_out, __nv_bfloat162 *h_out, cudaStream_t s) {
@@ -527,7 +576,8 @@ void conv_launch(const TI *in, const float2 *U, const int *fmap, const float2 *W
   const size_t smem = ((size_t)5 * kin * kout + (size_t)kin * S) * sizeof(float2);
   MG_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   const long long tiles = ((long long)L0 * L1 + S - 1) / S;
-  long long gx = (152 * 3 + nf - 1) / nf;
+  long long gx = 152 * 3 / nf;
+  if (gx < 1) gx = 1;
   if (gx > tiles) gx = tiles;
   fn<<<dim3((unsigned int)gx, nf), kConvThreads, smem, s>>>(in, U, fmap, W, kin, kout, L0, L1, a_prev, a_out, h_out);
   MG_LAUNCHED();
@@ -556,7 +606,7 @@ void launch_ptconv_bwd_weight(const float2 *ga, const void *h_in, const float2 *
                                                   co2, L0, L1, partials);
   MG_LAUNCHED();
   const int ne = 5 * co2 * ci2;
-  sum_partials_kernel<<<blocks_for(ne, 256), 256, 0, s>>>(partials, nparts, ne, gW);
+  sum_partials_kernel<<<blocks_for(ne, 32), 256, 0, s>>>(partials, nparts, ne, gW);
   MG_LAUNCHED();
 }
 
