@@ -42,80 +42,125 @@ __device__ __forceinline__ void warp_sum2(R &a, R &b) {
   }
 }
 
-// sum of (a, b) over the CTA, returned to every thread (fixed order: deterministic)
-__device__ __forceinline__ void block_sum2(double &a, double &b, double (*red)[32]) {
-  warp_sum2(a, b);
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  if (lane == 0) {
-    red[0][w] = a;
-    red[1][w] = b;
-  }
-  __syncthreads();
-  a = 0.0;
-  b = 0.0;
-  for (int i = 0; i < nw; ++i) {
-    a += red[0][i];
-    b += red[1][i];
-  }
-  __syncthreads();
-}
-
 }  // namespace
 
-// ---------------------------------------------------------------------------
-// restriction r_c[b][c] = sum_{s, d6} conj(V[b][c][s][d6]) r[x(b, s)][6 chi + d6]:
-// the block's fine values are staged in shared memory, a warp reduces one column
-// ---------------------------------------------------------------------------
+// a 16-byte word of a column of V (Nh = 6 bvol is even, so every column starts on one)
 template <typename R>
-__global__ void __launch_bounds__(256) restrict4_kernel(const Cx<R> *__restrict__ V, const Cx<R> *__restrict__ fine,
+struct alignas(16) Pack {
+  static constexpr int n = 16 / sizeof(Cx<R>);
+  Cx<R> c[n];
+};
+
+// ---------------------------------------------------------------------------
+// restriction r_c[b][c] = sum_{s, d6} conj(V[b][c][s][d6]) r[x(b, s)][6 chi + d6] of VB
+// vectors: their values in the block are staged in shared memory by chirality, a warp
+// reduces two columns. DRAM-bound on V; a CTA per block and vector with the vectors in the
+// slow grid index read V once per vector (12 FP32 vectors, 16^3 x 32, Nv = 24: 570 us, V's
+// 302 MB twelve times over). Here VB vectors share a read and the CTAs of a block's
+// vectors run side by side, so that the others find V in L2: 184 us.
+// ---------------------------------------------------------------------------
+template <typename R, int VB>
+__global__ void __launch_bounds__(256, 2) restrict4_kernel(const Cx<R> *__restrict__ V, const Cx<R> *__restrict__ fine,
                                                         Cx<R> *__restrict__ coarse, Block4 g, long long fine_ld,
-                                                        long long coarse_ld) {
+                                                        long long coarse_ld, int nvec) {
+  using P = Pack<R>;
   extern __shared__ __align__(16) unsigned char sm_raw[];
-  Cx<R> *sm = reinterpret_cast<Cx<R> *>(sm_raw);
-  const int b = blockIdx.x;
-  fine += blockIdx.y * fine_ld;
-  coarse += blockIdx.y * coarse_ld;
-  const int N = 2 * g.Nv, Nh = g.bvol * 6;
-  for (int e = threadIdx.x; e < g.bvol * 12; e += blockDim.x) {
-    const int s = e / 12, d = e - s * 12;
-    sm[e] = fine[(long long)fine_site4(g, b, s) * 12 + d];
+  Cx<R> *sm = reinterpret_cast<Cx<R> *>(sm_raw);  // [vector][chirality][s][d6]
+  const int nch = (nvec + VB - 1) / VB, b = blockIdx.x / nch, v0 = (blockIdx.x - b * nch) * VB;
+  const int nv = min(VB, nvec - v0), N = 2 * g.Nv, Nh = g.bvol * 6;
+  fine += v0 * fine_ld;
+  coarse += v0 * coarse_ld + (long long)b * N;
+  for (int e = threadIdx.x; e < 2 * Nh; e += blockDim.x) {
+    const int s = e / 12, d = e - s * 12, chi = d / 6;
+    const Cx<R> *f = fine + (long long)fine_site4(g, b, s) * 12 + d;
+    Cx<R> *q = sm + chi * Nh + s * 6 + d - 6 * chi;
+#pragma unroll
+    for (int v = 0; v < VB; ++v) q[v * 2 * Nh] = v < nv ? f[v * fine_ld] : mk((R)0, (R)0);
   }
   __syncthreads();
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  for (int c = warp; c < N; c += nw) {
-    const int chi = c / g.Nv;
-    const Cx<R> *Vc = V + ((long long)b * N + c) * Nh;
-    R re = 0, im = 0;
-    for (int e = lane; e < Nh; e += 32) {
-      const int s = e / 6, d6 = e - s * 6;
-      const Cx<R> v = Vc[e], f = sm[s * 12 + 6 * chi + d6];
-      re += v.re * f.re + v.im * f.im;
-      im += v.re * f.im - v.im * f.re;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5, pairs = (g.Nv + 1) / 2;
+  for (int q = warp; q < 2 * pairs; q += nw) {
+    const int chi = q / pairs, k = 2 * (q - chi * pairs), c = chi * g.Nv + k;
+    const bool two = k + 1 < g.Nv;
+    const P *V0 = reinterpret_cast<const P *>(V + ((long long)b * N + c) * Nh);
+    const P *V1 = two ? V0 + Nh / P::n : V0;
+    const P *f = reinterpret_cast<const P *>(sm + chi * Nh);
+    Cx<R> acc[2][VB];
+#pragma unroll
+    for (int v = 0; v < VB; ++v) acc[0][v] = acc[1][v] = mk((R)0, (R)0);
+#pragma unroll 4
+    for (int p = lane; p < Nh / P::n; p += 32) {
+      const P a0 = V0[p], a1 = V1[p];
+#pragma unroll
+      for (int v = 0; v < VB; ++v) {
+        const P x = f[v * (2 * Nh / P::n) + p];
+#pragma unroll
+        for (int t = 0; t < P::n; ++t) {
+          cmac_conj(acc[0][v], a0.c[t], x.c[t]);
+          cmac_conj(acc[1][v], a1.c[t], x.c[t]);
+        }
+      }
     }
-    warp_sum2(re, im);
-    if (lane == 0) coarse[(long long)b * N + c] = mk(re, im);
+#pragma unroll
+    for (int v = 0; v < VB; ++v) {
+      warp_sum2(acc[0][v].re, acc[0][v].im);
+      warp_sum2(acc[1][v].re, acc[1][v].im);
+      if (lane == 0 && v < nv) {
+        coarse[v * coarse_ld + c] = acc[0][v];
+        if (two) coarse[v * coarse_ld + c + 1] = acc[1][v];
+      }
+    }
   }
 }
 
-// prolongation fine[x(b, s)][6 chi + d6] += sum_k V[b][chi Nv + k][s][d6] e[b][chi Nv + k]
-template <typename R>
+// prolongation fine[x(b, s)][6 chi + d6] += sum_k V[b][chi Nv + k][s][d6] e[b][chi Nv + k] of VB
+// vectors, a thread per word of V's columns; the vectors share V as in the restriction (12 FP32
+// vectors as there: 510 -> 164 us). FP32 fields start on 16 bytes.
+template <typename R, int VB>
 __global__ void __launch_bounds__(256) prolong4_kernel(const Cx<R> *__restrict__ V, const Cx<R> *__restrict__ coarse,
                                                        Cx<R> *__restrict__ fine, Block4 g, long long fine_ld,
-                                                       long long coarse_ld) {
-  __shared__ Cx<R> es[128];
-  const int b = blockIdx.x;
-  fine += blockIdx.y * fine_ld;
-  coarse += blockIdx.y * coarse_ld;
-  const int N = 2 * g.Nv, Nh = g.bvol * 6;
-  for (int c = threadIdx.x; c < N; c += blockDim.x) es[c] = coarse[(long long)b * N + c];
+                                                       long long coarse_ld, int nvec) {
+  using P = Pack<R>;
+  __shared__ __align__(16) Cx<R> es[64][VB];
+  const int nch = (nvec + VB - 1) / VB, b = blockIdx.x / nch, v0 = (blockIdx.x - b * nch) * VB;
+  const int nv = min(VB, nvec - v0), N = 2 * g.Nv, Nh = g.bvol * 6, NhP = Nh / P::n;
+  fine += v0 * fine_ld;
+  coarse += v0 * coarse_ld + (long long)b * N;
+  for (int q = threadIdx.x; q < N * VB; q += blockDim.x) {
+    const int v = q / N, c = q - v * N;
+    es[c][v] = v < nv ? coarse[v * coarse_ld + c] : mk((R)0, (R)0);
+  }
   __syncthreads();
-  for (int e = threadIdx.x; e < 2 * Nh; e += blockDim.x) {
-    const int chi = e / Nh, r = e - chi * Nh, s = r / 6, d6 = r - s * 6;
-    const Cx<R> *Vb = V + ((long long)b * N + chi * g.Nv) * Nh + r;
-    Cx<R> acc = mk((R)0, (R)0);
-    for (int k = 0; k < g.Nv; ++k) cmac(acc, Vb[(long long)k * Nh], es[chi * g.Nv + k]);
+  for (int e = threadIdx.x; e < 2 * NhP; e += blockDim.x) {
+    const int chi = e / NhP, r = e - chi * NhP, s = r * P::n / 6, d6 = r * P::n - s * 6;
+    const P *Vb = reinterpret_cast<const P *>(V + ((long long)b * N + chi * g.Nv) * Nh) + r;
+    P acc[VB];
+#pragma unroll
+    for (int v = 0; v < VB; ++v)
+#pragma unroll
+      for (int t = 0; t < P::n; ++t) acc[v].c[t] = mk((R)0, (R)0);
+#pragma unroll 4
+    for (int k = 0; k < g.Nv; ++k) {
+      const P a = Vb[(long long)k * NhP];
+#pragma unroll
+      for (int v = 0; v < VB; ++v)
+#pragma unroll
+        for (int t = 0; t < P::n; ++t) cmac(acc[v].c[t], a.c[t], es[chi * g.Nv + k][v]);
+    }
     Cx<R> *f = fine + (long long)fine_site4(g, b, s) * 12 + 6 * chi + d6;
-    *f = *f + acc;
+#pragma unroll
+    for (int v = 0; v < VB; ++v) {
+      if (v >= nv) break;
+      if constexpr (P::n == 1) {
+        f[v * fine_ld] = f[v * fine_ld] + acc[v].c[0];
+      } else {
+        P *fp = reinterpret_cast<P *>(f + v * fine_ld);
+        P x = *fp;
+#pragma unroll
+        for (int t = 0; t < P::n; ++t) x.c[t] = x.c[t] + acc[v].c[t];
+        *fp = x;
+      }
+    }
   }
 }
 
@@ -135,35 +180,69 @@ __global__ void gather_split4_kernel(const Cx<double> *__restrict__ vecs, long l
 }
 
 // modified Gram-Schmidt in k order, run twice, on the Nv columns of one (block, chirality)
+// FP64-bound (8 multiply-adds per entry and pair of columns, 12 ms of them at 16^3 x 32 with Nv = 24). A thread owns
+// kGsOwn entries of every column: the column in work stays in its registers, and with few threads per CTA the sums
+// over them, which are FP64 work as well, stay small. Re-reading both columns for each product with 256 threads per
+// CTA took 28.4 ms, this 14.2 ms.
+constexpr int kGsOwn = 12;
+
 __global__ void __launch_bounds__(256) block_gs4_kernel(Cx<double> *__restrict__ V, Block4 g) {
-  __shared__ double red[2][32];
+  __shared__ double red[2][8][2];  // two sets in turn: one barrier per sum
   const int b = blockIdx.x, chi = blockIdx.y, N = 2 * g.Nv, Nh = g.bvol * 6;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
   Cx<double> *base = V + ((long long)b * N + chi * g.Nv) * Nh;
+  int set = 0;
+  // sum over the CTA of (re, im), to every thread (fixed order): half the lanes of a warp take either part
+  auto sum2 = [&](double &re, double &im) {
+    const bool up = lane & 16;
+    double t = (up ? im : re) + __shfl_xor_sync(0xffffffffu, up ? re : im, 16);
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    if ((lane & 15) == 0) red[set][w][lane >> 4] = t;
+    __syncthreads();
+    re = red[set][0][0];
+    im = red[set][0][1];
+    for (int i = 1; i < nw; ++i) {
+      re += red[set][i][0];
+      im += red[set][i][1];
+    }
+    set ^= 1;
+  };
   for (int pass = 0; pass < 2; ++pass) {
     for (int k = 0; k < g.Nv; ++k) {
       Cx<double> *vk = base + (long long)k * Nh;
+      Cx<double> c[kGsOwn];
+#pragma unroll
+      for (int t = 0; t < kGsOwn; ++t) {
+        const int e = threadIdx.x + t * blockDim.x;
+        c[t] = e < Nh ? vk[e] : mk(0.0, 0.0);
+      }
       for (int j = 0; j < k; ++j) {
         const Cx<double> *vj = base + (long long)j * Nh;
-        double re = 0.0, im = 0.0;  // <v_j, v_k>
-        for (int e = threadIdx.x; e < Nh; e += blockDim.x) {
-          const Cx<double> a = vj[e], c = vk[e];
-          re += a.re * c.re + a.im * c.im;
-          im += a.re * c.im - a.im * c.re;
+        Cx<double> d = mk(0.0, 0.0);  // <v_j, v_k>
+#pragma unroll
+        for (int t = 0; t < kGsOwn; ++t) {
+          const int e = threadIdx.x + t * blockDim.x;
+          if (e < Nh) cmac_conj(d, vj[e], c[t]);
         }
-        block_sum2(re, im, red);
-        for (int e = threadIdx.x; e < Nh; e += blockDim.x) {
-          const Cx<double> a = vj[e];
-          Cx<double> c = vk[e];
-          c.re -= re * a.re - im * a.im;
-          c.im -= re * a.im + im * a.re;
-          vk[e] = c;
+        sum2(d.re, d.im);
+        const Cx<double> md = mk(-d.re, -d.im);
+#pragma unroll
+        for (int t = 0; t < kGsOwn; ++t) {
+          const int e = threadIdx.x + t * blockDim.x;
+          if (e < Nh) cmac(c[t], md, vj[e]);
         }
       }
       double n2 = 0.0, zero = 0.0;
-      for (int e = threadIdx.x; e < Nh; e += blockDim.x) n2 += norm2(vk[e]);
-      block_sum2(n2, zero, red);
+#pragma unroll
+      for (int t = 0; t < kGsOwn; ++t) n2 += norm2(c[t]);
+      sum2(n2, zero);
       const double inv = 1.0 / sqrt(n2);
-      for (int e = threadIdx.x; e < Nh; e += blockDim.x) vk[e] = inv * vk[e];
+#pragma unroll
+      for (int t = 0; t < kGsOwn; ++t) {
+        const int e = threadIdx.x + t * blockDim.x;
+        if (e < Nh) vk[e] = inv * c[t];
+      }
     }
   }
 }
@@ -663,24 +742,47 @@ __global__ void prolongator4_to_canonical_kernel(const Cx<double> *__restrict__ 
 // ---------------------------------------------------------------------------
 // launchers
 // ---------------------------------------------------------------------------
+namespace {
+
+// vectors of a batch that share a read of V: a CTA stages at most 196 KB of them (blocks of 512 sites)
+template <typename R>
+constexpr int kShare4 = 16 / sizeof(R);
+
+template <typename R, int VB>
+void restrict4(const Cx<R> *V, const Cx<R> *fine, Cx<R> *coarse, const Block4 &g, cudaStream_t s, int nvec) {
+  const size_t smem = (size_t)g.bvol * 12 * sizeof(Cx<R>) * VB;
+  if (smem > 48 * 1024)
+    MG_CUDA(cudaFuncSetAttribute(restrict4_kernel<R, VB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  const unsigned int grid = (unsigned int)g.nblocks * ((nvec + VB - 1) / VB);
+  restrict4_kernel<R, VB><<<grid, 256, smem, s>>>(V, fine, coarse, g, (long long)g.nblocks * g.bvol * 12,
+                                                  (long long)g.nblocks * 2 * g.Nv, nvec);
+  MG_LAUNCHED();
+}
+
+template <typename R, int VB>
+void prolong4(const Cx<R> *V, const Cx<R> *coarse, Cx<R> *fine, const Block4 &g, cudaStream_t s, int nvec) {
+  const unsigned int grid = (unsigned int)g.nblocks * ((nvec + VB - 1) / VB);
+  prolong4_kernel<R, VB><<<grid, 256, 0, s>>>(V, coarse, fine, g, (long long)g.nblocks * g.bvol * 12,
+                                              (long long)g.nblocks * 2 * g.Nv, nvec);
+  MG_LAUNCHED();
+}
+
+}  // namespace
+
 template <typename R>
 void launch_restrict4(const Cx<R> *V, const Cx<R> *fine, Cx<R> *coarse, const Block4 &g, cudaStream_t s, int nvec) {
-  const size_t smem = (size_t)g.bvol * 12 * sizeof(Cx<R>);
-  static bool attr = false;  // one opt-in per process for more than 48 KB
-  if (!attr) {
-    MG_CUDA(cudaFuncSetAttribute(restrict4_kernel<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024));
-    attr = true;
-  }
-  const long long nf = (long long)g.nblocks * g.bvol * 12;
-  restrict4_kernel<R><<<dim3(g.nblocks, nvec), 256, smem, s>>>(V, fine, coarse, g, nf, (long long)g.nblocks * 2 * g.Nv);
-  MG_LAUNCHED();
+  if (nvec > 1)
+    restrict4<R, kShare4<R>>(V, fine, coarse, g, s, nvec);
+  else
+    restrict4<R, 1>(V, fine, coarse, g, s, nvec);
 }
 
 template <typename R>
 void launch_prolong4(const Cx<R> *V, const Cx<R> *coarse, Cx<R> *fine, const Block4 &g, cudaStream_t s, int nvec) {
-  const long long nf = (long long)g.nblocks * g.bvol * 12;
-  prolong4_kernel<R><<<dim3(g.nblocks, nvec), 256, 0, s>>>(V, coarse, fine, g, nf, (long long)g.nblocks * 2 * g.Nv);
-  MG_LAUNCHED();
+  if (nvec > 1)
+    prolong4<R, kShare4<R>>(V, coarse, fine, g, s, nvec);
+  else
+    prolong4<R, 1>(V, coarse, fine, g, s, nvec);
 }
 
 void launch_gather_split4(const Cx<double> *vecs, long long vstride, Cx<double> *V, const Block4 &g, cudaStream_t s) {
@@ -691,7 +793,9 @@ void launch_gather_split4(const Cx<double> *vecs, long long vstride, Cx<double> 
 }
 
 void launch_block_gs4(Cx<double> *V, const Block4 &g, cudaStream_t s) {
-  block_gs4_kernel<<<dim3(g.nblocks, 2), 256, 0, s>>>(V, g);
+  // blocks have at most 512 sites: 3072 entries a column, 256 threads
+  const int own = 32 * kGsOwn, threads = 32 * ((g.bvol * 6 + own - 1) / own);
+  block_gs4_kernel<<<dim3(g.nblocks, 2), threads, 0, s>>>(V, g);
   MG_LAUNCHED();
 }
 
