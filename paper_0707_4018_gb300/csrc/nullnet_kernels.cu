@@ -97,12 +97,16 @@ __device__ __forceinline__ void adj_hop(int dir, int z0, int z1, int L0, int L1,
 // ---------------------------------------------------------------------------
 // The transported convolution as a tiled product: for a tile of S sites and one direction the
 // transported inputs v_x[k] = phase_x in_{nb(x)}[k] are staged in shared memory (site fastest), the
-// weights of all directions once per CTA, and a thread accumulates the two spin rows of one channel
-// at four sites: one 16-byte weight load and two 16-byte input loads for 8 complex multiply-adds.
-// FP32 issue bounds it; with a warp per site and a lane per output row the weights' rows met in one
-// bank and every input took two shuffles (16 fields of 128^2, one layer: 2.1 ms forward, 2.5 ms
-// backward; a whole gradient, with the loss and weight kernels below, 22.1 ms before and 6.3 now). Every output sums its terms in the order direction, input, as fused multiply-adds, so
-// the values that are rounded to bfloat16 do not depend on the tiling.
+// weights of all directions once per CTA, and a thread accumulates the spin rows of two channels at SP sites: with
+// SP = 4 two 16-byte loads of weights and two of inputs for 16 complex multiply-adds, whose 64 instructions take
+// as long as the loads' 16 cycles of shared memory (with one channel 12 cycles of loads met 8 of arithmetic). A thread
+// stages one site: its neighbour and phase are worked out once per direction, for all of its channels, and the
+// entries are requested while the direction before is multiplied.
+// FP32 issue bounds it (150 us of multiply-adds per layer at 16 fields of 128^2, 32 entries): 271 us forward, 264 us
+// for the adjoint; with one channel to a thread and a neighbour per entry 328 and 312, with a warp per site, a lane
+// per output row and two shuffles per input 2.1 and 2.5 ms. A whole gradient with the loss and weight kernels below:
+// 22.1 ms then, 3.8 now. Every output sums its terms in the order direction, input, as fused multiply-adds, so the
+// values that are rounded to bfloat16 do not depend on the tiling.
 // ---------------------------------------------------------------------------
 enum class Conv {
   kHidden,  // bf16 in; gated bf16 out, pre-activation out if asked for
@@ -111,139 +115,166 @@ enum class Conv {
 };
 
 constexpr int kConvThreads = 256;
-constexpr int kSites = 4;      // sites of a thread
-constexpr int kMaxTile = 128;  // sites of a tile
+constexpr int kAhead = 8;  // channels of a thread's site: 32 / 2 entries over at least two rows of threads, or 16 / 2
 
-// sites of a tile for `channels` output channels
-__host__ __device__ inline int conv_tile(int channels) {
-  const int s = kConvThreads / channels * kSites;
-  return s < kMaxTile ? s : kMaxTile;
+// sites of a tile for c2 pairs of output channels, SP sites to a thread and kin inputs; a thread stages one site, so
+// a tile has at most kConvThreads, and half of them where a thread would stage more than kAhead channels
+__host__ __device__ inline int conv_tile(int c2, int sp, int kin) {
+  const int s = kConvThreads / c2 * sp, most = kin <= 2 * kAhead ? kConvThreads : kConvThreads / 2;
+  return s < most ? s : most;
 }
 
-__device__ __forceinline__ void load_pair(const __nv_bfloat162 *p, float2 &a, float2 &b) {
-  const uint2 w = *reinterpret_cast<const uint2 *>(p);
+// the two spin entries of a channel as they are stored
+template <typename TI>
+struct RawPair {
+  using T = uint2;
+};
+template <>
+struct RawPair<float2> {
+  using T = float4;
+};
+__device__ __forceinline__ void unpack(uint2 w, float2 &a, float2 &b) {
   a = bf2f(*reinterpret_cast<const __nv_bfloat162 *>(&w.x));
   b = bf2f(*reinterpret_cast<const __nv_bfloat162 *>(&w.y));
 }
-__device__ __forceinline__ void load_pair(const float2 *p, float2 &a, float2 &b) {
-  const float4 w = *reinterpret_cast<const float4 *>(p);
+__device__ __forceinline__ void unpack(float4 w, float2 &a, float2 &b) {
   a = make_float2(w.x, w.y);
   b = make_float2(w.z, w.w);
 }
 
-// kin / kout: channel-spin entries (even) of the input and output of this product
-template <Conv M, typename TI>
-__global__ void __launch_bounds__(kConvThreads, 3) ptconv_kernel(const TI *__restrict__ in, const float2 *__restrict__ U,
+// kin / kout: channel-spin entries (even, at most 32) of the input and output of this product
+template <Conv M, typename TI, int SP>
+__global__ void __launch_bounds__(kConvThreads, 2) ptconv_kernel(const TI *__restrict__ in, const float2 *__restrict__ U,
                                                               const int *__restrict__ fmap,
                                                               const float2 *__restrict__ W, int kin, int kout, int L0,
                                                               int L1, const float2 *__restrict__ a_prev,
                                                               float2 *__restrict__ a_out,
                                                               __nv_bfloat162 *__restrict__ h_out) {
+  using Raw = typename RawPair<TI>::T;
   extern __shared__ float4 conv_smem[];
-  const int C = kout / 2, S = conv_tile(C), V = L0 * L1, f = blockIdx.y;
-  float2 *Ws = reinterpret_cast<float2 *>(conv_smem);  // [dir][k][out]
-  float2 *Vs = Ws + 5 * kin * kout;                    // [k][S]
-  for (int q = threadIdx.x; q < 5 * kin * kout; q += kConvThreads) {
-    const int dir = q / (kin * kout), r = q - dir * kin * kout;
-    if (M == Conv::kAdjoint) {  // W[dir][k][out]: rows of the layer's weights are this product's inputs
-      Ws[q] = conjf2(W[q]);
-    } else {  // W[dir][out][k]
-      const int o = r / kin, k = r - o * kin;
-      Ws[(dir * kin + k) * kout + o] = W[q];
+  const int C = kout / 2, C2 = (C + 1) / 2, S = conv_tile(C2, SP, kin), V = L0 * L1, f = blockIdx.y;
+  // [dir][k][channel parity][pair][spin]: a quarter warp's 16-byte loads are consecutive; zero past the last channel
+  float2 *Ws = reinterpret_cast<float2 *>(conv_smem);
+  float2 *Vs = Ws + 5 * kin * 4 * C2;  // [k][S]
+  for (int q = threadIdx.x; q < 5 * kin * 4 * C2; q += kConvThreads) {
+    const int dk = q / (4 * C2), r = q - dk * 4 * C2, half = r / (2 * C2);
+    const int o = 4 * ((r - half * 2 * C2) >> 1) + 2 * half + (r & 1);
+    float2 w = make_float2(0.f, 0.f);
+    if (o < kout) {
+      if (M == Conv::kAdjoint) {  // W[dir][k][out]: rows of the layer's weights are this product's inputs
+        w = conjf2(W[dk * kout + o]);
+      } else {  // W[dir][out][k]
+        const int dir = dk / kin, k = dk - dir * kin;
+        w = W[(dir * kout + o) * kin + k];
+      }
     }
+    Ws[q] = w;
   }
   const float2 *Uf = U + (size_t)(fmap ? fmap[f] : f) * 2 * V;
   in += (size_t)f * V * kin;
-  const int c = threadIdx.x % C, grp = threadIdx.x / C;
-  const bool works = grp * kSites < S;
-  // raw inputs and phases of this thread's first kAhead channels of the next direction to be staged (16 fields of
-  // 128^2, 32 channels: the adjoint 470 -> 408 us)
-  constexpr int kAhead = 4;
-  float2 ra[kAhead], rb[kAhead], rp[kAhead];
-  const int work = S * (kin / 2);  // a thread stages the two entries of a channel at a site; consecutive threads,
-                                   // consecutive sites
-  auto get = [&](int q, int x0, int dir, float2 &a, float2 &b, float2 &ph) {
-    const int ch = q / S, x = x0 + q - ch * S;
-    a = b = ph = make_float2(0.f, 0.f);
-    if (q < work && x < V) {
-      const int y1 = x / L0, y0 = x - y1 * L0;
-      long long nb;
+  const int c2 = threadIdx.x % C2, grp = threadIdx.x / C2;
+  const bool works = grp * SP < S;
+  // staging: this thread's site of the tile and its channels row, row + rows, ...
+  const int rows = kConvThreads / S, ss = threadIdx.x % S, row = threadIdx.x / S;
+  Raw raw[kAhead];
+  float2 ph;
+  int y0 = 0, y1 = 0;
+  bool there = false;
+  auto ahead = [&](int x0, int dir) {
+    if (dir == 0) {
+      const int x = x0 + ss;
+      there = row < rows && x < V;
+      y1 = x / L0;
+      y0 = x - y1 * L0;
+    }
+    ph = make_float2(0.f, 0.f);
+    long long nb = 0;
+    if (there) {
       if (M == Conv::kAdjoint)
         adj_hop(dir, y0, y1, L0, L1, Uf, nb, ph);
       else
         fwd_hop(dir, y0, y1, L0, L1, Uf, nb, ph);
-      load_pair(in + nb * kin + 2 * ch, a, b);
     }
-  };
-  auto put = [&](int q, float2 a, float2 b, float2 ph) {
-    const int ch = q / S, s = q - ch * S;
-    Vs[2 * ch * S + s] = cmulf(ph, a);
-    Vs[(2 * ch + 1) * S + s] = cmulf(ph, b);
-  };
-  auto ahead = [&](int x0, int dir) {
 #pragma unroll
-    for (int u = 0; u < kAhead; ++u) get(threadIdx.x + u * kConvThreads, x0, dir, ra[u], rb[u], rp[u]);
+    for (int u = 0; u < kAhead; ++u) {
+      const int ch = row + u * rows;
+      raw[u] = Raw{};
+      if (there && ch < kin / 2) raw[u] = *reinterpret_cast<const Raw *>(in + nb * kin + 2 * ch);
+    }
   };
   ahead(blockIdx.x * S, 0);
   for (int x0 = blockIdx.x * S; x0 < V; x0 += gridDim.x * S) {
-    float2 acc[kSites][2];
+    float2 acc[SP][4];
 #pragma unroll
-    for (int s = 0; s < kSites; ++s) acc[s][0] = acc[s][1] = make_float2(0.f, 0.f);
+    for (int s = 0; s < SP; ++s)
+#pragma unroll
+      for (int e = 0; e < 4; ++e) acc[s][e] = make_float2(0.f, 0.f);
     for (int dir = 0; dir < 5; ++dir) {
       __syncthreads();
 #pragma unroll
-      for (int u = 0; u < kAhead; ++u)
-        if ((int)threadIdx.x + u * kConvThreads < work) put(threadIdx.x + u * kConvThreads, ra[u], rb[u], rp[u]);
-      for (int q = threadIdx.x + kAhead * kConvThreads; q < work; q += kConvThreads) {
-        float2 a, b, ph;
-        get(q, x0, dir, a, b, ph);
-        put(q, a, b, ph);
+      for (int u = 0; u < kAhead; ++u) {
+        const int ch = row + u * rows;
+        if (row < rows && ch < kin / 2) {
+          float2 a, b;
+          unpack(raw[u], a, b);
+          Vs[2 * ch * S + ss] = cmulf(ph, a);
+          Vs[(2 * ch + 1) * S + ss] = cmulf(ph, b);
+        }
       }
       __syncthreads();
-      // requested while this direction's products run
       if (dir < 4)
         ahead(x0, dir + 1);
       else
         ahead(x0 + gridDim.x * S, 0);
       if (works) {
-        const float4 *wp = reinterpret_cast<const float4 *>(Ws + dir * kin * kout) + c;
-        const float4 *vp = reinterpret_cast<const float4 *>(Vs) + grp * (kSites / 2);
+        const float4 *wp = reinterpret_cast<const float4 *>(Ws + dir * kin * 4 * C2) + c2;
+        const float4 *vp = reinterpret_cast<const float4 *>(Vs) + grp * (SP / 2);
 #pragma unroll 4
         for (int k = 0; k < kin; ++k) {
-          const float4 w = wp[k * C], v01 = vp[k * (S / 2)], v23 = vp[k * (S / 2) + 1];
-          const float2 v[kSites] = {make_float2(v01.x, v01.y), make_float2(v01.z, v01.w), make_float2(v23.x, v23.y),
-                                    make_float2(v23.z, v23.w)};
+          const float4 w0 = wp[k * 2 * C2], w1 = wp[k * 2 * C2 + C2];
+          const float2 w[4] = {make_float2(w0.x, w0.y), make_float2(w0.z, w0.w), make_float2(w1.x, w1.y),
+                               make_float2(w1.z, w1.w)};
+          float2 v[SP];
 #pragma unroll
-          for (int s = 0; s < kSites; ++s) {
-            cmacf(acc[s][0], make_float2(w.x, w.y), v[s]);
-            cmacf(acc[s][1], make_float2(w.z, w.w), v[s]);
+          for (int s = 0; s < SP; s += 2) {
+            const float4 t = vp[k * (S / 2) + s / 2];
+            v[s] = make_float2(t.x, t.y);
+            v[s + 1] = make_float2(t.z, t.w);
           }
+#pragma unroll
+          for (int s = 0; s < SP; ++s)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) cmacf(acc[s][e], w[e], v[s]);
         }
       }
     }
     if (!works) continue;
 #pragma unroll
-    for (int s = 0; s < kSites; ++s) {
-      const int x = x0 + grp * kSites + s;
+    for (int s = 0; s < SP; ++s) {
+      const int x = x0 + grp * SP + s;
       if (x >= V) break;
-      const float2 p = acc[s][0], q = acc[s][1];
-      const size_t o = ((size_t)f * V + x) * kout + 2 * c;
-      if (M == Conv::kAdjoint) {
-        const float4 a = *reinterpret_cast<const float4 *>(a_prev + o);
-        const float sq = (a.x * a.x + a.y * a.y) + (a.z * a.z + a.w * a.w);
-        const float re = (a.x * p.x + a.y * p.y) + (a.z * q.x + a.w * q.y);
-        const float g = rsqrtf(1.f + sq);
-        const float dg2 = -g * g * g * re;  // 2 g'(s) Re(a^dagger gh), g' = -g^3 / 2
-        *reinterpret_cast<float4 *>(a_out + o) =
-            make_float4(g * p.x + dg2 * a.x, g * p.y + dg2 * a.y, g * q.x + dg2 * a.z, g * q.y + dg2 * a.w);
-      } else {
-        if (M == Conv::kLast || a_out != nullptr)
-          *reinterpret_cast<float4 *>(a_out + o) = make_float4(p.x, p.y, q.x, q.y);
-        if (M == Conv::kHidden) {
-          const float s0 = norm2f(p), s1 = norm2f(q);
-          const float g = rsqrtf(1.f + (s0 + s1));
-          __nv_bfloat162 h[2] = {f2bf(make_float2(p.x * g, p.y * g)), f2bf(make_float2(q.x * g, q.y * g))};
-          *reinterpret_cast<uint2 *>(h_out + o) = *reinterpret_cast<const uint2 *>(h);
+#pragma unroll
+      for (int half = 0; half < 2; ++half) {
+        if (2 * c2 + half >= C) break;
+        const float2 p = acc[s][2 * half], q = acc[s][2 * half + 1];
+        const size_t o = ((size_t)f * V + x) * kout + 4 * c2 + 2 * half;
+        if (M == Conv::kAdjoint) {
+          const float4 a = *reinterpret_cast<const float4 *>(a_prev + o);
+          const float sq = (a.x * a.x + a.y * a.y) + (a.z * a.z + a.w * a.w);
+          const float re = (a.x * p.x + a.y * p.y) + (a.z * q.x + a.w * q.y);
+          const float g = rsqrtf(1.f + sq);
+          const float dg2 = -g * g * g * re;  // 2 g'(s) Re(a^dagger gh), g' = -g^3 / 2
+          *reinterpret_cast<float4 *>(a_out + o) =
+              make_float4(g * p.x + dg2 * a.x, g * p.y + dg2 * a.y, g * q.x + dg2 * a.z, g * q.y + dg2 * a.w);
+        } else {
+          if (M == Conv::kLast || a_out != nullptr)
+            *reinterpret_cast<float4 *>(a_out + o) = make_float4(p.x, p.y, q.x, q.y);
+          if (M == Conv::kHidden) {
+            const float s0 = norm2f(p), s1 = norm2f(q);
+            const float g = rsqrtf(1.f + (s0 + s1));
+            __nv_bfloat162 h[2] = {f2bf(make_float2(p.x * g, p.y * g)), f2bf(make_float2(q.x * g, q.y * g))};
+            *reinterpret_cast<uint2 *>(h_out + o) = *reinterpret_cast<const uint2 *>(h);
+          }
         }
       }
     }
@@ -254,7 +285,8 @@ __global__ void __launch_bounds__(kConvThreads, 3) ptconv_kernel(const TI *__res
 // contiguous range of (field, site) pairs; partials[cta][entry] (entry = (dir co2 + lo) ci2 + li)
 // A thread owns input entry li (its lane) and output rows lo0 .. lo0 + 3 of every direction: per staged
 // site two 16-byte broadcast loads of g and five loads of T h for 20 complex multiply-adds. The next group's
-// rows are requested while this one's are multiplied (16 fields of 128^2, 32 channels: 361 -> 261 us).
+// rows are requested while this one's are multiplied (16 fields of 128^2, 32 entries: 361 -> 261 us; eight rows to a
+// thread with 4 warps to a CTA took 300 us).
 constexpr int kWG = 16;  // sites staged per group
 __global__ void __launch_bounds__(256, 2) ptconv_bwd_weight_kernel(const float2 *__restrict__ ga,
                                                                    const __nv_bfloat162 *__restrict__ h_in,
@@ -566,21 +598,34 @@ __global__ void to_float2_kernel(const Cx<double> *__restrict__ a, long long n, 
 
 int blocks_for(long long n, int t) { return (int)((n + t - 1) / t); }
 
-// CTAs per field: at most the three resident on each of 152 SMs over all fields (each stages the weights
-// once; eight more than that ran a second wave of their own: 420 instead of 328 us a layer)
-template <Conv M, typename TI>
-void conv_launch(const TI *in, const float2 *U, const int *fmap, const float2 *W, int kin, int kout, int L0, int L1,
-                 int nf, const float2 *a_prev, float2 *a_out, __nv_bfloat162 *h_out, cudaStream_t s) {
-  auto fn = ptconv_kernel<M, TI>;
-  const int S = conv_tile(kout / 2);
-  const size_t smem = ((size_t)5 * kin * kout + (size_t)kin * S) * sizeof(float2);
+template <Conv M, typename TI, int SP>
+void conv_launch_tile(const TI *in, const float2 *U, const int *fmap, const float2 *W, int kin, int kout, int L0,
+                      int L1, int nf, const float2 *a_prev, float2 *a_out, __nv_bfloat162 *h_out, cudaStream_t s) {
+  const int c2 = (kout / 2 + 1) / 2, S = conv_tile(c2, SP, kin);
+  const auto fn = ptconv_kernel<M, TI, SP>;
+  const size_t smem = ((size_t)5 * kin * 4 * c2 + (size_t)kin * S) * sizeof(float2);
   MG_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  // CTAs per field: at most the two resident on each of 152 SMs over all fields (each stages the weights once; a
+  // few CTAs more would run a second wave of their own)
   const long long tiles = ((long long)L0 * L1 + S - 1) / S;
-  long long gx = 152 * 3 / nf;
+  long long gx = 152 * 2 / nf;
   if (gx < 1) gx = 1;
   if (gx > tiles) gx = tiles;
   fn<<<dim3((unsigned int)gx, nf), kConvThreads, smem, s>>>(in, U, fmap, W, kin, kout, L0, L1, a_prev, a_out, h_out);
   MG_LAUNCHED();
+}
+
+// four sites to a thread, or two where tiles of the wider form would not give every SM one (a gradient with 32
+// entries: one field of 64^2, 32 tiles: 436 us wide, 390 narrow; 128^2, 128 tiles: 524 both; eight fields of 64^2,
+// 256 tiles: 734 and 765)
+template <Conv M, typename TI>
+void conv_launch(const TI *in, const float2 *U, const int *fmap, const float2 *W, int kin, int kout, int L0, int L1,
+                 int nf, const float2 *a_prev, float2 *a_out, __nv_bfloat162 *h_out, cudaStream_t s) {
+  const int S = conv_tile((kout / 2 + 1) / 2, 4, kin);
+  if (((long long)L0 * L1 + S - 1) / S * nf >= 152)
+    conv_launch_tile<M, TI, 4>(in, U, fmap, W, kin, kout, L0, L1, nf, a_prev, a_out, h_out, s);
+  else
+    conv_launch_tile<M, TI, 2>(in, U, fmap, W, kin, kout, L0, L1, nf, a_prev, a_out, h_out, s);
 }
 
 }  // namespace
