@@ -44,15 +44,40 @@ inline int mr_blocks(long long full) { return (int)(full < kMrGrid ? full : kMrG
 // reach more SMs (64^2 in FP64, bound by the FP64 rate: an MR iteration on 16 of 152 SMs took 16 us).
 inline int site_threads(long long sites) { return sites <= 64LL * 152 ? 64 : 256; }
 
+// the warp's sums of v[0], v[1] and v[2], in the lanes with lane & 3 = 0, 1 and 2: the values part over the lanes of a
+// group of four first, 6 additions (each holds an FP64 pipe for 16 cycles) where three butterflies take 15
+template <typename R>
+__device__ __forceinline__ R warp_reduce3(const R (&v)[3]) {
+  const bool hi = (threadIdx.x & 2) != 0, odd = (threadIdx.x & 1) != 0;
+  const R a = (hi ? v[2] : v[0]) + __shfl_xor_sync(0xffffffffu, hi ? v[0] : v[2], 2);
+  const R b = (hi ? (R)0 : v[1]) + __shfl_xor_sync(0xffffffffu, hi ? v[1] : (R)0, 2);
+  R k = (odd ? b : a) + __shfl_xor_sync(0xffffffffu, odd ? a : b, 1);
+#pragma unroll
+  for (int o = 4; o < 32; o <<= 1) k += __shfl_xor_sync(0xffffffffu, k, o);
+  return k;
+}
+
+// sum over the block of the values that lanes 0, 1 and 2 of every warp hold, in threads 0, 1 and 2 (sh: 32 x 3)
+template <typename R>
+__device__ __forceinline__ R block_sum3(R k, R *sh) {
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  if (lane < 3) sh[wid * 3 + lane] = k;
+  __syncthreads();
+  R t = (R)0;
+  if (threadIdx.x < 3)
+    for (int w = 0; w < nw; ++w) t += sh[w * 3 + threadIdx.x];
+  return t;
+}
+
 // this block's (<A r, r> re, im, |A r|^2) into part_out[3 blockIdx.x ..]
 template <typename R>
-__device__ __forceinline__ void mr_publish(R (&v)[3], R *part_out, R *sh) {
-  block_reduce<3, R>(v, sh);
-  if (threadIdx.x == 0) {
-    part_out[3 * blockIdx.x] = v[0];
-    part_out[3 * blockIdx.x + 1] = v[1];
-    part_out[3 * blockIdx.x + 2] = v[2];
-  }
+__device__ __forceinline__ void mr_publish_lanes(R k, R *part_out, R *sh) {
+  const R t = block_sum3<R>(k, sh);
+  if (threadIdx.x < 3) part_out[3 * blockIdx.x + threadIdx.x] = t;
+}
+template <typename R>
+__device__ __forceinline__ void mr_publish(const R (&v)[3], R *part_out, R *sh) {
+  mr_publish_lanes<R>(warp_reduce3<R>(v), part_out, sh);
 }
 
 // alpha = omega <A r, r> / |A r|^2 from the `nb` block partials of the previous launch:
@@ -66,12 +91,11 @@ __device__ __forceinline__ Cx<R> mr_alpha(const R *part_in, int nb, double omega
     v[1] += __ldcg(part_in + 3 * b + 1);
     v[2] += __ldcg(part_in + 3 * b + 2);
   }
-  block_reduce<3, R>(v, sh);
+  const R t = block_sum3<R>(warp_reduce3<R>(v), sh);
   __shared__ R s_alpha[2];
-  if (threadIdx.x == 0) {
-    const R den = v[2];
-    s_alpha[0] = den > (R)0 ? (R)omega * v[0] / den : (R)0;
-    s_alpha[1] = den > (R)0 ? (R)omega * v[1] / den : (R)0;
+  if (threadIdx.x < 32) {
+    const R den = __shfl_sync(0xffffffffu, t, 2);
+    if (threadIdx.x < 2) s_alpha[threadIdx.x] = den > (R)0 ? (R)omega * t / den : (R)0;
   }
   __syncthreads();
   return mk(s_alpha[0], s_alpha[1]);
