@@ -149,7 +149,13 @@ __global__ void __launch_bounds__(256, 8) dslash_half_kernel(const __half2 *__re
   const unsigned int x0 = x % l0;
   const unsigned int up = x + l0 < V ? x + l0 : x + l0 - V, dn = x >= l0 ? x - l0 : x + V - l0;
   const unsigned int right = x0 + 1 == l0 ? x + 1 - l0 : x + 1, left = x0 == 0 ? x + l0 - 1 : x - 1;
-  const uint2 l = __ldg(reinterpret_cast<const uint2 *>(U) + x);
+  uint2 l;  // links may start on 4 bytes (one branch for the whole grid), spinors start on 8
+  if ((reinterpret_cast<uintptr_t>(U) & 7) == 0) {
+    l = __ldg(reinterpret_cast<const uint2 *>(U) + x);
+  } else {
+    l.x = __ldg(reinterpret_cast<const unsigned int *>(U) + 2 * x);
+    l.y = __ldg(reinterpret_cast<const unsigned int *>(U) + 2 * x + 1);
+  }
   const float2 p = h2f(l.x), q = h2f(l.y);
   const Pair<float> o =
       wilson_raw(raw_load(in, in_nrm, x), raw_load(in, in_nrm, right), raw_load(in, in_nrm, up),
