@@ -1212,7 +1212,7 @@ def main():
     ap.add_argument("--no-learned", action="store_true", help="skip the learned near-null setup evaluation")
     ap.add_argument("--no-config2", action="store_true", help="skip the many-configuration x many-source batch")
     ap.add_argument("--no-paper", action="store_true", help="skip the paper's MG-CG experiment")
-    ap.add_argument("--only", default=None, choices=["paper", "step", "dslash4-sweep", "dslash-f16", "dslash-f32", "dslash-f64", "dslash4-f32", "dslash4-f64", "solve", "vcycle",
+    ap.add_argument("--only", default=None, choices=["paper", "step", "dslash-f16", "dslash-f32", "dslash-f64", "dslash4-f32", "dslash4-f64", "solve", "vcycle",
                                                       "transfer", "coarse-tc", "coarse-tc4", "su3", "su3-prof",
                                                       "su3-batch-prof", "mixed-sizes", "learned", "large",
                                                       "config2"],
