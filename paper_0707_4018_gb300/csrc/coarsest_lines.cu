@@ -12,7 +12,8 @@
 // the dense factorisation of n = 2048 dofs is 23 GFLOP and its triangular solves are a chain of
 // 2048 steps; the ring of 16 lines x 128 dofs takes 1.8 GFLOP and a chain of 4 levels.
 // Measured at n = 2048 (16 x 16 sites, N = 8): one solve 68 us (dense triangular solves: 3.4 ms);
-// a 64^2 two-level FP64 setup and solve, 5 factorisations and 64 solves, 29.9 ms (dense: 524 ms).
+// a 64^2 two-level FP64 setup and solve, 5 factorisations and 64 solves, 29.9 ms (dense: 524 ms), 22.8 with the
+// other kernels of that path as they are now.
 //
 //  * D_e^-1: Gauss-Jordan over 16 x 16 sub-blocks, a CTA per 16 x 16 tile and line, one launch per
 //    sub-block column; the CTA that finishes the next pivot block inverts it (partial pivoting

@@ -204,12 +204,13 @@ void launch_prolong_add(const Cx<R> *V, const Cx<R> *coarse, Cx<R> *fine, BlockG
 // block Gram-Schmidt (modified, twice, k order) of Nv level vectors into V[b][k][i]; FP64
 void launch_block_mgs(const Cx<double> *vecs, long long vec_stride, Cx<double> *V, BlockGeo bg, int Nv,
                       double *min_norm_dev, cudaStream_t s);
-// Galerkin coarse operator Yc[b][dir][col][row] (internal layout) of P^dagger A P; FP64 inputs and
-// output, arithmetic in FP64 or (fp32_arith, the hierarchies of mixed-precision cycles) FP32
-void launch_galerkin_wilson(const Cx<double> *U, double diag, const Cx<double> *V, Cx<double> *Yc, BlockGeo bg,
-                            int Nv, cudaStream_t s, bool fp32_arith = false);
-void launch_galerkin_stencil(const Cx<double> *Y, const Cx<double> *V, Cx<double> *Yc, BlockGeo bg, int Nv,
-                             cudaStream_t s, bool fp32_arith = false);
+// Galerkin coarse operator Yc[b][dir][col][row] (internal layout) of P^dagger A P; inputs and arithmetic in CT
+// (double, or float in the hierarchies of mixed-precision cycles), output FP64
+template <typename CT>
+void launch_galerkin_wilson(const Cx<CT> *U, double diag, const Cx<CT> *V, Cx<double> *Yc, BlockGeo bg, int Nv,
+                            cudaStream_t s);
+template <typename CT>
+void launch_galerkin_stencil(const Cx<CT> *Y, const Cx<CT> *V, Cx<double> *Yc, BlockGeo bg, int Nv, cudaStream_t s);
 
 // ---- layout conversions at the boundary ----
 // internal Y[j][dir][col][row] <-> canonical Y[j][dir][row][col]

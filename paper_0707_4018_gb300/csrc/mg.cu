@@ -205,6 +205,27 @@ static bool galerkin_f32(const mg_ctx &c) {
 
 static double diag_of(const mg_ctx &c) { return c.geom.d + c.m; }
 
+// the Galerkin operator of level l + 1 from level l's operator and prolongator; in FP32 arithmetic from FP32 copies of
+// them, made here
+static void galerkin(mg_ctx &c, int l) {
+  Level &L = c.lv[l];
+  Cx<double> *Yc = c.lv[l + 1].Y64.p;
+  if (!galerkin_f32(c)) {
+    if (l == 0)
+      launch_galerkin_wilson<double>(c.U64.p, diag_of(c), L.V64.p, Yc, L.bg, L.Nv, c.s);
+    else
+      launch_galerkin_stencil<double>(L.Y64.p, L.V64.p, Yc, L.bg, L.Nv, c.s);
+    return;
+  }
+  launch_convert<float, double>(L.V64.p, L.V32.p, L.V64.n, c.s);
+  if (l == 0) {
+    launch_galerkin_wilson<float>(c.U32.p, diag_of(c), L.V32.p, Yc, L.bg, L.Nv, c.s);
+  } else {
+    launch_convert<float, double>(L.Y64.p, L.Y32.p, L.Y64.n, c.s);
+    launch_galerkin_stencil<float>(L.Y32.p, L.V32.p, Yc, L.bg, L.Nv, c.s);
+  }
+}
+
 template <typename R>
 static Work<R> &work(Level &L);
 template <>
@@ -1149,12 +1170,8 @@ static void prepare_coarsest(mg_ctx &c) {
 // block Gram-Schmidt of the level's vectors and the Galerkin operator of l+1
 static void build_level(mg_ctx &c, int l) {
   Level &L = c.lv[l];
-  Level &C = c.lv[l + 1];
   launch_block_mgs(L.nullv.p, L.n, L.V64.p, L.bg, L.Nv, L.mgs_min.p, c.s);
-  if (l == 0)
-    launch_galerkin_wilson(c.U64.p, diag_of(c), L.V64.p, C.Y64.p, L.bg, L.Nv, c.s, galerkin_f32(c));
-  else
-    launch_galerkin_stencil(L.Y64.p, L.V64.p, C.Y64.p, L.bg, L.Nv, c.s, galerkin_f32(c));
+  galerkin(c, l);
 }
 
 // One adaptive-setup level in the context precision. In FP32 mode the relaxation
@@ -1901,13 +1918,7 @@ int mg_update_mass(mg_ctx *c, double m) {
     c->m = m;
     MG_CUDA(cudaStreamSynchronize(c->s));  // no replay of the old graphs is still in flight
     drop_graphs(*c);
-    for (int l = 0; l + 1 < c->p.levels; ++l) {
-      Level &L = c->lv[l];
-      if (l == 0)
-        launch_galerkin_wilson(c->U64.p, diag_of(*c), L.V64.p, c->lv[1].Y64.p, L.bg, L.Nv, c->s, galerkin_f32(*c));
-      else
-        launch_galerkin_stencil(L.Y64.p, L.V64.p, c->lv[l + 1].Y64.p, L.bg, L.Nv, c->s, galerkin_f32(*c));
-    }
+    for (int l = 0; l + 1 < c->p.levels; ++l) galerkin(*c, l);
     prepare_coarsest(*c);
     make_fp32_copies(*c);
     MG_CUDA(cudaStreamSynchronize(c->s));
@@ -1933,10 +1944,7 @@ int mg_clone(mg_ctx *src, double m, void *stream, mg_ctx **out) {
       MG_CUDA(cudaMemcpyAsync(L.nullv.p, S.nullv.p, L.nullv.n * sizeof(Cx<double>), cudaMemcpyDeviceToDevice, c->s));
       MG_CUDA(cudaMemcpyAsync(L.V64.p, S.V64.p, L.V64.n * sizeof(Cx<double>), cudaMemcpyDeviceToDevice, c->s));
       // Galerkin operators at the clone's mass, level by level (level l + 1 needs Y of level l)
-      if (l == 0)
-        launch_galerkin_wilson(c->U64.p, diag_of(*c), L.V64.p, c->lv[1].Y64.p, L.bg, L.Nv, c->s, galerkin_f32(*c));
-      else
-        launch_galerkin_stencil(L.Y64.p, L.V64.p, c->lv[l + 1].Y64.p, L.bg, L.Nv, c->s, galerkin_f32(*c));
+      galerkin(*c, l);
     }
     prepare_coarsest(*c);
     make_fp32_copies(*c);

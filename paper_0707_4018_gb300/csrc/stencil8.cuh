@@ -5,7 +5,7 @@
 // load per direction, so a warp reads each 512-byte block in one instruction (with 8-byte loads of
 // one row, 10 per thread, the loads' issue and their index arithmetic bounded the kernel: 690
 // instructions per warp and site). At 256 x 192 sites (126 MB of blocks) the apply takes 23 us (39
-// before), an MR iteration 36 us (121 before, 92 with the capped grid of mr.cuh). The q sum is a
+// before), an MR iteration 34 us (121 before, 92 with the capped grid of mr.cuh). The q sum is a
 // reduce-scatter: 4 shuffles, after which a lane holds one real number of the result.
 #pragma once
 

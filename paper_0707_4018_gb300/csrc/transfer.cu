@@ -262,10 +262,11 @@ __device__ __forceinline__ NbrInfo neighbour_in_blocks(const BlockGeo &g, int x0
   return n;
 }
 
-// parts for the fine Wilson level (n_int = 2); arithmetic in CT (FP64, or FP32 for the
-// setup of mixed-precision hierarchies), inputs and output FP64
+// parts for the fine Wilson level (n_int = 2); inputs and arithmetic in CT (FP64, or FP32 for the
+// setup of mixed-precision hierarchies). With FP64 inputs to FP32 arithmetic the conversions, two per product at the
+// FP64 rate, were most of the kernel (225 us at 256^2, and 144 us for the next level; 111 and 36 from FP32 copies).
 template <typename CT>
-__device__ void galerkin_parts_wilson(const Cx<double> *__restrict__ U, double diag, const Cx<double> *__restrict__ V,
+__device__ void galerkin_parts_wilson(const Cx<CT> *__restrict__ U, double diag, const Cx<CT> *__restrict__ V,
                                       const BlockGeo &g, int Nv, long long b, int lane, Cx<CT> *parts) {
   const long long pstride = (long long)Nv * g.Nb;  // parts[dir][k][i]
   for (int i = lane; i < g.Nb; i += 32) {
@@ -274,19 +275,24 @@ __device__ void galerkin_parts_wilson(const Cx<double> *__restrict__ U, double d
     const int x0 = (int)(x % g.L0), x1 = (int)(x / g.L0);
     NbrInfo nb[5];
     Cx<CT> link[5];
+#pragma unroll
     for (int dir = 1; dir <= 4; ++dir) {
       nb[dir] = neighbour_in_blocks(g, x0, x1, dir);
       // +mu: U_x^mu; -mu: U_{x-mu}^mu (conjugated inside hop_scalar)
-      link[dir] = cvt<CT, double>((dir == 1)   ? U[2 * x]
-                                  : (dir == 2) ? U[2 * nb[2].site]
-                                  : (dir == 3) ? U[2 * x + 1]
-                                               : U[2 * nb[4].site + 1]);
+      link[dir] = (dir == 1)   ? U[2 * x]
+                  : (dir == 2) ? U[2 * nb[2].site]
+                  : (dir == 3) ? U[2 * x + 1]
+                               : U[2 * nb[4].site + 1];
     }
+#pragma unroll 2
     for (int k = 0; k < Nv; ++k) {
-      Cx<CT> self = (CT)diag * cvt<CT, double>(V[(b * Nv + k) * (long long)g.Nb + i]);
+      Cx<CT> self = (CT)diag * V[(b * Nv + k) * (long long)g.Nb + i];
+#pragma unroll
       for (int dir = 1; dir <= 4; ++dir) {
-        const Cx<double> *Vs = V + (nb[dir].src_b * Nv + k) * (long long)g.Nb + 2 * nb[dir].src_s;
-        const Cx<CT> t = hop_scalar<CT>(dir, link[dir], cvt<CT, double>(Vs[0]), cvt<CT, double>(Vs[1]));
+        // a site's two entries in one load: Nb = 2 x sites is even
+        const Cx<CT> *Vk = V + (nb[dir].src_b * Nv + k) * (long long)g.Nb;
+        const Pair<CT> ws = reinterpret_cast<const Pair<CT> *>(Vk)[nb[dir].src_s];
+        const Cx<CT> t = hop_scalar<CT>(dir, link[dir], ws.a, ws.b);
         Cx<CT> comp = spin == 0 ? t : hop_lower<CT>(dir, t);
         comp = (CT)-0.5 * comp;
         if (nb[dir].face) {
@@ -301,44 +307,53 @@ __device__ void galerkin_parts_wilson(const Cx<double> *__restrict__ U, double d
   }
 }
 
-// parts for a coarse stencil level (n_int = N, Y internal [j][dir][col][row]); arithmetic in CT
-template <typename CT>
-__device__ void galerkin_parts_stencil(const Cx<double> *__restrict__ Y, const Cx<double> *__restrict__ V,
+// parts for a coarse stencil level (n_int = N, Y internal [j][dir][col][row]); inputs and arithmetic in CT. NC: N at
+// compile time (8), so that a lane holds its eight entries of a block of Y for all vectors, or 0
+template <typename CT, int NC>
+__device__ void galerkin_parts_stencil(const Cx<CT> *__restrict__ Y, const Cx<CT> *__restrict__ V,
                                        const BlockGeo &g, int Nv, long long b, int lane, Cx<CT> *parts) {
-  const int N = g.nint;
+  const int N = NC > 0 ? NC : g.nint;
   const long long pstride = (long long)Nv * g.Nb;
   for (int i = lane; i < g.Nb; i += 32) {
     const int s = i / N, arow = i - s * N;
     const long long x = fine_site_of(g, b, s);
     const int x0 = (int)(x % g.L0), x1 = (int)(x / g.L0);
-    for (int k = 0; k < Nv; ++k) {
-      // self term: X(arow, c) W_k(x, c)
-      Cx<CT> self = mk((CT)0, (CT)0);
-      {
-        const Cx<double> *Yd = Y + (x * 5 + 0) * (long long)N * N;
-        const Cx<double> *Ws = V + (b * Nv + k) * (long long)g.Nb + (long long)s * N;
-        for (int c = 0; c < N; ++c) cmac(self, cvt<CT, double>(Yd[(long long)c * N + arow]), cvt<CT, double>(Ws[c]));
-      }
-      for (int dir = 1; dir <= 4; ++dir) {
-        const NbrInfo nb = neighbour_in_blocks(g, x0, x1, dir);
-        const Cx<double> *Yd = Y + (x * 5 + dir) * (long long)N * N;
-        const Cx<double> *Ws = V + (nb.src_b * Nv + k) * (long long)g.Nb + (long long)nb.src_s * N;
+    for (int dir = 0; dir <= 4; ++dir) {
+      // self term: X(arow, c) W_k(x, c), then the hops
+      NbrInfo nb = {b, s, x, false};
+      if (dir > 0) nb = neighbour_in_blocks(g, x0, x1, dir);
+      const Cx<CT> *Yd = Y + (x * 5 + dir) * (long long)N * N + arow;
+      const Cx<CT> *Ws = V + nb.src_b * Nv * (long long)g.Nb + (long long)nb.src_s * N;
+      Cx<CT> y[NC > 0 ? NC : 1];
+#pragma unroll
+      for (int c = 0; c < NC; ++c) y[c] = Yd[c * NC];
+#pragma unroll 4
+      for (int k = 0; k < Nv; ++k) {
+        const Cx<CT> *Wk = Ws + (long long)k * g.Nb;
         Cx<CT> comp = mk((CT)0, (CT)0);
-        for (int c = 0; c < N; ++c) cmac(comp, cvt<CT, double>(Yd[(long long)c * N + arow]), cvt<CT, double>(Ws[c]));
-        if (nb.face) {
-          parts[dir * pstride + (long long)k * g.Nb + i] = comp;
+        if (NC > 0) {
+#pragma unroll
+          for (int c = 0; c < NC; c += 2) {
+            const Pair<CT> w = reinterpret_cast<const Pair<CT> *>(Wk)[c / 2];
+            cmac(comp, y[c], w.a);
+            cmac(comp, y[c + (NC > 1)], w.b);
+          }
         } else {
-          self = self + comp;
-          parts[dir * pstride + (long long)k * g.Nb + i] = mk((CT)0, (CT)0);
+          for (int c = 0; c < N; ++c) cmac(comp, Yd[(long long)c * N], Wk[c]);
         }
+        Cx<CT> *p = parts + (long long)k * g.Nb + i;
+        if (dir == 0)
+          *p = comp;
+        else if (!nb.face)
+          *p = *p + comp;
+        if (dir > 0) p[dir * pstride] = nb.face ? comp : mk((CT)0, (CT)0);
       }
-      parts[(long long)k * g.Nb + i] = self;
     }
   }
 }
 
-template <bool WILSON, typename CT>
-__global__ void galerkin_kernel(const Cx<double> *__restrict__ U_or_Y, double diag, const Cx<double> *__restrict__ V,
+template <bool WILSON, typename CT, int NC>
+__global__ void galerkin_kernel(const Cx<CT> *__restrict__ U_or_Y, double diag, const Cx<CT> *__restrict__ V,
                                 Cx<double> *__restrict__ Yc, BlockGeo g, int Nv) {
   extern __shared__ __align__(16) unsigned char smem_gal_raw[];
   Cx<CT> *smem_gal = reinterpret_cast<Cx<CT> *>(smem_gal_raw);
@@ -346,19 +361,29 @@ __global__ void galerkin_kernel(const Cx<double> *__restrict__ U_or_Y, double di
   const long long b = blockIdx.x * (long long)(blockDim.x >> 5) + warp;
   if (b >= g.nblocks) return;
   Cx<CT> *parts = smem_gal + (long long)warp * 5 * Nv * g.Nb;
-  if (WILSON)
+  if constexpr (WILSON)
     galerkin_parts_wilson<CT>(U_or_Y, diag, V, g, Nv, b, lane, parts);
   else
-    galerkin_parts_stencil<CT>(U_or_Y, V, g, Nv, b, lane, parts);
+    galerkin_parts_stencil<CT, NC>(U_or_Y, V, g, Nv, b, lane, parts);
   __syncwarp();
   const long long pstride = (long long)Nv * g.Nb;
-  const Cx<double> *Vb = V + b * (long long)Nv * g.Nb;
+  const Cx<CT> *Vb = V + b * (long long)Nv * g.Nb;
   for (int o = lane; o < 5 * Nv * Nv; o += 32) {
     const int dir = o / (Nv * Nv), rem = o - dir * Nv * Nv, k = rem / Nv, kp = rem - k * Nv;
     Cx<CT> acc = mk((CT)0, (CT)0);
     const Cx<CT> *p = parts + dir * pstride + (long long)k * g.Nb;
-    const Cx<double> *vk = Vb + (long long)kp * g.Nb;
-    for (int i = 0; i < g.Nb; ++i) cmac_conj(acc, cvt<CT, double>(vk[i]), p[i]);
+    const Cx<CT> *vk = Vb + (long long)kp * g.Nb;
+    if (sizeof(CT) == 4 && (g.Nb & 1) == 0) {  // 16-byte loads of two entries
+#pragma unroll 4
+      for (int i = 0; i < g.Nb / 2; ++i) {
+        const Pair<CT> v = reinterpret_cast<const Pair<CT> *>(vk)[i], q = reinterpret_cast<const Pair<CT> *>(p)[i];
+        cmac_conj(acc, v.a, q.a);
+        cmac_conj(acc, v.b, q.b);
+      }
+    } else {
+#pragma unroll 4
+      for (int i = 0; i < g.Nb; ++i) cmac_conj(acc, vk[i], p[i]);
+    }
     // internal layout [b][dir][col = k][row = kp]
     Yc[((b * 5 + dir) * Nv + k) * (long long)Nv + kp] = cvt<double, CT>(acc);
   }
@@ -408,7 +433,8 @@ __device__ __forceinline__ void philox10(uint32_t c[4], uint32_t k0, uint32_t k1
 
 // Vectors (k0 + blockIdx.z) of the seeds blockIdx.y: FP64-bound (log, sqrt, sincospi per draw). One launch for
 // all vectors, because one of 32768 draws occupies the chip for a launch's latency only: 128 launches took
-// 8.8 us each with cos and sin of 2 pi u2 and 7.5 us with sincospi, whose reduction of the angle is exact; as one launch they take 0.45 ms of 0.96.
+// 8.8 us each with cos and sin of 2 pi u2 and 7.5 us with sincospi, whose reduction of the angle is exact; as one
+// launch they take 0.55 ms.
 struct GaussianSeeds {
   unsigned long long v[kGaussianSeeds];
 };
@@ -484,35 +510,41 @@ void launch_block_mgs(const Cx<double> *vecs, long long vec_stride, Cx<double> *
   MG_LAUNCHED();
 }
 
-template <bool WILSON, typename CT>
-static void launch_galerkin_impl(const Cx<double> *UY, double diag, const Cx<double> *V, Cx<double> *Yc, BlockGeo bg,
-                                 int Nv, cudaStream_t s) {
+template <bool WILSON, typename CT, int NC>
+static void launch_galerkin_impl(const Cx<CT> *UY, double diag, const Cx<CT> *V, Cx<double> *Yc, BlockGeo bg, int Nv,
+                                 cudaStream_t s) {
+  const auto fn = galerkin_kernel<WILSON, CT, NC>;
   const size_t per_warp = (size_t)5 * Nv * bg.Nb * sizeof(Cx<CT>);
   const int warps = warps_for_smem(per_warp, 200 * 1024);
   if (warps < 1) fail(MG_ERR_UNSUPPORTED, "Galerkin build: block too large for shared memory");
   const size_t smem = per_warp * warps;
-  MG_CUDA(cudaFuncSetAttribute(galerkin_kernel<WILSON, CT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  MG_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   const unsigned int grid = (unsigned int)((bg.nblocks + warps - 1) / warps);
-  galerkin_kernel<WILSON, CT><<<grid, 32 * warps, smem, s>>>(UY, diag, V, Yc, bg, Nv);
+  fn<<<grid, 32 * warps, smem, s>>>(UY, diag, V, Yc, bg, Nv);
   MG_LAUNCHED();
 }
 
-void launch_galerkin_wilson(const Cx<double> *U, double diag, const Cx<double> *V, Cx<double> *Yc, BlockGeo bg,
-                            int Nv, cudaStream_t s, bool fp32_arith) {
+template <typename CT>
+void launch_galerkin_wilson(const Cx<CT> *U, double diag, const Cx<CT> *V, Cx<double> *Yc, BlockGeo bg, int Nv,
+                            cudaStream_t s) {
   if (bg.nint != 2) fail(MG_ERR_INVALID_ARG, "Galerkin (Wilson): n_int must be 2");
-  if (fp32_arith)
-    launch_galerkin_impl<true, float>(U, diag, V, Yc, bg, Nv, s);
-  else
-    launch_galerkin_impl<true, double>(U, diag, V, Yc, bg, Nv, s);
+  launch_galerkin_impl<true, CT, 0>(U, diag, V, Yc, bg, Nv, s);
 }
 
-void launch_galerkin_stencil(const Cx<double> *Y, const Cx<double> *V, Cx<double> *Yc, BlockGeo bg, int Nv,
-                             cudaStream_t s, bool fp32_arith) {
-  if (fp32_arith)
-    launch_galerkin_impl<false, float>(Y, 0.0, V, Yc, bg, Nv, s);
+template <typename CT>
+void launch_galerkin_stencil(const Cx<CT> *Y, const Cx<CT> *V, Cx<double> *Yc, BlockGeo bg, int Nv, cudaStream_t s) {
+  if (bg.nint == 8)
+    launch_galerkin_impl<false, CT, 8>(Y, 0.0, V, Yc, bg, Nv, s);
   else
-    launch_galerkin_impl<false, double>(Y, 0.0, V, Yc, bg, Nv, s);
+    launch_galerkin_impl<false, CT, 0>(Y, 0.0, V, Yc, bg, Nv, s);
 }
+
+#define MG_INST_GALERKIN(CT)                                                                                         \
+  template void launch_galerkin_wilson<CT>(const Cx<CT> *, double, const Cx<CT> *, Cx<double> *, BlockGeo, int,      \
+                                           cudaStream_t);                                                            \
+  template void launch_galerkin_stencil<CT>(const Cx<CT> *, const Cx<CT> *, Cx<double> *, BlockGeo, int, cudaStream_t);
+MG_INST_GALERKIN(double)
+MG_INST_GALERKIN(float)
 
 void launch_coarse_to_canonical(const Cx<double> *Yi, Cx<double> *Yc, long long nsites, int N, cudaStream_t s) {
   coarse_to_canonical_kernel<<<grid_for(nsites * 5LL * N * N, 256), 256, 0, s>>>(Yi, Yc, nsites, N);
