@@ -358,17 +358,25 @@ __global__ void __launch_bounds__(256) coarsest_gcr_kernel(CgArgs<VT> a) {
 // per site with 16-byte loads, the next site's blocks requested while one is summed (stencil8.cuh),
 // the vector work by a thread per dof. Gram-Schmidt is classical in one pass, with a second one only
 // where |w'|^2 < |w|^2 / 2 (every CTA decides from the same sums), so an iteration is one grid sum
-// and one barrier; sums inside a warp are FP32, across warps and CTAs FP64, as in the cluster kernel.
+// and one barrier; every sum is FP64.
+// With FP32 sums inside the warps (the form the figures below are of) a 1024 x 768 solve takes 3 ms less, but loses the precision.
 // The thread-per-row form on a quarter of the SMs, two passes always, took 563 us per solve at 98304
 // dofs (1024 x 768 fine lattice), this one 200 us (a whole fine solve 81.5 -> 64.5 ms; on half or a
 // quarter of the SMs 65.9 and 68.6 ms).
 // ---------------------------------------------------------------------------
 constexpr int kGcr8Warps = 16;
 
-__device__ __forceinline__ void warp_put32(float t, int s, double *swarp) {
+// the warp's sums of v[0 .. nv) (nv <= 4) as slots s, s + 1, ...: the values part over the lanes of a group of
+// four first, 6 FP64 additions where four butterflies take 20 (the kernel waits for these at the FP64 rate)
+__device__ __forceinline__ void warp_put4(const double (&v)[4], int nv, int s, double *swarp) {
+  const bool hi = (threadIdx.x & 2) != 0, odd = (threadIdx.x & 1) != 0;
+  const double a = (hi ? v[2] : v[0]) + __shfl_xor_sync(0xffffffffu, hi ? v[0] : v[2], 2);
+  const double b = (hi ? v[3] : v[1]) + __shfl_xor_sync(0xffffffffu, hi ? v[1] : v[3], 2);
+  double k = (odd ? b : a) + __shfl_xor_sync(0xffffffffu, odd ? a : b, 1);
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-  if ((threadIdx.x & 31) == 0) swarp[(threadIdx.x >> 5) * kSlots + s] = (double)t;
+  for (int o = 4; o < 32; o <<= 1) k += __shfl_xor_sync(0xffffffffu, k, o);
+  const int lane = threadIdx.x & 31;
+  if (lane < nv) swarp[(threadIdx.x >> 5) * kSlots + s + lane] = k;
 }
 
 // f(j, value) for every site j of the chunk: the lane's component of (A M v)_j (v through L2: other
@@ -430,27 +438,27 @@ __global__ void __launch_bounds__(32 * kGcr8Warps, 1) coarsest_gcr8_kernel(CgArg
       double inv = 0.0, ar = 0.0, ai = 0.0;
       for (int pass = 0;; ++pass) {
         __syncthreads();
-        for (int q = 0; q < k; ++q) {
-          const Cx<float> *Wq = a.W + (long long)q * n;
-          float re = 0.f, im = 0.f;
+        for (int q = 0; q < k; q += 2) {  // two basis vectors share the read of w and the warp sums
+          const int q1 = q + 1 < k ? q + 1 : q;
+          const Cx<float> *Wa = a.W + (long long)q * n, *Wb = a.W + (long long)q1 * n;
+          double t[4] = {0.0, 0.0, 0.0, 0.0};
           for (long long i = d0; i < d1; i += kStep) {
-            const Cx<float> wj = Wq[i], w = Wk[i];
-            re = fmaf(wj.re, w.re, fmaf(wj.im, w.im, re));
-            im = fmaf(wj.re, w.im, fmaf(-wj.im, w.re, im));
+            const Cx<float> w = Wk[i], wa = Wa[i], wb = Wb[i];
+            t[0] += (double)(wa.re * w.re + wa.im * w.im);
+            t[1] += (double)(wa.re * w.im - wa.im * w.re);
+            t[2] += (double)(wb.re * w.re + wb.im * w.im);
+            t[3] += (double)(wb.re * w.im - wb.im * w.re);
           }
-          warp_put32(re, 3 + 2 * q, swarp);
-          warp_put32(im, 4 + 2 * q, swarp);
+          warp_put4(t, q1 > q ? 4 : 2, 3 + 2 * q, swarp);
         }
-        float nn = 0.f, wr = 0.f, wi = 0.f;
+        double t[4] = {0.0, 0.0, 0.0, 0.0};
         for (long long i = d0; i < d1; i += kStep) {
           const Cx<float> w = Wk[i], ri = a.r[i];
-          nn = fmaf(w.re, w.re, fmaf(w.im, w.im, nn));
-          wr = fmaf(w.re, ri.re, fmaf(w.im, ri.im, wr));
-          wi = fmaf(w.re, ri.im, fmaf(-w.im, ri.re, wi));
+          t[0] += (double)norm2(w);
+          t[1] += (double)(w.re * ri.re + w.im * ri.im);
+          t[2] += (double)(w.re * ri.im - w.im * ri.re);
         }
-        warp_put32(nn, 0, swarp);
-        warp_put32(wr, 1, swarp);
-        warp_put32(wi, 2, swarp);
+        warp_put4(t, 3, 0, swarp);
         grid_sum(a, 3 + 2 * k, swarp, stage, sres, ok);
         if (!ok) return;
         double nw2 = sres[0];
@@ -502,9 +510,9 @@ __global__ void __launch_bounds__(32 * kGcr8Warps, 1) coarsest_gcr8_kernel(CgArg
       if (l.writes) reinterpret_cast<float *>(a.r)[e] = (float)(reinterpret_cast<const double *>(a.b)[e] - (double)v);
     });
     __syncthreads();
-    float tr = 0.f;
-    for (long long i = d0; i < d1; i += kStep) tr += norm2(a.r[i]);
-    warp_put32(tr, 0, swarp);
+    double tr = 0.0;
+    for (long long i = d0; i < d1; i += kStep) tr += (double)norm2(a.r[i]);
+    warp_put(tr, 0, swarp);
     grid_sum(a, 1, swarp, stage, sres, ok);
     if (!ok) return;
     rn2 = sres[0];
