@@ -29,6 +29,7 @@
 #include <algorithm>
 #include <cmath>
 #include <string>
+#include <utility>
 
 #include "coarsest_lines.h"
 #include "kernels.h"
@@ -421,8 +422,11 @@ std::vector<LineLevel> line_levels(int r, int b, long long *ws) {
   return lv;
 }
 
-void line_plan(LineSolver &f, Geo2 g, int N, bool nine, cudaStream_t s) {
-  if (f.planned) return;
+// The plan is made aside and taken over whole: solvers of batched masses are planned inside a solve, and an
+// allocation that fails there must leave the solver as one that was never planned.
+void line_plan(LineSolver &solver, Geo2 g, int N, bool nine, cudaStream_t s) {
+  if (solver.planned) return;
+  LineSolver f;
   f.N = N;
   f.L0 = g.L0;
   f.L1 = g.L1;
@@ -434,6 +438,7 @@ void line_plan(LineSolver &f, Geo2 g, int N, bool nine, cudaStream_t s) {
   f.planned = true;
   if (r < 3) {
     pool_ready();
+    solver = std::move(f);
     return;
   }
   long long ws = 0;
@@ -517,6 +522,7 @@ void line_plan(LineSolver &f, Geo2 g, int N, bool nine, cudaStream_t s) {
   f.jobs_dev.alloc(f.jobs.size());
   pool_ready();
   MG_CUDA(cudaMemcpyAsync(f.jobs_dev.p, f.jobs.data(), f.jobs.size() * sizeof(LineJob), cudaMemcpyHostToDevice, s));
+  solver = std::move(f);
 }
 
 // Dinv of `count` blocks at src (stride in entries)
@@ -631,7 +637,7 @@ bool line_factor(LineSolver &f, const Cx<double> *Y, Geo2 g, int N, bool nine, d
   line_plan(f, g, N, nine, s);
   f.lines = line_try(f, Y, nine, shift, work, s);
   if (!f.lines) {
-    if (f.LU.p == nullptr) {
+    if (f.ipiv.p == nullptr) {  // the later of the two: both are there or both are made
       f.LU.alloc((size_t)f.n * f.n);
       f.ipiv.alloc((size_t)f.n);
       pool_ready();
