@@ -25,10 +25,14 @@ struct Error {
 
 [[noreturn]] inline void fail(int code, const std::string &msg) { throw Error{code, msg}; }
 
+// A call that failed (an allocation of pinned memory, say) is reported here and not once more by the next launch.
 #define MG_CUDA(call)                                                                            \
   do {                                                                                           \
     cudaError_t e_ = (call);                                                                     \
-    if (e_ != cudaSuccess) ::mg::fail(MG_ERR_CUDA, std::string(#call) + ": " + cudaGetErrorString(e_)); \
+    if (e_ != cudaSuccess) {                                                                     \
+      (void)cudaGetLastError();                                                                  \
+      ::mg::fail(MG_ERR_CUDA, std::string(#call) + ": " + cudaGetErrorString(e_));               \
+    }                                                                                            \
   } while (0)
 
 extern std::atomic<long long> g_launches;

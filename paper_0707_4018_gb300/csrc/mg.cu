@@ -871,13 +871,14 @@ struct DevSolve {
 static void alloc_batch(mg_ctx &c);
 
 static void devloop_buffers(mg_ctx &c, int nb) {
-  if (c.dl_ctl.p == nullptr) {
+  // the last buffer of each set tells whether the set was made: an allocation may have failed in the middle of it
+  if (c.dl_w.p == nullptr) {
     c.dl_ctl.alloc(4);
     c.dl_st.alloc(4);
     c.dl_w.alloc(c.lv[0].n);
   }
-  if (nb > 1 && (long long)c.dl_wb.n < nb * c.lv[0].n) {
-    if (c.bZ.p == nullptr) alloc_batch(c);
+  if (nb > 1 && c.dl_coef.p == nullptr) {
+    if (c.bhost == nullptr) alloc_batch(c);
     c.dl_wb.alloc((size_t)c.p.max_rhs * c.lv[0].n);
     c.dl_act.alloc((size_t)c.p.max_rhs);
     c.dl_stv.alloc((size_t)2 * c.p.max_rhs);
@@ -1849,7 +1850,7 @@ int mg_solve_batch(mg_ctx *c, int nrhs, const void *chi, void *psi, const double
     }
     if (nrhs < 1 || nrhs > c->p.max_rhs) fail(MG_ERR_INVALID_ARG, "nrhs must be in [1, max_rhs]");
     check_fresh(*c);
-    if (c->bZ.p == nullptr) alloc_batch(*c);
+    if (c->bhost == nullptr) alloc_batch(*c);  // the last of its buffers
     std::vector<double> sh(nrhs, 0.0);
     for (int v = 0; v < nrhs; ++v) {
       if (mass != nullptr) sh[v] = mass[v] - c->m;

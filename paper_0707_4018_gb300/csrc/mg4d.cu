@@ -1014,7 +1014,6 @@ namespace {
 void alloc_batch(Engine4 &e) {
   auto &b = e.bt;
   const int nb = std::max(1, e.p.max_rhs), ro = e.p.gcr_restart, rc = e.p.coarsest_restart;
-  b.cap = nb;
   b.Z.alloc((size_t)ro * nb * e.nf);
   b.W.alloc((size_t)ro * nb * e.nf);
   b.r.alloc((size_t)nb * e.nf);
@@ -1063,8 +1062,9 @@ void alloc_batch(Engine4 &e) {
   b.ws.capacity = 2LL * rows * nb * 64;
   b.part.alloc((size_t)b.ws.capacity + 16);
   b.tickets.alloc((size_t)b.ws.tickets);
-  MG_CUDA(cudaMallocHost(&b.host, ((size_t)nb * 2 * (ro + 3) + nb * 4) * sizeof(double)));
-  MG_CUDA(cudaMallocHost(&b.chost, ((size_t)nb * 2 * (rc + 3) + nb * 4) * sizeof(double)));
+  if (b.host == nullptr) MG_CUDA(cudaMallocHost(&b.host, ((size_t)nb * 2 * (ro + 3) + nb * 4) * sizeof(double)));
+  if (b.chost == nullptr)
+    MG_CUDA(cudaMallocHost(&b.chost, ((size_t)nb * 2 * (rc + 3) + nb * 4) * sizeof(double)));
   pool_ready();
   MG_CUDA(cudaMemsetAsync(b.tickets.p, 0, b.ws.tickets * sizeof(unsigned int), e.s));
   b.ws.partials = b.part.p;
@@ -1073,6 +1073,7 @@ void alloc_batch(Engine4 &e) {
   // x 64 blocks of 1.5 elements per thread, and the batched dots took 164 us per launch
   b.wsc = b.ws;
   b.wsc.max_blocks = 8;
+  b.cap = nb;  // last: a failed allocation above leaves a batch that is made again
 }
 
 // operand precision of the batched tensor-core coarse apply (launch_coarse4_apply_tc's split):
@@ -1087,7 +1088,7 @@ static int tc_split() {
 // the multi-vector coarse operands after a Galerkin build: BF16 fragments (hi, and lo when
 // a split-operator apply wants them) and an FP32 copy of Y
 static void ensure_mrhs(Engine4 &e, bool lo) {
-  if (e.Ypk4.p == nullptr) {
+  if (e.Y32.p == nullptr) {  // the later of the two
     e.Ypk4.alloc((size_t)e.cg.nsites * 9 * 2 * 9 * 32);
     e.Y32.alloc(e.Y64.n);
     pool_ready();

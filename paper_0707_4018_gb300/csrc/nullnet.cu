@@ -38,6 +38,7 @@ constexpr int kWeightParts = 152 * 2;  // CTAs of partial weight-gradient sums
 
 void nn_ensure(mg_nullnet &n, long long nfV, int nf, long long nblocks) {
   if (nfV > n.cap) {
+    n.cap = 0;  // an allocation that fails below leaves nothing that a smaller call could take for usable
     for (int l = 0; l < 4; ++l) {
       n.h[l].alloc((size_t)nfV * 2 * n.ci[l]);
       n.a[l].alloc((size_t)nfV * 2 * n.co[l]);

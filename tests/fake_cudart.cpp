@@ -45,8 +45,12 @@ cudaError_t launched(const void *f, void **args) {
     if (zero_pivot && arg<int>(args, 2) == 0) *arg<int *>(args, 4) = 1;
   }
   if (has("tri_tile_kernel") || has("permute_kernel")) used(arg<void *>(args, 0), 1);
+  if (has("pack_noise_kernel")) {
+    used(arg<void *>(args, 0), 1);
+    used(arg<void *>(args, 4), 1);
+  }
   // norms of one, so that a solve reaches its preconditioner
-  if (has("norm2_batch_kernel"))
+  if (has("norm2_batch_kernel") && used(arg<void *>(args, 3), 1) == cudaSuccess)
     for (int v = 0; v < 2; ++v) arg<double *>(args, 3)[v] = 1.0;
   return cudaSuccess;
 }

@@ -1,4 +1,4 @@
-"""Failures on the host side of the exact coarsest solve: allocations that fail in the middle of a plan. The library's objects run against a CUDA runtime
+"""Failures on the host side: allocations that fail in the middle of a plan or of the buffers that a first call makes. The library's objects run against a CUDA runtime
 whose memory is host memory and whose launches do nothing (fake_cudart.cpp), so no device is involved."""
 import ctypes
 import glob
@@ -11,7 +11,8 @@ import pytest
 from paper_0707_4018_gb300 import binding, build
 
 HERE = os.path.dirname(os.path.abspath(__file__))
-OOM, NOT_CONVERGED = 3, 4
+FAILED = (2, 3)  # pinned host memory, device memory
+NOT_CONVERGED = 4
 DIMS = (16, 12)
 
 
@@ -31,6 +32,10 @@ def lib(tmp_path_factory):
     return so
 
 
+def _at(a):
+    return ctypes.c_void_p(a.ctypes.data)
+
+
 class Ctx:
     def __init__(self, lib, max_rhs):
         self.lib, self.p = lib, ctypes.c_void_p()
@@ -40,17 +45,13 @@ class Ctx:
         p.Nv[0], p.n_pass, p.max_rhs, p.max_iter = 4, 1, max_rhs, 2
         self.U = np.zeros((DIMS[0] * DIMS[1], 2), dtype=np.complex128)
         self.v = np.zeros((4, DIMS[0] * DIMS[1], 2), dtype=np.complex128)
-        rc = lib.mg_setup(ctypes.byref(self.p), ctypes.byref(binding.make_geom(DIMS)), self._at(self.U),
+        rc = lib.mg_setup(ctypes.byref(self.p), ctypes.byref(binding.make_geom(DIMS)), _at(self.U),
                           ctypes.c_double(0.1), ctypes.byref(p), None)
         assert rc == 0, lib.mg_last_error()
 
-    @staticmethod
-    def _at(a):
-        return ctypes.c_void_p(a.ctypes.data)
-
     def batch(self, *masses):
         m = (ctypes.c_double * len(masses))(*masses)
-        return self.lib.mg_solve_batch(self.p, len(masses), self._at(self.v), self._at(self.v[2:]), m,
+        return self.lib.mg_solve_batch(self.p, len(masses), _at(self.v), _at(self.v[2:]), m,
                                        ctypes.c_double(1e-10), None)
 
     def close(self):
@@ -65,7 +66,7 @@ def _reset(lib):
 
 
 @pytest.mark.parametrize("reject", [0, 1])  # the cyclic reduction's plan, and the dense factors behind it too
-@pytest.mark.parametrize("max_rhs", [2])
+@pytest.mark.parametrize("max_rhs", [1, 2])  # a limit of one: the buffers of batches are made by the first batch
 def test_a_failed_allocation_leaves_nothing_half_made(lib, max_rhs, reject):
     nth, failures = 0, 0
     while True:
@@ -76,12 +77,62 @@ def test_a_failed_allocation_leaves_nothing_half_made(lib, max_rhs, reject):
         lib.fake_fail_at(nth)
         rc = ctx.batch(*masses)
         lib.fake_fail_at(0)
-        if rc == OOM:
+        if rc in FAILED:
             failures += 1
             assert ctx.batch(*masses) in (0, NOT_CONVERGED), (nth, lib.mg_last_error())
         ctx.close()
         lib.fake_factor(0, 0)
         assert lib.fake_nulls() == 0, nth
-        if rc != OOM:
+        if rc not in FAILED:
             break
     assert failures >= 7  # mem, tmp, pinv, chk, berr, info and the job list of one slot at least
+
+
+def test_a_failed_allocation_of_a_4d_batch_is_made_up_for(lib):
+    dims = (4, 4, 4, 4)
+    U, v = np.zeros((256, 4, 3, 3), dtype=np.complex128), np.zeros((4, 256, 4, 3), dtype=np.complex128)
+    p = binding.mg_params()
+    lib.mg_default_params(ctypes.byref(p))
+    for i in range(4):
+        p.block[0][i] = 2
+    p.Nv[0], p.n_pass, p.nu_setup, p.chiral_split, p.max_iter, p.coarsest_max_iter = 2, 1, 1, 1, 2, 2
+    nth, rc = 0, FAILED[0]
+    while rc in FAILED:
+        nth += 1
+        ctx = ctypes.c_void_p()
+        assert lib.mg_setup(ctypes.byref(ctx), ctypes.byref(binding.make_geom(dims, 3)), _at(U), ctypes.c_double(0.1),
+                            ctypes.byref(p), None) == 0, lib.mg_last_error()
+        solve = lambda: lib.mg_solve_batch(ctx, 1, _at(v), _at(v[2:]), None, ctypes.c_double(1e-10), None)
+        lib.fake_fail_at(nth)
+        rc = solve()
+        lib.fake_fail_at(0)
+        if rc in FAILED:
+            assert solve() in (0, NOT_CONVERGED), (nth, lib.mg_last_error())
+        lib.mg_destroy(ctx)
+        assert lib.fake_nulls() == 0, nth
+    assert nth > 20
+
+
+def test_a_failed_growth_of_the_network_buffers_is_made_up_for(lib):
+    dims, block = (8, 8), (ctypes.c_int * 2)(4, 4)
+    U, tgt = np.zeros((2, 64, 2), dtype=np.complex128), np.zeros((2, 2, 64, 2), dtype=np.complex128)
+    nth, rc = 0, FAILED[0]
+    while rc in FAILED:
+        nth += 1
+        net = ctypes.c_void_p()
+        assert lib.mg_nullnet_create(ctypes.byref(net), 2, 2, 2, ctypes.c_uint64(1)) == 0
+
+        def gradient(fields):
+            seeds = (ctypes.c_uint64 * fields)(*range(fields))
+            loss = ctypes.c_double()
+            return lib.mg_nullnet_gradient(net, ctypes.byref(binding.make_geom(dims)), fields, _at(U), seeds, _at(tgt),
+                                           block, ctypes.byref(loss), None, None)
+        assert gradient(1) == 0
+        lib.fake_fail_at(nth)
+        rc = gradient(2)
+        lib.fake_fail_at(0)
+        if rc in FAILED:
+            assert gradient(1) == 0, (nth, lib.mg_last_error())
+        lib.mg_nullnet_destroy(net)
+        assert lib.fake_nulls() == 0, nth
+    assert nth > 10
