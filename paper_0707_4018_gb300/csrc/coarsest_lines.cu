@@ -633,10 +633,10 @@ long long line_work_size(Geo2 g, int N) {
 
 bool line_factor(LineSolver &f, const Cx<double> *Y, Geo2 g, int N, bool nine, double shift, Cx<double> *work,
                  cudaStream_t s, const char *what) {
-  const bool first = !f.planned, was = f.lines;
+  f.kind = LineSolver::Kind::kNone;
   line_plan(f, g, N, nine, s);
-  f.lines = line_try(f, Y, nine, shift, work, s);
-  if (!f.lines) {
+  const bool lines = line_try(f, Y, nine, shift, work, s);
+  if (!lines) {
     if (f.ipiv.p == nullptr) {  // the later of the two: both are there or both are made
       f.LU.alloc((size_t)f.n * f.n);
       f.ipiv.alloc((size_t)f.n);
@@ -652,11 +652,14 @@ bool line_factor(LineSolver &f, const Cx<double> *Y, Geo2 g, int N, bool nine, d
     MG_CUDA(cudaStreamSynchronize(s));
     if (info != 0) fail(MG_ERR_NAN, std::string(what) + ": zero pivot at column " + std::to_string(info - 1));
   }
-  return !first && was != f.lines;
+  const LineSolver::Kind was = f.last;
+  f.kind = f.last = lines ? LineSolver::Kind::kLines : LineSolver::Kind::kDense;
+  return was != LineSolver::Kind::kNone && was != f.last;
 }
 
 void line_solve(const LineSolver &f, const Cx<double> *b, Cx<double> *x, int nvec, Cx<double> *work, cudaStream_t s) {
-  if (f.lines) {
+  if (f.kind == LineSolver::Kind::kNone) fail(MG_ERR_STATE, "the coarsest level has no factors: factoring it failed");
+  if (f.kind == LineSolver::Kind::kLines) {
     line_reduce_solve(f, b, x, nvec, work, s);
     return;
   }

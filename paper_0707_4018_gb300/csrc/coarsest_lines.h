@@ -30,8 +30,10 @@ struct LineJob {
 struct LineSolver {
   int N = 0, L0 = 0, L1 = 0, n = 0;
   int axis = 1, Q = 0, b = 0;  // line coordinate (1: lines along x0, one per x1), sites per line, dofs per line
-  bool lines = false;          // the factors in use: cyclic reduction, or the dense LU
   bool planned = false;
+  enum class Kind { kNone, kLines, kDense };
+  Kind kind = Kind::kNone;     // the factors in use; none before the first factorisation and after a failed one
+  Kind last = Kind::kNone;     // of the last factorisation that succeeded: what a captured graph may hold
   std::vector<LineLevel> lv;
   std::vector<LineJob> jobs;
   DevBuf<Cx<double>> mem, tmp, pinv, chk;
@@ -46,11 +48,12 @@ struct LineSolver {
 long long line_work_size(Geo2 g, int N);
 // Factors the 5-point stencil Y[j][dir][col][row] + shift (nine = false) or the 9-point stencil
 // Y[j][o][row][col] (nine = true). work: workspace of one right-hand side. Synchronises s.
-// Returns true when the kind of factors changed (a graph captured with the old ones is stale);
-// fails with MG_ERR_NAN ("... zero pivot at column k") on a singular matrix.
+// Returns true when the kind of factors is another than at the last success (a graph captured with those is
+// stale; a failure in between changes nothing about it); fails with MG_ERR_NAN ("... zero pivot at column k") on a singular matrix.
 bool line_factor(LineSolver &f, const Cx<double> *Y, Geo2 g, int N, bool nine, double shift, Cx<double> *work,
                  cudaStream_t s, const char *what);
-// x_v = A^{-1} b_v for nvec vectors of stride n (b and x may be equal); work: nvec workspaces
+// x_v = A^{-1} b_v for nvec vectors of stride n (b and x may be equal); work: nvec workspaces. Fails with
+// MG_ERR_STATE where the last factorisation failed.
 void line_solve(const LineSolver &f, const Cx<double> *b, Cx<double> *x, int nvec, Cx<double> *work, cudaStream_t s);
 
 }  // namespace mg

@@ -666,8 +666,10 @@ static void precondition(mg_ctx &c, const Cx<double> *r, Cx<double> *z) {
 // batched solves: nb systems (D + shift_v) psi_v = chi_v sharing one hierarchy
 // ---------------------------------------------------------------------------
 
-// the captured V-cycles hold the launches of one kind of coarsest solve: dropped when it changes
-static void reset_graphs(mg_ctx &c) {
+// Captured V-cycles hold the fine diagonal d + m as a kernel argument and the launches of one kind of exact
+// coarsest solve: a new mass and another kind of factors need new graphs (every buffer they touch is unchanged, the
+// coarse operators are rebuilt in place).
+static void drop_graphs(mg_ctx &c) {
   for (GraphCache &g : c.pre) g.reset();
   for (auto &v : c.preb)
     for (GraphCache &g : v) g.reset();
@@ -683,7 +685,7 @@ static void prepare_slots(mg_ctx &c, int nb, const double *shift) {
     if (c.use_lu) {
       if (line_factor(c.blu[v], L.Y64.p, L.geo, L.nint, false, shift[v], c.lu_work.p, c.s,
                       "coarsest LU (batched mass)"))
-        reset_graphs(c);
+        drop_graphs(c);
     } else {
       prepare_coarsest_gcr(L.Y64.p, L.geo, L.nint, c.bMinv.p + v * m2, c.cg_batch ? nullptr : c.bYt.p + v * 5 * m2,
                            c.cg_work.p, c.cg_info.p, c.s, shift[v]);
@@ -1165,7 +1167,7 @@ static void prepare_coarsest(mg_ctx &c) {
     if (info != 0) fail(MG_ERR_NAN, "coarsest level: a self block is singular");
     return;
   }
-  if (line_factor(c.lu, L.Y64.p, L.geo, L.nint, false, 0.0, c.lu_work.p, c.s, "coarsest LU")) reset_graphs(c);
+  if (line_factor(c.lu, L.Y64.p, L.geo, L.nint, false, 0.0, c.lu_work.p, c.s, "coarsest LU")) drop_graphs(c);
 }
 
 // block Gram-Schmidt of the level's vectors and the Galerkin operator of l+1
@@ -1895,16 +1897,6 @@ int mg_solve_batch(mg_ctx *c, int nrhs, const void *chi, void *psi, const double
     return status;
   }
   return rc;
-}
-
-// Captured V-cycles hold the fine diagonal d + m as a kernel argument: a new mass
-// needs new graphs (every buffer they touch is unchanged, the coarse operators are
-// rebuilt in place).
-static void drop_graphs(mg_ctx &c) {
-  for (auto &g : c.pre) g.reset();
-  for (auto &g : c.setup_vc) g.reset();
-  for (auto &v : c.preb)
-    for (auto &g : v) g.reset();
 }
 
 int mg_update_mass(mg_ctx *c, double m) {

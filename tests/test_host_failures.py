@@ -1,4 +1,5 @@
-"""Failures on the host side: allocations that fail in the middle of a plan or of the buffers that a first call makes. The library's objects run against a CUDA runtime
+"""Failures on the host side: allocations that fail in the middle of a plan or of the buffers that a first call makes,
+factorisations that fail, and captured V-cycles when the kind of factors changes. The library's objects run against a CUDA runtime
 whose memory is host memory and whose launches do nothing (fake_cudart.cpp), so no device is involved."""
 import ctypes
 import glob
@@ -12,7 +13,7 @@ from paper_0707_4018_gb300 import binding, build
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 FAILED = (2, 3)  # pinned host memory, device memory
-NOT_CONVERGED = 4
+NOT_CONVERGED, NAN, STATE = 4, 5, 7
 DIMS = (16, 12)
 
 
@@ -53,6 +54,12 @@ class Ctx:
         m = (ctypes.c_double * len(masses))(*masses)
         return self.lib.mg_solve_batch(self.p, len(masses), _at(self.v), _at(self.v[2:]), m,
                                        ctypes.c_double(1e-10), None)
+
+    def vcycle(self):
+        return self.lib.mg_vcycle(self.p, _at(self.v), _at(self.v[2:]))
+
+    def update_mass(self, m):
+        return self.lib.mg_update_mass(self.p, ctypes.c_double(m))
 
     def close(self):
         self.lib.mg_destroy(self.p)
@@ -136,3 +143,30 @@ def test_a_failed_growth_of_the_network_buffers_is_made_up_for(lib):
         lib.mg_nullnet_destroy(net)
         assert lib.fake_nulls() == 0, nth
     assert nth > 10
+
+
+def test_a_failed_mass_update_does_not_leave_missing_factors_in_use(lib):
+    ctx = Ctx(lib, 1)
+    assert ctx.vcycle() == 0
+    lib.fake_factor(1, 0)
+    lib.fake_fail_at(1)  # the dense factors
+    assert ctx.update_mass(0.2) in FAILED
+    assert ctx.vcycle() == STATE
+    assert ctx.update_mass(0.2) == 0 and ctx.vcycle() == 0
+    lib.fake_factor(0, 0)
+    assert ctx.update_mass(0.3) == 0 and ctx.vcycle() == 0
+    assert lib.fake_nulls() == 0
+    ctx.close()
+
+
+def test_a_failed_factorisation_drops_captured_cycles_of_the_other_kind(lib):
+    ctx = Ctx(lib, 2)
+    assert ctx.batch(0.2, 0.3) == NOT_CONVERGED
+    captured = lib.fake_graphs()
+    assert ctx.batch(0.2, 0.3) == NOT_CONVERGED and lib.fake_graphs() == captured  # replayed
+    lib.fake_factor(1, 1)
+    assert ctx.batch(0.4, 0.3) == NAN
+    lib.fake_factor(1, 0)
+    assert ctx.batch(0.4, 0.3) == NOT_CONVERGED
+    assert lib.fake_graphs() > captured  # the captured cycle held the reduction's launches
+    ctx.close()
