@@ -682,6 +682,7 @@ static void prepare_slots(mg_ctx &c, int nb, const double *shift) {
   const long long m2 = L.geo.nsites * (long long)L.nint * L.nint;
   for (int v = 0; v < nb; ++v) {
     if (c.slot_shift[v] == shift[v]) continue;
+    c.slot_shift[v] = std::nan("");  // what is there is overwritten, also by a preparation that fails
     if (c.use_lu) {
       if (line_factor(c.blu[v], L.Y64.p, L.geo, L.nint, false, shift[v], c.lu_work.p, c.s,
                       "coarsest LU (batched mass)"))

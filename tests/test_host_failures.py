@@ -170,3 +170,15 @@ def test_a_failed_factorisation_drops_captured_cycles_of_the_other_kind(lib):
     assert ctx.batch(0.4, 0.3) == NOT_CONVERGED
     assert lib.fake_graphs() > captured  # the captured cycle held the reduction's launches
     ctx.close()
+
+
+def test_a_failed_factorisation_is_not_taken_for_the_one_before(lib):
+    ctx = Ctx(lib, 2)
+    assert ctx.batch(0.2, 0.3) == NOT_CONVERGED
+    lib.fake_factor(1, 1)
+    assert ctx.batch(0.4, 0.3) == NAN
+    lib.fake_factor(0, 0)
+    checks = lib.fake_checks()
+    assert ctx.batch(0.2, 0.3) == NOT_CONVERGED
+    assert lib.fake_checks() == checks + 1  # the first slot's factors were overwritten, the second's were not
+    ctx.close()
