@@ -83,8 +83,10 @@ void launch_coarse_apply_tc(const uint2 *Ypk, const Cx<float> *in, Cx<float> *ou
 // ---- half-precision storage with per-site norms (wilson_half.cu) ----
 void launch_dslash_half(const void *U, const void *in, void *out, Geo2 g, double diag, cudaStream_t s);
 // fine level of FP32 V-cycles with half storage (MG_FP16 contexts; wilson_half.cu): the fused MR
-// iteration and its last step on half r / A r fields (12 V bytes per field of a batch), the
-// residual apply on FP32 vectors with half links
+// iteration and its last step on half r / A r fields, the residual apply on FP32 vectors with half links
+// bytes from one field of a batch to the next: 12 per site, and a whole number of 8-byte words (a site's two spin
+// components are read as one), which an odd volume by itself is not
+__host__ __device__ constexpr long long half_field_bytes(long long V) { return (12 * V + 7) / 8 * 8; }
 void launch_mr_iteration_half(const void *U16, Geo2 g, double diag, const double *shift, bool step,
                               const Cx<float> *b, void *r_old, void *Ar_old, const float *part_in, double omega,
                               Cx<float> *x, bool x_init, void *r_new, void *Ar_new, float *part_out,

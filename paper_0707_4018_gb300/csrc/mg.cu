@@ -116,7 +116,7 @@ struct mg_ctx {
   // A r in half with per-site norms (12 V bytes per field); half_now while such a cycle is built
   bool half_fine = false, half_now = false;
   mg::DevBuf<float> U16;             // 2 V floats: V x (U^0, U^1) half2 pairs
-  mg::DevBuf<float> hr[2], hA[2];    // 3 V floats per field, max_rhs fields
+  mg::DevBuf<float> hr[2], hA[2];    // max_rhs fields of half_field_bytes
   // coarsest
   bool use_lu = false;
   int nc = 0;
@@ -1422,8 +1422,8 @@ static std::unique_ptr<mg_ctx> create(const mg_geom *g, double m, const mg_param
   if (c->half_fine) {
     c->U16.alloc(F.geo.nsites * 2);
     for (int i = 0; i < 2; ++i) {
-      c->hr[i].alloc(F.geo.nsites * 3 * (size_t)p->max_rhs);
-      c->hA[i].alloc(F.geo.nsites * 3 * (size_t)p->max_rhs);
+      c->hr[i].alloc(half_field_bytes(F.geo.nsites) / sizeof(float) * p->max_rhs);
+      c->hA[i].alloc(half_field_bytes(F.geo.nsites) / sizeof(float) * p->max_rhs);
     }
   }
   // coarsest

@@ -14,7 +14,8 @@
 // The same storage serves the fine level of FP32 V-cycles in MG_FP16 contexts: the MR
 // smoother's vectors r and A r (read at five sites per iteration) and the links are half,
 // the smoother's iterate x, the cycle's input and the residual handed to the restriction stay
-// FP32, every sum is FP32. A batch of half fields is stored field after field, 12 V bytes each.
+// FP32, every sum is FP32. A batch of half fields is stored field after field
+// (half_field_bytes).
 #include <cuda_fp16.h>
 
 #include "kernels.h"
@@ -237,9 +238,9 @@ struct HalfField {
   float *n;
 };
 
-// field v of a batch at base (12 V bytes per field: V half2 pairs, then V norms)
+// field v of a batch at base: V half2 pairs, then V norms
 __device__ __forceinline__ HalfField half_field(void *base, long long V, int v) {
-  char *p = static_cast<char *>(base) + (long long)v * 12 * V;
+  char *p = static_cast<char *>(base) + v * half_field_bytes(V);
   return {reinterpret_cast<__half2 *>(p), reinterpret_cast<float *>(p + 8 * V)};
 }
 
