@@ -79,15 +79,28 @@ __global__ void mr_update_kernel(const double *__restrict__ sc, double omega, Cx
   }
 }
 
-// This thread's part of <a, b> (SAME: |a|^2, real): the FP64 rate bounds these reductions (two multiply-adds
-// per clock and SM), so exactly four of them per complex product, two for a norm; as sums of products
-// they were six DP instructions for every row. Four elements are in flight per thread.
+// This thread's part of <a, b> (SAME: |a|^2, real), summed in FP64: the FP64 rate bounds these reductions (two
+// multiply-adds per clock and SM), so exactly four of them per complex product of FP64 vectors, two for a norm; as
+// sums of products they were six DP instructions for every row. FP32 vectors: an element's two products of a part are
+// added in FP32, everything else in FP64. Four elements are in flight per thread.
 template <typename VT>
 __device__ __forceinline__ void dot_part(const Cx<VT> *__restrict__ a, const Cx<VT> *__restrict__ b, bool same,
-                                         long long n, VT &t0, VT &t1) {
+                                         long long n, double &t0, double &t1) {
   const long long step = (long long)gridDim.x * blockDim.x;
   long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (same) {
+  if constexpr (sizeof(VT) == 4) {
+    if (same) {
+#pragma unroll 4
+      for (; i < n; i += step) t0 += (double)norm2(a[i]);
+    } else {
+#pragma unroll 4
+      for (; i < n; i += step) {
+        const Cx<VT> x = a[i], y = b[i];
+        t0 += (double)(x.re * y.re + x.im * y.im);
+        t1 += (double)(x.re * y.im - x.im * y.re);
+      }
+    }
+  } else if (same) {
 #pragma unroll 4
     for (; i < n; i += step) {
       const Cx<VT> x = a[i];
@@ -112,8 +125,6 @@ __device__ __forceinline__ void dot_part(const Cx<VT> *__restrict__ a, const Cx<
 static int dot_blocks(long long n, int per) { return reduce_blocks((n + 7) / 8, per); }
 
 // rows j < k: <W_j, w>; row k: <w, w>; row k + 1: <w, r>; row k + 2: <r, r>  (blockIdx.y = row)
-// (VT = float: FP32 vectors; each thread sums its few products in FP32, the block and grid
-// trees sum in FP64)
 // (kdev: k read from device memory, for loops replayed by a graph; the grid then has rows
 // for the longest basis, and the rows above k + 2 return at once, all blocks of a row alike)
 template <typename VT>
@@ -128,9 +139,8 @@ __global__ void __launch_bounds__(kReduceThreads) gcr_dots_kernel(const Cx<VT> *
   if (row > k + 2) return;
   const Cx<VT> *a = row < k ? W + (long long)row * n : (row == k + 2 ? r : w);
   const Cx<VT> *b = row > k ? r : w;
-  VT t0 = (VT)0, t1 = (VT)0;
-  dot_part<VT>(a, b, row == k || row == k + 2, n, t0, t1);
-  double v[2] = {(double)t0, (double)t1};
+  double v[2] = {0.0, 0.0};
+  dot_part<VT>(a, b, row == k || row == k + 2, n, v[0], v[1]);
   grid_finish<2>(v, partials + (long long)row * pstride, out + 2 * row, ticket + row, sh);
 }
 
@@ -263,7 +273,6 @@ __global__ void __launch_bounds__(kReduceThreads) norm2_batch_kernel(const Cx<VT
 
 // vector v = blockIdx.z, row = blockIdx.y: rows j < k <W_j, w>, row k |w|^2, row k + 1 <w, r>,
 // row k + 2 |r|^2; results at out[v * 2 (k + 3) + 2 row]
-// (VT = float: FP32 vectors, each thread's products summed in FP32, the trees in FP64)
 template <typename VT>
 __global__ void __launch_bounds__(kReduceThreads) gcr_dots_batch_kernel(const Cx<VT> *__restrict__ W,
                                                                         const Cx<VT> *__restrict__ r, int k,
@@ -275,9 +284,8 @@ __global__ void __launch_bounds__(kReduceThreads) gcr_dots_batch_kernel(const Cx
   const Cx<VT> *rv = r + (long long)v * n;
   const Cx<VT> *a = row < k ? W + ((long long)row * nb + v) * n : (row == k + 2 ? rv : w);
   const Cx<VT> *b = row > k ? rv : w;
-  VT t0 = (VT)0, t1 = (VT)0;
-  dot_part<VT>(a, b, row == k || row == k + 2, n, t0, t1);
-  double acc[2] = {(double)t0, (double)t1};
+  double acc[2] = {0.0, 0.0};
+  dot_part<VT>(a, b, row == k || row == k + 2, n, acc[0], acc[1]);
   const long long slot = (long long)v * rows + row;
   grid_finish<2>(acc, partials + slot * 2 * gridDim.x, out + 2 * slot, ticket + slot, sh);
 }
@@ -623,9 +631,8 @@ __global__ void __launch_bounds__(kReduceThreads) gcr_dots_batch_devk_kernel(
   const Cx<VT> *rv = r + (long long)v * n;
   const Cx<VT> *a = row < k ? W + ((long long)row * nb + v) * n : (row == k + 2 ? rv : wv);
   const Cx<VT> *b = row > k ? rv : wv;
-  VT t0 = (VT)0, t1 = (VT)0;
-  dot_part<VT>(a, b, row == k || row == k + 2, n, t0, t1);
-  double acc[2] = {(double)t0, (double)t1};
+  double acc[2] = {0.0, 0.0};
+  dot_part<VT>(a, b, row == k || row == k + 2, n, acc[0], acc[1]);
   const long long slot = (long long)v * rows + row;
   grid_finish<2>(acc, partials + slot * 2 * gridDim.x, out + 2 * slot, ticket + slot, sh);
 }

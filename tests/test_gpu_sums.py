@@ -1,0 +1,68 @@
+"""Where FP32 values are summed, and in what: the Krylov reductions of FP32 vectors (FP64). The inputs are integers whose products are exact in FP32 and among which one is large, so that an addition in FP32 next to
+it loses the small ones. The launchers are the library's internal C++ functions."""
+import ctypes
+
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+BIG = 2.0 ** 24  # FP32 counts in steps of two from here on
+
+
+class ReduceWs(ctypes.Structure):
+    _fields_ = [("partials", ctypes.c_void_p), ("ticket", ctypes.c_void_p), ("max_blocks", ctypes.c_int),
+                ("capacity", ctypes.c_longlong), ("tickets", ctypes.c_longlong)]
+
+
+class Geo4(ctypes.Structure):
+    _fields_ = [("L", ctypes.c_int * 4), ("nsites", ctypes.c_longlong)]
+
+
+class BlockGeo(ctypes.Structure):
+    _fields_ = [(n, ctypes.c_int) for n in ("L0", "L1", "B0", "B1", "nb0", "nb1", "bvol", "nint", "Nb")] + [
+        ("nblocks", ctypes.c_longlong)]
+
+
+def _fn(name):
+    import paper_0707_4018_gb300 as mg
+    f = getattr(mg.load(), name)
+    f.restype = None
+    return f
+
+
+def _p(t):
+    return ctypes.c_void_p(t.data_ptr() if t is not None else 0)
+
+
+def _stream():
+    import torch
+    return ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
+
+
+@pytest.mark.parametrize("n", [1, 7, 1000, 16385, 24576, 70000])
+@pytest.mark.parametrize("batch", [False, True])
+def test_krylov_reductions_of_fp32_vectors_sum_in_fp64(n, batch):
+    import torch
+    k = 2
+    rng = np.random.default_rng(n)
+    W, r = rng.integers(-3, 4, (k + 1, n, 2)).astype(np.float32), rng.integers(-3, 4, (n, 2)).astype(np.float32)
+    for v in (*W, r):  # an element's products are small whole numbers, in every fifth one times 2^20
+        v[::5] *= 2.0 ** 10
+    Wc, rc = W[..., 0] + 1j * W[..., 1].astype(np.complex128), r[..., 0] + 1j * r[..., 1].astype(np.complex128)
+    want = np.array([*(np.vdot(Wc[j], Wc[k]) for j in range(k)), np.vdot(Wc[k], Wc[k]), np.vdot(Wc[k], rc),
+                     np.vdot(rc, rc)])
+    dW, dr = torch.from_numpy(W).cuda(), torch.from_numpy(r).cuda()
+    out = torch.zeros(2 * (k + 3), dtype=torch.float64, device="cuda")
+    part = torch.zeros(1 << 16, dtype=torch.float64, device="cuda")
+    tick = torch.zeros(64, dtype=torch.int32, device="cuda")
+    ws = ReduceWs(part.data_ptr(), tick.data_ptr(), 64, part.numel(), 64)
+    if batch:
+        _fn("_ZN2mg21launch_gcr_dots_batchIfEEvPKNS_2CxIT_EES5_iixPdRKNS_8ReduceWsEP11CUstream_st")(
+            _p(dW), _p(dr), k, 1, ctypes.c_longlong(n), _p(out), ctypes.byref(ws), _stream())
+    else:
+        _fn("_ZN2mg15launch_gcr_dotsEPKNS_2CxIfEES3_S3_ixPdRKNS_8ReduceWsEP11CUstream_st")(
+            _p(dW), _p(dW[k]), _p(dr), k, ctypes.c_longlong(n), _p(out), ctypes.byref(ws), _stream())
+    got = out.cpu().numpy()
+    # the two products of an element have few digits, the sums are whole numbers below 2^53: nothing rounds
+    assert np.array_equal(got[0::2], want.real) and np.array_equal(got[1::2], want.imag)
