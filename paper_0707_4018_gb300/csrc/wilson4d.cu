@@ -445,8 +445,8 @@ __device__ __forceinline__ void row_hops(const Cx<float> (&p)[12], const Cx<floa
 }  // namespace
 
 // SUMS: also the step length of an MR iteration on each vector, omega <out, in> / |out|^2, from the
-// values the kernel holds anyway: per-thread and per-block sums in FP32, FP64 partials, final sum and
-// quotient, into mr.alpha[v]
+// values the kernel holds anyway: FP32 sums over a site and the 64 sites of a tile, FP64 over the CTA's tiles, the
+// partials, the final sum and the quotient, into mr.alpha[v]
 struct MrStep {
   double *partials;       // [vector][CTA][3]
   unsigned int *tickets;  // [vector], zero
@@ -526,7 +526,7 @@ __global__ void __launch_bounds__(32 * kTiles, 2)
   in += v0 * ldv;
   out += v0 * ldv;
   if (b != nullptr) b += v0 * ldv;
-  __shared__ float sh[SUMS ? kMaxChunk : 1][kTiles][3];
+  __shared__ float sh[SUMS ? kMaxChunk : 1][kTiles][3];  // a tile's sums
   for (int v = v0; v < v1; ++v) {
     const float dg = SHIFT ? diag + (float)shift[v] : diag;
     float sums[3] = {0.f, 0.f, 0.f};
@@ -583,16 +583,21 @@ __global__ void __launch_bounds__(32 * kTiles, 2)
         Cx<float>(&p)[12] = half ? pB : pA;
         Cx<float>(&acc)[12] = half ? aB : aA;
         const int x = half ? xB : xA;
+        float site[3] = {0.f, 0.f, 0.f};
 #pragma unroll
         for (int i = 0; i < 12; ++i) {
           const Cx<float> o =
               mk(a * (dg * p[i].re - 0.5f * acc[i].re), a * (dg * p[i].im - 0.5f * acc[i].im));
           if (SUMS) {
-            sums[0] += o.re * p[i].re + o.im * p[i].im;
-            sums[1] += o.re * p[i].im - o.im * p[i].re;
-            sums[2] += o.re * o.re + o.im * o.im;
+            site[0] += o.re * p[i].re + o.im * p[i].im;
+            site[1] += o.re * p[i].im - o.im * p[i].re;
+            site[2] += o.re * o.re + o.im * o.im;
           }
           p[i] = o;
+        }
+        if (SUMS) {
+#pragma unroll
+          for (int k = 0; k < 3; ++k) sums[k] += site[k];
         }
         if (b != nullptr) {
           Cx<float> q[12];
@@ -625,10 +630,10 @@ __global__ void __launch_bounds__(32 * kTiles, 2)
       double *part = mr.partials + (long long)v * gridDim.x * 3;
 #pragma unroll
       for (int k = 0; k < 3; ++k) {
-        float t = 0.f;
+        double t = 0.0;
 #pragma unroll
-        for (int q = 0; q < kTiles; ++q) t += sh[j][q][k];
-        part[blockIdx.x * 3 + k] = (double)t;
+        for (int q = 0; q < kTiles; ++q) t += (double)sh[j][q][k];
+        part[blockIdx.x * 3 + k] = t;
       }
       __threadfence();
       last[j] = atomicAdd(mr.tickets + v, 1u) == gridDim.x - 1;

@@ -1,4 +1,5 @@
-"""Where FP32 values are summed, and in what: the Krylov reductions of FP32 vectors (FP64). The inputs are integers whose products are exact in FP32 and among which one is large, so that an addition in FP32 next to
+"""Where FP32 values are summed, and in what: the Krylov reductions of FP32 vectors (FP64) and the MR sums of the
+tiled 4d apply (FP32 inside a tile of 64 sites, FP64 across). The inputs are integers whose products are exact in FP32 and among which one is large, so that an addition in FP32 next to
 it loses the small ones. The launchers are the library's internal C++ functions."""
 import ctypes
 
@@ -66,3 +67,24 @@ def test_krylov_reductions_of_fp32_vectors_sum_in_fp64(n, batch):
     got = out.cpu().numpy()
     # the two products of an element have few digits, the sums are whole numbers below 2^53: nothing rounds
     assert np.array_equal(got[0::2], want.real) and np.array_equal(got[1::2], want.imag)
+
+
+@pytest.mark.parametrize("dims", [(8, 4, 4, 2), (8, 2, 2, 6)])  # four tiles of a CTA, and three
+def test_mr_sums_of_the_tiled_4d_apply_are_fp64_across_tiles(dims):
+    import torch
+    V = int(np.prod(dims))
+    U = torch.zeros((V, 4, 3, 3), dtype=torch.complex64, device="cuda")  # D r = diag r
+    r = torch.zeros((V, 12), dtype=torch.complex64, device="cuda")
+    r[0, 0] = 2.0 ** 12  # tile 0 sums to 2^24
+    r[V - 1, 5] = 1.0    # the last tile to 1
+    Ar = torch.empty_like(r)
+    alpha = torch.zeros(2, dtype=torch.float32, device="cuda")
+    part = torch.zeros(3 * (V // 64), dtype=torch.float64, device="cuda")
+    tick = torch.zeros(1, dtype=torch.int32, device="cuda")
+    f = _fn("_ZN2mg17launch_dslash4_mrEPKNS_2CxIfEES3_PS1_NS_4Geo4EdidP6float2PdxPjP11CUstream_st")
+    f.restype = ctypes.c_bool
+    assert f(_p(U), _p(r), _p(Ar), Geo4((ctypes.c_int * 4)(*dims), V), ctypes.c_double(1.0), 1, ctypes.c_double(0.5),
+             _p(alpha), _p(part), ctypes.c_longlong(part.numel()), _p(tick), _stream())
+    got = part.cpu().numpy()[:3]
+    assert np.array_equal(got, [BIG + 1, 0.0, BIG + 1])
+    assert alpha.cpu().numpy().tolist() == [0.5, 0.0]
