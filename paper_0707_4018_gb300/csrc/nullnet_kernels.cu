@@ -416,6 +416,31 @@ struct LossSmem {
   float2 A[kLossBlocks][kMaxNv * kMaxNv];
 };
 
+// A lane's four sums over 2^LEVEL rows, from `first` on and 32 / 2^LEVEL apart (LEVEL 5: all rows), as a tree of
+// additions: five roundings on the way of a product, where a chain over the rows has up to 32.
+template <int LEVEL>
+__device__ __forceinline__ void loss_sums(const LossSmem &sm, int first, int rows, int k, int j, float2 &g0, float2 &g1,
+                                          float2 &c0, float2 &c1) {
+  if constexpr (LEVEL == 0) {
+    g0 = g1 = c0 = c1 = make_float2(0.f, 0.f);
+    if (first < rows) {
+      const float2 a = sm.w[first][k], e = sm.w[first][k + 4], wj = sm.w[first][j], vj = sm.v[first][j];
+      cmacf_conj(g0, a, wj);
+      cmacf_conj(g1, e, wj);
+      cmacf_conj(c0, a, vj);
+      cmacf_conj(c1, e, vj);
+    }
+  } else {
+    float2 h0, h1, d0, d1;
+    loss_sums<LEVEL - 1>(sm, first, rows, k, j, g0, g1, c0, c1);
+    loss_sums<LEVEL - 1>(sm, first + (32 >> LEVEL), rows, k, j, h0, h1, d0, d1);
+    g0 = make_float2(g0.x + h0.x, g0.y + h0.y);
+    g1 = make_float2(g1.x + h1.x, g1.y + h1.y);
+    c0 = make_float2(c0.x + d0.x, c0.y + d0.y);
+    c1 = make_float2(c1.x + d1.x, c1.y + d1.y);
+  }
+}
+
 __global__ void __launch_bounds__(32 * kLossWarps) nullnet_loss_kernel(const float2 *__restrict__ y,
                                                                        const float2 *__restrict__ target,
                                                                        const int *__restrict__ fmap, int nv,
@@ -446,15 +471,8 @@ __global__ void __launch_bounds__(32 * kLossWarps) nullnet_loss_kernel(const flo
     }
     __syncwarp();
     const int k0 = lane >> 3, j = lane & 7;
-    float2 g0 = zero, g1 = zero, c0 = zero, c1 = zero;
-#pragma unroll 4
-    for (int r = 0; r < rows; ++r) {
-      const float2 a = sm.w[r][k0], e = sm.w[r][k0 + 4], wj = sm.w[r][j], vj = sm.v[r][j];
-      cmacf_conj(g0, a, wj);
-      cmacf_conj(g1, e, wj);
-      cmacf_conj(c0, a, vj);
-      cmacf_conj(c1, e, vj);
-    }
+    float2 g0, g1, c0, c1;
+    loss_sums<5>(sm, 0, rows, k0, j, g0, g1, c0, c1);
     // unused vectors: an identity block, so that the factorisation runs over all eight rows
     const bool in0 = k0 < nv && j < nv, in1 = k0 + 4 < nv && j < nv;
     sm.G[b][lane] = in0 ? make_double2(g0.x, g0.y) : make_double2(k0 == j ? 1.0 : 0.0, 0.0);

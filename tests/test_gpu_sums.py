@@ -1,5 +1,6 @@
-"""Where FP32 values are summed, and in what: the Krylov reductions of FP32 vectors (FP64) and the MR sums of the
-tiled 4d apply (FP32 inside a tile of 64 sites, FP64 across). The inputs are integers whose products are exact in FP32 and among which one is large, so that an addition in FP32 next to
+"""Where FP32 values are summed, and in what: the Krylov reductions of FP32 vectors (FP64), the MR sums of the tiled 4d
+apply (FP32 inside a tile of 64 sites, FP64 across) and the block loss's products (FP32, as a tree over the rows). The
+inputs are integers whose products are exact in FP32 and among which one is large, so that an addition in FP32 next to
 it loses the small ones. The launchers are the library's internal C++ functions."""
 import ctypes
 
@@ -88,3 +89,22 @@ def test_mr_sums_of_the_tiled_4d_apply_are_fp64_across_tiles(dims):
     got = part.cpu().numpy()[:3]
     assert np.array_equal(got, [BIG + 1, 0.0, BIG + 1])
     assert alpha.cpu().numpy().tolist() == [0.5, 0.0]
+
+
+@pytest.mark.parametrize("rows", [2, 8, 18, 32])
+def test_block_loss_products_are_summed_as_a_tree(rows):
+    import torch
+    B0, B1 = {2: (1, 1), 8: (2, 2), 18: (3, 3), 32: (4, 4)}[rows]
+    y = torch.ones((B0 * B1, 2, 1, 2), dtype=torch.float32, device="cuda")  # [x][2 nv] float2, one vector
+    y[..., 1] = 0.0
+    y.view(-1, 2)[0, 0] = 2.0 ** 12
+    tgt = torch.zeros((1, B0 * B1, 2, 2), dtype=torch.float32, device="cuda")
+    tgt.view(-1, 2)[0, 0] = 1.0
+    gy, loss = torch.zeros_like(y), torch.zeros(1, dtype=torch.float64, device="cuda")
+    bg = BlockGeo(B0, B1, B0, B1, 1, 1, B0 * B1, 2, 2 * B0 * B1, 1)
+    _fn("_ZN2mg19launch_nullnet_lossEPK6float2S2_PKiiRKNS_8BlockGeoEifPS0_PdP11CUstream_st")(
+        _p(y), _p(tgt), _p(None), 1, ctypes.byref(bg), 1, ctypes.c_float(1.0), _p(gy), _p(loss), _stream())
+    # loss = 1 - |c|^2 / (g (1 + 1e-7)), c = 2^12 and g = 2^24 + rows - 1
+    g = BIG / ((1.0 - float(loss.cpu()[0])) * (1.0 + 1e-7))
+    # five additions of half a step (one above 2^24) and FP64 rounding; summed in a chain g stays at 2^24
+    assert abs(g - (BIG + rows - 1)) <= 5.0 + 1e-6
