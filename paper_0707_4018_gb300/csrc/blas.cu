@@ -79,27 +79,30 @@ __global__ void mr_update_kernel(const double *__restrict__ sc, double omega, Cx
   }
 }
 
-// This thread's part of <a, b> (SAME: |a|^2, real), summed in FP64: the FP64 rate bounds these reductions (two
-// multiply-adds per clock and SM), so exactly four of them per complex product of FP64 vectors, two for a norm; as
-// sums of products they were six DP instructions for every row. FP32 vectors: an element's two products of a part are
-// added in FP32, everything else in FP64. Four elements are in flight per thread.
+// This thread's part of <a, b> (same: |a|^2, real). FP64 vectors: the FP64 rate bounds these reductions (two
+// multiply-adds per clock and SM), so exactly four of them per complex product, two for a norm; as sums of products
+// they were six DP instructions for every row. FP32 vectors: a thread's elements, few (dot_blocks), are summed in
+// FP32. Four elements are in flight per thread.
 template <typename VT>
 __device__ __forceinline__ void dot_part(const Cx<VT> *__restrict__ a, const Cx<VT> *__restrict__ b, bool same,
                                          long long n, double &t0, double &t1) {
   const long long step = (long long)gridDim.x * blockDim.x;
   long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   if constexpr (sizeof(VT) == 4) {
+    VT u0 = (VT)0, u1 = (VT)0;
     if (same) {
 #pragma unroll 4
-      for (; i < n; i += step) t0 += (double)norm2(a[i]);
+      for (; i < n; i += step) u0 += norm2(a[i]);
     } else {
 #pragma unroll 4
       for (; i < n; i += step) {
         const Cx<VT> x = a[i], y = b[i];
-        t0 += (double)(x.re * y.re + x.im * y.im);
-        t1 += (double)(x.re * y.im - x.im * y.re);
+        u0 += x.re * y.re + x.im * y.im;
+        u1 += x.re * y.im - x.im * y.re;
       }
     }
+    t0 = (double)u0;
+    t1 = (double)u1;
   } else if (same) {
 #pragma unroll 4
     for (; i < n; i += step) {
@@ -119,10 +122,16 @@ __device__ __forceinline__ void dot_part(const Cx<VT> *__restrict__ a, const Cx<
   }
 }
 
-// Blocks per reduction: at least eight elements per thread, so that the block and grid trees (FP64
+// Blocks per reduction. FP64 vectors: at least eight elements per thread, so that the block and grid trees (FP64
 // too) stay small beside the products; one element per thread and 512 blocks per row took 50 us at
-// n = 131072 (256^2), more than its products by a factor of eight.
-static int dot_blocks(long long n, int per) { return reduce_blocks((n + 7) / 8, per); }
+// n = 131072 (256^2), more than its products by a factor of eight. FP32 vectors: as few elements per thread as `per`
+// blocks allow, because FP64 takes over where the thread's own sum ends. Eight of them summed in FP64 per thread
+// instead, two additions and two conversions each, cost the 4d batch (24576 entries, 8 blocks) 515 ms where this
+// takes 502.
+template <typename VT>
+static int dot_blocks(long long n, int per) {
+  return reduce_blocks(sizeof(VT) == 4 ? n : (n + 7) / 8, per);
+}
 
 // rows j < k: <W_j, w>; row k: <w, w>; row k + 1: <w, r>; row k + 2: <r, r>  (blockIdx.y = row)
 // (kdev: k read from device memory, for loops replayed by a graph; the grid then has rows
@@ -187,7 +196,7 @@ static void gcr_dots_any(const Cx<VT> *W, const Cx<VT> *w, const Cx<VT> *r, int 
   int per = (int)(ws.capacity / (2 * rows));
   if (per > ws.max_blocks) per = ws.max_blocks;
   if (per < 1) per = 1;
-  dim3 grid(dot_blocks(n, per), rows);
+  dim3 grid(dot_blocks<VT>(n, per), rows);
   gcr_dots_kernel<VT><<<grid, kReduceThreads, 0, s>>>(W, w, r, k, nullptr, n, ws.partials, out, ws.ticket,
                                                       2 * (int)grid.x);
   MG_LAUNCHED();
@@ -202,7 +211,7 @@ void launch_gcr_dots_kdev(const Cx<VT> *W, const Cx<VT> *w, const Cx<VT> *r, con
   int per = (int)(ws.capacity / (2 * rows));
   if (per > ws.max_blocks) per = ws.max_blocks;
   if (per < 1) per = 1;
-  dim3 grid(dot_blocks(n, per), rows);
+  dim3 grid(dot_blocks<VT>(n, per), rows);
   gcr_dots_kernel<VT><<<grid, kReduceThreads, 0, s>>>(W, w, r, 0, kdev, n, ws.partials, out, ws.ticket,
                                                       2 * (int)grid.x);
   MG_LAUNCHED();
@@ -385,7 +394,7 @@ void launch_gcr_dots_batch(const Cx<VT> *W, const Cx<VT> *r, int k, int nb, long
   int per = (int)(ws.capacity / (2LL * rows * nb));
   if (per > ws.max_blocks) per = ws.max_blocks;
   if (per < 1) fail(MG_ERR_STATE, "gcr_dots_batch: reduction workspace too small");
-  gcr_dots_batch_kernel<VT><<<dim3(dot_blocks(n, per), rows, nb), kReduceThreads, 0, s>>>(W, r, k, nb, n,
+  gcr_dots_batch_kernel<VT><<<dim3(dot_blocks<VT>(n, per), rows, nb), kReduceThreads, 0, s>>>(W, r, k, nb, n,
                                                                                              ws.partials, out,
                                                                                              ws.ticket);
   MG_LAUNCHED();
@@ -444,7 +453,7 @@ void launch_xmy(const Cx<R> *x, Cx<R> *y, long long n, cudaStream_t s) {
 }
 template <typename R>
 void launch_dot_norm(const Cx<R> *a, const Cx<R> *b, long long n, double *out, const ReduceWs &ws, cudaStream_t s) {
-  dot_norm_kernel<R><<<dot_blocks(n, ws.max_blocks), kReduceThreads, 0, s>>>(a, b, n, ws.partials, out, ws.ticket);
+  dot_norm_kernel<R><<<dot_blocks<double>(n, ws.max_blocks), kReduceThreads, 0, s>>>(a, b, n, ws.partials, out, ws.ticket);
   MG_LAUNCHED();
 }
 template <typename R>
@@ -576,7 +585,7 @@ void launch_gcr_dots_devk(const Cx<double> *W, const Cx<double> *w, const Cx<dou
   int per = (int)(ws.capacity / (2 * rows));
   if (per > ws.max_blocks) per = ws.max_blocks;
   if (per < 1) per = 1;
-  dim3 grid(dot_blocks(n, per), rows);
+  dim3 grid(dot_blocks<double>(n, per), rows);
   gcr_dots_devk_kernel<<<grid, kReduceThreads, 0, s>>>(W, w, r, ctl, n, ws.partials, out, ws.ticket, 2 * (int)grid.x);
   MG_LAUNCHED();
 }
@@ -729,7 +738,7 @@ void launch_gcr_dots_batch_devk(const Cx<VT> *W, const Cx<VT> *w, const Cx<VT> *
   if (per > ws.max_blocks) per = ws.max_blocks;
   if (per < 1) per = 1;
   if ((long long)rows * nb > ws.tickets) fail(MG_ERR_UNSUPPORTED, "gcr_dots_batch: too many reduction slots");
-  gcr_dots_batch_devk_kernel<VT><<<dim3(dot_blocks(n, per), rows, nb), kReduceThreads, 0, s>>>(
+  gcr_dots_batch_devk_kernel<VT><<<dim3(dot_blocks<VT>(n, per), rows, nb), kReduceThreads, 0, s>>>(
       W, w, r, ctl, nb, restart, n, ws.partials, out, ws.ticket);
   MG_LAUNCHED();
 }
