@@ -25,7 +25,10 @@
 // Pivots stay inside a 16 x 16 sub-block, which the near-positive Wilson operators do not mind
 // but an arbitrary matrix may: every factorisation is followed by a solve for a fixed vector whose
 // componentwise backward error must stay below kBackward; otherwise (and for rings of fewer than
-// three lines) the dense LU with partial pivoting takes over.
+// three lines) the dense LU with partial pivoting takes over. The bound is what that LU gives itself: on the same
+// vector and the operators of 64^2 and smaller lattices at the couplings' masses the reduction has 3e-16 to 9.5e-16
+// (n = 96 to 2048), the LU 7e-16 to 2.8e-15. Where the operator is indefinite (m = -1, -1.7) the reduction reaches
+// 1.2e-12 and the LU 7.8e-15.
 #include <algorithm>
 #include <cmath>
 #include <string>
@@ -39,7 +42,7 @@ namespace mg {
 namespace {
 
 constexpr int kT = 16;                // tile edge
-constexpr double kBackward = 1e-12;   // largest accepted |b - A x| / (|A| |x| + |b|), entry by entry
+constexpr double kBackward = 2e-15;   // largest accepted |b - A x| / (|A| |x| + |b|), entry by entry
 
 // position of dof i of line p in a level-0 vector (site-major); compact levels: axis 1
 struct LineMap {
