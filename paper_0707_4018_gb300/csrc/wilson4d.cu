@@ -362,7 +362,8 @@ __device__ __forceinline__ void reconstruct4(const Cx<float> (&t)[6], Cx<float> 
 namespace {
 
 // staged links, in 16-byte units: a site's four links (288 B, padded), and one link of a face site
-// as the 80 bytes around it that start on a 16-byte boundary (72 mu rounded down)
+// as the 80 bytes around it that start on a 16-byte boundary. U16: the links start on 16 bytes; else (on an odd 8) a
+// record begins 8 bytes before its site, so that it too is copied in whole units, and fills its padding.
 constexpr int kRec = 19, kHalo = 5;
 constexpr int kHaloX = 0, kHaloY = 8, kHaloZ = 40, kHaloT = 72, kHaloSites = 104;
 constexpr int kTiles = 4;      // tiles of a CTA
@@ -370,18 +371,26 @@ constexpr int kMaxChunk = 32;  // vectors of a CTA
 constexpr int kTileUnits = 64 * kRec + kHaloSites * kHalo;
 constexpr size_t kPairSmem = (size_t)kTiles * kTileUnits * 16;
 
-// first 16-byte unit of link mu in a record; links 1 and 3 start 8 bytes into it
-__host__ __device__ constexpr int link_unit(int mu) { return mu == 0 ? 0 : mu == 1 ? 4 : mu == 2 ? 9 : 13; }
+// first 16-byte unit of link mu in a record; every second link starts 8 bytes into it
+template <bool U16>
+__host__ __device__ constexpr int link_unit(int mu) { return (72 * mu + (U16 ? 0 : 8)) / 16; }
 
-__device__ __forceinline__ void copy16(float4 *dst, const char *src) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned int)__cvta_generic_to_shared(dst)),
-               "l"(src)
-               : "memory");
+// one unit of the links, which lie in [U, end): the units of links on an odd 8 bytes that reach over either end are
+// copied by the half that is inside
+template <bool U16>
+__device__ __forceinline__ void copy16(float4 *dst, const char *src, const char *U, const char *end) {
+  const unsigned int d = (unsigned int)__cvta_generic_to_shared(dst);
+  if (!U16 && src < U)
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(d + 8), "l"(src + 8) : "memory");
+  else if (!U16 && src + 16 > end)
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(d), "l"(src) : "memory");
+  else
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(src) : "memory");
 }
 
-template <int MU>
+template <int MU, bool U16>
 __device__ __forceinline__ void staged_link(const float4 *q, Cx<float> (&u)[9]) {
-  if (MU % 2 == 0) {
+  if ((MU % 2 == 0) == U16) {
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
       const float4 w = q[i];
@@ -412,7 +421,7 @@ __device__ __forceinline__ void rotate6(const Cx<float> (&s)[6], int src, Cx<flo
 // beyond the row that the lane read (first lane: the one after the last, last lane: the one before
 // the first; others none), fsrc / bsrc the lanes holding x + mu and x - mu (cyclic in the row), own /
 // face the staged links of the site and of the site before the first one
-template <int MU>
+template <int MU, bool U16>
 __device__ __forceinline__ void row_hops(const Cx<float> (&p)[12], const Cx<float> (&q)[12], bool first, bool last,
                                          int fsrc, int bsrc, const float4 *own, const float4 *face,
                                          Cx<float> (&acc)[12]) {
@@ -430,13 +439,13 @@ __device__ __forceinline__ void row_hops(const Cx<float> (&p)[12], const Cx<floa
 #pragma unroll
   for (int i = 0; i < 6; ++i) h[i] = mk(first ? e[i].re : h[i].re, first ? e[i].im : h[i].im);
   rotate6(h, fsrc, t);
-  staged_link<MU>(own + link_unit(MU), u);
+  staged_link<MU, U16>(own + link_unit<U16>(MU), u);
   link_times4<false>(u, t, h);
   reconstruct4<MU, true>(h, acc);
   project4<MU, false>(p, h);
 #pragma unroll
   for (int i = 0; i < 6; ++i) h[i] = mk(last ? e[i].re : h[i].re, last ? e[i].im : h[i].im);
-  staged_link<MU>(last ? face : own + link_unit(MU), u);
+  staged_link<MU, U16>(last ? face : own + link_unit<U16>(MU), u);
   link_times4<true>(u, h, t);
   rotate6(t, bsrc, h);
   reconstruct4<MU, false>(h, acc);
@@ -455,7 +464,7 @@ struct MrStep {
 };
 
 // out_v = a (D in_v) + c b_v for the vectors [chunk blockIdx.y, ...) of nvec (stride ldv complex)
-template <bool A32, bool SHIFT, bool SUMS>
+template <bool A32, bool SHIFT, bool SUMS, bool U16>
 __global__ void __launch_bounds__(32 * kTiles, 2)
     dslash4_pair_kernel(const Cx<float> *__restrict__ U, const Cx<float> *__restrict__ in, Cx<float> *__restrict__ out,
                         Geo4 g, float diag, const Cx<float> *__restrict__ b, float a, float c, long long ldv,
@@ -481,21 +490,22 @@ __global__ void __launch_bounds__(32 * kTiles, 2)
   const int p3 = o3 + 2 == g.L[3] ? 0 : o3 + 2, m3 = o3 == 0 ? g.L[3] - 1 : o3 - 1;
   float4 *rec = staged + w * kTileUnits, *halo = rec + 64 * kRec;
   if (live) {
-    const char *Ub = reinterpret_cast<const char *>(U);
+    const char *U0 = reinterpret_cast<const char *>(U), *U1 = U0 + g.nsites * 288, *Ub = U16 ? U0 : U0 - 8;
+    constexpr int n = U16 ? 18 : 19;  // units of a record
     const long long org = o0 + (long long)o1 * s1 + (long long)o2 * s2 + (long long)o3 * s3;
-    // own links: 8 rows of 8 sites, 144 units each
+    // own links: 8 rows of 8 sites
 #pragma unroll 4
-    for (int it = 0; it < 36; ++it) {
-      const int idx = it * 32 + lane, row = idx / 144, k = idx - row * 144, site = k / 18;
+    for (int it = 0; it < 2 * n; ++it) {
+      const int idx = it * 32 + lane, row = idx / (8 * n), k = idx - row * 8 * n, site = k / n;
       const long long x = org + (row & 1) * s1 + ((row >> 1) & 1) * s2 + (row >> 2) * s3;
-      copy16(rec + (row * 8 + site) * kRec + (k - site * 18), Ub + x * 288 + k * 16);
+      copy16<U16>(rec + (row * 8 + site) * kRec + (k - site * n), Ub + x * 288 + k * 16 - (n - 18) * 16 * site, U0, U1);
     }
     // backward faces: 8 sites of the x0 face, 4 rows of 8 sites of each other face
 #pragma unroll
     for (int it = 0; it < 2; ++it) {
       const int idx = it * 32 + lane, e = idx / kHalo, k = idx - e * kHalo;
       const long long x = org - o0 + m0 + (e & 1) * s1 + ((e >> 1) & 1) * s2 + (e >> 2) * s3;
-      if (idx < 8 * kHalo) copy16(halo + idx, Ub + x * 288 + k * 16);
+      if (idx < 8 * kHalo) copy16<U16>(halo + idx, Ub + x * 288 + k * 16, U0, U1);
     }
 #pragma unroll
     for (int mu = 1; mu < 4; ++mu) {
@@ -507,7 +517,7 @@ __global__ void __launch_bounds__(32 * kTiles, 2)
       for (int it = 0; it < 5; ++it) {
         const int idx = it * 32 + lane, row = idx / 40, e = (idx - row * 40) / kHalo, k = idx % kHalo;
         const long long x = face + (row & 1) * sa + (row >> 1) * sb + e;
-        copy16(halo + h0 + idx, Ub + x * 288 + (link_unit(mu) + k) * 16);
+        copy16<U16>(halo + h0 + idx, Ub + x * 288 + (link_unit<U16>(mu) + k) * 16, U0, U1);
       }
     }
   }
@@ -550,29 +560,29 @@ __global__ void __launch_bounds__(32 * kTiles, 2)
         asm volatile("cp.async.wait_all;" ::: "memory");
         __syncwarp();
       }
-      row_hops<0>(pA, qA, l0 == 0, l0 == 7, fX, bX, recA, hX, aA);
-      row_hops<0>(pB, qB, l0 == 0, l0 == 7, fX, bX, recB, hX + 4 * kHalo, aB);
+      row_hops<0, U16>(pA, qA, l0 == 0, l0 == 7, fX, bX, recA, hX, aA);
+      row_hops<0, U16>(pB, qB, l0 == 0, l0 == 7, fX, bX, recB, hX + 4 * kHalo, aB);
       load_spinor32<A32>(in, outZ, qA);
-      row_hops<1>(pA, nA, l1 == 0, l1 == 1, lane ^ 8, lane ^ 8, recA, hY, aA);
+      row_hops<1, U16>(pA, nA, l1 == 0, l1 == 1, lane ^ 8, lane ^ 8, recA, hY, aA);
       load_spinor32<A32>(in, outZ + s3, qB);
-      row_hops<1>(pB, nB, l1 == 0, l1 == 1, lane ^ 8, lane ^ 8, recB, hY + 16 * kHalo, aB);
+      row_hops<1, U16>(pB, nB, l1 == 0, l1 == 1, lane ^ 8, lane ^ 8, recB, hY + 16 * kHalo, aB);
       load_spinor32<A32>(in, xA + (m3 - o3) * s3, nA);
-      row_hops<2>(pA, qA, l2 == 0, l2 == 1, lane ^ 16, lane ^ 16, recA, hZ, aA);
+      row_hops<2, U16>(pA, qA, l2 == 0, l2 == 1, lane ^ 16, lane ^ 16, recA, hZ, aA);
       load_spinor32<A32>(in, xA + (p3 - o3) * s3, nB);
-      row_hops<2>(pB, qB, l2 == 0, l2 == 1, lane ^ 16, lane ^ 16, recB, hZ + 16 * kHalo, aB);
+      row_hops<2, U16>(pB, qB, l2 == 0, l2 == 1, lane ^ 16, lane ^ 16, recB, hZ + 16 * kHalo, aB);
       {  // direction 3: the neighbours inside the tile are the lane's own two sites
         Cx<float> h[6], t[6], t2[6], u[9];
-        staged_link<3>(recA + link_unit(3), u);
+        staged_link<3, U16>(recA + link_unit<U16>(3), u);
         project4<3, true>(pB, h);
         link_times4<false>(u, h, t);
         reconstruct4<3, true>(t, aA);
         project4<3, false>(pA, h);
         link_times4<true>(u, h, t);
-        staged_link<3>(hT, u);
+        staged_link<3, U16>(hT, u);
         project4<3, false>(nA, h);
         link_times4<true>(u, h, t2);
         reconstruct4<3, false>(t2, aA);
-        staged_link<3>(recB + link_unit(3), u);
+        staged_link<3, U16>(recB + link_unit<U16>(3), u);
         project4<3, true>(nB, h);
         link_times4<false>(u, h, t2);
         reconstruct4<3, true>(t2, aB);
@@ -680,10 +690,10 @@ int pair_chunk(const Geo4 &g, int nvec) {
   return best;
 }
 
-template <bool A32, bool SHIFT, bool SUMS>
+template <bool A32, bool SHIFT, bool SUMS, bool U16 = true>
 void launch_pair(const Cx<float> *U, const Cx<float> *in, Cx<float> *out, Geo4 g, double diag, const Cx<float> *b,
                  double a, double c, cudaStream_t s, int nvec, const double *shift, MrStep mr) {
-  auto fn = dslash4_pair_kernel<A32, SHIFT, SUMS>;
+  auto fn = dslash4_pair_kernel<A32, SHIFT, SUMS, U16>;
   MG_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPairSmem));
   const int chunk = pair_chunk(g, nvec);
   fn<<<dim3(pair_ctas(g), (nvec + chunk - 1) / chunk), 32 * kTiles, kPairSmem, s>>>(
@@ -693,10 +703,9 @@ void launch_pair(const Cx<float> *U, const Cx<float> *in, Cx<float> *out, Geo4 g
 
 bool aligned(const void *p, uintptr_t n) { return (reinterpret_cast<uintptr_t>(p) & (n - 1)) == 0; }
 
-// the tiled kernel takes lattices of whole 8 x 2 x 2 x 2 tiles with 16-byte aligned links (its
-// asynchronous copies); other shapes and links at an odd 8-byte offset run the warp gather
-bool pair_takes(const Cx<float> *U, const Geo4 &g) {
-  return g.L[0] % 8 == 0 && g.L[1] % 2 == 0 && g.L[2] % 2 == 0 && g.L[3] % 2 == 0 && aligned(U, 16) &&
+// the tiled kernel takes lattices of whole 8 x 2 x 2 x 2 tiles; other shapes run the warp gather
+bool pair_takes(const Geo4 &g) {
+  return g.L[0] % 8 == 0 && g.L[1] % 2 == 0 && g.L[2] % 2 == 0 && g.L[3] % 2 == 0 &&
          std::getenv("MG_DSLASH4_GATHER") == nullptr;
 }
 
@@ -705,10 +714,15 @@ bool pair_takes(const Cx<float> *U, const Geo4 &g) {
 // true when the tiled kernel took the apply
 static bool try_tile4(const Cx<float> *U, const Cx<float> *in, Cx<float> *out, Geo4 g, double diag,
                       const Cx<float> *b, double a, double c, cudaStream_t s, int nvec, const double *shift) {
-  if (!pair_takes(U, g)) return false;
+  if (!pair_takes(g)) return false;
   const bool a32 = aligned(in, 32) && aligned(out, 32) && aligned(b, 32);
   auto run = [&](auto fn) { fn(U, in, out, g, diag, b, a, c, s, nvec, shift, MrStep{}); };
-  if (a32)
+  // links on an odd 8 bytes come from a caller's own buffer (mg_dslash), never with shifts: their records begin 8
+  // bytes before the site (32^3 x 64: 340 us; 8-byte copies 371, the warp gather 417, the tiled kernel before 355)
+  if (!aligned(U, 16)) {
+    if (shift != nullptr) return false;
+    run(launch_pair<false, false, false, false>);
+  } else if (a32)
     shift != nullptr ? run(launch_pair<true, true, false>) : run(launch_pair<true, false, false>);
   else
     shift != nullptr ? run(launch_pair<false, true, false>) : run(launch_pair<false, false, false>);
@@ -718,7 +732,7 @@ static bool try_tile4(const Cx<float> *U, const Cx<float> *in, Cx<float> *out, G
 bool launch_dslash4_mr(const Cx<float> *U, const Cx<float> *r, Cx<float> *Ar, Geo4 g, double diag, int nvec,
                        double omega, float2 *alpha, double *partials, long long partials_cap, unsigned int *tickets,
                        cudaStream_t s) {
-  if (!pair_takes(U, g) || (long long)pair_ctas(g) * 3 * nvec > partials_cap) return false;
+  if (!pair_takes(g) || !aligned(U, 16) || (long long)pair_ctas(g) * 3 * nvec > partials_cap) return false;
   const MrStep mr{partials, tickets, omega, alpha};
   if (aligned(r, 32) && aligned(Ar, 32))
     launch_pair<true, false, true>(U, r, Ar, g, diag, nullptr, 1.0, 0.0, s, nvec, nullptr, mr);
