@@ -55,13 +55,13 @@ __global__ void __launch_bounds__(256) coarse_apply_kernel(const Cx<R> *__restri
   out[t] = o;
 }
 
-// N = 8: four threads per (site, row), a warp per site (10 of the 40 terms each,
+// N = 8 in FP64: four threads per (site, row), a warp per site (10 of the 40 terms each,
 // combined by shuffles)
-template <typename R>
-__global__ void __launch_bounds__(256) coarse_apply8_kernel(const Cx<R> *__restrict__ Y, const Cx<R> *__restrict__ in,
-                                                            Cx<R> *__restrict__ out, int L0, int L1,
-                                                            const Cx<R> *__restrict__ b, R a, R c, long long ldv,
-                                                            const double *__restrict__ shift) {
+__global__ void __launch_bounds__(256) coarse_apply8_kernel(const Cx<double> *__restrict__ Y,
+                                                            const Cx<double> *__restrict__ in,
+                                                            Cx<double> *__restrict__ out, int L0, int L1,
+                                                            const Cx<double> *__restrict__ b, double a, double c,
+                                                            long long ldv, const double *__restrict__ shift) {
   in += blockIdx.y * ldv;
   out += blockIdx.y * ldv;
   if (b != nullptr) b += blockIdx.y * ldv;
@@ -74,7 +74,7 @@ __global__ void __launch_bounds__(256) coarse_apply8_kernel(const Cx<R> *__restr
   const long long xm0 = rowo + (x0 == 0 ? L0 - 1 : x0 - 1);
   const long long xp1 = (x1 + 1 == L1 ? 0 : rowo + L0) + x0;
   const long long xm1 = (x1 == 0 ? (long long)(L1 - 1) * L0 : rowo - L0) + x0;
-  Cx<R> acc = mk((R)0, (R)0);
+  Cx<double> acc = mk(0.0, 0.0);
 #pragma unroll
   for (int u = 0; u < 10; ++u) {
     const int term = q * 10 + u, dir = term >> 3, col = term & 7;
@@ -89,14 +89,14 @@ __global__ void __launch_bounds__(256) coarse_apply8_kernel(const Cx<R> *__restr
   if (q != 0) return;
   const long long t = j * 8 + row;
   if (shift != nullptr) {
-    const R sv = (R)shift[blockIdx.y];
-    const Cx<R> xt = in[t];
+    const double sv = shift[blockIdx.y];
+    const Cx<double> xt = in[t];
     acc.re = fma(sv, xt.re, acc.re);
     acc.im = fma(sv, xt.im, acc.im);
   }
-  Cx<R> o = mk(a * acc.re, a * acc.im);
+  Cx<double> o = mk(a * acc.re, a * acc.im);
   if (b != nullptr) {
-    const Cx<R> bb = b[t];
+    const Cx<double> bb = b[t];
     o = mk(o.re + c * bb.re, o.im + c * bb.im);
   }
   out[t] = o;
@@ -153,12 +153,13 @@ void launch_coarse_apply(const Cx<R> *Y, const Cx<R> *in, Cx<R> *out, Geo2 g, in
       MG_LAUNCHED();
       return;
     }
+  } else if (N == 8) {
+    coarse_apply8_kernel<<<dim3(grid_for(g.nsites * 32, threads), nvec), threads, 0, s>>>(Y, in, out, g.L0, g.L1, b, a,
+                                                                                         c, ldv, shift);
+    MG_LAUNCHED();
+    return;
   }
-  if (N == 8)
-    coarse_apply8_kernel<R><<<dim3(grid_for(g.nsites * 32, threads), nvec), threads, 0, s>>>(Y, in, out, g.L0, g.L1, b,
-                                                                                            (R)a, (R)c, ldv, shift);
-  else
-    coarse_apply_kernel<R, 0><<<grid, threads, 0, s>>>(Y, in, out, g.L0, g.L1, N, b, (R)a, (R)c, ldv, shift);
+  coarse_apply_kernel<R, 0><<<grid, threads, 0, s>>>(Y, in, out, g.L0, g.L1, N, b, (R)a, (R)c, ldv, shift);
   MG_LAUNCHED();
 }
 

@@ -307,18 +307,6 @@ __device__ __forceinline__ void store_spinor32(Cx<float> *f, int x, const Cx<flo
   }
 }
 
-// h = psi_up - A_mu psi_dn (MINUS, the forward hop's (1 - gamma_mu)) or psi_up + A_mu psi_dn
-template <int MU, bool MINUS>
-__device__ __forceinline__ void project4(const Cx<float> (&p)[12], Cx<float> (&h)[6]) {
-#pragma unroll
-  for (int c = 0; c < 3; ++c) {
-    Cx<float> a0, a1;
-    a_times<float, MU>(p[6 + c], p[9 + c], a0, a1);
-    h[c] = MINUS ? p[c] - a0 : p[c] + a0;
-    h[3 + c] = MINUS ? p[3 + c] - a1 : p[3 + c] + a1;
-  }
-}
-
 // t = U h (DAG false) or U^dagger h, for both spin rows of h
 template <bool DAG>
 __device__ __forceinline__ void link_times4(const Cx<float> (&u)[9], const Cx<float> (&h)[6], Cx<float> (&t)[6]) {
@@ -435,14 +423,14 @@ __device__ __forceinline__ void row_hops(const Cx<float> (&p)[12], const Cx<floa
     e[c] = mk(fmaf(sg, a0.re, q[c].re), fmaf(sg, a0.im, q[c].im));
     e[3 + c] = mk(fmaf(sg, a1.re, q[3 + c].re), fmaf(sg, a1.im, q[3 + c].im));
   }
-  project4<MU, true>(p, h);
+  hop_project<float, MU, true>(p, h);
 #pragma unroll
   for (int i = 0; i < 6; ++i) h[i] = mk(first ? e[i].re : h[i].re, first ? e[i].im : h[i].im);
   rotate6(h, fsrc, t);
   staged_link<MU, U16>(own + link_unit<U16>(MU), u);
   link_times4<false>(u, t, h);
   reconstruct4<MU, true>(h, acc);
-  project4<MU, false>(p, h);
+  hop_project<float, MU, false>(p, h);
 #pragma unroll
   for (int i = 0; i < 6; ++i) h[i] = mk(last ? e[i].re : h[i].re, last ? e[i].im : h[i].im);
   staged_link<MU, U16>(last ? face : own + link_unit<U16>(MU), u);
@@ -573,17 +561,17 @@ __global__ void __launch_bounds__(32 * kTiles, 2)
       {  // direction 3: the neighbours inside the tile are the lane's own two sites
         Cx<float> h[6], t[6], t2[6], u[9];
         staged_link<3, U16>(recA + link_unit<U16>(3), u);
-        project4<3, true>(pB, h);
+        hop_project<float, 3, true>(pB, h);
         link_times4<false>(u, h, t);
         reconstruct4<3, true>(t, aA);
-        project4<3, false>(pA, h);
+        hop_project<float, 3, false>(pA, h);
         link_times4<true>(u, h, t);
         staged_link<3, U16>(hT, u);
-        project4<3, false>(nA, h);
+        hop_project<float, 3, false>(nA, h);
         link_times4<true>(u, h, t2);
         reconstruct4<3, false>(t2, aA);
         staged_link<3, U16>(recB + link_unit<U16>(3), u);
-        project4<3, true>(nB, h);
+        hop_project<float, 3, true>(nB, h);
         link_times4<false>(u, h, t2);
         reconstruct4<3, true>(t2, aB);
         reconstruct4<3, false>(t, aB);

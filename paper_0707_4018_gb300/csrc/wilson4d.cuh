@@ -96,20 +96,20 @@ __device__ __forceinline__ void hop_dispatch(int hop, const Cx<R> (&p)[12], cons
 
 // h = psi_up - A_mu psi_dn (MINUS, the forward hop's (1 - gamma_mu)) or psi_up + A_mu psi_dn
 template <typename R, int MU, bool MINUS>
-__device__ __forceinline__ void hop_project(const Cx<R> (&p)[12], Cx<R> (&h)[2][3]) {
+__device__ __forceinline__ void hop_project(const Cx<R> (&p)[12], Cx<R> (&h)[6]) {
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
     Cx<R> a0, a1;
     a_times<R, MU>(p[6 + c], p[9 + c], a0, a1);
-    h[0][c] = MINUS ? p[c] - a0 : p[c] + a0;
-    h[1][c] = MINUS ? p[3 + c] - a1 : p[3 + c] + a1;
+    h[c] = MINUS ? p[c] - a0 : p[c] + a0;
+    h[3 + c] = MINUS ? p[3 + c] - a1 : p[3 + c] + a1;
   }
 }
 
 // forward hop of direction MU: t = U (1 - gamma_mu) psi_{x+mu}, upper half
 template <typename R, int MU>
 __device__ __forceinline__ void hop_fwd(const Cx<R> (&p)[12], const Cx<R> *link, Cx<R> (&t)[2][3]) {
-  Cx<R> h[2][3];
+  Cx<R> h[6];
   hop_project<R, MU, true>(p, h);
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
@@ -118,8 +118,8 @@ __device__ __forceinline__ void hop_fwd(const Cx<R> (&p)[12], const Cx<R> *link,
 #pragma unroll
     for (int b = 0; b < 3; ++b) {
       const Cx<R> u = link[a * 3 + b];  // U_ab
-      cmac(t[0][a], u, h[0][b]);
-      cmac(t[1][a], u, h[1][b]);
+      cmac(t[0][a], u, h[b]);
+      cmac(t[1][a], u, h[3 + b]);
     }
   }
 }
@@ -131,7 +131,7 @@ __device__ __forceinline__ void hop_fwd(const Cx<R> (&p)[12], const Cx<R> *link,
 template <typename R, int MU>
 __device__ __forceinline__ void hop_bwd(const Cx<R> (&p)[12], const Cx<R> *link, const Cx<R> (&t)[2][3],
                                         Cx<R> (&acc)[12]) {
-  Cx<R> h[2][3];
+  Cx<R> h[6];
   hop_project<R, MU, false>(p, h);
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
@@ -139,8 +139,8 @@ __device__ __forceinline__ void hop_bwd(const Cx<R> (&p)[12], const Cx<R> *link,
 #pragma unroll
     for (int b = 0; b < 3; ++b) {
       const Cx<R> u = link[b * 3 + a];  // (U^dagger)_ab = conj(U_ba)
-      cmac_conj(s0, u, h[0][b]);
-      cmac_conj(s1, u, h[1][b]);
+      cmac_conj(s0, u, h[b]);
+      cmac_conj(s1, u, h[3 + b]);
     }
     const R m2 = (R)-2;
     const Cx<R> d0 = mk(fma(m2, t[0][a].re, s0.re), fma(m2, t[0][a].im, s0.im));
