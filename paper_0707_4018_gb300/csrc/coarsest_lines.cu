@@ -42,6 +42,7 @@ namespace mg {
 namespace {
 
 constexpr int kT = 16;                // tile edge
+constexpr int kGridY = 65535;         // lines or products of one launch: the most that a grid's second extent takes
 constexpr double kBackward = 2e-15;   // largest accepted |b - A x| / (|A| |x| + |b|), entry by entry
 
 // position of dof i of line p in a level-0 vector (site-major); compact levels: axis 1
@@ -54,14 +55,14 @@ struct LineMap {
   }
 };
 
-// blocks of the finest ring from the stencil: which = 0 (self), 1 (next line), 2 (previous line)
+// blocks of the finest ring's lines p0, p0 + 1, ... from the stencil: which = 0 (self), 1 (next line), 2 (previous line)
 __global__ void line_blocks_kernel(const Cx<double> *__restrict__ Y, Cx<double> *__restrict__ D,
                                    Cx<double> *__restrict__ R, Cx<double> *__restrict__ L, int L0, int L1, int N,
-                                   int axis, int Q, int b, bool nine, double shift) {
+                                   int axis, int Q, int b, int p0, bool nine, double shift) {
   const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   if (t >= (long long)b * b) return;
   const int i = (int)(t / b), k = (int)(t - (long long)i * b);
-  const int p = blockIdx.y, which = blockIdx.z;
+  const int p = p0 + blockIdx.y, which = blockIdx.z;
   const int q = i / N, a = i - q * N, qq = k / N, c = k - qq * N;
   const long long j = axis == 1 ? (long long)q + (long long)L0 * p : (long long)p + (long long)L0 * q;
   Cx<double> v = mk(0.0, 0.0);
@@ -536,10 +537,21 @@ void line_inverse(LineSolver &f, const Cx<double> *src, long long stride, int co
   MG_LAUNCHED();
   for (int k = 0; k < nt; ++k) {
     Cx<double> *dst = (nt - 1 - k) % 2 == 0 ? Dinv : f.tmp.p;
-    gj_step_kernel<<<dim3(nt * nt, count), kT * kT, 0, s>>>(src, stride, dst, b2, b, k, f.pinv.p, f.info.p);
-    MG_LAUNCHED();
+    for (int c = 0; c < count; c += kGridY) {
+      gj_step_kernel<<<dim3(nt * nt, std::min(count - c, kGridY)), kT * kT, 0, s>>>(
+          src + c * stride, stride, dst + c * b2, b2, b, k, f.pinv.p + (long long)c * 2 * kT * kT, f.info.p);
+      MG_LAUNCHED();
+    }
     src = dst;
     stride = b2;
+  }
+}
+
+void line_products(const LineSolver &f, long long first, int count, cudaStream_t s) {
+  const int nt = (f.b + kT - 1) / kT;
+  for (int c = 0; c < count; c += kGridY) {
+    line_product_kernel<<<dim3(nt * nt, std::min(count - c, kGridY)), kT * kT, 0, s>>>(f.jobs_dev.p + first + c, f.b);
+    MG_LAUNCHED();
   }
 }
 
@@ -594,10 +606,11 @@ bool line_try(LineSolver &f, const Cx<double> *Y, bool nine, double shift, Cx<do
   MG_CUDA(cudaMemsetAsync(f.info.p, 0, sizeof(int), s));
   MG_CUDA(cudaMemsetAsync(f.berr.p, 0, sizeof(double), s));
   LineLevel &t = f.lv[0];
-  line_blocks_kernel<<<dim3(grid_for(b2, 256), t.r, 3), 256, 0, s>>>(Y, t.D, t.R, t.L, f.L0, f.L1, f.N, f.axis, f.Q,
-                                                                     f.b, nine, shift);
-  MG_LAUNCHED();
-  const int nt = (f.b + kT - 1) / kT;
+  for (int p = 0; p < t.r; p += kGridY) {
+    line_blocks_kernel<<<dim3(grid_for(b2, 256), std::min(t.r - p, kGridY), 3), 256, 0, s>>>(
+        Y, t.D, t.R, t.L, f.L0, f.L1, f.N, f.axis, f.Q, f.b, p, nine, shift);
+    MG_LAUNCHED();
+  }
   for (size_t k = 0; k < f.lv.size(); ++k) {
     LineLevel &l = f.lv[k];
     if (l.r == 1) {
@@ -605,10 +618,8 @@ bool line_try(LineSolver &f, const Cx<double> *Y, bool nine, double shift, Cx<do
       break;
     }
     line_inverse(f, l.D + b2, 2 * b2, l.E, l.Dinv, s);
-    line_product_kernel<<<dim3(nt * nt, l.n_w), kT * kT, 0, s>>>(f.jobs_dev.p + l.w_jobs, f.b);
-    MG_LAUNCHED();
-    line_product_kernel<<<dim3(nt * nt, l.n_u), kT * kT, 0, s>>>(f.jobs_dev.p + l.u_jobs, f.b);
-    MG_LAUNCHED();
+    line_products(f, l.w_jobs, l.n_w, s);
+    line_products(f, l.u_jobs, l.n_u, s);
   }
   check_vector_kernel<<<grid_for(f.n, 256), 256, 0, s>>>(f.chk.p, f.n);
   MG_LAUNCHED();

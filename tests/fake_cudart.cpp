@@ -31,7 +31,9 @@ template <typename T>
 T arg(void **args, int i) {
   return *static_cast<T *>(args[i]);
 }
-cudaError_t launched(const void *f, void **args) {
+cudaError_t launched(const void *f, dim3 g, void **args) {
+  if (g.x == 0 || g.y == 0 || g.z == 0 || g.x > 0x7fffffffu || g.y > 65535 || g.z > 65535)
+    return error = cudaErrorInvalidConfiguration;
   const std::string &n = names()[f];
   auto has = [&](const char *s) { return n.find(s) != std::string::npos; };
   if (has("line_product_kernel")) used(arg<void *>(args, 0), 1);
@@ -181,11 +183,13 @@ cudaError_t __cudaPopCallConfiguration(dim3 *g, dim3 *b, size_t *smem, void *s) 
 cudaError_t __cudaGetKernel(cudaKernel_t *k, const void *f) {
   return *k = reinterpret_cast<cudaKernel_t>(const_cast<void *>(f)), cudaSuccess;
 }
-cudaError_t __cudaLaunchKernel(cudaKernel_t k, dim3, dim3, void **args, size_t, cudaStream_t) {
-  return launched(k, args);
+cudaError_t __cudaLaunchKernel(cudaKernel_t k, dim3 g, dim3, void **args, size_t, cudaStream_t) {
+  return launched(k, g, args);
 }
-cudaError_t cudaLaunchKernel(const void *f, dim3, dim3, void **args, size_t, cudaStream_t) { return launched(f, args); }
-cudaError_t cudaLaunchCooperativeKernel(const void *f, dim3, dim3, void **args, size_t, cudaStream_t) {
-  return launched(f, args);
+cudaError_t cudaLaunchKernel(const void *f, dim3 g, dim3, void **args, size_t, cudaStream_t) {
+  return launched(f, g, args);
+}
+cudaError_t cudaLaunchCooperativeKernel(const void *f, dim3 g, dim3, void **args, size_t, cudaStream_t) {
+  return launched(f, g, args);
 }
 }

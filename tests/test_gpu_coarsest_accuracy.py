@@ -32,3 +32,24 @@ def test_backward_error_of_the_exact_coarsest_solve(ext, N, m):
         r = np.abs(rhs - (A.astype(np.clongdouble) @ got.astype(np.clongdouble)))
         assert (r <= TOL * (np.abs(A) @ np.abs(got) + np.abs(rhs))).all()
     ctx.close()
+
+
+def test_a_ring_of_more_lines_than_a_grid_has_rows():
+    # a coarse lattice of 1 x 70000 sites with two dofs each
+    import torch
+    import paper_0707_4018_gb300 as mg
+    dims, n, N = (2, 140000), 70000, 2
+    p = mg.mg_default_params(levels=2, blocks=[(2, 2)], Nv=[N], n_pass=1, nu_setup=2, coarsest_lu_max=n * N)
+    ctx = mg.Context.setup(to_dev(inputs.hot_links(*dims, seed=19)), 0.1, dims, p)
+    Y = to_host(ctx.coarse_op(1))
+    b = inputs.gaussian_spinor(n, N, 44, 0)
+    x = torch.empty((n, N), dtype=torch.complex128, device="cuda")
+    ctx.coarsest_solve(to_dev(b), x)
+    x = to_host(x)
+    r, size = b.astype(np.clongdouble), np.abs(b)
+    for d, o in enumerate((0, 0, 0, 1, -1)):  # both hops along the extent of one lead back to the site
+        v = np.roll(x, -o, 0)
+        r = r - np.einsum("jab,jb->ja", Y[:, d].astype(np.clongdouble), v.astype(np.clongdouble))
+        size = size + np.einsum("jab,jb->ja", np.abs(Y[:, d]), np.abs(v))
+    assert (np.abs(r) <= TOL * size).all()
+    ctx.close()

@@ -38,15 +38,17 @@ def _at(a):
 
 
 class Ctx:
-    def __init__(self, lib, max_rhs):
+    def __init__(self, lib, max_rhs, dims=DIMS, **params):
         self.lib, self.p = lib, ctypes.c_void_p()
         p = binding.mg_params()
         lib.mg_default_params(ctypes.byref(p))
         p.block[0][0] = p.block[0][1] = 2
         p.Nv[0], p.n_pass, p.max_rhs, p.max_iter = 4, 1, max_rhs, 2
-        self.U = np.zeros((DIMS[0] * DIMS[1], 2), dtype=np.complex128)
-        self.v = np.zeros((4, DIMS[0] * DIMS[1], 2), dtype=np.complex128)
-        rc = lib.mg_setup(ctypes.byref(self.p), ctypes.byref(binding.make_geom(DIMS)), _at(self.U),
+        for k, v in params.items():
+            setattr(p, k, v)
+        self.U = np.zeros((dims[0] * dims[1], 2), dtype=np.complex128)
+        self.v = np.zeros((4, dims[0] * dims[1], 2), dtype=np.complex128)
+        rc = lib.mg_setup(ctypes.byref(self.p), ctypes.byref(binding.make_geom(dims)), _at(self.U),
                           ctypes.c_double(0.1), ctypes.byref(p), None)
         assert rc == 0, lib.mg_last_error()
 
@@ -181,4 +183,11 @@ def test_a_failed_factorisation_is_not_taken_for_the_one_before(lib):
     checks = lib.fake_checks()
     assert ctx.batch(0.2, 0.3) == NOT_CONVERGED
     assert lib.fake_checks() == checks + 1  # the first slot's factors were overwritten, the second's were not
+    ctx.close()
+
+
+def test_a_ring_of_more_lines_than_a_grid_has_rows(lib):
+    # a coarse lattice of 1 x 70000 sites: more lines, and products of them, than the second extent of a grid takes
+    ctx = Ctx(lib, 1, dims=(2, 140000), nu_setup=1, nu_pre=1, nu_post=1, coarsest_lu_max=300000)
+    assert ctx.vcycle() == 0
     ctx.close()
