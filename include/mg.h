@@ -95,7 +95,7 @@ typedef struct {
   int nu_setup;                     /* MR iterations of the null-space relaxation (paper: Eq. relax) */
   int gcr_restart;                  /* outer flexible GCR restart length */
   int max_iter;                     /* outer iteration limit */
-  int coarsest_lu_max;              /* coarsest dimension up to which a dense LU is used */
+  int coarsest_lu_max;              /* coarsest dimension up to which the coarsest level is factored */
   double coarsest_tol;              /* relative residual of the iterative coarsest solve */
   int coarsest_restart;             /* restart length of the iterative coarsest solve (1..32) */
   int coarsest_max_iter;            /* iteration limit of the iterative coarsest solve */
@@ -127,7 +127,7 @@ typedef struct {
 typedef struct mg_ctx mg_ctx;
 
 /* Defaults: 2 levels, 4x4 blocks, Nv = 8, MR 4 + 4 with omega = 0.8, 5 passes,
- * nu_setup = 8, GCR(16), max_iter 500, coarsest LU up to 2048, coarsest GCR
+ * nu_setup = 8, GCR(16), max_iter 500, coarsest factorisation up to 2048, coarsest GCR
  * tol 1e-12 / restart 16 / 20000 iterations, FP64, seed 20070704, max_rhs 1. */
 void mg_default_params(mg_params *p);
 
@@ -305,10 +305,12 @@ int mg_prolong(mg_ctx *ctx, int level, const void *coarse, void *fine);
 int mg_vcycle(mg_ctx *ctx, const void *b, void *x);
 
 /* One coarsest-level solve x = A_c^{-1} b (paper: the coarsest level of the
- * V-cycle is an exact solve), FP64, coarsest-level layout [site][a]: dense LU
- * when the coarsest dimension is <= coarsest_lu_max, else the persistent GCR
+ * V-cycle is an exact solve), FP64, coarsest-level layout [site][a]: direct when
+ * the coarsest dimension is <= coarsest_lu_max (cyclic reduction over lattice
+ * lines, or dense LU where that is less accurate), else the persistent GCR
  * kernel to relative residual coarsest_tol. iters (may be NULL): iterations of
- * the iterative solve (0 for LU). ms (may be NULL): device time of the solve,
+ * the iterative solve (0 for the direct one). MG_ERR_STATE when the last
+ * factorisation (mg_update_mass) failed. ms (may be NULL): device time of the solve,
  * from CUDA events recorded on the context's stream around it. */
 int mg_coarsest_solve(mg_ctx *ctx, const void *b, void *x, long long *iters, double *ms);
 
@@ -450,8 +452,8 @@ int mg_convergence_rate(mg_ctx *ctx, int steps, uint64_t seed, double *rate);
  * level by level); the coarse operators P^dagger A P are 9-point stencils (D^dagger D reaches the
  * diagonal neighbours); every non-coarsest level relaxes with the degree-2 MR polynomial whose
  * coefficients come from two MR steps (omega) on a fixed Philox vector and are then held fixed, so
- * R = R^dagger and the V-cycle is hermitian; the coarsest level is solved by dense LU (at most 4096
- * dofs). All arithmetic is FP64.
+ * R = R^dagger and the V-cycle is hermitian; the coarsest level (at most 4096 dofs) is solved
+ * directly, as in mg_coarsest_solve. All arithmetic is FP64.
  *   mg_cg_setup: g (d = 2, Nc = 1), U device complex128 [x][mu] (copied), mass m, parameters p
  *     (levels, block, Nv, n_pass, nu_setup, omega and seed are used; blocks at least 2 x 2, and
  *     every coarse extent at least 3). Errors: INVALID_ARG, UNSUPPORTED, OOM, CUDA, NAN.

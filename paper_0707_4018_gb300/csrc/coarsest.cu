@@ -358,11 +358,14 @@ __global__ void __launch_bounds__(256) coarsest_gcr_kernel(CgArgs<VT> a) {
 // per site with 16-byte loads, the next site's blocks requested while one is summed (stencil8.cuh),
 // the vector work by a thread per dof. Gram-Schmidt is classical in one pass, with a second one only
 // where |w'|^2 < |w|^2 / 2 (every CTA decides from the same sums), so an iteration is one grid sum
-// and one barrier; every sum is FP64.
-// With FP32 sums inside the warps (the form the figures below are of) a 1024 x 768 solve takes 3 ms less, but loses the precision.
-// The thread-per-row form on a quarter of the SMs, two passes always, took 563 us per solve at 98304
-// dofs (1024 x 768 fine lattice), this one 200 us (a whole fine solve 81.5 -> 64.5 ms; on half or a
-// quarter of the SMs 65.9 and 68.6 ms).
+// and one barrier. An element's two products of a part are added in FP32, every other sum is FP64.
+// At 98304 dofs (1024 x 768 fine lattice) a solve takes 207 us; a thread per row on a quarter of the SMs
+// with two passes always took 563. Every SM is the best grid for one context and for several whose solves
+// share the chip, and for the thread-per-row form that other N run (fine solves in ms on all, half and a
+// quarter of the SMs):
+//   1024 x 768, N = 8: one context 47.9, 49.9, 54.9; three in one launch 144, 150, 165
+//   512 x 512, N = 8: one 23.5, 24.2, 25.7; three 69.9, 72.0, 76.8
+//   N = 6: 1024 x 768 76.5, 83.8, 97.6; 512 x 512 37.1, 40.4, 43.8
 // ---------------------------------------------------------------------------
 constexpr int kGcr8Warps = 16;
 

@@ -457,7 +457,7 @@ static GcrOut outer_fgcr(mg_ctx &c, const Cx<double> *b, Cx<double> *x, double t
   return out;
 }
 
-// exact solve on the coarsest level (FP64): dense LU or GCR to coarsest_tol. Slot 0 holds
+// exact solve on the coarsest level (FP64): direct (coarsest_lines.h) or GCR to coarsest_tol. Slot 0 holds
 // the factors / preconditioner at the context mass, slot 1 + v those of batched vector v.
 static void coarsest_solve64(mg_ctx &c, const Cx<double> *b, Cx<double> *x, int slot = 0) {
   const int l = c.p.levels - 1;

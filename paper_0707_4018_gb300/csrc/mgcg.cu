@@ -297,7 +297,7 @@ static void cg_build(CgEngine &e, int l) {
 }
 
 // frozen smoother coefficients of every non-coarsest level (two MR steps on A x = b_l from 0,
-// b_l Philox vector 0x2C of level l) and the LU factors of the coarsest level
+// b_l Philox vector 0x2C of level l) and the factors of the coarsest level
 static void cg_prepare(CgEngine &e) {
   for (int l = 0; l + 1 < (int)e.lv.size(); ++l) {
     CgLevel &L = e.lv[l];
@@ -360,7 +360,7 @@ static std::unique_ptr<CgEngine> cg_create(const mg_geom *g, const void *U, doub
     }
   }
   const long long nc = e->lv.back().n;
-  if (nc > 4096) fail(MG_ERR_UNSUPPORTED, "MG-CG: the coarsest level is solved by dense LU (at most 4096 dofs)");
+  if (nc > 4096) fail(MG_ERR_UNSUPPORTED, "MG-CG: the coarsest level is solved directly (at most 4096 dofs)");
   e->lu_work.alloc((size_t)line_work_size(e->lv.back().geo, e->lv.back().nint));
   const long long nf = e->lv[0].n;
   e->U.alloc((size_t)e->lv[0].geo.nsites * 2);

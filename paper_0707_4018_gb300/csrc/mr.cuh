@@ -35,8 +35,10 @@ __device__ __forceinline__ void block_reduce(T (&v)[NOUT], T *sh) {
 // Blocks of one MR launch per vector; a block strides over the rest of a larger lattice. Every block of
 // the next launch sums all of a vector's partials, so one block per 256 units would make that sum
 // quadratic in the lattice: at 1024 x 768 it was 60 to 75 % of an iteration (level 0: 45 us with it,
-// 11 without; level 1: 121 and 47). Up to 1216 partials (5 loads per thread) it is small beside the
-// rest: a solve there took 122 ms without the cap, 100 with it, 108 / 112 / 111 with 608 / 304 / 2432.
+// 11 without; level 1: 121 and 47). Up to 1216 partials (5 loads per thread) it is small beside the rest.
+// Solves in ms with 304 / 608 / 1216 / 2432 / 4864 blocks: 512 x 512 20.1 / 20.1 / 22.4 / 24.3 / 24.3,
+// 1024 x 768 46.7 / 43.0 / 44.0 / 51.4 / 64.3, 2048 x 1024 111 / 99.0 / 97.7 / 107 / 136; four sources at
+// 1024 x 768 199 / 202 / 211 / 243 / 276.
 constexpr int kMrGrid = 1216;
 inline int mr_blocks(long long full) { return (int)(full < kMrGrid ? full : kMrGrid); }
 

@@ -259,7 +259,7 @@ __global__ void __launch_bounds__(32 * DSLASH4_WARPS, sizeof(R) == 4 ? 5 : 2) ds
 // warp twice the loads in flight, and a direction's outside spinors are requested while the one
 // before it is worked on: with so few warps the loads' latency is what bounds it (L1 path 40 % busy,
 // issue slots 40 %). 32^3 x 64: 250 us (4.0 TB/s), the one-site form 353 us. 24 vectors on 16^3 x 32
-// with the MR step (mr_step_batch_kernel): 525 us, before 850 us; without the early requests and with
+// with the MR step (mr_step_batch_kernel): 528 us, before 836 us; without the early requests and with
 // the sums met in a block reduction per vector 691 us; with the step applied while r is read (6
 // vector passes, not 7) 677 us, the doubled face loads costing what the pass saves; 12 warps of 168
 // registers sharing the staged links 718 us.

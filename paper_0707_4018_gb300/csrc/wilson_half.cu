@@ -138,10 +138,10 @@ __device__ __forceinline__ uint2 pack_site(const Pair<float> &p, float &nu) {
   return raw;
 }
 
-// One site per thread: rows of odd length (a pair of sites is then aligned in every second row only) and
-// fields that are not 16-byte aligned. Rows x1 +- 1 are x +- L0 in the linear index, modulo the volume.
-// Instruction issue bounds it, not HBM: 3071 x 2049 in 46.1 us (4365 GB/s), 47.1 before with the norms applied
-// to whole spinors and two-dimensional neighbour indices.
+// One site per thread: rows of odd length (a pair of sites has its own words aligned then, but not those of the
+// rows x1 +- 1, x +- L0 in the linear index modulo the volume) and fields that are not 16-byte aligned.
+// Instruction issue bounds it, not HBM: 3071 x 2049 in 46.2 us (4.36 TB/s). Norms applied to the projected half
+// spinors and linear neighbour indices brought it there from 47.1.
 __global__ void __launch_bounds__(256, 8) dslash_half_kernel(const __half2 *__restrict__ U,
                                                              const __half2 *__restrict__ in,
                                                              const float *__restrict__ in_nrm,
